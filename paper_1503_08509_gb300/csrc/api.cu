@@ -599,7 +599,7 @@ int fep3m_create(const fep3m_config* cfg, void* stream, fep3m_ctx** out) {
       (e = cudaEventCreateWithFlags(&c->ev_join2, cudaEventDisableTiming)) != cudaSuccess)
     return fail(from_cuda(e));
   if (box) {
-    if ((st = box_create(c, cfg->n_el, (cfg->flags & FEP3M_NEUMANN) != 0)) != FEP3M_OK) return fail(st);
+    if ((st = box_create(c, cfg->n_el, (cfg->flags & FEP3M_NEUMANN) != 0, Hw.data())) != FEP3M_OK) return fail(st);
   } else {
     // the forward solver also pairs the forward and adjoint right-hand sides (tensor-core
     // fast diagonalisation); the second solver serves the multigrid path and fep3m_vjp
@@ -656,6 +656,10 @@ int fep3m_set_particles(fep3m_ctx* c, int64_t N, const double* pos, const double
   if (flag) return FEP3M_EINVAL;
   if (!c->box && !(c->cfg.flags & FEP3M_NEUTRALIZE) && std::fabs(sums[0]) > 1e-12 * sums[1])
     return FEP3M_ENOTNEUTRAL;
+  // within 2^-100 .. 2^100, so that the scale is exact and finite in FP32 too
+  c->q_scale = sums[1] > 0 && std::isfinite(sums[1])
+                   ? std::ldexp(1.0, std::max(-100, std::min(100, -std::ilogb(sums[1] / (double)N))))
+                   : 1.0;
   c->have_particles = true;
   if (c->timing) c->stats.ms_bin = ev_ms(c, 6, 7);
   return FEP3M_OK;

@@ -19,8 +19,8 @@
 //     charges' screens outside the box are not loads of the box problem;
 //   boundary values: h (g - Phi^sr) at each boundary node, from the singular
 //     sum over the node's block and the screen field at the node (the
-//     vertex-regrouped contraction of the pair kernel for the node's element,
-//     in FP64), one CTA per boundary element;
+//     vertex-regrouped contraction of the pair kernel for the node's element),
+//     in double-float arithmetic, one CTA per boundary element;
 //   Neumann load: s at the face nodes, per face element by a tensor
 //     Gauss-Legendre rule (BOX_NGL points per axis) of g less the normal
 //     derivative of Phi^sr (singular sum over the point's block and the
@@ -30,7 +30,8 @@
 //     boundary values fixed (Dirichlet), or K phi = b + s less its component
 //     along the node integrals (the constant null space) on all (3 nb + 1)^3
 //     nodes with int phi = 0 (Neumann), by iterative refinement: the residual
-//     in FP64 (separable banded passes over the whole node grid), the
+//     in FP64 or, mixed, double-float arithmetic (the periodic solver's fused
+//     apply on the open node grid), the
 //     correction by the FP32 fast-diagonalisation solve of the solved nodes
 //     with the box eigenbasis (Dirichlet: no null mode; the periodic solve's
 //     transform passes, on the tensor cores unless FEP3M_CUDA_CORES);
@@ -39,9 +40,11 @@
 // Mesh values are in element units (h Phi), as on the periodic path.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
+#include "df.cuh"
 
 namespace fep3m {
 
@@ -106,95 +109,251 @@ __global__ void k_box_load_axis(int nb, int axis, int d0, int d1, int d2, int64_
   out[g] = (Tout)(scale * (double)acc);
 }
 
+// Short-range part at the boundary.  Both kernels below take one CTA of BT
+// threads per boundary (or face) element and work on its block, the elements
+// within n_sr of it that lie in the box: the block's charges are staged in
+// shared memory a chunk at a time (a row of the block along x is one
+// contiguous run of sorted charges), and the sums run in double-float
+// arithmetic on the FP32 pipes (df.cuh) with FP64 totals.  The charges are
+// scaled by a power of two near the inverse of their mean magnitude, so that
+// the pairs' low words stay normal FP32 numbers whatever the charges' unit.
+constexpr int BROWS = 81;   // rows (y, z) of a block, n_sr <= 4
+
+// a thread's running sum: a pair, on the FP64 path three floats
+template <class T> struct Sum {
+  typedef typename std::conditional<sizeof(T) == 4, df, tf>::type type;
+};
+
+__device__ __forceinline__ void negate(df& s) { s = {-s.h, -s.l}; }
+__device__ __forceinline__ void negate(tf& s) { s = {-s.h, -s.m, -s.l}; }
+// s += a, running sums of two threads
+__device__ __forceinline__ void add_part(df& s, df a) { s = df_add(s, a); }
+__device__ __forceinline__ void add_part(tf& s, tf a) {
+  const df t = df_two_sum(s.h, a.h), u = df_two_sum(s.m, a.m), w = df_two_sum(t.l, u.h);
+  s.h = t.h;
+  s.m = w.h;
+  s.l += a.l + (w.l + u.l);
+}
+
+// the runs of the block's rows: j0[r] the first sorted charge of row r, pre[r]
+// the charges of the rows before it; returns their number.  By the CTA.
+__device__ int block_rows(int n, int nb, int n_sr, const int E[3], const int* __restrict__ start, int* j0, int* pre) {
+  const int nbk = 2 * n_sr + 1, nrow = nbk * nbk;
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    const int x0 = max(E[0] - n_sr, 0), x1 = min(E[0] + n_sr, nb - 1);
+    int carry = 0;
+    for (int base = 0; base < nrow; base += 32) {
+      const int r = base + lane;
+      int first = 0, cnt = 0;
+      if (r < nrow) {
+        const int y = E[1] + r % nbk - n_sr, z = E[2] + r / nbk - n_sr;
+        if (y >= 0 && z >= 0 && y < nb && z < nb) {
+          // x1 + 1 <= nb is an element of the padded row: its start ends the run
+          const int64_t row = (int64_t)n * (y + (int64_t)n * z);
+          first = start[row + x0];
+          cnt = start[row + x1 + 1] - first;
+        }
+      }
+      int x = cnt;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += v;
+      }
+      if (r < nrow) {
+        j0[r] = first;
+        pre[r] = carry + x - cnt;
+      }
+      carry += __shfl_sync(0xffffffffu, x, 31);
+    }
+    if (lane == 0) pre[nrow] = carry;
+  }
+  __syncthreads();
+  return pre[nrow];
+}
+
+// sorted index of the block's charge s (0 <= s < pre[nrow])
+__device__ __forceinline__ int block_charge(int s, int nrow, const int* j0, const int* pre) {
+  int lo = 0, hi = nrow;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (pre[mid] <= s) lo = mid;
+    else hi = mid;
+  }
+  return j0[lo] + (s - pre[lo]);
+}
+
+// Vertex amplitudes of element E's block as pairs: A[o] = the corner terms
+// C[v - k][k] at vertex v = E - o of the block's elements, times scale
+template <class T>
+__device__ void block_amplitudes(int n, int n_sr, const int E[3], T scale, const T* __restrict__ Cv, df* A) {
+  const int keep = n_sr + 1, noff = 2 * n_sr + 2, no3 = noff * noff * noff;
+  for (int o = threadIdx.x; o < no3; o += BT) {
+    const int ox = o % noff - keep, oy = (o / noff) % noff - keep, oz = o / (noff * noff) - keep;
+    const int64_t v = wrapb(E[0] - ox, n) + (int64_t)n * (wrapb(E[1] - oy, n) + (int64_t)n * wrapb(E[2] - oz, n));
+    // the corner's element v - k is in the block: |o + k| <= n_sr per axis
+    const unsigned mx = ox == -keep ? 0xAAu : (ox == n_sr ? 0x55u : 0xFFu);
+    const unsigned my = oy == -keep ? 0xCCu : (oy == n_sr ? 0x33u : 0xFFu);
+    const unsigned mz = oz == -keep ? 0xF0u : (oz == n_sr ? 0x0Fu : 0xFFu);
+    const unsigned mask = mx & my & mz;
+    typedef typename vec4<T>::type V4;
+    const V4 a = reinterpret_cast<const V4*>(Cv + 8 * v)[0], b = reinterpret_cast<const V4*>(Cv + 8 * v)[1];
+    const T c[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    if constexpr (sizeof(T) == 4) {
+      df s = {0.f, 0.f};
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const df t = df_two_sum(s.h, ((mask >> k) & 1u) ? c[k] * scale : 0.f);
+        s = {t.h, s.l + t.l};
+      }
+      A[o] = s;
+    } else {
+      double s = 0.0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) s += ((mask >> k) & 1u) ? c[k] : 0.0;
+      A[o] = df_split(s * scale);
+    }
+  }
+}
+
 // Boundary values of the mesh problem (Eq. bcadjust), element units:
 //   phi[node] = h g[node] - sum_{j in block} Q_j / |x_node - x_j| (element
 //   units) + sum_o A_e(o) H(o, m),
 // the last term the screen field of the block's charges at node m of the
-// node's element e (H the absolute FP64 vertex table [offset][node], A_e(o)
-// the vertex amplitudes: the corner terms C[v - k][k] at vertex v = e - o of
-// the block's elements).  One CTA (128 threads) per boundary element; the
-// element writes the boundary nodes it owns (per axis local nodes 0 .. 2, and
-// 3 on the last element: the binning rule min(i / 3, nb - 1)), one warp per
-// node.  A charge at a boundary node makes that node's value infinite.
-//
-// The screen field of element E's block at E's 64 nodes, sum_o A_E(o) H(o, m),
-// into G[0 .. 63] (element units), by a CTA of 128 threads; A: noff^3 + 128
-// doubles of shared scratch.  Ends with a barrier.
+// node's element e (Hdf the absolute vertex table [offset][node] as pairs).
+// The element writes the boundary nodes it owns (per axis local nodes 0 .. 2,
+// and 3 on the last element: the binning rule min(i / 3, nb - 1)): 9 on a
+// face element, up to 37 at a corner.  Thread (k, part) sums node k over the
+// charges and the offsets part, part + nparts, ...: with M nodes, nparts =
+// BT / M, so nearly all threads work whatever M is.  A charge at a boundary
+// node makes that node's value infinite.  Bound by FP32 issue (about 80
+// operations per node and charge, 11 per node and offset); rock salt in a
+// 32^3 box: 1722 -> 132 us against FP64 sums with one lane per block element.
+constexpr int BCH = 256;    // charges staged at once
+struct BoxSrc {             // a staged charge at its largest (FP64 positions)
+  tf x[3];
+  df q;
+};
 template <class T>
-__device__ void element_screen_field(int n, int n_sr, const int E[3], const T* __restrict__ Cv,
-                                     const double* __restrict__ Hw, double* A, double* G) {
-  const int keep = n_sr + 1, noff = 2 * n_sr + 2, no3 = noff * noff * noff;
-  const int tid = threadIdx.x;
-  for (int o = tid; o < no3; o += blockDim.x) {
-    const int oa[3] = {o % noff - keep, (o / noff) % noff - keep, o / (noff * noff) - keep};
-    const int64_t v = wrapb(E[0] - oa[0], n) + (int64_t)n * (wrapb(E[1] - oa[1], n) + (int64_t)n * wrapb(E[2] - oa[2], n));
-    double a = 0.0;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      // the corner's element v - k is in the block: |e - (v - k)| = |o + k| <= n_sr per axis
-      if (abs(oa[0] + (k & 1)) <= n_sr && abs(oa[1] + ((k >> 1) & 1)) <= n_sr && abs(oa[2] + (k >> 2)) <= n_sr)
-        a += (double)Cv[8 * v + k];
-    }
-    A[o] = a;
-  }
-  __syncthreads();
-  double* Gp = A + no3;
-  {
-    const int m = tid & 63, half = tid >> 6;
-    double s = 0.0;
-    for (int o = half; o < no3; o += 2) s = fma(A[o], Hw[(int64_t)o * 64 + m], s);
-    Gp[half * 64 + m] = s;
-  }
-  __syncthreads();
-  if (tid < 64) G[tid] = Gp[tid] + Gp[64 + tid];
-  __syncthreads();
-}
-
-template <class T>
-__global__ void __launch_bounds__(128) k_box_boundary(int n, int nb, int n_sr, double h, const int* __restrict__ bel,
-                                                      const int* __restrict__ start, const int* __restrict__ count,
-                                                      const typename vec4<T>::type* __restrict__ part,
-                                                      const T* __restrict__ Cv, const double* __restrict__ Hw,
-                                                      const double* __restrict__ g, double* __restrict__ phi) {
-  extern __shared__ double A[];   // noff^3 vertex amplitudes and 128 partial sums, then G (64)
-  const int noff = 2 * n_sr + 2, no3 = noff * noff * noff, nbk = 2 * n_sr + 1;
+__global__ void __launch_bounds__(BT) k_box_boundary(int n, int nb, int n_sr, double h, double scale,
+                                                     double inv_scale, const int* __restrict__ bel, const int* __restrict__ start,
+                                                     const int* __restrict__ ecoord,
+                                                     const typename vec4<T>::type* __restrict__ part,
+                                                     const T* __restrict__ Cv, const float2* __restrict__ Hdf,
+                                                     const double* __restrict__ g, double* __restrict__ phi) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int noff = 2 * n_sr + 2, no3 = noff * noff * noff, nrow = (2 * n_sr + 1) * (2 * n_sr + 1);
+  df* A = reinterpret_cast<df*>(smem);                                  // no3
+  // a charge's coordinates from E's corner: an FP32 one plus a whole number is a
+  // pair exactly, an FP64 one takes three floats
+  typedef typename std::conditional<sizeof(T) == 4, df, tf>::type X1;
+  struct Src {
+    X1 x[3];
+    df q;
+  };
+  struct Part {
+    typename Sum<T>::type s;
+    double far;
+  };
+  Src* ch = reinterpret_cast<Src*>(A + no3);                            // [BCH]
+  Part* red = reinterpret_cast<Part*>(smem + no3 * sizeof(df) + BCH * sizeof(BoxSrc));   // BT
+  __shared__ int j0[BROWS], pre[BROWS + 1], list[64], nlist;
   const int e = bel[blockIdx.x];
   const int E[3] = {e % n, (e / n) % n, e / (n * n)};
-  const int tid = threadIdx.x;
-  double* G = A + no3 + 128;
-  element_screen_field<T>(n, n_sr, E, Cv, Hw, A, G);
-  const int lane = tid & 31, warp = tid >> 5, Nn = 3 * nb + 1, nb3 = nbk * nbk * nbk;
-  for (int m = warp; m < 64; m += 4) {
-    const int mm[3] = {m & 3, (m >> 2) & 3, m >> 4};
-    bool own = true, bnd = false;
-    int gi[3];
+  const int tid = threadIdx.x, Nn = 3 * nb + 1;
+  if (tid < 32) {   // the boundary nodes E owns, in order
+    int base = 0;
+    for (int m = tid; m < 64; m += 32) {
+      const int mm[3] = {m & 3, (m >> 2) & 3, m >> 4};
+      bool own = true, bnd = false;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      own = own && (mm[d] < 3 || E[d] == nb - 1);
-      gi[d] = 3 * E[d] + mm[d];
-      bnd = bnd || gi[d] == 0 || gi[d] == 3 * nb;
+      for (int d = 0; d < 3; ++d) {
+        own = own && (mm[d] < 3 || E[d] == nb - 1);
+        const int gi = 3 * E[d] + mm[d];
+        bnd = bnd || gi == 0 || gi == 3 * nb;
+      }
+      const unsigned b = __ballot_sync(0xffffffffu, own && bnd);
+      if (own && bnd) list[base + __popc(b & ((1u << tid) - 1u))] = m;
+      base += __popc(b);
     }
-    if (!own || !bnd) continue;   // uniform across the warp
-    const double tn[3] = {mm[0] / 3.0, mm[1] / 3.0, mm[2] / 3.0};
-    double s = 0.0;
-    for (int b = lane; b < nb3; b += 32) {
-      const int d[3] = {b % nbk - n_sr, (b / nbk) % nbk - n_sr, b / (nbk * nbk) - n_sr};
-      const int sx = E[0] + d[0], sy = E[1] + d[1], sz = E[2] + d[2];
-      if (sx < 0 || sy < 0 || sz < 0 || sx >= nb || sy >= nb || sz >= nb) continue;
-      const int64_t se = sx + (int64_t)n * (sy + (int64_t)n * sz);
-      const int j0 = start[se], j1 = j0 + count[se];
-      for (int j = j0; j < j1; ++j) {
-        const typename vec4<T>::type pj = part[j];
-        const double rx = (d[0] + (double)pj.x) - tn[0], ry = (d[1] + (double)pj.y) - tn[1],
-                     rz = (d[2] + (double)pj.z) - tn[2];
-        s += (double)pj.w / sqrt(rx * rx + ry * ry + rz * rz);
+    if (tid == 0) nlist = base;
+  }
+  block_amplitudes<T>(n, n_sr, E, (T)scale, Cv, A);
+  const int total = block_rows(n, nb, n_sr, E, start, j0, pre);   // ends with a barrier
+  const int M = nlist, nparts = BT / M, k = tid % M, p = tid / M;
+  const bool on = p < nparts;
+  const int m = list[k], mm[3] = {m & 3, (m >> 2) & 3, m >> 4};
+  X1 tn[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    // (mm / 3 by selection: an FP64 division here costs as much as the sums)
+    const int q = mm[a];
+    constexpr float h1 = (float)(1.0 / 3.0), h2 = (float)(2.0 / 3.0);
+    constexpr float m1 = (float)(1.0 / 3.0 - h1), m2 = (float)(2.0 / 3.0 - h2);
+    constexpr float l1 = (float)(1.0 / 3.0 - h1 - m1), l2 = (float)(2.0 / 3.0 - h2 - m2);
+    const float th = q == 0 ? 0.f : (q == 1 ? h1 : (q == 2 ? h2 : 1.f));
+    const float tm = q == 1 ? m1 : (q == 2 ? m2 : 0.f);
+    if constexpr (sizeof(T) == 4) tn[a] = df{-th, -tm};
+    else tn[a] = tf{th, tm, q == 1 ? l1 : (q == 2 ? l2 : 0.f)};
+  }
+  auto diff = [&](const X1& x, int a) -> df {
+    if constexpr (sizeof(T) == 4) return df_add(x, tn[a]);
+    else return tf_diff(x, tn[a]);
+  };
+  typename Sum<T>::type acc = {};   // screen field
+  double far = 0.0;      // terms outside the pairs' range
+  if (on) {
+#pragma unroll 4
+    for (int o = p; o < no3; o += nparts) {
+      const float2 hv = Hdf[(int64_t)o * 64 + m];
+      df_fma(acc, A[o], df{hv.x, hv.y});
+    }
+  }
+  typename Sum<T>::type sing = {};
+  for (int c0 = 0; c0 < total; c0 += BCH) {
+    const int nc = min(BCH, total - c0);
+    if (c0) __syncthreads();
+    if (tid < nc) {
+      const int j = block_charge(c0 + tid, nrow, j0, pre);
+      const typename vec4<T>::type pj = part[j];
+      const int ec = ecoord[j];
+      const int d[3] = {(ec & 1023) - E[0], ((ec >> 10) & 1023) - E[1], (ec >> 20) - E[2]};
+      const T pp[3] = {pj.x, pj.y, pj.z};
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        if constexpr (sizeof(T) == 4) ch[tid].x[a] = df_two_sum((float)d[a], pp[a]);
+        else ch[tid].x[a] = tf_split((double)d[a] + pp[a]);
+      }
+      if constexpr (sizeof(T) == 4) ch[tid].q = {pj.w * (float)scale, 0.f};
+      else ch[tid].q = df_split(pj.w * scale);
+    }
+    __syncthreads();
+    if (on) {
+#pragma unroll 2
+      for (int c = p; c < nc; c += nparts) {
+        df r2 = df_sqr(diff(ch[c].x[0], 0));
+        r2 = df_add(r2, df_sqr(diff(ch[c].x[1], 1)));
+        r2 = df_add(r2, df_sqr(diff(ch[c].x[2], 2)));
+        if (df_in_range(r2)) df_fma(sing, ch[c].q, df_rsqrt<sizeof(T) == 8>(r2));
+        else far += df_value(ch[c].q) / sqrt(df_value(r2));
       }
     }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-      const int64_t node = gi[0] + (int64_t)Nn * (gi[1] + (int64_t)Nn * gi[2]);
-      phi[node] = h * g[node] - s + G[m];
+  }
+  negate(sing);
+  add_part(sing, acc);      // screen field less the singular sum
+  red[tid] = {sing, far};   // threads off: zero
+  __syncthreads();
+  if (tid < M) {
+    typename Sum<T>::type t = red[tid].s;
+    double f = far;
+    for (int q = 1; q < nparts; ++q) {
+      add_part(t, red[q * M + tid].s);
+      if (red[q * M + tid].far != 0.0) f += red[q * M + tid].far;   // also NaN
     }
+    const double s = df_value(t) - f;
+    const int gx = 3 * E[0] + mm[0], gy = 3 * E[1] + mm[1], gz = 3 * E[2] + mm[2];
+    const int64_t node = gx + (int64_t)Nn * (gy + (int64_t)Nn * gz);
+    phi[node] = h * g[node] + s * inv_scale;
   }
 }
 
@@ -204,80 +363,151 @@ __global__ void __launch_bounds__(128) k_box_boundary(int n, int nb, int n_sr, d
 // over the BOX_NGL^2 Gauss-Legendre points p of a face element (weights w_p on
 // the unit square), D_p the normal derivative of Phi^sr in element units:
 // -sum_{j in block} Q_j (r . n) / |r|^3 (r the point less x_j) less the
-// screen field's derivative sum_m G_m du_m/dn at the point.  One CTA (128
-// threads) per face element fe = (face, e1, e2), face = 2 axis + side (side 1:
-// the face at L, outward normal +axis), e1 and e2 along the next two axes
-// (e2 fastest); the point data g in the same order, points (i, j) with i along
-// the first of those axes.  Writes the 16 face-node sums (node i1 + 4 i2).
+// screen field's derivative there.  One CTA per face element fe = (face, e1,
+// e2), face = 2 axis + side (side 1: the face at L, outward normal +axis), e1
+// and e2 along the next two axes (e2 fastest); the point data g in the same
+// order, points (i, j) with i along the first of those axes.  Writes the 16
+// face-node sums (node i1 + 4 i2).
+//
+// On a face r . n is one number per charge and |r|^2 = (t_i - x1)^2 +
+// ((t_j - x2)^2 + (r . n)^2) takes 8 + 8 values per charge over the 64
+// points, so these are staged per charge and a (point, charge) pair costs
+// one sum, the power -3/2 and one multiply-add: about 40 FP32 operations.
+// The screen field's normal derivative needs the table contracted along the
+// normal axis only once, on the host: Hface[face][offset][16 face nodes].
+// Thread (point, group of four) walks every fourth charge.  Bound by FP32
+// issue; rock salt in a 32^3 box (77 M pairs): 14603 -> 216 us against FP64
+// terms with the 64 nodes' gradient at every point.
+constexpr int FCH = 64;     // charges staged at once
 template <class T>
-__global__ void __launch_bounds__(128) k_box_flux(int n, int nb, int n_sr, double h, BoxQuad qd,
-                                                  const int* __restrict__ start, const int* __restrict__ count,
-                                                  const typename vec4<T>::type* __restrict__ part,
-                                                  const T* __restrict__ Cv, const double* __restrict__ Hw,
-                                                  const double* __restrict__ g, double* __restrict__ sface) {
-  extern __shared__ double A[];   // noff^3 + 128 scratch, G (64), point values (BOX_NGL^2)
-  const int noff = 2 * n_sr + 2, no3 = noff * noff * noff, nbk = 2 * n_sr + 1, nb3 = nbk * nbk * nbk;
-  constexpr int NP = BOX_NGL * BOX_NGL;
+__global__ void __launch_bounds__(BT) k_box_flux(int n, int nb, int n_sr, double h, double scale, double inv_scale, BoxQuad qd,
+                                                 const int* __restrict__ start, const int* __restrict__ ecoord,
+                                                 const typename vec4<T>::type* __restrict__ part,
+                                                 const T* __restrict__ Cv, const float2* __restrict__ Hface,
+                                                 const double* __restrict__ g, double* __restrict__ sface) {
+  constexpr int NP = BOX_NGL * BOX_NGL, NG = BT / NP;
+  static_assert(BOX_NGL == 8 && BT == 4 * FCH && NG == 4, "the thread mapping below");
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int noff = 2 * n_sr + 2, no3 = noff * noff * noff, nrow = (2 * n_sr + 1) * (2 * n_sr + 1);
+  df* A = reinterpret_cast<df*>(smem);   // no3
+  __shared__ df sA[FCH][BOX_NGL + 1], sB[FCH][BOX_NGL + 1], sW[FCH];   // odd rows: no bank conflicts
+  __shared__ double red[BT], G[16], fp[NP], half[32];
+  __shared__ int j0[BROWS], pre[BROWS + 1];
   const int fe = blockIdx.x, face = fe / (nb * nb), e1 = (fe / nb) % nb, e2 = fe % nb;
   const int ax = face >> 1, side = face & 1, a1 = (ax + 1) % 3, a2 = (ax + 2) % 3;
   int E[3];
-  E[ax] = side ? nb - 1 : 0;
-  E[a1] = e1;
-  E[a2] = e2;
-  double* G = A + no3 + 128;
-  double* fp = G + 64;
-  element_screen_field<T>(n, n_sr, E, Cv, Hw, A, G);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  E[0] = ax == 0 ? (side ? nb - 1 : 0) : (a1 == 0 ? e1 : e2);
+  E[1] = ax == 1 ? (side ? nb - 1 : 0) : (a1 == 1 ? e1 : e2);
+  E[2] = ax == 2 ? (side ? nb - 1 : 0) : (a1 == 2 ? e1 : e2);
+  const int tid = threadIdx.x;
   const double sgn = side ? 1.0 : -1.0;   // outward normal along ax
-  for (int p = warp; p < NP; p += 4) {
-    double tau[3];
-    tau[ax] = side;
-    tau[a1] = qd.t[p / BOX_NGL];
-    tau[a2] = qd.t[p % BOX_NGL];
-    double sg = 0.0;   // sum_j Q_j (r . n) / |r|^3, element units
-    for (int b = lane; b < nb3; b += 32) {
-      const int d[3] = {b % nbk - n_sr, (b / nbk) % nbk - n_sr, b / (nbk * nbk) - n_sr};
-      const int sx = E[0] + d[0], sy = E[1] + d[1], sz = E[2] + d[2];
-      if (sx < 0 || sy < 0 || sz < 0 || sx >= nb || sy >= nb || sz >= nb) continue;
-      const int64_t se = sx + (int64_t)n * (sy + (int64_t)n * sz);
-      const int j0 = start[se], j1 = j0 + count[se];
-      for (int j = j0; j < j1; ++j) {
-        const typename vec4<T>::type pj = part[j];
-        const double r[3] = {tau[0] - (d[0] + (double)pj.x), tau[1] - (d[1] + (double)pj.y),
-                             tau[2] - (d[2] + (double)pj.z)};
-        const double ir = 1.0 / sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
-        sg += (double)pj.w * (sgn * r[ax]) * ir * ir * ir;
+  block_amplitudes<T>(n, n_sr, E, (T)scale, Cv, A);
+  const int total = block_rows(n, nb, n_sr, E, start, j0, pre);   // ends with a barrier
+  {
+    // the screen field's slope along ax at the 16 face nodes, in 16 parts
+    const int m = tid & 15, q = tid >> 4;
+    const float2* Hf = Hface + (int64_t)face * no3 * 16;
+    typename Sum<T>::type acc = {};
+#pragma unroll 4
+    for (int o = q; o < no3; o += BT / 16) {
+      const float2 hv = Hf[o * 16 + m];
+      df_fma(acc, A[o], df{hv.x, hv.y});
+    }
+    red[tid] = df_value(acc);
+    __syncthreads();
+    if (tid < 16) {
+      double s = 0.0;
+      for (int k = 0; k < BT / 16; ++k) s += red[16 * k + tid];
+      G[tid] = s;
+    }
+  }
+  const int p = tid & (NP - 1), pi = p >> 3, pj = p & 7, grp = tid / NP;
+  typename Sum<T>::type acc = {};   // sum_j Q_j (r . n) / |r|^3, element units
+  double far = 0.0;      // terms outside the pairs' range
+  for (int c0 = 0; c0 < total; c0 += FCH) {
+    const int nc = min(FCH, total - c0);
+    __syncthreads();
+    const int c = tid >> 2, sub = tid & 3;   // four threads per charge: two points of each axis
+    if (c < nc) {
+      const int j = block_charge(c0 + c, nrow, j0, pre);
+      const typename vec4<T>::type q = part[j];
+      const int ec = ecoord[j];
+      const int d[3] = {(ec & 1023) - E[0], ((ec >> 10) & 1023) - E[1], (ec >> 20) - E[2]};
+      const T x3[3] = {q.x, q.y, q.z};
+      const int dn = ax == 0 ? d[0] : (ax == 1 ? d[1] : d[2]), d1 = a1 == 0 ? d[0] : (a1 == 1 ? d[1] : d[2]),
+                d2 = a2 == 0 ? d[0] : (a2 == 1 ? d[1] : d[2]);
+      const T xn = ax == 0 ? x3[0] : (ax == 1 ? x3[1] : x3[2]), x1 = a1 == 0 ? x3[0] : (a1 == 1 ? x3[1] : x3[2]),
+              x2 = a2 == 0 ? x3[0] : (a2 == 1 ? x3[1] : x3[2]);
+      if constexpr (sizeof(T) == 4) {
+        // dn + xn etc. exactly as pairs; the point's coordinate less the charge's
+        const df rn = df_two_sum((float)(side - dn), -xn), X1 = df_two_sum((float)(-d1), -x1),
+                 X2 = df_two_sum((float)(-d2), -x2), rn2 = df_sqr(rn);
+#pragma unroll
+        for (int k = 2 * sub; k < 2 * sub + 2; ++k) {
+          const df t = {qd.th[k], qd.tl[k]};
+          sA[c][k] = df_sqr(df_add(t, X1));
+          sB[c][k] = df_add(df_sqr(df_add(t, X2)), rn2);
+        }
+        if (sub == 0) {
+          const float w = q.w * (float)scale, s = (float)sgn * w, ph = s * rn.h;
+          sW[c] = {ph, fmaf(s, rn.l, fmaf(s, rn.h, -ph))};
+        }
+      } else {
+        const double rn = side - (dn + xn), X1 = d1 + x1, X2 = d2 + x2;
+#pragma unroll
+        for (int k = 2 * sub; k < 2 * sub + 2; ++k) {
+          const double u = qd.t[k] - X1, v = qd.t[k] - X2;
+          sA[c][k] = df_split(u * u);
+          sB[c][k] = df_split(fma(v, v, rn * rn));
+        }
+        if (sub == 0) sW[c] = df_split(q.w * scale * (sgn * rn));
       }
     }
-    for (int o = 16; o > 0; o >>= 1) sg += __shfl_xor_sync(0xffffffffu, sg, o);
-    if (lane == 0) {
-      // screen field's normal derivative: only the ax factor is differentiated
-      double v[3][4], dv[4];
-      for (int a = 0; a < 3; ++a) q3_values<double>(tau[a], v[a]);
-      q3_derivs<double>(tau[ax], dv);
-      double sd = 0.0;
-      for (int m = 0; m < 64; ++m) {
-        const int mm[3] = {m & 3, (m >> 2) & 3, m >> 4};
-        double u = 1.0;
-        for (int a = 0; a < 3; ++a) u *= a == ax ? dv[mm[a]] : v[a][mm[a]];
-        sd = fma(G[m], u, sd);
+    __syncthreads();
+#pragma unroll 2
+    for (int k = grp; k < nc; k += NG) {
+      const df a = sA[k][pi], b = sB[k][pj], s = df_two_sum(a.h, b.h);
+      const df r2 = {s.h, s.l + (a.l + b.l)};
+      if (df_in_range(r2)) {
+        df_fma(acc, sW[k], df_rsqrt3<sizeof(T) == 8>(r2));
+      } else {
+        const double ir = 1.0 / sqrt(df_value(r2));
+        far += df_value(sW[k]) * ir * ir * ir;
       }
-      const double D = -sg - sgn * sd;
-      const double w = qd.w[p / BOX_NGL] * qd.w[p % BOX_NGL];
-      fp[p] = w * (h * h * g[(int64_t)fe * NP + p] - D);
     }
   }
   __syncthreads();
-  if (tid < 16) {
-    const int i1 = tid & 3, i2 = tid >> 2;
-    double s = 0.0;
-    for (int p = 0; p < NP; ++p) {
-      double l1[4], l2[4];
-      q3_values<double>(qd.t[p / BOX_NGL], l1);
-      q3_values<double>(qd.t[p % BOX_NGL], l2);
-      s = fma(fp[p], l1[i1] * l2[i2], s);
+  red[tid] = df_value(acc) + far;
+  __syncthreads();
+  if (tid < NP) {
+    double sg = 0.0, sd = 0.0;
+#pragma unroll
+    for (int k = 0; k < NG; ++k) sg += red[k * NP + p];
+#pragma unroll
+    for (int i2 = 0; i2 < 4; ++i2) {
+      double row = 0.0;
+#pragma unroll
+      for (int i1 = 0; i1 < 4; ++i1) row = fma(G[i1 + 4 * i2], qd.l[pi][i1], row);
+      sd = fma(row, qd.l[pj][i2], sd);
     }
-    sface[(int64_t)fe * 16 + tid] = s;
+    const double D = -(sg + sgn * sd) * inv_scale;
+    fp[p] = qd.w[pi] * qd.w[pj] * (h * h * g[(int64_t)fe * NP + p] - D);
+  }
+  __syncthreads();
+  if (tid < 32) {   // s_(i1, i2) = sum_i l_i1(t_i) sum_j l_i2(t_j) fp(i, j): first over i
+    const int i1 = tid & 3, j = tid >> 2;
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < BOX_NGL; ++i) s = fma(fp[i * BOX_NGL + j], qd.l[i][i1], s);
+    half[tid] = s;
+    __syncwarp();
+    if (tid < 16) {
+      const int i2 = tid >> 2;
+      s = 0.0;
+#pragma unroll
+      for (int k = 0; k < BOX_NGL; ++k) s = fma(half[i1 + 4 * k], qd.l[k][i2], s);
+      sface[(int64_t)fe * 16 + tid] = s;
+    }
   }
 }
 
@@ -316,42 +546,6 @@ __global__ void k_box_plain_bvals(int Nn, double h, const double* __restrict__ g
   phi[i] = bnd ? h * g[i] : 0.0;
 }
 
-// One axis of a separable banded apply on the box's node grid:
-//   out = A_axis(in) [+ B_axis(in2) + C_axis(in3)], then out = base - out with
-// base; rows by node type (tap o couples node g to g + o - 3), taps past the
-// grid's ends dropped and the end rows' diagonals those of one element: the
-// rows of the open matrices.
-__global__ void k_box_band(int Nn, int axis, BoxBand bd, int ma, const double* __restrict__ in, int mb,
-                           const double* __restrict__ in2, int mc, const double* __restrict__ in3,
-                           const double* __restrict__ base, double* __restrict__ out) {
-  const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (g >= (int64_t)Nn * Nn * Nn) return;
-  const int idx[3] = {(int)(g % Nn), (int)((g / Nn) % Nn), (int)(g / ((int64_t)Nn * Nn))};
-  const int64_t st[3] = {1, Nn, (int64_t)Nn * Nn};
-  const int ga = idx[axis], t = ga % 3;
-  const int64_t b0 = g - (int64_t)ga * st[axis];
-  const double* rows[3] = {ma ? bd.bK[t] : bd.bM[t], mb ? bd.bK[t] : bd.bM[t], mc ? bd.bK[t] : bd.bM[t]};
-  const int end = ga == 0 ? 0 : (ga == Nn - 1 ? 1 : -1);   // the first and last rows: one element's diagonal
-  double acc = 0.0;
-#pragma unroll
-  for (int o = 0; o < 7; ++o) {
-    const int ja = ga + o - 3;
-    if (ja < 0 || ja >= Nn) continue;
-    const int64_t j = b0 + (int64_t)ja * st[axis];
-    double w0 = rows[0][o], w1 = rows[1][o], w2 = rows[2][o];
-    if (o == 3 && end >= 0) {
-      w0 = ma ? bd.dK[end] : bd.dM[end];
-      w1 = mb ? bd.dK[end] : bd.dM[end];
-      w2 = mc ? bd.dK[end] : bd.dM[end];
-    }
-    double v = w0 * in[j];
-    if (in2) v += w1 * in2[j];
-    if (in3) v += w2 * in3[j];
-    acc += v;
-  }
-  out[g] = base ? base[g] - acc : acc;
-}
-
 // node of solved index i: the Ns^3 solved nodes start at index off per axis
 // (Dirichlet: the interior, off = 1; Neumann: all nodes, off = 0)
 __device__ __forceinline__ int64_t solved_node(int64_t i, int Ns, int Nn, int off) {
@@ -364,12 +558,17 @@ __device__ __forceinline__ double box_w1(int g, int Nn, const BoxBand& bd) {
   return (g == 0 || g == Nn - 1) ? bd.wend : bd.wn[g % 3];
 }
 
-// deterministic FP64 sums: mode 0, sum of squares of v at the solved nodes;
-// mode 1, sum of v over all nodes; mode 2, sum of w3 v over all nodes (w3
-// the 3-D node integrals).  Per-block partials, then one block adds them in order
-__global__ void k_box_partial(int mode, int Ns, int Nn, int off, BoxBand bd, const double* __restrict__ v,
-                              double* __restrict__ partial) {
+// deterministic FP64 sums: mode 0, sum of squares of v at the solved nodes
+// into *out, with the power of two near the inverse RMS and its inverse into
+// scale[0], scale[1]; mode 1, sum of v over all nodes; mode 2, sum of w3 v
+// over all nodes (w3 the 3-D node integrals).  Per-block partials; the last
+// block to finish adds them in a fixed order.
+__global__ void __launch_bounds__(BT) k_box_sum(int mode, int Ns, int Nn, int off, BoxBand bd,
+                                                const double* __restrict__ v, double* __restrict__ partial,
+                                                unsigned int* __restrict__ counter, double* __restrict__ out,
+                                                float* __restrict__ scale) {
   __shared__ double sh[BT / 32];
+  __shared__ bool last;
   const int64_t len = mode == 0 ? (int64_t)Ns * Ns * Ns : (int64_t)Nn * Nn * Nn;
   double acc = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x) {
@@ -383,36 +582,60 @@ __global__ void k_box_partial(int mode, int Ns, int Nn, int off, BoxBand bd, con
       acc = fma(box_w1(x, Nn, bd) * box_w1(y, Nn, bd) * box_w1(z, Nn, bd), v[i], acc);
     }
   }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
+  auto block_sum = [&](double a) -> double {   // in thread 0
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x == 0)
+      for (int k = 0; k < BT / 32; ++k) s += sh[k];
+    return s;
+  };
+  double s = block_sum(acc);
   if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int k = 0; k < BT / 32; ++k) s += sh[k];
     partial[blockIdx.x] = s;
+    __threadfence();
+    last = atomicAdd(counter, 1u) == gridDim.x - 1;
   }
-}
-__global__ void k_box_final(int nb, const double* __restrict__ partial, double* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int k = 0; k < nb; ++k) s += partial[k];
-    *out = s;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  acc = 0.0;
+  for (unsigned k = threadIdx.x; k < gridDim.x; k += BT) acc += ((volatile double*)partial)[k];
+  s = block_sum(acc);
+  if (threadIdx.x != 0) return;
+  *counter = 0u;
+  *out = s;
+  if (mode == 0) {
+    const double rms = sqrt(s / (double)len);
+    int k = rms > 0.0 && isfinite(rms) ? ilogb(rms) : 0;
+    k = max(-100, min(100, k));
+    scale[0] = (float)ldexp(1.0, -k);
+    scale[1] = (float)ldexp(1.0, k);
   }
 }
 
-// the residual at the solved nodes, scaled into FP32; the FP32 correction added back
-__global__ void k_box_round(int Ns, int Nn, int off, const double* __restrict__ res, double scale,
+// the first residual at the solved nodes, scaled into FP32; the FP32
+// correction added back (pairs: the new iterate as float pairs too)
+__global__ void k_box_round(int Ns, int Nn, int off, const double* __restrict__ res, const float* __restrict__ scale,
                             float* __restrict__ out) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < (int64_t)Ns * Ns * Ns) out[i] = (float)(res[solved_node(i, Ns, Nn, off)] * scale);
+  if (i < (int64_t)Ns * Ns * Ns) out[i] = (float)(res[solved_node(i, Ns, Nn, off)] * (double)scale[0]);
 }
-__global__ void k_box_add(int Ns, int Nn, int off, const float* __restrict__ x, double scale,
-                          double* __restrict__ phi) {
+__global__ void k_box_add(int Ns, int Nn, int off, const float* __restrict__ x, const float* __restrict__ scale,
+                          double* __restrict__ phi, df* __restrict__ pairs) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < (int64_t)Ns * Ns * Ns) {
     const int64_t j = solved_node(i, Ns, Nn, off);
-    phi[j] += (double)x[i] * scale;
+    const double v = phi[j] + (double)(x[i] * scale[1]);   // the scale is a power of two
+    phi[j] = v;
+    if (pairs) pairs[j] = df_split(v);
   }
+}
+__global__ void k_box_clear(int Ns, int Nn, int off, double* __restrict__ phi) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < (int64_t)Ns * Ns * Ns) phi[solved_node(i, Ns, Nn, off)] = 0.0;
 }
 
 // out = in - s w3 (w3 the node integrals: the load of a constant density, the
@@ -453,78 +676,96 @@ double box_rtol(const fep3m_ctx* c) {
   return c->cfg.mg_rtol > 0 ? c->cfg.mg_rtol : (c->precision == FEP3M_FP64 ? 1e-13 : 1e-10);
 }
 
-struct BoxReducer {
-  Box* B;
-  int nblk;
-  // the sum of the given mode into dst (device); no sync
-  void run(int mode, const double* v, double* dst, cudaStream_t s) {
-    FEP3M_CL k_box_partial<<<nblk, BT, 0, s>>>(mode, B->Ns, B->Nn, B->off, B->band, v, B->red);
-    FEP3M_CL k_box_final<<<1, 32, 0, s>>>(nblk, B->red, dst);
-  }
-  double host_norm2(const double* v, cudaStream_t s) {
-    run(0, v, B->red + 1024, s);
-    cudaMemcpyAsync(B->host_red, B->red + 1024, sizeof(double), cudaMemcpyDeviceToHost, s);
-    cudaStreamSynchronize(s);
-    return *B->host_red;
-  }
-};
+// B->red: partials of the sums (1024) or of the fused applies from PART on
+// (box_apply_blocks), and before them the sums' results and the scale
+constexpr int RED_SUM = 1024, RED_SCALE = 1027, RED_NORM = 1028, PART = 1060;   // norms: the start's, one per sweep
+constexpr int MAX_SWEEPS = PART - RED_NORM - 1;
 
-BoxReducer box_reducer(Box* B) {
+void box_sum(Box* B, int mode, const double* v, double* dst, cudaStream_t s) {
   const int64_t len = (int64_t)B->Nn * B->Nn * B->Nn;
-  return BoxReducer{B, (int)std::min<int64_t>(1024, std::max<int64_t>(1, len / (BT * 8)))};
-}
-
-// r = rhs - K phi with K = K1 (x) M1 (x) M1 + M1 (x) K1 (x) M1 + M1 (x) M1 (x) K1
-// (interior rows): a = M_z phi, b = K_z phi; c = M_y a, d = K_y a, f = M_y b;
-// r = rhs - (K_x c + M_x d + M_x f)
-void box_residual(Box* B, const double* rhs, const double* phi, double* r, cudaStream_t s) {
-  const int Nn = B->Nn;
-  const int64_t len = (int64_t)Nn * Nn * Nn;
-  double *a = B->t[0], *b = B->t[1], *c = B->t[2], *d = B->t[3];
-  FEP3M_CL k_box_band<<<gsz(len), BT, 0, s>>>(Nn, 2, B->band, 0, phi, 0, nullptr, 0, nullptr, nullptr, a);
-  FEP3M_CL k_box_band<<<gsz(len), BT, 0, s>>>(Nn, 2, B->band, 1, phi, 0, nullptr, 0, nullptr, nullptr, b);
-  FEP3M_CL k_box_band<<<gsz(len), BT, 0, s>>>(Nn, 1, B->band, 0, a, 0, nullptr, 0, nullptr, nullptr, c);
-  FEP3M_CL k_box_band<<<gsz(len), BT, 0, s>>>(Nn, 1, B->band, 1, a, 0, nullptr, 0, nullptr, nullptr, d);
-  FEP3M_CL k_box_band<<<gsz(len), BT, 0, s>>>(Nn, 1, B->band, 0, b, 0, nullptr, 0, nullptr, nullptr, a);
-  FEP3M_CL k_box_band<<<gsz(len), BT, 0, s>>>(Nn, 0, B->band, 1, c, 0, d, 0, a, rhs, r);
+  const int nblk = (int)std::min<int64_t>(1024, std::max<int64_t>(1, len / (BT * 8)));
+  FEP3M_CL k_box_sum<<<nblk, BT, 0, s>>>(mode, B->Ns, B->Nn, B->off, B->band, v, B->red, B->counter, dst,
+                                         (float*)(B->red + RED_SCALE));
 }
 
 // K phi = rhs at the solved nodes (Dirichlet: the interior, phi's boundary
-// values held; Neumann: all, rhs compatible): iterative refinement around the
-// FP32 fast-diagonalisation solve; sets B->sweeps and B->relres (the residual
-// relative to that of phi's starting values)
+// values held; Neumann: all, rhs compatible; phi zero at the solved nodes):
+// iterative refinement around the FP32 fast-diagonalisation solve, the
+// residuals scaled by one power of two near the first one's inverse RMS.  In
+// MIXED the residual is formed in double-float arithmetic (as the periodic
+// solver's; about 2e-14 relative) from a copy of the iterate as float pairs.
+// The norms stay on the device: they are read once after as many sweeps as
+// the last solve took (and after each further one).  Sets B->sweeps and
+// B->relres (the residual relative to that of phi's starting values)
 cudaError_t box_refine(fep3m_ctx* c, Box* B, const double* rhs, double* phi) {
-  const int Ns = B->Ns;
-  const int64_t len = (int64_t)Ns * Ns * Ns;
+  const int Ns = B->Ns, Nn = B->Nn;
+  const int64_t len = (int64_t)Ns * Ns * Ns, nn3 = (int64_t)Nn * Nn * Nn;
   cudaStream_t s = c->stream;
-  BoxReducer red = box_reducer(B);
   const double rtol = box_rtol(c);
-  const int max_sweeps = c->cfg.mg_max_cycles > 0 ? c->cfg.mg_max_cycles : 10;
-  box_residual(B, rhs, phi, B->res, s);
-  const double n0 = std::sqrt(red.host_norm2(B->res, s));
+  const int max_sweeps = std::min(c->cfg.mg_max_cycles > 0 ? c->cfg.mg_max_cycles : 10, MAX_SWEEPS);
+  const bool mixed = c->precision == FEP3M_MIXED;
+  df* pairs = mixed ? (df*)c->phi_hl : nullptr;
+  float* scale = (float*)(B->red + RED_SCALE);
+  double* norm = B->red + RED_NORM;
+  cudaError_t e;
+  if (mixed && (e = split_pairs(nn3, rhs, B->t[0], s)) != cudaSuccess) return e;
+  if (mixed && (e = split_pairs(nn3, phi, pairs, s)) != cudaSuccess) return e;
+  BoxApply ap;
+  ap.N = Nn;
+  ap.Ns = Ns;
+  ap.off = B->off;
+  ap.pairs = mixed;
+  ap.x = mixed ? (const void*)pairs : phi;
+  ap.b = mixed ? (const void*)B->t[0] : rhs;
+  ap.partials = B->red + PART;
+  ap.counter = B->counter;
+  const double* r0 = rhs;   // Neumann: phi is zero
+  if (!B->neumann) {
+    ap.r64 = B->res;
+    if ((e = box_apply(ap, s)) != cudaSuccess) return e;
+    ap.r64 = nullptr;
+    r0 = B->res;
+  }
+  box_sum(B, 0, r0, norm, s);
+  FEP3M_CL k_box_round<<<gsz(len), BT, 0, s>>>(Ns, Nn, B->off, r0, scale, B->r32);
+  ap.scale = scale;
+  ap.r = B->r32;
   B->sweeps = 0;
   B->relres = 0.0;
-  if (!(n0 > 0.0)) return cudaGetLastError();   // zero (or, for non-finite data, NaN) residual: nothing to solve
-  double nr = n0;
+  int read = std::max(1, std::min(B->plan, max_sweeps));   // sweeps before the norms are looked at
   for (int k = 0; k < max_sweeps; ++k) {
-    // scale the residual by a power of two near 1 / RMS into FP32
-    const double sc = std::ldexp(1.0, -std::ilogb(nr / std::sqrt((double)len)));
-    FEP3M_CL k_box_round<<<gsz(len), BT, 0, s>>>(Ns, B->Nn, B->off, B->res, sc, B->r32);
-    cudaError_t e = fdm_apply(B->fdm, B->r32, B->x32, B->w1, B->w2, s);
-    if (e != cudaSuccess) return e;
-    FEP3M_CL k_box_add<<<gsz(len), BT, 0, s>>>(Ns, B->Nn, B->off, B->x32, 1.0 / sc, phi);
-    box_residual(B, rhs, phi, B->res, s);
-    nr = std::sqrt(red.host_norm2(B->res, s));
+    if ((e = fdm_apply(B->fdm, B->r32, B->x32, B->w1, B->w2, s)) != cudaSuccess) return e;
+    FEP3M_CL k_box_add<<<gsz(len), BT, 0, s>>>(Ns, Nn, B->off, B->x32, scale, phi, pairs);
+    ap.norm = norm + 1 + k;
+    if ((e = box_apply(ap, s)) != cudaSuccess) return e;
+    if (k + 1 < read) continue;
+    // host_red: the scale (two floats), then the norms
+    cudaMemcpyAsync(B->host_red, B->red + RED_SCALE, (k + 3) * sizeof(double), cudaMemcpyDeviceToHost, s);
+    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+    const double n0 = std::sqrt(B->host_red[1]), sc = *(const float*)B->host_red;
+    if (!(n0 > 0.0)) {
+      // a zero (or, for non-finite data, NaN) residual: nothing to solve.  MIXED: an infinite
+      // boundary value is NaN in the float pairs, reported as not converged, as in FP64
+      if (mixed && !(n0 == 0.0)) B->relres = n0;
+      FEP3M_CL k_box_clear<<<gsz(len), BT, 0, s>>>(Ns, Nn, B->off, phi);
+      return cudaGetLastError();
+    }
+    bool done = false;
+    for (int j = 0; j <= k && !done; ++j) {   // the sweeps that were needed: the next solve's plan
+      const double rel = std::sqrt(B->host_red[2 + j]) / (sc * n0);
+      done = !(rel > rtol);
+      B->plan = j + 1;
+    }
     B->sweeps = k + 1;
-    B->relres = nr / n0;
-    if (!(B->relres > rtol)) break;
+    B->relres = std::sqrt(B->host_red[2 + k]) / (sc * n0);
+    if (done || !(B->relres > rtol)) break;
   }
   return cudaGetLastError();
 }
 
 }  // namespace
 
-int box_create(fep3m_ctx* c, int nb, bool neumann) {
+int box_create(fep3m_ctx* c, int nb, bool neumann, const double* Hw) {
   Box* B = new (std::nothrow) Box();
   if (!B) return FEP3M_ENOMEM;
   c->box = B;
@@ -534,19 +775,9 @@ int box_create(fep3m_ctx* c, int nb, bool neumann) {
   B->neumann = neumann;
   B->Ns = neumann ? B->Nn : B->NI;
   B->off = neumann ? 0 : 1;
-  // rows of the open order-3 matrices (h = 1): the periodic stencils inside,
-  // one element's diagonal at the two ends; node integrals
+  // mixed mass and node integrals (h = 1)
   double Me[4][4], Ke[4][4], Mpq[4][2];
   element_matrices_q3(Me, Ke, Mpq);
-  for (int t = 0; t < 3; ++t)
-    for (int j = 0; j < 7; ++j) {
-      B->band.bM[t][j] = c->st.M[t][j];
-      B->band.bK[t][j] = c->st.K[t][j];
-    }
-  B->band.dM[0] = Me[0][0];
-  B->band.dK[0] = Ke[0][0];
-  B->band.dM[1] = Me[3][3];
-  B->band.dK[1] = Ke[3][3];
   for (int i = 0; i < 4; ++i)
     for (int j = 0; j < 2; ++j) B->band.Mpq[i][j] = Mpq[i][j];
   double rs[4] = {0, 0, 0, 0};   // element row sums: the integrals of the shape functions
@@ -562,6 +793,33 @@ int box_create(fep3m_ctx* c, int nb, bool neumann) {
     for (int k = 0; k < BOX_NGL; ++k) {
       B->quad.t[k] = x[k];
       B->quad.w[k] = w[k];
+      q3_values<double>(x[k], B->quad.l[k]);
+      const df t = df_split(x[k]);
+      B->quad.th[k] = t.h;
+      B->quad.tl[k] = t.l;
+    }
+  }
+  // the vertex table [offset][64 nodes] as pairs (Dirichlet), or contracted
+  // along each face's normal axis with the shape functions' derivatives there:
+  // [face][offset][16 face nodes] (Neumann)
+  const int no3 = c->noff * c->noff * c->noff;
+  std::vector<df> tab;
+  if (!neumann) {
+    tab.resize((size_t)no3 * 64);
+    for (size_t i = 0; i < tab.size(); ++i) tab[i] = df_split(Hw[i]);
+  } else {
+    tab.resize((size_t)6 * no3 * 16);
+    for (int face = 0; face < 6; ++face) {
+      const int ax = face >> 1, st[3] = {1, 4, 16};
+      double dv[4];
+      q3_derivs<double>(face & 1, dv);
+      for (int o = 0; o < no3; ++o)
+        for (int m = 0; m < 16; ++m) {
+          const double* Ho = Hw + (size_t)o * 64 + (m & 3) * st[(ax + 1) % 3] + (m >> 2) * st[(ax + 2) % 3];
+          double v = 0.0;
+          for (int k = 0; k < 4; ++k) v += dv[k] * Ho[k * st[ax]];
+          tab[((size_t)face * no3 + o) * 16 + m] = df_split(v);
+        }
     }
   }
   // boundary elements (padded-grid ids)
@@ -589,30 +847,28 @@ int box_create(fep3m_ctx* c, int nb, bool neumann) {
   al((void**)&B->w1, ns3 * sizeof(float));
   al((void**)&B->w2, ns3 * sizeof(float));
   al((void**)&B->bel, bel.size() * sizeof(int));
-  al((void**)&B->red, 1040 * sizeof(double));
+  al((void**)&B->red, (PART + box_apply_blocks(B->Nn)) * sizeof(double));
+  al((void**)&B->counter, sizeof(unsigned int));
+  al((void**)&B->tab, tab.size() * sizeof(df));
   if (neumann) al((void**)&B->sface, (size_t)6 * nb * nb * 16 * sizeof(double));
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? FEP3M_ENOMEM : FEP3M_ECUDA;
-  if (cudaMallocHost(&B->host_red, sizeof(double)) != cudaSuccess) return FEP3M_ENOMEM;
+  if (cudaMallocHost(&B->host_red, (MAX_SWEEPS + 2) * sizeof(double)) != cudaSuccess) return FEP3M_ENOMEM;
+  cudaMemset(B->counter, 0, sizeof(unsigned int));
+  if ((e = box_apply_setup(c->st)) != cudaSuccess) return FEP3M_ECUDA;
   cudaMemset(B->g, 0, box_data_size(c) * sizeof(double));
   cudaMemcpy(B->bel, bel.data(), bel.size() * sizeof(int), cudaMemcpyHostToDevice);
+  cudaMemcpy(B->tab, tab.data(), tab.size() * sizeof(df), cudaMemcpyHostToDevice);
   std::vector<double> lam, V;
   box_eigen(3, nb, !neumann, lam, V);
   e = fdm_setup(B->fdm, B->Ns, lam, V, 1, !(c->cfg.flags & FEP3M_CUDA_CORES), neumann);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? FEP3M_ENOMEM : FEP3M_ECUDA;
-  const int noff = c->noff;
-  const size_t smem = ((size_t)noff * noff * noff + 128 + 64 + BOX_NGL * BOX_NGL) * sizeof(double);
-  if (cudaFuncSetAttribute(k_box_boundary<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-      cudaFuncSetAttribute(k_box_boundary<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-      cudaFuncSetAttribute(k_box_flux<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-      cudaFuncSetAttribute(k_box_flux<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return FEP3M_ECUDA;
   return FEP3M_OK;
 }
 
 void box_destroy(fep3m_ctx* c) {
   Box* B = c->box;
   if (!B) return;
-  void* p[] = {B->g, B->gstage, B->b, B->rhs, B->res, B->r32, B->x32, B->w1, B->w2, B->bel, B->red, B->sface};
+  void* p[] = {B->g, B->gstage, B->b, B->rhs, B->res, B->r32, B->x32, B->w1, B->w2, B->bel, B->red, B->sface, B->tab, B->counter};
   for (void* x : p)
     if (x) cudaFree(x);
   for (double* t : B->t)
@@ -668,16 +924,14 @@ static void box_load(fep3m_ctx* c, Box* B, cudaStream_t s) {
 static void box_project(Box* B, double* rhs, cudaStream_t s) {
   const int64_t nn3 = (int64_t)B->Nn * B->Nn * B->Nn;
   const double w3 = (double)B->nb * B->nb * B->nb;   // the box's volume, h = 1
-  BoxReducer red = box_reducer(B);
-  red.run(1, rhs, B->red + 1025, s);
-  FEP3M_CL k_box_sub<<<gsz(nn3), BT, 0, s>>>(B->Nn, B->band, B->red + 1025, 1.0 / w3, 0, rhs, rhs);
+  box_sum(B, 1, rhs, B->red + RED_SUM, s);
+  FEP3M_CL k_box_sub<<<gsz(nn3), BT, 0, s>>>(B->Nn, B->band, B->red + RED_SUM, 1.0 / w3, 0, rhs, rhs);
 }
 static void box_zero_mean(Box* B, double* phi, cudaStream_t s) {
   const int64_t nn3 = (int64_t)B->Nn * B->Nn * B->Nn;
   const double w3 = (double)B->nb * B->nb * B->nb;
-  BoxReducer red = box_reducer(B);
-  red.run(2, phi, B->red + 1026, s);
-  FEP3M_CL k_box_sub<<<gsz(nn3), BT, 0, s>>>(B->Nn, B->band, B->red + 1026, 1.0 / w3, 1, phi, phi);
+  box_sum(B, 2, phi, B->red + RED_SUM, s);
+  FEP3M_CL k_box_sub<<<gsz(nn3), BT, 0, s>>>(B->Nn, B->band, B->red + RED_SUM, 1.0 / w3, 1, phi, phi);
 }
 
 int box_compute(fep3m_ctx* c, double* phi_dev, double* U_dev) {
@@ -691,30 +945,34 @@ int box_compute(fep3m_ctx* c, double* phi_dev, double* U_dev) {
   // singular sums and screen field of the targets (need no mesh solution)
   if ((e = pair_screen(c, 0, s, false)) != cudaSuccess) return FEP3M_ECUDA;
   if (cudaMemsetAsync(c->phi64, 0, nn3 * sizeof(double), s) != cudaSuccess) return FEP3M_ECUDA;
-  const size_t smem = ((size_t)c->noff * c->noff * c->noff + 128 + 64 + BOX_NGL * BOX_NGL) * sizeof(double);
+  const size_t asz = (size_t)c->noff * c->noff * c->noff * sizeof(df);
   const bool f32 = c->precision == FEP3M_MIXED;
   const double* rhs = B->b;
   if (!B->neumann) {
     // boundary values (Eq. bcadjust), then the interior solve
+    const size_t smem = asz + BCH * sizeof(BoxSrc) + BT * (sizeof(double) + 2 * sizeof(df));
     if (f32)
-      FEP3M_CL k_box_boundary<float><<<B->nbel, 128, smem, s>>>(c->n, B->nb, c->n_sr, c->h, B->bel, c->start,
-                                                               c->count, (const float4*)c->part, (const float*)c->Cv,
-                                                               c->Hw64, B->g, c->phi64);
+      FEP3M_CL k_box_boundary<float><<<B->nbel, BT, smem, s>>>(c->n, B->nb, c->n_sr, c->h, c->q_scale,
+                                                               1.0 / c->q_scale, B->bel, c->start,
+                                                               c->ecoord, (const float4*)c->part, (const float*)c->Cv,
+                                                               (const float2*)B->tab, B->g, c->phi64);
     else
-      FEP3M_CL k_box_boundary<double><<<B->nbel, 128, smem, s>>>(c->n, B->nb, c->n_sr, c->h, B->bel, c->start,
-                                                                c->count, (const vec4<double>::type*)c->part,
-                                                                (const double*)c->Cv, c->Hw64, B->g, c->phi64);
+      FEP3M_CL k_box_boundary<double><<<B->nbel, BT, smem, s>>>(c->n, B->nb, c->n_sr, c->h, c->q_scale,
+                                                                1.0 / c->q_scale, B->bel,
+                                                                c->start, c->ecoord, (const vec4<double>::type*)c->part,
+                                                                (const double*)c->Cv, (const float2*)B->tab, B->g,
+                                                                c->phi64);
   } else {
     // the adjusted flux as a boundary load, made compatible
     const unsigned nfe = (unsigned)(6 * B->nb * B->nb);
     if (f32)
-      FEP3M_CL k_box_flux<float><<<nfe, 128, smem, s>>>(c->n, B->nb, c->n_sr, c->h, B->quad, c->start, c->count,
-                                                       (const float4*)c->part, (const float*)c->Cv, c->Hw64, B->g,
-                                                       B->sface);
+      FEP3M_CL k_box_flux<float><<<nfe, BT, asz, s>>>(c->n, B->nb, c->n_sr, c->h, c->q_scale, 1.0 / c->q_scale, B->quad, c->start,
+                                                      c->ecoord, (const float4*)c->part, (const float*)c->Cv,
+                                                      (const float2*)B->tab, B->g, B->sface);
     else
-      FEP3M_CL k_box_flux<double><<<nfe, 128, smem, s>>>(c->n, B->nb, c->n_sr, c->h, B->quad, c->start, c->count,
-                                                        (const vec4<double>::type*)c->part, (const double*)c->Cv,
-                                                        c->Hw64, B->g, B->sface);
+      FEP3M_CL k_box_flux<double><<<nfe, BT, asz, s>>>(c->n, B->nb, c->n_sr, c->h, c->q_scale, 1.0 / c->q_scale, B->quad, c->start,
+                                                       c->ecoord, (const vec4<double>::type*)c->part,
+                                                       (const double*)c->Cv, (const float2*)B->tab, B->g, B->sface);
     FEP3M_CL k_box_sgather<<<gsz(nn3), BT, 0, s>>>(B->nb, B->b, B->sface, B->rhs);
     box_project(B, B->rhs, s);
     rhs = B->rhs;

@@ -225,17 +225,32 @@ struct OrderQ {
 // The box [0, L]^3 with Dirichlet data (box.cu): order-3 mesh of nb elements
 // per axis, Nn = 3 nb + 1 nodes, the NI = 3 nb - 1 interior ones solved for.
 struct BoxBand {
-  double bM[3][7];      // 1-D order-3 mass row of node type t = g mod 3: tap o -> node g + o - 3
-  double bK[3][7];      // the same for the stiffness (interior rows of the open matrices)
-  double dM[2], dK[2];  // diagonals of the open matrices' first and last rows (one element each)
   double Mpq[4][2];     // element mixed mass int l^3_i l^1_j (h = 1)
   double wn[3];         // node integrals by node type t (t = 0: a vertex shared by two elements)
   double wend;          // the node integral of the first and last node
+};
+// one residual r = b - K x on the open mesh (box_apply, mesh.cu): x and b in
+// FP64 or float pairs; r64: the FP64 residual of every node; else r receives
+// scale times it at the solved nodes (Ns per axis from index off), packed, in
+// FP32, and norm the sum of its squares
+struct BoxApply {
+  int N = 0, Ns = 0, off = 0;
+  bool pairs = false;
+  const void* x = nullptr;
+  const void* b = nullptr;
+  float* r = nullptr;
+  double* r64 = nullptr;
+  const float* scale = nullptr;   // device
+  double* partials = nullptr;     // box_apply_blocks(N)
+  unsigned int* counter = nullptr;
+  double* norm = nullptr;
 };
 // Gauss-Legendre rule on [0, 1] of the Neumann face integrals
 constexpr int BOX_NGL = 8;
 struct BoxQuad {
   double t[BOX_NGL], w[BOX_NGL];
+  float th[BOX_NGL], tl[BOX_NGL];   // t as hi + lo floats
+  double l[BOX_NGL][4];   // the order-3 shape functions at the points
 };
 struct Box {
   int nb = 0, Nn = 0, NI = 0;
@@ -251,15 +266,20 @@ struct Box {
   double* rhs = nullptr;      // Nn^3 Neumann right-hand side: b + s, made compatible
   double* phi = nullptr;      // Nn^3 mesh potential (element units: h Phi^sm)
   double* res = nullptr;      // Nn^3 residual b - K phi (interior rows)
-  double* t[4] = {};          // Nn^3 scratch of the stiffness apply and the load passes
+  double* t[2] = {};          // Nn^3 scratch of the load passes; MIXED: t[0] then holds the refinement's
+                              // right-hand side as float pairs
   float* r32 = nullptr;       // Ns^3 FP32 inner solve: right-hand side, correction, scratch
   float* x32 = nullptr;
   float* w1 = nullptr;
   float* w2 = nullptr;
+  void* tab = nullptr;        // float pairs: the vertex table [offset][64 nodes] (Dirichlet), or its normal
+                              // derivatives at the faces [face][offset][16 face nodes] (Neumann)
   int* bel = nullptr;         // boundary elements (ids in the padded grid)
   int nbel = 0;
-  double* red = nullptr;      // reduction partials
-  double* host_red = nullptr; // pinned: one reduction result
+  double* red = nullptr;      // reduction partials and results (box.cu)
+  double* host_red = nullptr; // pinned: the norms of one refinement
+  unsigned int* counter = nullptr;   // last-block counter of the reductions
+  int plan = 0;               // refinement sweeps of the last solve: the next one's before its first check
   FineFDM fdm;                // box eigenbasis of the solved nodes (Dirichlet: no null mode)
   int sweeps = 0;
   double relres = 0;
@@ -280,6 +300,7 @@ struct fep3m_ctx {
   double* Hw64 = nullptr;
   // particles
   int64_t N = 0, cap = 0;
+  double q_scale = 1;            // power of two near the inverse mean |Q| of the charges last set
   bool have_particles = false, have_forward = false, have_grad = false;
   double* pos_in = nullptr;      // N*3 (staging for host inputs)
   double* Q_in = nullptr;        // N
@@ -435,6 +456,8 @@ void pair_adjoint_table(int n_sr, const double* Hw, double* Hd, float* H0);
 // singular adjoint of the energy's weights Q / 2)
 cudaError_t pair_screen(fep3m_ctx* c, int want_grad, cudaStream_t s, bool energy_adjoint);
 cudaError_t pair_prepare(fep3m_ctx* c);
+// n FP64 values as hi + lo floats
+cudaError_t split_pairs(int64_t n, const double* v, void* out, cudaStream_t s);
 // tensor-core row GEMM with transposed output (mesh.cu): out[(i - cb) R + r]
 // = sum_{a < K} in[r K + a] B[i][a] for the columns cb <= i < ce; B in split
 // bf16 pieces per column tile of nt
@@ -459,12 +482,16 @@ void orderq_destroy(fep3m_ctx* c);
 int orderq_compute(fep3m_ctx* c, double* phi_dev, double* U_dev);
 int orderq_solve(fep3m_ctx* c, const double* b_dev, double* phi_dev);
 // the box (box.cu); n is the padded grid's, nb the box's elements per axis
-int box_create(fep3m_ctx* c, int nb, bool neumann);
+// Hw: the vertex table [offset][64 nodes]
+int box_create(fep3m_ctx* c, int nb, bool neumann, const double* Hw);
 int64_t box_data_size(const fep3m_ctx* c);
 void box_destroy(fep3m_ctx* c);
 int box_set_boundary(fep3m_ctx* c, const double* g_dev);
 int box_compute(fep3m_ctx* c, double* phi_dev, double* U_dev);
 int box_solve(fep3m_ctx* c, double* rhs_dev, double* phi_dev);   // rhs_dev may be overwritten
+int box_apply_blocks(int N);
+cudaError_t box_apply_setup(const Stencils& st);
+cudaError_t box_apply(const BoxApply& a, cudaStream_t s);
 cudaError_t box_binning(fep3m_ctx* c, int* count_out, int* cell_out);
 cudaError_t box_coeffs(fep3m_ctx* c, double* out);
 }  // namespace fep3m

@@ -502,6 +502,12 @@ struct ApplyDot {
   int post;
   double* wout = nullptr;
   double invW = 0.0;
+  // box: the solved nodes (Ns per axis from index off) that the packed FP32
+  // residual and its sum take, their scale, or (out64) the FP64 residual of
+  // every node instead
+  int Ns = 0, off = 0;
+  const float* bscale = nullptr;
+  double* out64 = nullptr;
 };
 
 
@@ -582,6 +588,14 @@ __device__ __forceinline__ void st_MK(const T* v, T& sm, T& sk) {
   }
 }
 
+// minus half a stencil's diagonal: what the end rows of an open 1-D matrix
+// lack of the periodic row (one element's part of two equal ones)
+template <class T>
+__device__ __forceinline__ T half_diag(T d) {
+  if constexpr (std::is_same<T, dfv>::value) return {-0.5f * d.h, -0.5f * d.l};
+  else return T(-0.5) * d;
+}
+
 // sum_j M(t, j) u[j]
 template <class T, int t>
 __device__ __forceinline__ T st_M(const T* u) {
@@ -658,14 +672,22 @@ __device__ __forceinline__ T apply_epilogue(int64_t g, T y, T bg, T dg, T xg, T*
 // F32IN (dfv, EPI_RESID: the first refinement sweep, whose iterate is the
 // FP32 correction e over the power-of-two scale s): x points at e (floats),
 // the apply reads the pairs (e / s, 0) and writes them to xo as the iterate.
-template <class T, int EPI, bool DOT = false, bool F32IN = false>
+//
+// BOX (EPI_RESID): the open mesh of a box, N = 3 nb + 1 nodes per axis.
+// Nodes past the ends read as zero, the first and last rows of each 1-D matrix
+// have one element's diagonal, half the periodic one, and the last element
+// step holds the far vertex alone (dt: what is written and summed).  32^3 box
+// (885 k nodes), per residual: six separable FP64 passes 264 us, fused in
+// double-float 59 us.
+template <class T, int EPI, bool DOT = false, bool F32IN = false, bool BOX = false>
 __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
     k_apply_el(int N, int steps, const T* __restrict__ x, T* __restrict__ out, const T* __restrict__ b,
                T* __restrict__ d, T* __restrict__ xo, T c0, T c1, T c2, double* __restrict__ scal, ApplyDot dt,
                int64_t vs) {
   PDL_PROLOGUE
-  static_assert(!DOT || EPI == EPI_Y || EPI == EPI_CHEB || (EPI == EPI_RESID && std::is_same<T, dfv>::value),
-                "fused dots: EPI_Y, EPI_CHEB and the double-float residual");
+  static_assert(!DOT || EPI == EPI_Y || EPI == EPI_CHEB || (EPI == EPI_RESID && (BOX || std::is_same<T, dfv>::value)),
+                "fused dots: EPI_Y, EPI_CHEB, the double-float residual and a box's");
+  static_assert(!BOX || (EPI == EPI_RESID && DOT && !F32IN && !std::is_same<T, float>::value), "box: residuals only");
   static_assert(!F32IN || (EPI == EPI_RESID && std::is_same<T, dfv>::value), "FP32 input: the double-float residual");
   extern __shared__ __align__(16) unsigned char apply_smem_raw[];
   ApplySmem<T, EPI, DOT>& S = *reinterpret_cast<ApplySmem<T, EPI, DOT>*>(apply_smem_raw);
@@ -673,7 +695,7 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
   double dacc = 0.0;
   float facc = 0.f;          // EPI_RESID dot: |r|^2 in FP32
   dfv wacc = {0.f, 0.f};     // EPI_RESID dot with dt.wout: the iterate's integral
-  const int n = N / 3;
+  const int n = BOX ? (N + 2) / 3 : N / 3;
   const int64_t NN = (int64_t)N * N;
   const int x0 = blockIdx.x * AFX, y0 = blockIdx.y * AFY;
   // several vectors (vs: their stride in nodes; scalars in blocks of 64): the z blocks of vector v follow those of v - 1
@@ -694,13 +716,19 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
   }
   const int tid = threadIdx.x;
   float rs = 0.0f;   // power-of-two scale of the refinement residual (FP64, double-float)
-  if constexpr (!std::is_same<T, float>::value) rs = reinterpret_cast<const float*>(scal + SC_DERIVED_F)[SD_SCALE];
+  if constexpr (BOX) rs = dt.bscale ? *dt.bscale : 1.f;
+  else if constexpr (!std::is_same<T, float>::value) rs = reinterpret_cast<const float*>(scal + SC_DERIVED_F)[SD_SCALE];
   float ris = 0.0f;  // F32IN: 1 / s
   if constexpr (F32IN) ris = reinterpret_cast<const float*>(scal + SC_DERIVED_F)[SD_INVSCALE];
   const float* xf = reinterpret_cast<const float*>(x);   // F32IN: the correction e
   auto ldx = [&](int64_t off) -> T {
     if constexpr (F32IN) return T{xf[off] * ris, 0.f};
     else return x[off];
+  };
+  // plane zz of halo column k (BOX: zero outside the box)
+  auto ldz = [&](int zz, int col) -> T {
+    if constexpr (BOX) return col < 0 || (unsigned)zz >= (unsigned)N ? T{} : x[zz * NN + col];
+    else return ldx(zz * NN + col);
   };
   if constexpr (!std::is_same<T, dfv>::value) {
     if (tid < 27) S.dinv[tid] = Cst<T>::Dinv(tid);
@@ -712,12 +740,17 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
   for (int k = 0; k < APL; ++k) {
     const int i = tid + k * AT;
     const int hy = i / AHX, hx = i - hy * AHX;
-    const int gx = ((x0 + hx - 3) % N + N) % N, gy = ((y0 + hy - 3) % N + N) % N;
-    coff[k] = i < ANC ? gy * N + gx : 0;
+    if constexpr (BOX) {
+      const int gx = x0 + hx - 3, gy = y0 + hy - 3;
+      coff[k] = i < ANC && (unsigned)gx < (unsigned)N && (unsigned)gy < (unsigned)N ? gy * N + gx : -1;
+    } else {
+      const int gx = ((x0 + hx - 3) % N + N) % N, gy = ((y0 + hy - 3) % N + N) % N;
+      coff[k] = i < ANC ? gy * N + gx : 0;
+    }
   }
   // window slot s holds plane 3e - 3 + s (wrapped); N >= 9, so one wrap suffices
   int zs = 3 * e0 - 3;
-  if (zs < 0) zs += N;
+  if (!BOX && zs < 0) zs += N;
   // EPI_CHEB0: input c0 D^-1 b, scaled per column and plane type (a halo
   // column's x and y types are hx % 3 and hy % 3: the tile starts on a vertex)
   T fs[EPI == EPI_CHEB0 ? APL : 1][3];
@@ -734,10 +767,10 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
 #pragma unroll
   for (int s = 0; s < 7; ++s) {
     int zz = zs + s;
-    if (zz >= N) zz -= N;
+    if (!BOX && zz >= N) zz -= N;
 #pragma unroll
     for (int k = 0; k < APL; ++k) {
-      w[k][s] = ldx(zz * NN + coff[k]);
+      w[k][s] = ldz(zz, coff[k]);
       if (EPI == EPI_CHEB0) w[k][s] *= fs[k][s % 3];
     }
   }
@@ -755,9 +788,9 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
 #pragma unroll
       for (int s = 0; s < 3; ++s) {
         int zz = zs + 7 + s;
-        if (zz >= N) zz -= N;
+        if (!BOX && zz >= N) zz -= N;
 #pragma unroll
-        for (int k = 0; k < APL; ++k) nx[k][s] = ldx(zz * NN + coff[k]);
+        for (int k = 0; k < APL; ++k) nx[k][s] = ldz(zz, coff[k]);
       }
     }
     if (EPI == EPI_CHEB0 && e > e0) {   // planes 3e + 1 .. 3e + 3 arrived in the previous round
@@ -775,6 +808,7 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
         const int64_t g = (int64_t)(3 * e + p) * NN + (int64_t)gy * N + gx0;
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
+          if (BOX && (gx0 + r >= N || 3 * e + p >= N)) continue;
           cp_async<sizeof(T)>(&S.stg[0][p][x_yy][3 * x_ex + r], (EPI == EPI_Y ? x : b) + g + r);
           if constexpr (NST > 1) cp_async<sizeof(T)>(&S.stg[NST > 1 ? 1 : 0][p][x_yy][3 * x_ex + r], d + g + r);
           if constexpr (NST > 2) cp_async<sizeof(T)>(&S.stg[NST > 2 ? 2 : 0][p][x_yy][3 * x_ex + r], x + g + r);
@@ -791,6 +825,10 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
         st_MK<T, 0>(w[k], m0, k0);
         st_MK<T, 1>(w[k] + 1, m1, k1);
         st_MK<T, 2>(w[k] + 2, m2, k2);
+        if (BOX && (e == 0 || e == n - 1)) {
+          m0 += half_diag<T>(Cst<T>::M(0, 3)) * w[k][3];
+          k0 += half_diag<T>(Cst<T>::K(0, 3)) * w[k][3];
+        }
         (&S.tz[0][0][0])[i] = {m0, k0};
         (&S.tz[1][0][0])[i] = {m1, k1};
         (&S.tz[2][0][0])[i] = {m2, k2};
@@ -808,7 +846,13 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
           u[j] = q.a;
           v[j] = q.b;
         }
-        S.ac[p][3 * y_ey + 0][y_hx] = {st_M<T, 0>(u), st_KM<T, 0>(u, v)};
+        T a0 = st_M<T, 0>(u), c0y = st_KM<T, 0>(u, v);
+        if (BOX && (y0 + 3 * y_ey == 0 || y0 + 3 * y_ey == N - 1)) {
+          a0 += half_diag<T>(Cst<T>::M(0, 3)) * u[3];
+          c0y += half_diag<T>(Cst<T>::K(0, 3)) * u[3];
+          c0y += half_diag<T>(Cst<T>::M(0, 3)) * v[3];
+        }
+        S.ac[p][3 * y_ey + 0][y_hx] = {a0, c0y};
         S.ac[p][3 * y_ey + 1][y_hx] = {st_M<T, 1>(u + 1), st_KM<T, 1>(u + 1, v + 1)};
         S.ac[p][3 * y_ey + 2][y_hx] = {st_M<T, 2>(u + 2), st_KM<T, 2>(u + 2, v + 2)};
       }
@@ -832,6 +876,36 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
         y[0] = st_KM<T, 0>(u, v);
         y[1] = st_KM<T, 1>(u + 1, v + 1);
         y[2] = st_KM<T, 2>(u + 2, v + 2);
+        if constexpr (BOX) {
+          if (gx0 == 0 || gx0 == N - 1) {
+            y[0] += half_diag<T>(Cst<T>::K(0, 3)) * u[3];
+            y[0] += half_diag<T>(Cst<T>::M(0, 3)) * v[3];
+          }
+          const int iy = gy - dt.off, iz = 3 * e + p - dt.off;
+#pragma unroll
+          for (int r = 0; r < 3; ++r) {
+            if (gx0 + r >= N || 3 * e + p >= N) continue;
+            const T bg = S.stg[0][p][x_yy][3 * x_ex + r];
+            float rsd;
+            if constexpr (std::is_same<T, dfv>::value) {
+              dfv df = bg;
+              df += dfv{-y[r].h, -y[r].l};
+              if (dt.out64) dt.out64[g + r] = (double)df.h + (double)df.l;
+              rsd = (df.h + df.l) * rs;
+            } else {
+              const double df = bg - y[r];
+              if (dt.out64) dt.out64[g + r] = df;
+              rsd = (float)(df * (double)rs);
+            }
+            const int ix = gx0 + r - dt.off;
+            if (!dt.out64 && (unsigned)ix < (unsigned)dt.Ns && (unsigned)iy < (unsigned)dt.Ns &&
+                (unsigned)iz < (unsigned)dt.Ns) {
+              reinterpret_cast<float*>(out)[ix + (int64_t)dt.Ns * (iy + (int64_t)dt.Ns * iz)] = rsd;
+              facc = fmaf(rsd, rsd, facc);
+            }
+          }
+          continue;
+        }
         T dsum{};
         float dres = 0.f;
 #pragma unroll
@@ -844,7 +918,7 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
           float rsd = 0.f;
           const T f = apply_epilogue<T, EPI>(g + r, y[r], bg, dg, xg, out, d, xo, c0, c1, c2, dv[r], rs, rsd);
           if constexpr (F32IN) xo[g + r] = T{xf[g + r] * ris, 0.f};   // the iterate after the first sweep
-          if constexpr (DOT && EPI == EPI_RESID) {
+          if constexpr (DOT && EPI == EPI_RESID && !BOX) {
             if (dt.wout) {   // the node weight (1/4 or 3/8 per axis) times the iterate, as a two-product
               const float wn = (r ? 0.375f : 0.25f) * (ty3 ? 0.375f : 0.25f) * (p ? 0.375f : 0.25f);
               const T xv = ldx(g + r);
@@ -868,8 +942,9 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
       for (int s = 0; s < 3; ++s) w[k][4 + s] = nx[k][s];
     }
     zs += 3;
-    if (zs >= N) zs -= N;
+    if (!BOX && zs >= N) zs -= N;
   }
+  if (BOX && dt.out64) return;
   if constexpr (DOT) {
     const unsigned nbv = gridDim.x * gridDim.y * zsb;   // blocks per vector
     const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * (blockIdx.z - vi * zsb));
@@ -897,9 +972,9 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
   }
 }
 
-template <class T, int EPI, bool DOT = false, bool F32IN = false>
+template <class T, int EPI, bool DOT = false, bool F32IN = false, bool BOX = false>
 static cudaError_t apply_set_smem_one() {
-  return cudaFuncSetAttribute(k_apply_el<T, EPI, DOT, F32IN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(k_apply_el<T, EPI, DOT, F32IN, BOX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)sizeof(ApplySmem<T, EPI, DOT>));
 }
 
@@ -916,6 +991,8 @@ static cudaError_t apply_set_smem() {
   if (e == cudaSuccess) e = apply_set_smem_one<dfv, EPI_RESID, true>();
   if (e == cudaSuccess) e = apply_set_smem_one<dfv, EPI_RESID, false, true>();
   if (e == cudaSuccess) e = apply_set_smem_one<dfv, EPI_RESID, true, true>();
+  if (e == cudaSuccess) e = apply_set_smem_one<double, EPI_RESID, true, false, true>();
+  if (e == cudaSuccess) e = apply_set_smem_one<dfv, EPI_RESID, true, false, true>();
   // coarsest-level kernels at N = CP_MAX
   const int smp = 3 * CP_MAX * (CP_MAX + 1) * (int)sizeof(float);
   const int smq = (2 * CP_MAX * (CP_MAX + 1) + 2 * CP_MAX * (CP_PEN + 1)) * (int)sizeof(float);
@@ -2766,6 +2843,42 @@ void solver_destroy(Solver* s) {
   if (s->host_res) cudaFreeHost(s->host_res);
   s->scal = s->red_tmp = s->res64 = s->host_res = nullptr;
   s->red_counter = nullptr;
+}
+
+// ---- the open mesh of a box (box.cu)
+static int box_apply_steps(int N) { return std::min(apply_steps(N), (N + 2) / 3); }
+static dim3 box_apply_grid(int N) {
+  return apply_grid(N + 2, box_apply_steps(N));   // (N + 2) / 3 element steps, the last the far vertex alone
+}
+int box_apply_blocks(int N) {
+  const dim3 g = box_apply_grid(N);
+  return (int)(g.x * g.y * g.z);
+}
+cudaError_t box_apply_setup(const Stencils& st) {
+  upload_constants(st);
+  return apply_set_smem();
+}
+cudaError_t box_apply(const BoxApply& a, cudaStream_t s) {
+  ApplyDot dt = {a.partials, a.counter, a.norm, POST_NONE};
+  dt.Ns = a.Ns;
+  dt.off = a.off;
+  dt.bscale = a.scale;
+  dt.out64 = a.r64;
+  const dim3 g = box_apply_grid(a.N);
+  const int steps = box_apply_steps(a.N);
+  if (a.pairs) {
+    const dfv z = {0.f, 0.f};
+    launch_pdl(k_apply_el<dfv, EPI_RESID, true, false, true>, g, AT, sizeof(ApplySmem<dfv, EPI_RESID, true>), s, a.N,
+               steps, reinterpret_cast<const dfv*>(a.x), reinterpret_cast<dfv*>(a.r),
+               reinterpret_cast<const dfv*>(a.b), (dfv*)nullptr, (dfv*)nullptr, z, z, z, (double*)nullptr, dt,
+               (int64_t)0);
+  } else {
+    launch_pdl(k_apply_el<double, EPI_RESID, true, false, true>, g, AT, sizeof(ApplySmem<double, EPI_RESID, true>), s,
+               a.N, steps, reinterpret_cast<const double*>(a.x), reinterpret_cast<double*>(a.r),
+               reinterpret_cast<const double*>(a.b), (double*)nullptr, (double*)nullptr, 0.0, 0.0, 0.0,
+               (double*)nullptr, dt, (int64_t)0);
+  }
+  return cudaGetLastError();
 }
 
 cudaError_t element_lists(fep3m_ctx* c) {

@@ -26,6 +26,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "df.cuh"
 #include "tc.cuh"
 
 namespace fep3m {
@@ -44,14 +45,6 @@ __device__ __forceinline__ int wrapn(int i, int n) {
 }
 
 template <class T> __device__ __forceinline__ T rsq(T x);
-// the hardware estimate of 1 / sqrt(x) (PTX rsqrt.approx, relative error
-// about 2^-23; subnormal input and output flushed to zero, which the
-// squared distances of distinct charges never are)
-__device__ __forceinline__ float rsqrt_est(float x) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 // 1 / sqrt(x) in FP64 from the FP32 hardware estimate y, refined by one
 // third-order (Householder) step: with e = 1 - x y^2, 1 / sqrt(x) =
 // y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2 / 8 + O(e^3)), and the dropped term is
@@ -1781,13 +1774,18 @@ void pair_tc_table(int n_sr, const double* Hw, uint16_t* out) {
       }
 }
 
-// a box's FP64 mesh potential as hi + lo floats for the FP32 pair kernels
+// a box's FP64 mesh vectors as hi + lo floats
 __global__ void k_phi_hilo(int64_t n, const double* __restrict__ phi, float2* __restrict__ out) {
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (g >= n) return;
   const double v = phi[g];
   const float hi = (float)v;
   out[g] = make_float2(hi, (float)(v - (double)hi));
+}
+
+cudaError_t split_pairs(int64_t n, const double* v, void* out, cudaStream_t s) {
+  FEP3M_CL k_phi_hilo<<<gsz(n), PT, 0, s>>>(n, v, (float2*)out);
+  return cudaGetLastError();
 }
 
 cudaError_t pair_prepare(fep3m_ctx* c) {
