@@ -123,13 +123,14 @@ inline int gsz(int64_t n) { return (int)((n + PT - 1) / PT); }
 
 void free_particles(fep3m_ctx* c) {
   void* p[] = {c->pos_in, c->Q_in, c->cell, c->delta, c->perm, c->ecoord, c->part, c->phi_s, c->E_s, c->w_s,
-               c->psi_s, c->gpsi_s, c->out_tmp, c->Q_s, c->gphi_dev, c->w_s32};
+               c->psi_s, c->gpsi_s, c->out_tmp, c->Q_s, c->gphi_dev, c->w_s32, c->part_pairs};
   for (void* q : p) dfree(q);
   c->pos_in = c->Q_in = c->delta = c->phi_s = c->E_s = c->w_s = c->psi_s = c->gpsi_s = c->out_tmp = c->Q_s =
       c->gphi_dev = nullptr;
   c->cell = c->perm = c->ecoord = nullptr;
   c->part = nullptr;
   c->w_s32 = nullptr;
+  c->part_pairs = nullptr;
   c->cap = 0;
 }
 
@@ -144,6 +145,7 @@ int grow_particles(fep3m_ctx* c, int64_t N) {
   CK(dalloc(&c->perm, N));
   CK(dalloc(&c->ecoord, N));
   CK(cudaMalloc(&c->part, N * es));
+  if (c->precision == FEP3M_FP64) CK(cudaMalloc(&c->part_pairs, N * FEP3M_PAIR_CHARGE_BYTES));
   CK(dalloc(&c->phi_s, N));
   CK(dalloc(&c->E_s, 3 * N));
   CK(dalloc(&c->w_s, N));

@@ -45,6 +45,7 @@
 
 #include "common.cuh"
 #include "df.cuh"
+#include "gridsum.cuh"
 
 namespace fep3m {
 
@@ -128,12 +129,7 @@ __device__ __forceinline__ void negate(df& s) { s = {-s.h, -s.l}; }
 __device__ __forceinline__ void negate(tf& s) { s = {-s.h, -s.m, -s.l}; }
 // s += a, running sums of two threads
 __device__ __forceinline__ void add_part(df& s, df a) { s = df_add(s, a); }
-__device__ __forceinline__ void add_part(tf& s, tf a) {
-  const df t = df_two_sum(s.h, a.h), u = df_two_sum(s.m, a.m), w = df_two_sum(t.l, u.h);
-  s.h = t.h;
-  s.m = w.h;
-  s.l += a.l + (w.l + u.l);
-}
+__device__ __forceinline__ void add_part(tf& s, tf a) { tf_add(s, a); }
 
 // the runs of the block's rows: j0[r] the first sorted charge of row r, pre[r]
 // the charges of the rows before it; returns their number.  By the CTA.
@@ -561,14 +557,12 @@ __device__ __forceinline__ double box_w1(int g, int Nn, const BoxBand& bd) {
 // deterministic FP64 sums: mode 0, sum of squares of v at the solved nodes
 // into *out, with the power of two near the inverse RMS and its inverse into
 // scale[0], scale[1]; mode 1, sum of v over all nodes; mode 2, sum of w3 v
-// over all nodes (w3 the 3-D node integrals).  Per-block partials; the last
-// block to finish adds them in a fixed order.
+// over all nodes (w3 the 3-D node integrals)
 __global__ void __launch_bounds__(BT) k_box_sum(int mode, int Ns, int Nn, int off, BoxBand bd,
                                                 const double* __restrict__ v, double* __restrict__ partial,
                                                 unsigned int* __restrict__ counter, double* __restrict__ out,
                                                 float* __restrict__ scale) {
-  __shared__ double sh[BT / 32];
-  __shared__ bool last;
+  static_assert(BT == 256, "grid_sum256");
   const int64_t len = mode == 0 ? (int64_t)Ns * Ns * Ns : (int64_t)Nn * Nn * Nn;
   double acc = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x) {
@@ -582,37 +576,10 @@ __global__ void __launch_bounds__(BT) k_box_sum(int mode, int Ns, int Nn, int of
       acc = fma(box_w1(x, Nn, bd) * box_w1(y, Nn, bd) * box_w1(z, Nn, bd), v[i], acc);
     }
   }
-  auto block_sum = [&](double a) -> double {   // in thread 0
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
-    __syncthreads();
-    double s = 0.0;
-    if (threadIdx.x == 0)
-      for (int k = 0; k < BT / 32; ++k) s += sh[k];
-    return s;
-  };
-  double s = block_sum(acc);
-  if (threadIdx.x == 0) {
-    partial[blockIdx.x] = s;
-    __threadfence();
-    last = atomicAdd(counter, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  acc = 0.0;
-  for (unsigned k = threadIdx.x; k < gridDim.x; k += BT) acc += ((volatile double*)partial)[k];
-  s = block_sum(acc);
-  if (threadIdx.x != 0) return;
-  *counter = 0u;
-  *out = s;
-  if (mode == 0) {
-    const double rms = sqrt(s / (double)len);
-    int k = rms > 0.0 && isfinite(rms) ? ilogb(rms) : 0;
-    k = max(-100, min(100, k));
-    scale[0] = (float)ldexp(1.0, -k);
-    scale[1] = (float)ldexp(1.0, k);
+  double s;
+  if (grid_sum256(acc, gridDim.x, blockIdx.x, partial, counter, s)) {
+    *out = s;
+    if (mode == 0) rms_scale(s, (double)len, scale);
   }
 }
 

@@ -189,6 +189,7 @@ struct OQParams {
   double bM[6][13];     // 1-D periodic order-p mass row of node type t = g mod p: tap o -> node g + o - p
   double bK[6][13];     // the same for the stiffness
   double wn[6];         // node integrals by type
+  double lden[7];       // 1 / prod_{j != k} (k - j): the equispaced Lagrange functions' denominators
 };
 
 // host-side data of the order-q path (highorder.cpp)
@@ -207,17 +208,22 @@ struct OrderQ {
   double* b = nullptr;        // (p n)^3 load vector (element units)
   double* pb = nullptr;       // the load vector less its neutralising background
   double* phi = nullptr;      // (p n)^3 mesh potential (element units)
-  double* res = nullptr;      // refinement residual
-  double* t[4] = {};          // scratch of the stiffness apply
+  double* t[4] = {};          // scratch of the stiffness apply and the load passes
   float* r32 = nullptr;       // FP32 inner solve: right-hand side, solution, scratch
   float* x32 = nullptr;
   float* w1 = nullptr;
   float* w2 = nullptr;
-  double* S = nullptr;        // n^3 (p+1)^3 screen field at each element's order-p nodes
-  double* H = nullptr;        // U^3 (p+1)^3 node-regrouped tables
-  double* red = nullptr;      // reduction partials
-  double* host_red = nullptr; // pinned: one reduction result
+  double* S = nullptr;        // n^3 (p+1)^3 screen field at each element's order-p nodes, by parity
+  void* H = nullptr;          // the node-regrouped tables by parity block, float pairs
+  void* Cp = nullptr;         // C and r as float pairs, times the context's q_scale
+  void* rp = nullptr;
+  void* amps = nullptr;       // one piece of elements' block amplitudes by parity, float pairs
+  int piece = 0;              // elements per piece
+  double* red = nullptr;      // reduction results and partials (orderq.cu)
+  double* host_red = nullptr; // pinned: the norms of one refinement
+  unsigned int* counter = nullptr;   // last-block counter of the reductions
   FineFDM fdm;
+  int plan = 0;               // refinement sweeps of the last solve: the next one's before its first check
   int sweeps = 0;
   double relres = 0;
 };
@@ -312,6 +318,7 @@ struct fep3m_ctx {
   int* start = nullptr;          // n^3 + 1
   int* fill = nullptr;           // n^3
   void* part = nullptr;          // sorted (t, Q): double4 or float4, N
+  void* part_pairs = nullptr;    // FP64: the same for the singular sums in float pairs (pair.cu)
   void* scan_tmp = nullptr;
   size_t scan_tmp_bytes = 0;
   // element / vertex fields
@@ -379,6 +386,8 @@ struct fep3m_ctx {
   cudaEvent_t ev[11];
   bool ev_init = false;
 };
+
+#define FEP3M_PAIR_CHARGE_BYTES 48   // sizeof a charge of part_pairs
 
 namespace fep3m {
 // host setup (setup.cpp)
@@ -473,9 +482,8 @@ cudaError_t adjoint_vertex(fep3m_ctx* c, cudaStream_t s);
 cudaError_t adjoint_final(fep3m_ctx* c, double gU, double* dpos, double* dQ, double sign, cudaStream_t s);
 // U = 1/2 sum Q phi on stream s (the context's stream when null)
 cudaError_t energy(fep3m_ctx* c, double* U_dev, cudaStream_t s = nullptr);
-// sum_j w_j / r and sum_j w_j (x_j - x_t) / r^3 over each target's block, j != t
-// (sorted order; physical units)
-cudaError_t singular_sums(fep3m_ctx* c, const double* w, double* psi, double* gpsi, cudaStream_t s);
+// sum_j Q_j / r over each charge's block, j != t, into phi_s (sorted order; physical units)
+cudaError_t singular_sums(fep3m_ctx* c, cudaStream_t s);
 // the order-q path (orderq.cu)
 int orderq_create(fep3m_ctx* c);
 void orderq_destroy(fep3m_ctx* c);

@@ -33,6 +33,10 @@ __device__ __forceinline__ df df_sqr(df a) {
   const float p = a.h * a.h;
   return {p, fmaf(a.h + a.h, a.l, fmaf(a.h, a.h, -p))};
 }
+__device__ __forceinline__ df df_mul(df a, df b) {
+  const float p = a.h * b.h;
+  return {p, fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)))};
+}
 // s += a b, s unnormalised (h + l the running value)
 __device__ __forceinline__ void df_fma(df& s, df a, df b) {
   const float p = a.h * b.h;
@@ -40,6 +44,12 @@ __device__ __forceinline__ void df_fma(df& s, df a, df b) {
   const df t = df_two_sum(s.h, p);
   s.h = t.h;
   s.l += t.l + e;
+}
+// s += a, s unnormalised
+__device__ __forceinline__ void df_acc(df& s, df a) {
+  const df t = df_two_sum(s.h, a.h);
+  s.h = t.h;
+  s.l += t.l + a.l;
 }
 // the hardware estimate of 1 / sqrt(x) (PTX rsqrt.approx, relative error
 // about 2^-23; subnormals flushed to zero)
@@ -106,6 +116,19 @@ __device__ __forceinline__ void df_fma(tf& s, df a, df b) {
   s.h = t.h;
   s.m = w.h;
   s.l += w.l + u.l;
+}
+// s += a: a pair, or another running value
+__device__ __forceinline__ void tf_add(tf& s, df a) {
+  const df t = df_two_sum(s.h, a.h), u = df_two_sum(t.l, a.l), w = df_two_sum(s.m, u.h);
+  s.h = t.h;
+  s.m = w.h;
+  s.l += w.l + u.l;
+}
+__device__ __forceinline__ void tf_add(tf& s, tf a) {
+  const df t = df_two_sum(s.h, a.h), u = df_two_sum(s.m, a.m), w = df_two_sum(t.l, u.h);
+  s.h = t.h;
+  s.m = w.h;
+  s.l += a.l + (w.l + u.l);
 }
 __device__ __forceinline__ double df_value(tf a) { return (double)a.h + ((double)a.m + (double)a.l); }
 

@@ -103,76 +103,83 @@ constexpr int BX = 4, BY = 4, BZ = 4, BE = BX * BY * BZ;   // 64 elements per br
 constexpr int OCH = 32;                                      // offsets per chunk
 constexpr int MAXRUN = 2 * 81;                               // rows of the block (n_sr <= 4), 2 runs each
 
-// source weights of the singular sum: the charge itself, or an adjoint weight array
-template <class T> struct WeightQ {
-  __device__ __forceinline__ T operator()(int, const typename vec4<T>::type& pj) const { return pj.w; }
-};
-template <class T> struct WeightArr {
-  const double* w;
-  __device__ __forceinline__ T operator()(int j, const typename vec4<T>::type&) const { return (T)w[j]; }
-};
-
 template <class T>
 __device__ __forceinline__ void warp_sum(T& v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
 }
 
-// singular sum for one target over its block, lanes of one warp in parallel.
-// W(j) = source weight (Q_j, or the adjoint weight); returns sum W/r and
-// sum W (x_j - x_t)/r^3 in every lane.
-template <class T, bool GRAD, class WeightF>
+// The rows (y, z) of a target's block as runs of consecutive sorted charges,
+// two where a row wraps: run k's first charge in runs[k], the charges of the
+// runs before it in pre[k]; returns (and pre[2 rows] holds) their number.  By a warp.
+__device__ __forceinline__ int warp_runs(int n, int n_sr, int ex, int ey, int ez, const int* __restrict__ start,
+                                         int* runs /* MAXRUN */, int* pre /* MAXRUN + 1 */) {
+  const int lane = threadIdx.x & 31, nb = 2 * n_sr + 1, rows = nb * nb;
+  int carry = 0;
+  for (int r0 = 0; r0 < rows; r0 += 32) {
+    const int r = r0 + lane;
+    int a0 = 0, a1 = 0, b0 = 0, b1 = 0;
+    if (r < rows) {
+      const int dy = r % nb - n_sr, dz = r / nb - n_sr;
+      const int yy = wrapn(ey + dy, n), zz = wrapn(ez + dz, n);
+      const int64_t rowbase = (int64_t)n * (yy + (int64_t)n * zz);
+      const int x0 = ex - n_sr, x1 = ex + n_sr;
+      if (x0 < 0) {
+        a0 = start[rowbase + x0 + n]; a1 = start[rowbase + n];        // x0+n .. n-1
+        b0 = start[rowbase];          b1 = start[rowbase + x1 + 1];   // 0 .. x1
+      } else if (x1 >= n) {
+        a0 = start[rowbase + x0];     a1 = start[rowbase + n];        // x0 .. n-1
+        b0 = start[rowbase];          b1 = start[rowbase + x1 - n + 1];
+      } else {
+        a0 = start[rowbase + x0];     a1 = start[rowbase + x1 + 1];
+      }
+    }
+    const int ca = a1 - a0, cb = b1 - b0;
+    int x = ca + cb;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += v;
+    }
+    if (r < rows) {
+      runs[2 * r] = a0;
+      runs[2 * r + 1] = b0;
+      pre[2 * r] = carry + x - ca - cb;
+      pre[2 * r + 1] = carry + x - cb;
+    }
+    carry += __shfl_sync(0xffffffffu, x, 31);
+  }
+  if (lane == 0) pre[2 * rows] = carry;
+  __syncwarp();
+  return carry;
+}
+
+// the source's element less the target's, the nearest image
+__device__ __forceinline__ int block_delta(int d, int n, int n_sr) {
+  return d > n_sr ? d - n : (d < -n_sr ? d + n : d);
+}
+
+// Singular sum for one target over its block, lanes of one warp in parallel.
+// w[j]: source weights; returns sum w/r and (GRAD) sum w (x_j - x_t)/r^3 in
+// every lane, physical units, compensated per lane.
+template <class T, bool GRAD>
 __device__ __forceinline__ void warp_singular(int n, int n_sr, T h, int ex, int ey, int ez, int slot,
                                               typename vec4<T>::type pt, const int* __restrict__ start,
                                               const typename vec4<T>::type* __restrict__ part,
-                                              const int* __restrict__ ecoord, int* runs /* 2*MAXRUN */,
-                                              int* pre /* MAXRUN+1 */, WeightF W, T out[4]) {
-  const int lane = threadIdx.x & 31;
-  const int nb = 2 * n_sr + 1, rows = nb * nb;
-  // runs of consecutive element ids (split where the row wraps)
-  for (int r = lane; r < rows; r += 32) {
-    const int dy = r % nb - n_sr, dz = r / nb - n_sr;
-    const int yy = wrapn(ey + dy, n), zz = wrapn(ez + dz, n);
-    const int64_t rowbase = (int64_t)n * (yy + (int64_t)n * zz);
-    int x0 = ex - n_sr, x1 = ex + n_sr;
-    int a0, a1, b0 = 0, b1 = 0;
-    if (x0 < 0) {
-      a0 = start[rowbase + x0 + n]; a1 = start[rowbase + n];        // x0+n .. n-1
-      b0 = start[rowbase];          b1 = start[rowbase + x1 + 1];   // 0 .. x1
-    } else if (x1 >= n) {
-      a0 = start[rowbase + x0];     a1 = start[rowbase + n];        // x0 .. n-1
-      b0 = start[rowbase];          b1 = start[rowbase + x1 - n + 1];
-    } else {
-      a0 = start[rowbase + x0];     a1 = start[rowbase + x1 + 1];
-    }
-    runs[4 * r + 0] = a0; runs[4 * r + 1] = a1 - a0;
-    runs[4 * r + 2] = b0; runs[4 * r + 3] = b1 - b0;
-  }
-  __syncwarp();
-  if (lane == 0) {
-    int acc = 0;
-    for (int k = 0; k < 2 * rows; ++k) {
-      pre[k] = acc;
-      acc += runs[2 * k + 1];
-    }
-    pre[2 * rows] = acc;
-  }
-  __syncwarp();
-  const int total = pre[2 * rows];
+                                              const int* __restrict__ ecoord, int* runs, int* pre,
+                                              const double* __restrict__ w, T out[4]) {
+  const int total = warp_runs(n, n_sr, ex, ey, ez, start, runs, pre);
   Acc<T> ps, fx, fy, fz;
   int k = 0;
-  for (int f = lane; f < total; f += 32) {
+  for (int f = threadIdx.x & 31; f < total; f += 32) {
     while (pre[k + 1] <= f) ++k;
-    const int j = runs[2 * k] + (f - pre[k]);
+    const int j = runs[k] + (f - pre[k]);
     if (j == slot) continue;
     const typename vec4<T>::type pj = part[j];
     const int ec = ecoord[j];
-    int dx = (ec & 1023) - ex, dy = ((ec >> 10) & 1023) - ey, dz = (ec >> 20) - ez;
-    dx = dx > n_sr ? dx - n : (dx < -n_sr ? dx + n : dx);
-    dy = dy > n_sr ? dy - n : (dy < -n_sr ? dy + n : dy);
-    dz = dz > n_sr ? dz - n : (dz < -n_sr ? dz + n : dz);
+    const int dx = block_delta((ec & 1023) - ex, n, n_sr), dy = block_delta(((ec >> 10) & 1023) - ey, n, n_sr),
+              dz = block_delta((ec >> 20) - ez, n, n_sr);
     const T rx = (T(dx) + (pj.x - pt.x)) * h, ry = (T(dy) + (pj.y - pt.y)) * h, rz = (T(dz) + (pj.z - pt.z)) * h;
     const T ir = rsq<T>(rx * rx + ry * ry + rz * rz);
-    const T wj = W(j, pj);
+    const T wj = (T)w[j];
     ps.add(wj * ir);
     if (GRAD) {
       const T f3 = wj * ir * ir * ir;
@@ -185,8 +192,137 @@ __device__ __forceinline__ void warp_singular(int n, int n_sr, T h, int ex, int 
   out[1] = fx.get();
   out[2] = fy.get();
   out[3] = fz.get();
-  for (int i = 0; i < 4; ++i) warp_sum(out[i]);
+  for (int i = 0; i < (GRAD ? 4 : 1); ++i) warp_sum(out[i]);
   __syncwarp();
+}
+
+// ---------------------------------------------------- FP64 singular sums
+// An FP64 operation costs as much as 64 FP32 ones on this GPU, so the charges'
+// own singular sums of an FP64 context run in float pairs.  A charge for them:
+// per axis its local coordinate tau = a + bh + bl, a the multiple of 2^-20
+// nearest tau and bh + bl the rest (33 bits), so that a difference of two
+// coordinates plus a whole number is a float (exactly) plus a small pair; and
+// the charge times a power of two near the inverse mean charge
+// (fep3m_ctx::q_scale), so that low words stay normal numbers.
+struct __align__(16) PairCharge {
+  float a[3], bh[3], bl[3];
+  df q;
+  float pad;
+};
+static_assert(sizeof(PairCharge) == FEP3M_PAIR_CHARGE_BYTES, "the context's allocation");
+
+__global__ void k_pair_charges(int64_t N, const vec4<double>::type* __restrict__ part, double scale,
+                               PairCharge* __restrict__ out) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  const vec4<double>::type p = part[i];
+  const double x[3] = {p.x, p.y, p.z};
+  PairCharge c;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const double a = rint(x[k] * 1048576.0) * (1.0 / 1048576.0);
+    const df b = df_split(x[k] - a);
+    c.a[k] = (float)a;
+    c.bh[k] = b.h;
+    c.bl[k] = b.l;
+  }
+  c.q = df_split(p.w * scale);
+  c.pad = 0.f;
+  out[i] = c;
+}
+
+// x_s - x_t along axis k, the source's element d elements on
+__device__ __forceinline__ df charge_diff(const PairCharge& s, const PairCharge& t, int k, float d) {
+  const float A = (s.a[k] - t.a[k]) + d;   // exact: at most 23 bits
+  const df b = df_two_sum(s.bh[k], -t.bh[k]), v = df_two_sum(A, b.h);
+  return {v.h, v.l + (b.l + (s.bl[k] - t.bl[k]))};
+}
+
+// One warp per target: sum Q / r into phi_s, (GRAD) sum Q (x_j - x_t) / r^3
+// into E_s, and half of them to psi and gpsi when given (the singular adjoint
+// for the energy's weights Q / 2).  A lane sums sixteen charges at a time in
+// pairs (element units) and those sums in three floats; a distance outside the
+// pairs' range (df_in_range) takes FP64.  About 160 FP32 operations per pair;
+// bound by FP32 issue and, for few targets, by the latency of the loads.
+// 4000 charges, q = 2, potentials: 266 -> 42 us.
+template <bool GRAD>
+__global__ void __launch_bounds__(PT) k_singular64(int64_t N, int n, int n_sr, double h, double inv_scale,
+                                                   const int* __restrict__ start, const PairCharge* __restrict__ ch,
+                                                   const int* __restrict__ ecoord, double* __restrict__ phi_s,
+                                                   double* __restrict__ E_s, double* __restrict__ psi,
+                                                   double* __restrict__ gpsi) {
+  constexpr int NS = GRAD ? 4 : 1;
+  __shared__ int runs_all[PT / 32][MAXRUN];
+  __shared__ int pre_all[PT / 32][MAXRUN + 1];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t t = blockIdx.x * (int64_t)(PT / 32) + warp;
+  if (t >= N) return;
+  int *runs = runs_all[warp], *pre = pre_all[warp];
+  const int et = ecoord[t], ex = et & 1023, ey = (et >> 10) & 1023, ez = et >> 20;
+  const PairCharge ct = ch[t];
+  const int total = warp_runs(n, n_sr, ex, ey, ez, start, runs, pre);
+  tf tot[NS] = {};
+  double far[NS] = {};
+  int k = 0;
+  for (int f0 = lane; f0 < total; f0 += 32 * 16) {
+    df s[NS] = {};
+#pragma unroll 2
+    for (int f = f0; f < min(total, f0 + 32 * 16); f += 32) {
+      while (pre[k + 1] <= f) ++k;
+      const int j = runs[k] + (f - pre[k]);
+      if (j == (int)t) continue;
+      const PairCharge cj = ch[j];
+      const int ec = ecoord[j];
+      const df dx = charge_diff(cj, ct, 0, (float)block_delta((ec & 1023) - ex, n, n_sr)),
+               dy = charge_diff(cj, ct, 1, (float)block_delta(((ec >> 10) & 1023) - ey, n, n_sr)),
+               dz = charge_diff(cj, ct, 2, (float)block_delta((ec >> 20) - ez, n, n_sr));
+      const df r2 = df_add(df_add(df_sqr(dx), df_sqr(dy)), df_sqr(dz));
+      if (df_in_range(r2)) {
+        const df ir = df_rsqrt<true>(r2);
+        const df w = df_mul(cj.q, ir);
+        df_acc(s[0], w);
+        if constexpr (GRAD) {
+          const df g = df_mul(w, df_sqr(ir));
+          df_fma(s[1], g, dx);
+          df_fma(s[2], g, dy);
+          df_fma(s[3], g, dz);
+        }
+      } else {
+        const double ir = 1.0 / sqrt(df_value(r2)), w = df_value(cj.q) * ir;
+        far[0] += w;
+        if constexpr (GRAD) {
+          const double g = w * ir * ir;
+          far[1] += g * df_value(dx);
+          far[2] += g * df_value(dy);
+          far[3] += g * df_value(dz);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NS; ++i) tf_add(tot[i], s[i]);
+  }
+#pragma unroll
+  for (int i = 0; i < NS; ++i)
+    for (int o = 16; o > 0; o >>= 1)
+      tf_add(tot[i], tf{__shfl_xor_sync(0xffffffffu, tot[i].h, o), __shfl_xor_sync(0xffffffffu, tot[i].m, o),
+                        __shfl_xor_sync(0xffffffffu, tot[i].l, o)});
+  double out = 0.0;   // lane i takes sum i
+#pragma unroll
+  for (int i = 0; i < NS; ++i) {
+    // (the FP64 sums are zero unless some lane met such a distance; NaN counts as met)
+    if (__any_sync(0xffffffffu, far[i] != 0.0)) warp_sum(far[i]);
+    if (lane == i) out = df_value(tot[i]) + far[i];
+  }
+  if (lane >= NS) return;
+  const double ih = 1.0 / h;
+  out *= inv_scale * (lane == 0 ? ih : ih * ih);
+  if (lane == 0) {
+    phi_s[t] = out;
+    if (psi) psi[t] = 0.5 * out;
+  } else {
+    E_s[3 * t + lane - 1] = out;
+    if (gpsi) gpsi[3 * t + lane - 1] = 0.5 * out;
+  }
 }
 
 // Extended vertex field: per axis SW = 3 BX + 2 n_sr - 1 slots, the first
@@ -1450,27 +1586,28 @@ __global__ void __launch_bounds__(32 * AV_WARPS) k_adj_vertex(int n, int z0, int
   *dst = first ? acc_value(s) : *dst + acc_value(s);
 }
 
-template <class T>
+template <class T, bool GRAD>
 __global__ void __launch_bounds__(PT) k_pair_adj_warp(int64_t N, int n, int n_sr, T h, const int* __restrict__ start,
                                                       const typename vec4<T>::type* __restrict__ part,
                                                       const int* __restrict__ ecoord, const double* __restrict__ w,
                                                       double* __restrict__ psi, double* __restrict__ gpsi) {
-  __shared__ int runs_all[8 * 2 * MAXRUN];
-  __shared__ int pre_all[8 * (MAXRUN + 1)];
+  __shared__ int runs_all[PT / 32][MAXRUN];
+  __shared__ int pre_all[PT / 32][MAXRUN + 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t t = blockIdx.x * (int64_t)(PT / 32) + warp;
   if (t >= N) return;
   const typename vec4<T>::type pt = part[t];
   const int ec = ecoord[t];
   T sg[4];
-  WeightArr<T> wf{w};
-  warp_singular<T, true>(n, n_sr, h, ec & 1023, (ec >> 10) & 1023, ec >> 20, (int)t, pt, start, part, ecoord,
-                         runs_all + warp * 2 * MAXRUN, pre_all + warp * (MAXRUN + 1), wf, sg);
+  warp_singular<T, GRAD>(n, n_sr, h, ec & 1023, (ec >> 10) & 1023, ec >> 20, (int)t, pt, start, part, ecoord,
+                         runs_all[warp], pre_all[warp], w, sg);
   if (lane == 0) {
     psi[t] = (double)sg[0];
-    gpsi[3 * t + 0] = (double)sg[1];
-    gpsi[3 * t + 1] = (double)sg[2];
-    gpsi[3 * t + 2] = (double)sg[3];
+    if (GRAD) {
+      gpsi[3 * t + 0] = (double)sg[1];
+      gpsi[3 * t + 1] = (double)sg[2];
+      gpsi[3 * t + 2] = (double)sg[3];
+    }
   }
 }
 
@@ -1901,12 +2038,12 @@ cudaError_t adjoint_sweeps(fep3m_ctx* c, cudaStream_t s, bool singular) {
   if (c->precision == FEP3M_MIXED) {
     e = screen_adjoint<float>(c, (const float*)c->W_el, c->Ha64, (double*)c->A_el);
     if (e == cudaSuccess && singular)
-      FEP3M_CL k_pair_adj_warp<float><<<(unsigned)((N + 7) / 8), PT, 0, s>>>(N, n, c->n_sr, (float)c->h, c->start,
+      FEP3M_CL k_pair_adj_warp<float, true><<<(unsigned)((N + 7) / 8), PT, 0, s>>>(N, n, c->n_sr, (float)c->h, c->start,
                                                          (const float4*)c->part, c->ecoord, c->w_s, c->psi_s, c->gpsi_s);
   } else {
     e = screen_adjoint<double>(c, (const double*)c->W_el, c->Hw64, (double*)c->A_el);
     if (e == cudaSuccess && singular)
-      FEP3M_CL k_pair_adj_warp<double><<<(unsigned)((N + 7) / 8), PT, 0, s>>>(N, n, c->n_sr, c->h, c->start,
+      FEP3M_CL k_pair_adj_warp<double, true><<<(unsigned)((N + 7) / 8), PT, 0, s>>>(N, n, c->n_sr, c->h, c->start,
                                                           (const vec4<double>::type*)c->part, c->ecoord, c->w_s,
                                                           c->psi_s, c->gpsi_s);
   }
@@ -1921,16 +2058,24 @@ cudaError_t adjoint_vertex(fep3m_ctx* c, cudaStream_t s) {
   return vertex_adjoint(c, c->lam64, c->mu_v, L0.t1, L0.t2, s);
 }
 
-cudaError_t singular_sums(fep3m_ctx* c, const double* w, double* psi, double* gpsi, cudaStream_t s) {
+// the charges' singular sums of an FP64 context into phi_s (and, with grad, E_s;
+// half: also half of them into psi_s and gpsi_s)
+static cudaError_t singular64(fep3m_ctx* c, bool grad, bool half, cudaStream_t s) {
   const int64_t N = c->N;
-  if (c->precision == FEP3M_MIXED)
-    FEP3M_CL k_pair_adj_warp<float><<<(unsigned)((N + 7) / 8), PT, 0, s>>>(N, c->n, c->n_sr, (float)c->h, c->start,
-                                                                           (const float4*)c->part, c->ecoord, w, psi,
-                                                                           gpsi);
-  else
-    FEP3M_CL k_pair_adj_warp<double><<<(unsigned)((N + 7) / 8), PT, 0, s>>>(N, c->n, c->n_sr, c->h, c->start,
-                                                                            (const vec4<double>::type*)c->part,
-                                                                            c->ecoord, w, psi, gpsi);
+  PairCharge* ch = (PairCharge*)c->part_pairs;
+  FEP3M_CL k_pair_charges<<<gsz(N), PT, 0, s>>>(N, (const vec4<double>::type*)c->part, c->q_scale, ch);
+  double *psi = half ? c->psi_s : nullptr, *gpsi = half ? c->gpsi_s : nullptr;
+  auto k = grad ? k_singular64<true> : k_singular64<false>;
+  FEP3M_CL k<<<(unsigned)((N + 7) / 8), PT, 0, s>>>(N, c->n, c->n_sr, c->h, 1.0 / c->q_scale, c->start, ch, c->ecoord,
+                                                    c->phi_s, c->E_s, psi, gpsi);
+  return cudaGetLastError();
+}
+
+cudaError_t singular_sums(fep3m_ctx* c, cudaStream_t s) {
+  const int64_t N = c->N;
+  if (c->precision == FEP3M_FP64) return singular64(c, false, false, s);
+  FEP3M_CL k_pair_adj_warp<float, false><<<(unsigned)((N + 7) / 8), PT, 0, s>>>(
+      N, c->n, c->n_sr, (float)c->h, c->start, (const float4*)c->part, c->ecoord, c->Q_s, c->phi_s, nullptr);
   return cudaGetLastError();
 }
 
