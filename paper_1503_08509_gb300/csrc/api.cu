@@ -405,7 +405,8 @@ const char* fep3m_strerror(int s) {
 void fep3m_destroy(fep3m_ctx* c) {
   if (!c) return;
   free_particles(c);
-  void* p[] = {c->Hw64, c->count, c->start, c->fill, c->scan_tmp, c->C, c->rv, c->Cv, c->b64, c->phi64,
+  void* p[] = {c->HP, c->Vc, c->count, c->start, c->fill, c->scan_tmp, c->C,
+               c->precision == FEP3M_MIXED ? nullptr : c->rv, c->Cv, c->b64, c->phi64,
                c->res64, c->scal, c->iflags, c->phi_hl, c->W_el, c->A_el, c->mu_v, c->Gscr, c->Hb, c->HbA,
                c->Hdf, c->red_tmp, c->red_counter, c->D_adj, c->Ha64, c->H0df, c->Wsum};
   for (void* q : p) dfree(q);
@@ -520,14 +521,17 @@ int fep3m_create(const fep3m_config* cfg, void* stream, fep3m_ctx** out) {
   if (c->precision == FEP3M_MIXED) {
     pair_relative_table(c->n_sr, Hw.data(), Hrel.data());
     pair_adjoint_table(c->n_sr, Hw.data(), Hd.data(), H0.data());
-  } else {
-    Hrel = Hw;
   }
-  if ((st = from_cuda(dalloc(&c->Hw64, Hw.size()))) != FEP3M_OK) return fail(st);
-  cudaMemcpy(c->Hw64, Hw.data(), Hw.size() * 8, cudaMemcpyHostToDevice);
-  if (c->precision == FEP3M_FP64 || (cfg->flags & FEP3M_CUDA_CORES)) {
+  if (c->precision == FEP3M_FP64) {
+    const int kh = c->n_sr + 1;
+    std::vector<float> hp((size_t)2 * 64 * kh * kh * kh);
+    pair_parity_table(c->n_sr, Hw.data(), hp.data());
+    if ((st = from_cuda(cudaMalloc(&c->HP, hp.size() * 4))) != FEP3M_OK) return fail(st);
+    cudaMemcpy(c->HP, hp.data(), hp.size() * 4, cudaMemcpyHostToDevice);
+  }
+  if (c->precision == FEP3M_MIXED && (cfg->flags & FEP3M_CUDA_CORES)) {
     // hi = fl32(H), lo = fl32(H - hi): the operand pairs of the double-float
-    // screen contraction on the CUDA cores (MIXED: of the relative table)
+    // screen contraction on the CUDA cores (of the relative table)
     std::vector<float> hdf(2 * Hrel.size());
     for (size_t i = 0; i < Hrel.size(); ++i) {
       hdf[2 * i] = (float)Hrel[i];
@@ -562,8 +566,9 @@ int fep3m_create(const fep3m_config* cfg, void* stream, fep3m_ctx** out) {
   if ((e = dalloc(&c->count, ne)) != cudaSuccess || (e = dalloc(&c->start, ne + 1)) != cudaSuccess ||
       (e = dalloc(&c->fill, ne)) != cudaSuccess ||
       (e = cudaMalloc(&c->scan_tmp, scan_tmp_bytes(ne))) != cudaSuccess ||
-      (e = cudaMalloc(&c->C, ne * 8 * es)) != cudaSuccess || (e = cudaMalloc(&c->rv, ne * es)) != cudaSuccess ||
-      (e = cudaMalloc(&c->Cv, ne * 8 * es)) != cudaSuccess ||
+      (e = cudaMalloc(&c->C, ne * 8 * es)) != cudaSuccess || (e = cudaMalloc(&c->Vc, 27 * ne * es)) != cudaSuccess ||
+      (c->precision == FEP3M_FP64 && (e = cudaMalloc(&c->rv, ne * es)) != cudaSuccess) ||
+      (box && (e = cudaMalloc(&c->Cv, ne * 8 * es)) != cudaSuccess) ||
       (e = dalloc(&c->b64, 2 * nodes)) != cudaSuccess || (e = dalloc(&c->phi64, 2 * nodes)) != cudaSuccess ||
       (e = dalloc(&c->res64, nodes)) != cudaSuccess || (e = dalloc(&c->scal, 64)) != cudaSuccess ||
       (e = dalloc(&c->iflags, 16)) != cudaSuccess || (e = cudaMalloc(&c->W_el, ne * 64 * es)) != cudaSuccess ||
@@ -576,6 +581,7 @@ int fep3m_create(const fep3m_config* cfg, void* stream, fep3m_ctx** out) {
   // paired mesh solve takes both at one stride
   c->g64 = c->b64 + nodes;
   c->lam64 = c->phi64 + nodes;
+  if (c->precision == FEP3M_MIXED) c->rv = c->Vc;
   // MIXED: the element weight sums; a box's hi + lo copy of its FP64 mesh potential (the periodic
   // solver's output is float pairs already)
   if (c->precision == FEP3M_MIXED &&

@@ -301,9 +301,7 @@ struct fep3m_ctx {
   double L = 1, h = 1, inv_h = 1;
   int precision = FEP3M_FP64;
   fep3m::Stencils st;
-  // kept FE table (host copy) and its device copy in [offset][node] layout
-  std::vector<double> table_host;
-  double* Hw64 = nullptr;
+  std::vector<double> table_host;   // kept FE table
   // particles
   int64_t N = 0, cap = 0;
   double q_scale = 1;            // power of two near the inverse mean |Q| of the charges last set
@@ -323,8 +321,10 @@ struct fep3m_ctx {
   size_t scan_tmp_bytes = 0;
   // element / vertex fields
   void* C = nullptr;             // n^3 * 8 (T)
-  void* rv = nullptr;            // n^3 vertex density (T)
-  void* Cv = nullptr;            // n^3 * 8 (T): C regrouped by vertex, Cv[v][k] = C[v - k][k]
+  void* rv = nullptr;            // n^3 vertex density (T; MIXED: the first n^3 values of Vc)
+  void* Vc = nullptr;            // 27 n^3: the density's partial sums by class (k_vertex_density): FP32, or in
+                                 // FP64 contexts float pairs times q_scale
+  void* Cv = nullptr;            // box: n^3 * 8 (T): C regrouped by vertex, Cv[v][k] = C[v - k][k]
   // fine-level FP64 vectors
   // the periodic mesh vectors hold FP64 values, or in MIXED float pairs h + l
   // (the mixed solver's format, 8 bytes a node as well); a box's are FP64
@@ -354,8 +354,9 @@ struct fep3m_ctx {
   void* Gscr = nullptr;          // screen field at each brick element's 64 nodes, bricks * 4096 (T)
   void* Hb = nullptr;            // bf16 pieces of the table for the tensor-core contraction (MIXED)
   void* HbA = nullptr;           // the same for the screen adjoint's contraction (MIXED)
-  void* Hdf = nullptr;           // hi + lo float pairs of the table (MIXED: of Hrel), the double-float
+  void* Hdf = nullptr;           // MIXED with FEP3M_CUDA_CORES: hi + lo float pairs of Hrel, the double-float
                                  // screen contraction on the CUDA cores
+  void* HP = nullptr;            // FP64: the table by parity as float pairs (pair_parity_table)
   double* Ha64 = nullptr;        // MIXED: the screen adjoint's table relative to node 0 (pair_adjoint_table)
   void* H0df = nullptr;          // MIXED: H(o, 0) per vertex offset as hi + lo floats
   void* Wsum = nullptr;          // MIXED: per element, the sum of the adjoint weights as hi + lo floats
@@ -406,7 +407,7 @@ double estimate_lmax(const Stencils& st, int n);
 
 // device launches (return cudaGetLastError-style codes)
 cudaError_t bin_particles(fep3m_ctx* c, const double* pos, const double* Q, int use_fp32);
-// screen lists C and the vertex density (and its by-vertex copy Cv) of the binned charges
+// screen lists C and the vertex density (with its partial sums by class) of the binned charges
 cudaError_t element_lists(fep3m_ctx* c);
 cudaError_t assemble_forward(fep3m_ctx* c);
 // nv: right-hand sides the refinement buffers hold (2 for the paired solve, which
@@ -461,6 +462,8 @@ void pair_adj_table(int n_sr, const double* Hw, uint16_t* out);
 // floats, 2 per offset)
 void pair_relative_table(int n_sr, const double* Hw, double* Hrel);
 void pair_adjoint_table(int n_sr, const double* Hw, double* Hd, float* H0);
+// the FP64 path's table by parity, as hi + lo floats (2 x 64 (n_sr + 1)^3)
+void pair_parity_table(int n_sr, const double* Hw, float* out);
 // energy_adjoint: also leave half the singular sums in psi_s / gpsi_s (the
 // singular adjoint of the energy's weights Q / 2)
 cudaError_t pair_screen(fep3m_ctx* c, int want_grad, cudaStream_t s, bool energy_adjoint);

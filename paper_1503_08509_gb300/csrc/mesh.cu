@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "df.cuh"
 #include "tc.cuh"
 
 namespace fep3m {
@@ -123,23 +124,46 @@ __global__ void k_elem_coeff(int64_t ne, const int* __restrict__ start, const in
   for (int k = 0; k < 8; ++k) C[e * 8 + k] = acc[k];
 }
 
-// vertex density r_v = sum_k C[v - k][k], and the same eight terms stored by
-// vertex (Cv[v][k]) for the short-range kernel's partial (block-boundary) sums
+// Vertex density r_v = sum_k C[v - k][k], and for the short-range kernels the
+// partial sums that a vertex on a block's boundary has: along each axis both
+// corners (class 0), corner 1 only (1) or corner 0 only (2), Vc[cx + 3 cy + 9
+// cz][v], class 0 the density itself.  A vertex is at such a place of up to
+// eight blocks' boundaries, so the sums are formed here once instead of by each
+// block.  MIXED: Vc in FP32; FP64: Vc as float pairs times scale, the density in
+// FP64.  Cv (a box's): the eight terms by vertex.
 template <class T>
-__global__ void k_vertex_density(int n, const T* __restrict__ C, T* __restrict__ rv, T* __restrict__ Cv) {
+__global__ void k_vertex_density(int n, const T* __restrict__ C, double* __restrict__ rv, void* __restrict__ Vc,
+                                 T* __restrict__ Cv, double scale) {
   int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t ne = (int64_t)n * n * n;
   if (v >= ne) return;
   const int vx = (int)(v % n), vy = (int)((v / n) % n), vz = (int)(v / ((int64_t)n * n));
-  T acc = T(0);
+  T c[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     int ex = wrapi(vx - (k & 1), n), ey = wrapi(vy - ((k >> 1) & 1), n), ez = wrapi(vz - (k >> 2), n);
-    const T ck = C[(ex + (int64_t)n * (ey + (int64_t)n * ez)) * 8 + k];
-    Cv[v * 8 + k] = ck;
-    acc += ck;
+    c[k] = C[(ex + (int64_t)n * (ey + (int64_t)n * ez)) * 8 + k];
+    if (Cv) Cv[v * 8 + k] = c[k];
   }
-  rv[v] = acc;
+#pragma unroll
+  for (int q = 0; q < 27; ++q) {
+    const int cx = q % 3, cy = (q / 3) % 3, cz = q / 9;
+    T acc = T(0);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int kx = k & 1, ky = (k >> 1) & 1, kz = k >> 2;
+      if ((cx == 1 && !kx) || (cx == 2 && kx) || (cy == 1 && !ky) || (cy == 2 && ky) || (cz == 1 && !kz) ||
+          (cz == 2 && kz))
+        continue;
+      acc += c[k];
+    }
+    if constexpr (sizeof(T) == 8) {
+      if (q == 0) rv[v] = acc;
+      static_cast<df*>(Vc)[q * ne + v] = df_split(acc * scale);
+    } else {
+      static_cast<float*>(Vc)[q * ne + v] = acc;
+    }
+  }
 }
 
 // one axis of the order-3 x order-1 mixed mass: global order-3 node g -> up to
@@ -2887,12 +2911,11 @@ cudaError_t element_lists(fep3m_ctx* c) {
   cudaStream_t s = c->stream;
   if (c->precision == FEP3M_MIXED) {
     FEP3M_CL k_elem_coeff<float><<<grid_for(ne), TPB, 0, s>>>(ne, c->start, c->count, (const float4*)c->part, (float*)c->C);
-    FEP3M_CL k_vertex_density<float><<<grid_for(ne), TPB, 0, s>>>(n, (const float*)c->C, (float*)c->rv,
-                                                                   (float*)c->Cv);
+    FEP3M_CL k_vertex_density<float><<<grid_for(ne), TPB, 0, s>>>(n, (const float*)c->C, nullptr, c->Vc, (float*)c->Cv, 1.0);
   } else {
     FEP3M_CL k_elem_coeff<double><<<grid_for(ne), TPB, 0, s>>>(ne, c->start, c->count, (const vec4<double>::type*)c->part, (double*)c->C);
-    FEP3M_CL k_vertex_density<double><<<grid_for(ne), TPB, 0, s>>>(n, (const double*)c->C, (double*)c->rv,
-                                                                    (double*)c->Cv);
+    FEP3M_CL k_vertex_density<double><<<grid_for(ne), TPB, 0, s>>>(n, (const double*)c->C, (double*)c->rv, c->Vc,
+                                                                    (double*)c->Cv, c->q_scale);
   }
   return cudaGetLastError();
 }

@@ -68,7 +68,6 @@ template <> __device__ __forceinline__ float rsq<float>(float x) {
 
 // fused multiply-add in the working precision
 __device__ __forceinline__ float fmaw(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double fmaw(double a, double b, double c) { return fma(a, b, c); }
 
 // compensated (Kahan) accumulator; FP64 uses plain sums
 template <class T> struct Acc {
@@ -101,26 +100,37 @@ template <class T> struct Acc {
 // the nodes, contracted with the shape functions at each target.
 constexpr int BX = 4, BY = 4, BZ = 4, BE = BX * BY * BZ;   // 64 elements per brick
 constexpr int OCH = 32;                                      // offsets per chunk
-constexpr int MAXRUN = 2 * 81;                               // rows of the block (n_sr <= 4), 2 runs each
+constexpr int MAXROW = 81;                                   // rows (y, z) of the block (n_sr <= 4)
 
 template <class T>
 __device__ __forceinline__ void warp_sum(T& v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
 }
 
-// The rows (y, z) of a target's block as runs of consecutive sorted charges,
-// two where a row wraps: run k's first charge in runs[k], the charges of the
-// runs before it in pre[k]; returns (and pre[2 rows] holds) their number.  By a warp.
-__device__ __forceinline__ int warp_runs(int n, int n_sr, int ex, int ey, int ez, const int* __restrict__ start,
-                                         int* runs /* MAXRUN */, int* pre /* MAXRUN + 1 */) {
-  const int lane = threadIdx.x & 31, nb = 2 * n_sr + 1, rows = nb * nb;
+// the rows (dy, dz) of a block, by the CTA; ends with a barrier
+__device__ __forceinline__ void row_table(int n_sr, char2* rows /* MAXROW */) {
+  const int nb = 2 * n_sr + 1;
+  for (int r = threadIdx.x; r < nb * nb; r += blockDim.x) rows[r] = make_char2(r % nb - n_sr, r / nb - n_sr);
+  __syncthreads();
+}
+
+// The rows (y, z) of a target's block: row r's charges are a run of consecutive
+// sorted ones from rows[r].x on, and where the row wraps rows[r].y of them are
+// followed by a second run from rows[r].z on; pre[r] the charges of the rows
+// before it.  Returns (and pre[nrow] holds) their number.  By a warp.
+__device__ __forceinline__ int warp_rows(int n, int n_sr, const char2* tab, int ex, int ey, int ez,
+                                         const int* __restrict__ start, int4* rows /* MAXROW */,
+                                         int* pre /* MAXROW + 1 */) {
+  const int lane = threadIdx.x & 31, nb = 2 * n_sr + 1, nrow = nb * nb;
   int carry = 0;
-  for (int r0 = 0; r0 < rows; r0 += 32) {
+  for (int r0 = 0; r0 < nrow; r0 += 32) {
     const int r = r0 + lane;
     int a0 = 0, a1 = 0, b0 = 0, b1 = 0;
-    if (r < rows) {
-      const int dy = r % nb - n_sr, dz = r / nb - n_sr;
-      const int yy = wrapn(ey + dy, n), zz = wrapn(ez + dz, n);
+    if (r < nrow) {
+      const char2 d = tab[r];
+      int yy = ey + d.x, zz = ez + d.y;
+      yy += yy < 0 ? n : (yy >= n ? -n : 0);
+      zz += zz < 0 ? n : (zz >= n ? -n : 0);
       const int64_t rowbase = (int64_t)n * (yy + (int64_t)n * zz);
       const int x0 = ex - n_sr, x1 = ex + n_sr;
       if (x0 < 0) {
@@ -133,21 +143,19 @@ __device__ __forceinline__ int warp_runs(int n, int n_sr, int ex, int ey, int ez
         a0 = start[rowbase + x0];     a1 = start[rowbase + x1 + 1];
       }
     }
-    const int ca = a1 - a0, cb = b1 - b0;
-    int x = ca + cb;
+    const int cnt = a1 - a0 + b1 - b0;
+    int x = cnt;
     for (int o = 1; o < 32; o <<= 1) {
       const int v = __shfl_up_sync(0xffffffffu, x, o);
       if (lane >= o) x += v;
     }
-    if (r < rows) {
-      runs[2 * r] = a0;
-      runs[2 * r + 1] = b0;
-      pre[2 * r] = carry + x - ca - cb;
-      pre[2 * r + 1] = carry + x - cb;
+    if (r < nrow) {
+      rows[r] = make_int4(a0, a1 - a0, b0, 0);
+      pre[r] = carry + x - cnt;
     }
     carry += __shfl_sync(0xffffffffu, x, 31);
   }
-  if (lane == 0) pre[2 * rows] = carry;
+  if (lane == 0) pre[nrow] = carry;
   __syncwarp();
   return carry;
 }
@@ -161,17 +169,19 @@ __device__ __forceinline__ int block_delta(int d, int n, int n_sr) {
 // w[j]: source weights; returns sum w/r and (GRAD) sum w (x_j - x_t)/r^3 in
 // every lane, physical units, compensated per lane.
 template <class T, bool GRAD>
-__device__ __forceinline__ void warp_singular(int n, int n_sr, T h, int ex, int ey, int ez, int slot,
+__device__ __forceinline__ void warp_singular(int n, int n_sr, const char2* tab, T h, int ex, int ey, int ez, int slot,
                                               typename vec4<T>::type pt, const int* __restrict__ start,
                                               const typename vec4<T>::type* __restrict__ part,
-                                              const int* __restrict__ ecoord, int* runs, int* pre,
+                                              const int* __restrict__ ecoord, int4* rows, int* pre,
                                               const double* __restrict__ w, T out[4]) {
-  const int total = warp_runs(n, n_sr, ex, ey, ez, start, runs, pre);
+  const int total = warp_rows(n, n_sr, tab, ex, ey, ez, start, rows, pre);
   Acc<T> ps, fx, fy, fz;
   int k = 0;
   for (int f = threadIdx.x & 31; f < total; f += 32) {
     while (pre[k + 1] <= f) ++k;
-    const int j = runs[k] + (f - pre[k]);
+    const int i = f - pre[k];
+    const int4 r = rows[k];
+    const int j = i < r.y ? r.x + i : r.z + (i - r.y);
     if (j == slot) continue;
     const typename vec4<T>::type pj = part[j];
     const int ec = ecoord[j];
@@ -199,19 +209,21 @@ __device__ __forceinline__ void warp_singular(int n, int n_sr, T h, int ex, int 
 // ---------------------------------------------------- FP64 singular sums
 // An FP64 operation costs as much as 64 FP32 ones on this GPU, so the charges'
 // own singular sums of an FP64 context run in float pairs.  A charge for them:
-// per axis its local coordinate tau = a + bh + bl, a the multiple of 2^-20
-// nearest tau and bh + bl the rest (33 bits), so that a difference of two
-// coordinates plus a whole number is a float (exactly) plus a small pair; and
+// per axis its local coordinate tau = a + b + c, a the multiple of 2^-20 nearest
+// tau, b the multiple of 2^-42 nearest the rest and c what is left (below
+// 2^-43), so that the differences of two coordinates' parts (a's plus a whole
+// number) are exact in FP32, and a's difference is zero or larger than b's; and
 // the charge times a power of two near the inverse mean charge
 // (fep3m_ctx::q_scale), so that low words stay normal numbers.
 struct __align__(16) PairCharge {
-  float a[3], bh[3], bl[3];
+  float a[3], b[3], c[3];
   df q;
-  float pad;
+  float ex;   // the element's x coordinate
 };
 static_assert(sizeof(PairCharge) == FEP3M_PAIR_CHARGE_BYTES, "the context's allocation");
 
-__global__ void k_pair_charges(int64_t N, const vec4<double>::type* __restrict__ part, double scale,
+__global__ void k_pair_charges(int64_t N, const vec4<double>::type* __restrict__ part,
+                               const int* __restrict__ ecoord, double scale,
                                PairCharge* __restrict__ out) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
@@ -221,63 +233,83 @@ __global__ void k_pair_charges(int64_t N, const vec4<double>::type* __restrict__
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const double a = rint(x[k] * 1048576.0) * (1.0 / 1048576.0);
-    const df b = df_split(x[k] - a);
+    const double r = x[k] - a, b = rint(r * 4398046511104.0) * (1.0 / 4398046511104.0);   // 2^42
     c.a[k] = (float)a;
-    c.bh[k] = b.h;
-    c.bl[k] = b.l;
+    c.b[k] = (float)b;
+    c.c[k] = (float)(r - b);
   }
   c.q = df_split(p.w * scale);
-  c.pad = 0.f;
+  c.ex = (float)(ecoord[i] & 1023);
   out[i] = c;
 }
 
+// the same in FP64 (as exact as the coordinates)
+__device__ __forceinline__ double charge_diff64(const PairCharge& s, const PairCharge& t, int k, float d) {
+  return (double)((s.a[k] - t.a[k]) + d) +
+         ((double)(s.b[k] - t.b[k]) + (double)(s.c[k] - t.c[k]));
+}
 // x_s - x_t along axis k, the source's element d elements on
 __device__ __forceinline__ df charge_diff(const PairCharge& s, const PairCharge& t, int k, float d) {
-  const float A = (s.a[k] - t.a[k]) + d;   // exact: at most 23 bits
-  const df b = df_two_sum(s.bh[k], -t.bh[k]), v = df_two_sum(A, b.h);
-  return {v.h, v.l + (b.l + (s.bl[k] - t.bl[k]))};
+  const float A = (s.a[k] - t.a[k]) + d, B = s.b[k] - t.b[k];   // exact
+  const float h = A + B;
+  return {h, (B - (h - A)) + (s.c[k] - t.c[k])};
 }
 
 // One warp per target: sum Q / r into phi_s, (GRAD) sum Q (x_j - x_t) / r^3
 // into E_s, and half of them to psi and gpsi when given (the singular adjoint
 // for the energy's weights Q / 2).  A lane sums sixteen charges at a time in
-// pairs (element units) and those sums in three floats; a distance outside the
-// pairs' range (df_in_range) takes FP64.  About 160 FP32 operations per pair;
+// pairs (element units) and those sums in three floats.  A pair's term is good
+// to a few 2^-48; the few charges within three quarters of an element, whose terms are the
+// largest, take FP64 (as do distances outside df_in_range), so that the sums
+// are as good as all in FP64.  About 120 FP32 operations per pair;
 // bound by FP32 issue and, for few targets, by the latency of the loads.
 // 4000 charges, q = 2, potentials: 266 -> 42 us.
+constexpr float NEAR2 = 0.5625f;   // three quarters of an element, squared
 template <bool GRAD>
-__global__ void __launch_bounds__(PT) k_singular64(int64_t N, int n, int n_sr, double h, double inv_scale,
+__global__ void __launch_bounds__(PT) k_singular64(int64_t N, int n, int n_sr, double u0, double u1,
                                                    const int* __restrict__ start, const PairCharge* __restrict__ ch,
                                                    const int* __restrict__ ecoord, double* __restrict__ phi_s,
                                                    double* __restrict__ E_s, double* __restrict__ psi,
                                                    double* __restrict__ gpsi) {
   constexpr int NS = GRAD ? 4 : 1;
-  __shared__ int runs_all[PT / 32][MAXRUN];
-  __shared__ int pre_all[PT / 32][MAXRUN + 1];
+  __shared__ int4 rows_all[PT / 32][MAXROW];
+  __shared__ int pre_all[PT / 32][MAXROW + 1];
+  __shared__ char2 tab[MAXROW];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t t = blockIdx.x * (int64_t)(PT / 32) + warp;
+  row_table(n_sr, tab);
   if (t >= N) return;
-  int *runs = runs_all[warp], *pre = pre_all[warp];
+  int4* rows = rows_all[warp];
+  int* pre = pre_all[warp];
   const int et = ecoord[t], ex = et & 1023, ey = (et >> 10) & 1023, ez = et >> 20;
   const PairCharge ct = ch[t];
-  const int total = warp_runs(n, n_sr, ex, ey, ez, start, runs, pre);
+  const int total = warp_rows(n, n_sr, tab, ex, ey, ez, start, rows, pre);
+  // x displacement of a charge's element: its coordinate plus one of these (the period taken
+  // off in the first run of a row that wraps below, or the second of one that wraps above)
+  const float sx0 = (float)((ex - n_sr < 0 ? -n : 0) - ex), sx1 = (float)((ex - n_sr < 0 ? 0 : n) - ex);
   tf tot[NS] = {};
-  double far[NS] = {};
+  double s64[NS] = {};
+  bool met = false;   // some distance took FP64
   int k = 0;
   for (int f0 = lane; f0 < total; f0 += 32 * 16) {
     df s[NS] = {};
 #pragma unroll 2
     for (int f = f0; f < min(total, f0 + 32 * 16); f += 32) {
       while (pre[k + 1] <= f) ++k;
-      const int j = runs[k] + (f - pre[k]);
+      const int i = f - pre[k];
+      const int4 r = rows[k];
+      const bool first = i < r.y;
+      const int j = first ? r.x + i : r.z + (i - r.y);
       if (j == (int)t) continue;
       const PairCharge cj = ch[j];
-      const int ec = ecoord[j];
-      const df dx = charge_diff(cj, ct, 0, (float)block_delta((ec & 1023) - ex, n, n_sr)),
-               dy = charge_diff(cj, ct, 1, (float)block_delta(((ec >> 10) & 1023) - ey, n, n_sr)),
-               dz = charge_diff(cj, ct, 2, (float)block_delta((ec >> 20) - ez, n, n_sr));
-      const df r2 = df_add(df_add(df_sqr(dx), df_sqr(dy)), df_sqr(dz));
-      if (df_in_range(r2)) {
+      const char2 d = tab[k];
+      const float ddx = cj.ex + (first ? sx0 : sx1);
+      const df dx = charge_diff(cj, ct, 0, ddx), dy = charge_diff(cj, ct, 1, (float)d.x),
+               dz = charge_diff(cj, ct, 2, (float)d.y);
+      const df x2 = df_sqr(dx), y2 = df_sqr(dy), z2 = df_sqr(dz);
+      const df xy = df_two_sum(x2.h, y2.h), xyz = df_two_sum(xy.h, z2.h);
+      const df r2 = {xyz.h, xyz.l + ((xy.l + x2.l) + (y2.l + z2.l))};
+      if (r2.h >= NEAR2 && df_in_range(r2)) {
         const df ir = df_rsqrt<true>(r2);
         const df w = df_mul(cj.q, ir);
         df_acc(s[0], w);
@@ -288,34 +320,53 @@ __global__ void __launch_bounds__(PT) k_singular64(int64_t N, int n, int n_sr, d
           df_fma(s[3], g, dz);
         }
       } else {
-        const double ir = 1.0 / sqrt(df_value(r2)), w = df_value(cj.q) * ir;
-        far[0] += w;
+        const double x = charge_diff64(cj, ct, 0, ddx), y = charge_diff64(cj, ct, 1, (float)d.x),
+                     z = charge_diff64(cj, ct, 2, (float)d.y);
+        met = true;
+        const double ir = rsq<double>(x * x + y * y + z * z), w = df_value(cj.q) * ir;
+        s64[0] += w;
         if constexpr (GRAD) {
           const double g = w * ir * ir;
-          far[1] += g * df_value(dx);
-          far[2] += g * df_value(dy);
-          far[3] += g * df_value(dz);
+          s64[1] += g * x;
+          s64[2] += g * y;
+          s64[3] += g * z;
         }
       }
     }
 #pragma unroll
     for (int i = 0; i < NS; ++i) tf_add(tot[i], s[i]);
   }
+  auto with = [&](tf a, int o) -> tf {   // a plus lane ^ o's
+    tf_add(a, tf{__shfl_xor_sync(0xffffffffu, a.h, o), __shfl_xor_sync(0xffffffffu, a.m, o),
+                 __shfl_xor_sync(0xffffffffu, a.l, o)});
+    return a;
+  };
+  // the lanes' sums: with four, the lanes first split them, lane i (mod 4) adding up sum i
+  tf sum = tot[0];
+  if constexpr (GRAD) {
+    const bool b1 = lane & 1, b2 = lane & 2;
+    auto give = [&](const tf& keep, const tf& other, int o) -> tf {
+      tf a = keep;
+      tf_add(a, tf{__shfl_xor_sync(0xffffffffu, other.h, o), __shfl_xor_sync(0xffffffffu, other.m, o),
+                   __shfl_xor_sync(0xffffffffu, other.l, o)});
+      return a;
+    };
+    const tf e = give(b1 ? tot[1] : tot[0], b1 ? tot[0] : tot[1], 1), f = give(b1 ? tot[3] : tot[2], b1 ? tot[2] : tot[3], 1);
+    sum = give(b2 ? f : e, b2 ? e : f, 2);
+  } else {
+    sum = with(with(sum, 1), 2);
+  }
+  sum = with(with(with(sum, 4), 8), 16);
+  double out = df_value(sum);   // lane i's: sum i
+  if (__any_sync(0xffffffffu, met)) {
 #pragma unroll
-  for (int i = 0; i < NS; ++i)
-    for (int o = 16; o > 0; o >>= 1)
-      tf_add(tot[i], tf{__shfl_xor_sync(0xffffffffu, tot[i].h, o), __shfl_xor_sync(0xffffffffu, tot[i].m, o),
-                        __shfl_xor_sync(0xffffffffu, tot[i].l, o)});
-  double out = 0.0;   // lane i takes sum i
-#pragma unroll
-  for (int i = 0; i < NS; ++i) {
-    // (the FP64 sums are zero unless some lane met such a distance; NaN counts as met)
-    if (__any_sync(0xffffffffu, far[i] != 0.0)) warp_sum(far[i]);
-    if (lane == i) out = df_value(tot[i]) + far[i];
+    for (int i = 0; i < NS; ++i) {
+      warp_sum(s64[i]);
+      if (lane == i) out += s64[i];
+    }
   }
   if (lane >= NS) return;
-  const double ih = 1.0 / h;
-  out *= inv_scale * (lane == 0 ? ih : ih * ih);
+  out *= lane == 0 ? u0 : u1;   // physical units
   if (lane == 0) {
     phi_s[t] = out;
     if (psi) psi[t] = 0.5 * out;
@@ -721,7 +772,7 @@ template <class T, bool GRAD, bool TC>
 __global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_sr, T h, const int* __restrict__ start,
                                                              const int* __restrict__ count,
                                                              const typename vec4<T>::type* __restrict__ part,
-                                                             const T* __restrict__ Cv, const T* __restrict__ rv,
+                                                             const T* __restrict__ Vc,
                                                              const uint4* __restrict__ Hb, const float2* __restrict__ H0,
                                                              const float2* __restrict__ Hdf, T* __restrict__ Gscr, double* __restrict__ phi_s,
                                                              double* __restrict__ E_s, double* __restrict__ psi,
@@ -796,7 +847,9 @@ __global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_s
       if (sa < SF) v = E0[a] + sa - (n_sr - 1);
       else if (sa < SF + BX) v = E0[a] + (sa - SF) + keep;
       else v = E0[a] + (sa - SF - BX) - n_sr;
-      wv[i] = wrapn(v, n) * (a == 0 ? 1 : (a == 1 ? n : n * n));   // the vertex id's term of axis a
+      // the term of axis a in the index of the class sums Vc: its vertex coordinate and its class
+      const int cls = sa < SF ? 0 : (sa < SF + BX ? 1 : 2);
+      wv[i] = wrapn(v, n) * (a == 0 ? 1 : (a == 1 ? n : n * n)) + cls * (a == 0 ? 1 : (a == 1 ? 3 : 9)) * n * n * n;
     }
     for (int i = tid; i < 3 * HW; i += NT) {
       const int a = i / HW, ha = i % HW;
@@ -810,29 +863,10 @@ __global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_s
   int sx = tid % SW, sy = (tid / SW) % SW, sz = tid / (SW * SW);
 #pragma unroll 4
   for (int i = tid; i < SW * SW * SW; i += NT) {
-    // allowed corners k = kx + 2 ky + 4 kz as a bit mask: per axis both
-    // corners, corner 1 only (k with kx = 1: 0xAA) or corner 0 only (0x55)
-    const unsigned mx = sx < SF ? 0xFFu : (sx < SF + BX ? 0xAAu : 0x55u);
-    const unsigned my = sy < SF ? 0xFFu : (sy < SF + BX ? 0xCCu : 0x33u);
-    const unsigned mz = sz < SF ? 0xFFu : (sz < SF + BX ? 0xF0u : 0x0Fu);
-    const unsigned mask = mx & my & mz;
-    const int v = wv[sx] + wv[SW + sy] + wv[2 * SW + sz];   // < n^3 <= 2^30
-    T val = T(0);
-    if (mask == 0xFFu) {
-      val = rv[v];
-    } else {
-      // the vertex's eight corner terms are contiguous: two vector loads
-      const V4 c03 = reinterpret_cast<const V4*>(Cv + 8 * v)[0], c47 = reinterpret_cast<const V4*>(Cv + 8 * v)[1];
-      const T c8[8] = {c03.x, c03.y, c03.z, c03.w, c47.x, c47.y, c47.z, c47.w};
-#pragma unroll
-      for (int k = 0; k < 8; ++k) val += ((mask >> k) & 1u) ? c8[k] : T(0);
-    }
+    const T val = Vc[wv[sx] + wv[SW + sy] + wv[2 * SW + sz]];   // class and vertex: < 27 n^3 < 2^31
     if constexpr (!TC) {
-      // split once here into the hi + lo floats of the double-float
-      // contraction (each R value is read by several offsets; an FP32 value
-      // has lo = 0)
-      const float vh = (float)val;
-      reinterpret_cast<float2*>(R)[i] = make_float2(vh, (float)((double)val - (double)vh));
+      // the hi + lo floats of the double-float contraction (an FP32 value has lo = 0)
+      reinterpret_cast<float2*>(R)[i] = make_float2(val, 0.f);
     } else {
       R[i] = val;
     }
@@ -1089,18 +1123,126 @@ __global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_s
   }
 }
 
+// The screen field in an FP64 context.  The table is symmetric under reflection
+// of each axis about the element's centre, H(noff - 1 - o, 3 - m) = H(o, m), so
+// with the even and odd parts of the amplitudes and of the field along each axis
+//   A+-(i) = A(i) +- A(noff - 1 - i),  S(j) = S+(j) + S-(j),  S(3 - j) = S+(j) - S-(j)
+// the contraction falls into eight products (parities s = sx + 2 sy + 4 sz) of
+// (n_sr + 1)^3 amplitudes with two nodes per axis: an eighth of the
+// multiply-adds.  They run in float pairs on the FP32 pipes, 32 offsets at a
+// time in pairs and across those in three floats (relative to sum |A H| about
+// 1e-15).  One CTA per brick and parities (sy, sz), so that small meshes fill
+// the GPU too; it forms both parities along x.  As in k_pair_screen the brick's
+// extended vertex field R is in shared memory and A(e, o) = R[otab(o) +
+// lambda(e)]; R comes as pairs, times a power of two (fep3m_ctx::q_scale).
+// Gscr[brick][element][8 s + jx + 2 jy + 4 jz].  Bound by FP32 issue (about 105
+// operations per pair of parts staged, 12 per multiply-add).  Rock salt 32^3:
+// screen and singular sums took 2080 us in one kernel (the whole contraction in
+// pairs, FP64 singular terms); now 164 us here and 165 us in k_singular64.
+constexpr int SK = 32;   // offsets staged at once
+// row stride of R: 4 modulo 16 pairs, so that the four rows of four elements a
+// half-warp reads fall on different banks (even: the operands after R stay aligned)
+__host__ __device__ constexpr int screen64_row(int sw) { return sw + (20 - sw % 16) % 16; }
+static size_t screen64_smem(int n_sr) {
+  const int sw = 3 * BX + 2 * n_sr - 1, kh = n_sr + 1, K = kh * kh * kh;
+  return ((size_t)screen64_row(sw) * sw * sw + 2 * SK * (BE + 2) + 2 * K * 8) * sizeof(df) + (size_t)K * 8 * sizeof(int);
+}
+__global__ void __launch_bounds__(PT, 2) k_screen64(int n, int n_sr, const int* __restrict__ count,
+                                                    const df* __restrict__ Vc, const df* __restrict__ HP, double inv_scale,
+                                                    double* __restrict__ Gscr) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int nbx = (n + BX - 1) / BX, nby = (n + BY - 1) / BY;
+  const int E0[3] = {(int)(blockIdx.x % nbx) * BX, (int)((blockIdx.x / nbx) % nby) * BY,
+                     (int)(blockIdx.x / (nbx * nby)) * BZ};
+  const int sy = blockIdx.y & 1, sz = blockIdx.y >> 1;
+  const int kh = n_sr + 1, noff = 2 * kh, K = kh * kh * kh;
+  const int SW = 3 * BX + 2 * n_sr - 1, SF = BX + 2 * n_sr - 1, SW3 = SW * SW * SW;
+  const int RS = screen64_row(SW);
+  df* R = reinterpret_cast<df*>(smem_raw);
+  df(*As)[SK][BE + 2] = reinterpret_cast<df(*)[SK][BE + 2]>(R + RS * SW * SW);   // [2]: parity along x
+  df* Hs = reinterpret_cast<df*>(As + 2);                                            // [2][K][8]
+  int* otab = reinterpret_cast<int*>(Hs + 2 * K * 8);                                // [K][8] mirror images of an offset
+  __shared__ int wv[3][3 * BX + 8];
+  const int tid = threadIdx.x;
+  bool any = false;
+  if (tid < BE) {
+    const int lx = E0[0] + tid % BX, ly = E0[1] + (tid / BX) % BY, lz = E0[2] + tid / (BX * BY);
+    any = lx < n && ly < n && lz < n && count[lx + (int64_t)n * (ly + (int64_t)n * lz)] != 0;
+  }
+  if (!__syncthreads_or(any)) return;
+  auto slot = [&](int o) {   // R's slot of offset index o (0 .. noff - 1) of an axis
+    return o == 0 ? SF : (o == noff - 1 ? SF + BX : 2 * n_sr - o);
+  };
+  for (int i = tid; i < 3 * SW; i += PT) {
+    const int a = i / SW, sa = i % SW;
+    const int v = sa < SF ? E0[a] + sa - (n_sr - 1) : (sa < SF + BX ? E0[a] + (sa - SF) + kh : E0[a] + (sa - SF - BX) - n_sr);
+    // the term of axis a in the index of the class sums Vc: its vertex coordinate and its class
+    const int cls = sa < SF ? 0 : (sa < SF + BX ? 1 : 2);
+    wv[a][sa] = wrapn(v, n) * (a == 0 ? 1 : (a == 1 ? n : n * n)) + cls * (a == 0 ? 1 : (a == 1 ? 3 : 9)) * n * n * n;
+  }
+  for (int i = tid; i < 8 * K; i += PT) {
+    const int k = i >> 3, f = i & 7, kk[3] = {k % kh, (k / kh) % kh, k / (kh * kh)};
+    int idx = 0;
+    for (int a = 2; a >= 0; --a)
+      idx += slot((f >> a) & 1 ? noff - 1 - kk[a] : kk[a]) * (a == 0 ? 1 : (a == 1 ? RS : RS * SW));
+    otab[i] = idx;
+  }
+  for (int i = tid; i < 2 * K * 8; i += PT) Hs[i] = HP[(int64_t)(2 * sy + 4 * sz) * K * 8 + i];   // sx = 0, 1 follow
+  __syncthreads();
+#pragma unroll 4
+  for (int i = tid; i < SW3; i += PT) {
+    const int r = i / SW, x = i - r * SW, z = r / SW, y = r - z * SW;
+    R[x + RS * r] = Vc[wv[0][x] + wv[1][y] + wv[2][z]];
+  }
+  const int el = tid & 63, k4 = tid >> 6;   // staging: this thread's element, and every fourth offset
+  const int lam = (el % BX) + RS * (((el / BX) % BY) + SW * (el / (BX * BY)));
+  const int m = tid & 7, g = (tid >> 3) & 15, sx = tid >> 7;   // product: node part, four elements, parity along x
+  tf tot[4] = {};
+  for (int k0 = 0; k0 < K; k0 += SK) {
+    const int nk = min(SK, K - k0);
+    __syncthreads();
+#pragma unroll 2
+    for (int kk = k4; kk < nk; kk += 4) {
+      const int* o = otab + 8 * (k0 + kk);
+      df t[2];
+#pragma unroll
+      for (int f = 0; f < 2; ++f) {
+        const df a0 = R[o[f] + lam], a1 = R[o[f + 2] + lam], b0 = R[o[f + 4] + lam], b1 = R[o[f + 6] + lam];
+        const df a = df_add(a0, sy ? df{-a1.h, -a1.l} : a1), b = df_add(b0, sy ? df{-b1.h, -b1.l} : b1);
+        t[f] = df_add(a, sz ? df{-b.h, -b.l} : b);
+      }
+      As[0][kk][el] = df_add(t[0], t[1]);
+      As[1][kk][el] = df_add(t[0], df{-t[1].h, -t[1].l});
+    }
+    __syncthreads();
+    df acc[4] = {};
+    const df* Hm = Hs + (int64_t)sx * K * 8 + (int64_t)k0 * 8 + m;
+#pragma unroll 4
+    for (int kk = 0; kk < nk; ++kk) {
+      const df h = Hm[8 * kk];
+      const float4* ap = reinterpret_cast<const float4*>(&As[sx][kk][4 * g]);
+      const float4 v0 = ap[0], v1 = ap[1];
+      df_fma(acc[0], df{v0.x, v0.y}, h);
+      df_fma(acc[1], df{v0.z, v0.w}, h);
+      df_fma(acc[2], df{v1.x, v1.y}, h);
+      df_fma(acc[3], df{v1.z, v1.w}, h);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) tf_add(tot[j], acc[j]);
+  }
+  double* gb = Gscr + (int64_t)blockIdx.x * (BE * 64) + 8 * (sx + 2 * sy + 4 * sz) + m;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) gb[(4 * g + j) * 64] = df_value(tot[j]) * inv_scale;
+}
+
 // One CTA per brick, after the mesh solve: G = mesh potential - screen field
 // at the 64 nodes of each non-empty brick element, then four threads per
 // target charge each contract 16 of the nodes with the order-3 shape
 // functions (and their derivatives) at the charge; the mesh part is added to
-// the singular part the screen kernel left in phi_s / E_s.
+// the singular part the screen kernel left in phi_s / E_s (FP64 contexts:
+// k_pair_eval64).
 //
-// FP64 path: G is held in shared memory relative to its value G0 at the
-// element's first node (kept in FP64): the shape functions sum to one and
-// their gradients to zero, so G0 enters the potential alone and the rounding
-// acts on the variation of G only.
-//
-// FP32 path: the screen field arrives relative to the element's corners (the
+// The screen field arrives relative to the element's corners (the
 // field at node 0, corner fields relative to it, elsewhere the field less its
 // trilinear interpolant; pair_relative_table), and G is split the same way:
 // G0 and the corner values of G - G0 in FP64 (the mesh potential's hi + lo
@@ -1108,19 +1250,17 @@ __global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_s
 // FP32 (from the same pairs).  The trilinear part and its gradient at the
 // charge are evaluated in FP64; only the small remainder goes through the FP32
 // contraction.
-template <class T, bool GRAD>
-__global__ void __launch_bounds__(PT) k_pair_eval(int n, int Nm, T inv_h, const int* __restrict__ start,
-                                                  const int* __restrict__ count,
-                                                  const typename vec4<T>::type* __restrict__ part,
-                                                  const double* __restrict__ phi64, const float2* __restrict__ phi_hl,
-                                                  const T* __restrict__ Gscr,
+template <bool GRAD>
+__global__ void __launch_bounds__(PT) k_pair_eval(int n, int Nm, float inv_h, const int* __restrict__ start,
+                                                  const int* __restrict__ count, const float4* __restrict__ part,
+                                                  const float2* __restrict__ phi_hl, const float* __restrict__ Gscr,
                                                   const int* __restrict__ perm, double* __restrict__ phi_s,
                                                   double* __restrict__ E_s, double* __restrict__ phi_out) {
-  typedef typename vec4<T>::type V4;
-  constexpr bool F32 = sizeof(T) == 4;
+  typedef float T;
+  typedef float4 V4;
   __shared__ __align__(32) T G[BE * 64];
   __shared__ double G0[BE];
-  __shared__ double Gc[F32 ? BE * 8 : 1];   // FP32 path: corner values of G - G0
+  __shared__ double Gc[BE * 8];   // corner values of G - G0
   __shared__ int epre[BE + 1];
   __shared__ int wsum[PT / 32 + 1];
   const int nbx = (n + BX - 1) / BX, nby = (n + BY - 1) / BY;
@@ -1149,60 +1289,50 @@ __global__ void __launch_bounds__(PT) k_pair_eval(int n, int Nm, T inv_h, const 
     const int gx = 3 * ex + (m & 3), gy = 3 * ey + ((m >> 2) & 3), gz = 3 * ez + (m >> 4);   // < 3n + 3
     return (gx >= N ? gx - N : gx) + (int64_t)N * ((gy >= N ? gy - N : gy) + (int64_t)N * (gz >= N ? gz - N : gz));
   };
-  if constexpr (F32) {
-    auto phd = [&](int64_t k) -> double {
-      const float2 p = phi_hl[k];
-      return (double)p.x + (double)p.y;
-    };
-    if (tid < BE && epre[tid + 1] != epre[tid]) {
-      const double p00 = phd(node(tid, 0));
-      G0[tid] = p00 - (double)gb[tid * 64];
-      Gc[tid * 8] = 0.0;
+  auto phd = [&](int64_t k) -> double {
+    const float2 p = phi_hl[k];
+    return (double)p.x + (double)p.y;
+  };
+  if (tid < BE && epre[tid + 1] != epre[tid]) {
+    const double p00 = phd(node(tid, 0));
+    G0[tid] = p00 - (double)gb[tid * 64];
+    Gc[tid * 8] = 0.0;
 #pragma unroll
-      for (int c = 1; c < 8; ++c) {
-        const int mc = 3 * (c & 1) + 12 * ((c >> 1) & 1) + 48 * (c >> 2);
-        Gc[tid * 8 + c] = (phd(node(tid, mc)) - p00) - (double)gb[tid * 64 + mc];
-      }
-    }
-    // node differences of the mesh potential from its hi + lo floats
-    for (int i = tid; i < BE * 64; i += PT) {
-      const int l = i >> 6, m = i & 63;
-      if (epre[l + 1] == epre[l]) continue;   // empty (or outside the mesh): never read
-      const float2 p = phi_hl[node(l, m)], p0 = phi_hl[node(l, 0)];
-      G[i] = (p.x - p0.x) + (p.y - p0.y);
-    }
-    __syncthreads();
-    // remainder: the difference less its trilinear interpolant, less the screen
-    // remainder; zero at the corners
-    constexpr int PER = BE * 64 / PT;
-    float rem[PER];
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int i = tid + k * PT, l = i >> 6, m = i & 63;
-      const int mx = m & 3, my = (m >> 2) & 3, mz = m >> 4;
-      rem[k] = 0.f;
-      if (epre[l + 1] == epre[l]) continue;
-      if ((mx == 0 || mx == 3) && (my == 0 || my == 3) && (mz == 0 || mz == 3)) continue;
-      const float* g = G + l * 64;
-      const float tx = mx * (1.f / 3.f), ty = my * (1.f / 3.f), tz = mz * (1.f / 3.f);
-      // corners (0,0,0) 0, (3,0,0) 3, (0,3,0) 12, (3,3,0) 15, z + 48
-      const float x00 = fmaf(tx, g[3] - g[0], g[0]), x10 = fmaf(tx, g[15] - g[12], g[12]);
-      const float x01 = fmaf(tx, g[51] - g[48], g[48]), x11 = fmaf(tx, g[63] - g[60], g[60]);
-      const float y0 = fmaf(ty, x10 - x00, x00), y1 = fmaf(ty, x11 - x01, x01);
-      rem[k] = (g[m] - fmaf(tz, y1 - y0, y0)) - gb[i];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < PER; ++k) G[tid + k * PT] = rem[k];
-  } else {
-    if (tid < BE && epre[tid + 1] != epre[tid]) G0[tid] = phi64[node(tid, 0)] - gb[tid * 64];
-    __syncthreads();
-    for (int i = tid; i < BE * 64; i += PT) {
-      const int l = i >> 6, m = i & 63;
-      if (epre[l + 1] == epre[l]) continue;   // empty (or outside the mesh): never read
-      G[i] = (phi64[node(l, m)] - gb[i]) - G0[l];
+    for (int c = 1; c < 8; ++c) {
+      const int mc = 3 * (c & 1) + 12 * ((c >> 1) & 1) + 48 * (c >> 2);
+      Gc[tid * 8 + c] = (phd(node(tid, mc)) - p00) - (double)gb[tid * 64 + mc];
     }
   }
+  // node differences of the mesh potential from its hi + lo floats
+  for (int i = tid; i < BE * 64; i += PT) {
+    const int l = i >> 6, m = i & 63;
+    if (epre[l + 1] == epre[l]) continue;   // empty (or outside the mesh): never read
+    const float2 p = phi_hl[node(l, m)], p0 = phi_hl[node(l, 0)];
+    G[i] = (p.x - p0.x) + (p.y - p0.y);
+  }
+  __syncthreads();
+  // remainder: the difference less its trilinear interpolant, less the screen
+  // remainder; zero at the corners
+  constexpr int PER = BE * 64 / PT;
+  float rem[PER];
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int i = tid + k * PT, l = i >> 6, m = i & 63;
+    const int mx = m & 3, my = (m >> 2) & 3, mz = m >> 4;
+    rem[k] = 0.f;
+    if (epre[l + 1] == epre[l]) continue;
+    if ((mx == 0 || mx == 3) && (my == 0 || my == 3) && (mz == 0 || mz == 3)) continue;
+    const float* g = G + l * 64;
+    const float tx = mx * (1.f / 3.f), ty = my * (1.f / 3.f), tz = mz * (1.f / 3.f);
+    // corners (0,0,0) 0, (3,0,0) 3, (0,3,0) 12, (3,3,0) 15, z + 48
+    const float x00 = fmaf(tx, g[3] - g[0], g[0]), x10 = fmaf(tx, g[15] - g[12], g[12]);
+    const float x01 = fmaf(tx, g[51] - g[48], g[48]), x11 = fmaf(tx, g[63] - g[60], g[60]);
+    const float y0 = fmaf(ty, x10 - x00, x00), y1 = fmaf(ty, x11 - x01, x01);
+    rem[k] = (g[m] - fmaf(tz, y1 - y0, y0)) - gb[i];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < PER; ++k) G[tid + k * PT] = rem[k];
   __syncthreads();
   const int q = tid & 3;   // nodes 16 q .. 16 q + 15: mz = q, (mx, my) over 4 x 4
   for (int tb = 0; tb < ntarget; tb += PT / 4) {
@@ -1255,9 +1385,9 @@ __global__ void __launch_bounds__(PT) k_pair_eval(int n, int Nm, T inv_h, const 
       v4[i] += __shfl_xor_sync(0xffffffffu, v4[i], 2);
     }
     if (valid && q == 0) {
-      // FP32 path: the trilinear part of G - G0 and its gradient at the charge, in FP64
-      double tv = 0.0, tg[3] = {0.0, 0.0, 0.0};
-      if constexpr (F32) {
+      // the trilinear part of G - G0 and its gradient at the charge, in FP64
+      double tv, tg[3];
+      {
         const double* g = Gc + l * 8;
         const double x = pt.x, y = pt.y, z = pt.z;
         double a[4], b[4];   // x-lerps and x-differences of the corner pairs j = cy + 2 cz
@@ -1287,6 +1417,155 @@ __global__ void __launch_bounds__(PT) k_pair_eval(int n, int Nm, T inv_h, const 
   }
 }
 
+// The same in an FP64 context.  The screen field comes in its even and odd
+// parts (k_screen64); its nodal values are formed in shared memory, three
+// sums and differences each, and subtracted from the mesh potential.  Four
+// threads per target take the four z layers of nodes: each evaluates one shape
+// function and derivative per axis (shared by shuffles) and contracts its
+// layer along x, then y: about 400 FP64 operations per target where the terms
+// one by one took 3000 (rock salt 32^3 with forces: 98 -> 74 us; an FP64
+// operation costs as much as 64 FP32 ones here).
+__device__ __forceinline__ void q3_one(double t, int i, double& v, double& d) {
+  const double k = i == 0 ? -4.5 : (i == 1 ? 13.5 : (i == 2 ? -13.5 : 4.5));
+  const double r0 = i == 0 ? 1.0 / 3.0 : 0.0, r1 = i < 2 ? 2.0 / 3.0 : 1.0 / 3.0, r2 = i == 3 ? 2.0 / 3.0 : 1.0;
+  const double a = t - r0, b = t - r1, c = t - r2, ab = a * b;
+  v = k * (ab * c);
+  d = k * fma(c, a + b, ab);
+}
+template <bool GRAD>
+__global__ void __launch_bounds__(PT) k_pair_eval64(int n, int Nm, double inv_h, const int* __restrict__ start,
+                                                    const int* __restrict__ count,
+                                                    const vec4<double>::type* __restrict__ part,
+                                                    const double* __restrict__ phi64, const double* __restrict__ Gscr,
+                                                    const int* __restrict__ perm, double* __restrict__ phi_s,
+                                                    double* __restrict__ E_s, double* __restrict__ phi_out) {
+  typedef vec4<double>::type V4;
+  __shared__ __align__(32) double G[BE * 64];
+  __shared__ int epre[BE + 1];
+  __shared__ int wsum[PT / 32 + 1];
+  const int nbx = (n + BX - 1) / BX, nby = (n + BY - 1) / BY;
+  const int E0x = (blockIdx.x % nbx) * BX, E0y = ((blockIdx.x / nbx) % nby) * BY, E0z = (blockIdx.x / (nbx * nby)) * BZ;
+  const int tid = threadIdx.x;
+  int ntarget;
+  {
+    int c0 = 0;
+    if (tid < BE) {
+      const int lx = E0x + (tid % BX), ly = E0y + (tid / BX) % BY, lz = E0z + tid / (BX * BY);
+      if (lx < n && ly < n && lz < n) c0 = count[lx + (int64_t)n * (ly + (int64_t)n * lz)];
+    }
+    const int pre = block_scan_excl<PT>(c0, wsum, &ntarget);
+    if (tid < BE) epre[tid] = pre;
+    if (tid == 0) epre[BE] = ntarget;
+  }
+  if (ntarget == 0) return;
+  __syncthreads();
+  const double* gb = Gscr + (int64_t)blockIdx.x * (BE * 64);
+  constexpr int PER = BE * 64 / PT;
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int i = tid + k * PT;
+    G[i] = epre[(i >> 6) + 1] != epre[i >> 6] ? gb[i] : 0.0;
+  }
+  // part i = jx + 2 jy + 4 jz + 8 (sx + 2 sy + 4 sz): along each axis the even
+  // part's place takes their sum (node j), the odd part's the difference (node 3 - j)
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < PER / 2; ++k) {
+      const int i = tid + k * PT, bit = 8 << a;
+      const int e = ((i & ~(bit - 1)) << 1) | (i & (bit - 1));   // bit 3 + a clear
+      if (epre[(e >> 6) + 1] == epre[e >> 6]) continue;
+      const double x = G[e], y = G[e | bit];
+      G[e] = x + y;
+      G[e | bit] = x - y;
+    }
+  }
+  __syncthreads();
+  double val[PER];
+  int at[PER];
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int i = tid + k * PT, l = i >> 6;
+    int m[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int j = (i >> a) & 1;
+      m[a] = (i >> (3 + a)) & 1 ? 3 - j : j;
+    }
+    at[k] = l * 64 + m[0] + 4 * m[1] + 16 * m[2];
+    val[k] = 0.0;
+    if (epre[l + 1] == epre[l]) continue;   // empty (or outside the mesh): never read
+    // the node on the periodic mesh (Nm = 3 n) wrapped, on a box's (Nm = 3 nb + 1) never past the last
+    const int gx = 3 * (E0x + l % BX) + m[0], gy = 3 * (E0y + (l / BX) % BY) + m[1], gz = 3 * (E0z + l / (BX * BY)) + m[2];
+    val[k] = phi64[(gx >= Nm ? gx - Nm : gx) +
+                   (int64_t)Nm * ((gy >= Nm ? gy - Nm : gy) + (int64_t)Nm * (gz >= Nm ? gz - Nm : gz))] - G[i];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < PER; ++k) G[at[k]] = val[k];
+  __syncthreads();
+  const int q = tid & 3, lane0 = (tid & 31) & ~3;
+  for (int tb = 0; tb < ntarget; tb += PT / 4) {
+    const int k = tb + (tid >> 2);
+    const bool valid = k < ntarget;
+    int slot = 0, l = 0;
+    V4 pt;
+    pt.x = pt.y = pt.z = pt.w = 0.0;
+    if (valid) {
+      int lo = 0, hi2 = BE;
+      while (hi2 - lo > 1) {
+        const int mid = (lo + hi2) >> 1;
+        if (epre[mid] <= k) lo = mid;
+        else hi2 = mid;
+      }
+      l = lo;
+      const int ex = E0x + l % BX, ey = E0y + (l / BX) % BY, ez = E0z + l / (BX * BY);
+      slot = start[ex + (int64_t)n * (ey + (int64_t)n * ez)] + (k - epre[l]);
+      pt = part[slot];
+    }
+    double ux, uy, uz, dx, dy, dz;
+    q3_one(pt.x, q, ux, dx);
+    q3_one(pt.y, q, uy, dy);
+    q3_one(pt.z, q, uz, dz);
+    double X[4], DX[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      X[i] = __shfl_sync(0xffffffffu, ux, lane0 + i);
+      if (GRAD) DX[i] = __shfl_sync(0xffffffffu, dx, lane0 + i);
+    }
+    double v = 0.0, vx = 0.0, vy = 0.0;   // this layer: value, d/dx, d/dy
+#pragma unroll
+    for (int my = 0; my < 4; ++my) {
+      const V4 gv = *reinterpret_cast<const V4*>(G + l * 64 + 16 * q + 4 * my);
+      const double Y = __shfl_sync(0xffffffffu, uy, lane0 + my);
+      const double row = fma(gv.x, X[0], fma(gv.y, X[1], fma(gv.z, X[2], gv.w * X[3])));
+      v = fma(row, Y, v);
+      if (GRAD) {
+        const double DY = __shfl_sync(0xffffffffu, dy, lane0 + my);
+        vx = fma(fma(gv.x, DX[0], fma(gv.y, DX[1], fma(gv.z, DX[2], gv.w * DX[3]))), Y, vx);
+        vy = fma(row, DY, vy);
+      }
+    }
+    double v4[4] = {v * uz, vx * uz, vy * uz, v * dz};
+#pragma unroll
+    for (int i = 0; i < (GRAD ? 4 : 1); ++i) {
+      v4[i] += __shfl_xor_sync(0xffffffffu, v4[i], 1);
+      v4[i] += __shfl_xor_sync(0xffffffffu, v4[i], 2);
+    }
+    if (!valid) continue;
+    // thread q writes sum q
+    if (q == 0) {
+      const double phi = v4[0] * inv_h + phi_s[slot];
+      phi_s[slot] = phi;
+      if (phi_out) phi_out[perm[slot]] = phi;
+    } else if (GRAD) {
+      double* E = E_s + 3 * slot + (q - 1);
+      *E = (q == 1 ? v4[1] : (q == 2 ? v4[2] : v4[3])) * (inv_h * inv_h) + *E;
+    }
+  }
+}
+
 // ----------------------------------------------------------------- adjoint
 __global__ void k_weights(int64_t N, double gU, const double* __restrict__ gphi, const int* __restrict__ perm,
                           const double* __restrict__ Qs, double* __restrict__ w, float* __restrict__ w32) {
@@ -1301,38 +1580,77 @@ __global__ void k_weights(int64_t N, double gU, const double* __restrict__ gphi,
 // W[e][m] = sum_{t in e} w_t u_m(tau_t): the adjoint's point deposit, per
 // element.  wsum (FP32 path): sum_{t in e} w_t in FP64 as hi + lo floats, the
 // exact sum over m of W[e][m] (the shape functions sum to one).  wT: the
-// weights in the working precision (FP32: a copy, so that the 64 threads of
-// an element do not each convert them).
+// weights in the working precision.  A warp takes 32 consecutive elements,
+// whose charges are one run of the sorted arrays: it reads their starts and,
+// 32 at a time, the charges in one load each, then hands them round by
+// shuffles, two nodes per lane (with one thread per element and node each
+// element waited for three dependent loads: 262 144 charges on 64^3, 146 ->
+// 41 us, 10^6 on 128^3, 845 -> 145 us; FP64 rock salt 32^3, where every thread also evaluated twelve
+// shape functions, 208 -> 34 us).
 template <class T>
-__global__ void k_elem_deposit(int64_t ne, const int* __restrict__ start, const int* __restrict__ count,
-                               const typename vec4<T>::type* __restrict__ part, const double* __restrict__ w,
-                               const T* __restrict__ wT, T* __restrict__ W, float2* __restrict__ wsum) {
-  // wsum: the block's elements by the lanes of its first warp (an FP64
-  // instruction takes the FP64 pipe for a whole warp, however few lanes are on)
-  const int per = blockDim.x / 64;
-  if (wsum && threadIdx.x < per) {
-    const int64_t e = blockIdx.x * (int64_t)per + threadIdx.x;
-    if (e < ne) {
-      double ws = 0.0;
-      for (int j = start[e], j1 = start[e] + count[e]; j < j1; ++j) ws += w[j];
-      const float hi = (float)ws;
-      wsum[e] = make_float2(hi, (float)(ws - (double)hi));
+__global__ void __launch_bounds__(PT) k_elem_deposit(int64_t ne, const int* __restrict__ start,
+                                                     const int* __restrict__ count,
+                                                     const typename vec4<T>::type* __restrict__ part,
+                                                     const double* __restrict__ w, const T* __restrict__ wT,
+                                                     T* __restrict__ W, float2* __restrict__ wsum) {
+  const int lane = threadIdx.x & 31;
+  const int64_t e0 = (blockIdx.x * (int64_t)(PT / 32) + (threadIdx.x >> 5)) * 32;
+  if (e0 >= ne) return;
+  const int nel = (int)min((int64_t)32, ne - e0);
+  const int s0 = lane < nel ? start[e0 + lane] : 0, cnt = lane < nel ? count[e0 + lane] : 0;
+  if (wsum && lane < nel) {
+    double ws = 0.0;
+    for (int j = s0; j < s0 + cnt; ++j) ws += w[j];
+    const float hi = (float)ws;
+    wsum[e0 + lane] = make_float2(hi, (float)(ws - (double)hi));
+  }
+  // this lane's nodes: m = lane and lane + 32 (the same x and y index, z index 2 on)
+  const int mx = lane & 3, my = (lane >> 2) & 3, mz = lane >> 4;
+  // order-3 shape function i at t as q3_values forms it: k (t - r0) (t - r1) (t - r2)
+  auto one = [](T t, int i) -> T {
+    const T k = i == 0 ? T(-4.5) : (i == 1 ? T(13.5) : (i == 2 ? T(-13.5) : T(4.5)));
+    const T r0 = i == 0 ? T(1) / T(3) : T(0), r1 = i < 2 ? T(2) / T(3) : T(1) / T(3), r2 = i == 3 ? T(2) / T(3) : T(1);
+    return k * (t - r0) * (t - r1) * (t - r2);
+  };
+  const int first = __shfl_sync(0xffffffffu, s0, 0), end = __shfl_sync(0xffffffffu, s0 + cnt, nel - 1);
+  int base = first;                 // the charges base .. base + 31 are held, one per lane
+  typename vec4<T>::type pc;
+  T wc = T(0);
+  pc.x = pc.y = pc.z = pc.w = T(0);
+  auto hold = [&]() {
+    if (base + lane < end) {
+      pc = part[base + lane];
+      wc = wT[base + lane];
     }
+  };
+  hold();
+  for (int i = 0; i < nel; ++i) {
+    const int s = __shfl_sync(0xffffffffu, s0, i), c = __shfl_sync(0xffffffffu, cnt, i);
+    T a0 = T(0), a1 = T(0);
+    for (int j = s; j < s + c; ++j) {
+      if (j >= base + 32) {
+        base = j;
+        hold();
+      }
+      const int src = j - base;
+      const T x = __shfl_sync(0xffffffffu, pc.x, src), y = __shfl_sync(0xffffffffu, pc.y, src),
+              z = __shfl_sync(0xffffffffu, pc.z, src), wj = __shfl_sync(0xffffffffu, wc, src);
+      if constexpr (sizeof(T) == 4) {
+        const T xy = wj * one(x, mx) * one(y, my);
+        a0 += xy * one(z, mz);
+        a1 += xy * one(z, mz + 2);
+      } else {
+        // one shape function per lane (12 of them), then shuffles
+        const T u = one(lane < 4 ? x : (lane < 8 ? y : z), lane & 3);
+        const T xy = wj * __shfl_sync(0xffffffffu, u, mx) * __shfl_sync(0xffffffffu, u, 4 + my);
+        const T z0 = __shfl_sync(0xffffffffu, u, 8 + mz), z1 = __shfl_sync(0xffffffffu, u, 10 + mz);
+        a0 = fma(xy, z0, a0);
+        a1 = fma(xy, z1, a1);
+      }
+    }
+    W[(e0 + i) * 64 + lane] = a0;
+    W[(e0 + i) * 64 + lane + 32] = a1;
   }
-  const int64_t e = blockIdx.x * (int64_t)per + threadIdx.x / 64;
-  if (e >= ne) return;
-  const int m = threadIdx.x & 63, mx = m & 3, my = (m >> 2) & 3, mz = m >> 4;
-  const int s = start[e], cnt = count[e];
-  T acc = T(0);
-  for (int j = s; j < s + cnt; ++j) {
-    const typename vec4<T>::type p = part[j];
-    T ux[4], uy[4], uz[4];
-    q3_values<T>(p.x, ux);
-    q3_values<T>(p.y, uy);
-    q3_values<T>(p.z, uz);
-    acc += wT[j] * ux[mx] * uy[my] * uz[mz];
-  }
-  W[e * 64 + m] = acc;
 }
 
 // g[node] = sum over (element, local node) pairs at the node of W: in FP64,
@@ -1387,19 +1705,18 @@ __global__ void k_node_assemble(int n, const T* __restrict__ W, double* __restri
 //   D[o][e] = sum_m W[e][m] H(o, m)               (every element e, every vertex offset o)
 //   A[s][k] = sum_{o : o + k in block} D[o][s + k + o]
 // D[o][e] is the table field of element e's deposit seen from the vertex e - o
-// (k_adj_gemm on the CUDA cores, the tensor-core row GEMM in the FP32 path;
+// (the tensor-core row GEMM in the FP32 path, or k_adj_gemm; k_adj64 in FP64;
 // the gather is k_adj_vertex).
 constexpr int GT = 64;   // GEMM tile: 64 elements x 64 offsets, K = 64 nodes
 constexpr int ADJ_NT = 128;   // tensor-core column tile: offsets per tile
 
-// The products are summed in double-float arithmetic on the FP32 pipes in both
-// precisions, as in the screen contraction (hi + lo float pairs in shared
-// memory: the table's from FP64, an FP32 deposit has lo = 0; fused two-product
+// CUDA cores (MIXED with FEP3M_CUDA_CORES): the products are summed in
+// double-float arithmetic on the FP32 pipes (hi + lo float pairs in shared
+// memory: the table's from FP64, the FP32 deposit has lo = 0; fused two-product
 // with the cross terms, two-sum accumulation), in two halves of 32 nodes whose
-// sums are added in FP64; D is stored in T.
-template <class T>
-__global__ void __launch_bounds__(PT) k_adj_gemm(int64_t ne, int o0, int no, const T* __restrict__ W,
-                                                 const double* __restrict__ Hw, T* __restrict__ D) {
+// sums are added in FP64.
+__global__ void __launch_bounds__(PT) k_adj_gemm(int64_t ne, int o0, int no, const float* __restrict__ W,
+                                                 const double* __restrict__ Hw, float* __restrict__ D) {
   __shared__ float2 Ws2[64][GT + 1];   // [m][element]
   __shared__ float2 Hs2[64][GT + 1];   // [m][offset]
   const int64_t e0 = (int64_t)blockIdx.x * GT;
@@ -1461,7 +1778,7 @@ __global__ void __launch_bounds__(PT) k_adj_gemm(int64_t ne, int o0, int no, con
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int64_t e = e0 + te + 16 * i;
-      if (e < ne) D[(int64_t)(o - o0) * ne + e] = (T)acc[i][j];
+      if (e < ne) D[(int64_t)(o - o0) * ne + e] = (float)acc[i][j];
     }
   }
 }
@@ -1469,7 +1786,7 @@ __global__ void __launch_bounds__(PT) k_adj_gemm(int64_t ne, int o0, int no, con
 // Double-float accumulator (hi + lo floats, summed by two-sum): the FP32
 // path's screen adjoint sums, whose terms cancel to a small remainder.
 struct dfacc {
-  float h = 0.f, l = 0.f;
+  float h, l;
 };
 __device__ __forceinline__ void acc_add(dfacc& a, float b) {
   const float s = a.h + b, bb = s - a.h;
@@ -1481,9 +1798,102 @@ __device__ __forceinline__ void acc_merge(dfacc& a, const dfacc& b) {
   a.l += ((a.h - (s - bb)) + (b.h - bb)) + b.l;
   a.h = s;
 }
-__device__ __forceinline__ void acc_merge(double& a, double b) { a += b; }
 __device__ __forceinline__ double acc_value(const dfacc& a) { return (double)a.h + (double)a.l; }
-__device__ __forceinline__ double acc_value(double a) { return a; }
+
+// The FP64 path's D by parity (see k_screen64): with W+-(j) = W(j) +- W(3 - j)
+// along each axis, D+-(i) = sum_j E+-(i, j) W+-(j) and D(i) = D+(i) + D-(i),
+// D(noff - 1 - i) = D+(i) - D-(i): 4096 multiply-adds an element instead of 32
+// 768 (n_sr = 3), in float pairs, and three sums and differences per value.  A
+// CTA takes 32 consecutive elements, one per lane; a warp forms the eight
+// parities of two offsets i at a time for them and writes their sixteen
+// mirrored values of D as pairs (rows of 32 consecutive elements).  HP: the
+// table by parity, [s][i][j].  Bound by FP32 issue; rock salt 32^3: 778 ->
+// 143 us against the full product in pairs with D rounded to FP64.
+constexpr int AE = 32;
+static size_t adj64_smem(int n_sr) {
+  const int kh = n_sr + 1;
+  return (size_t)AE * 65 * sizeof(double) + (size_t)64 * AE * sizeof(df) + (size_t)kh * kh * kh * 64 * sizeof(df);
+}
+__global__ void __launch_bounds__(PT, 2) k_adj64(int64_t ne, int n_sr, int z0, int z1, const double* __restrict__ W,
+                                                 const df* __restrict__ HP, df* __restrict__ D) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int kh = n_sr + 1, noff = 2 * kh, K = kh * kh * kh, plane = noff * noff;
+  double(*Wd)[65] = reinterpret_cast<double(*)[65]>(smem_raw);                                      // [AE]
+  df(*Ws)[AE] = reinterpret_cast<df(*)[AE]>(smem_raw + AE * 65 * sizeof(double));                   // [64]: 8 s + j
+  df* Hs = reinterpret_cast<df*>(smem_raw + AE * 65 * sizeof(double) + 64 * AE * sizeof(df));       // [8][K][8]
+  const int64_t e0 = blockIdx.x * (int64_t)AE;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < 64 * K; i += PT) Hs[i] = HP[i];
+  for (int i = tid; i < AE * 64; i += PT) {
+    const int e = i >> 6;
+    Wd[e][i & 63] = e0 + e < ne ? W[(e0 + e) * 64 + (i & 63)] : 0.0;
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    __syncthreads();
+    for (int i = tid; i < AE * 32; i += PT) {
+      // node pair: index j (0, 1) along axis a and its mirror image 3 - j
+      const int e = i & 31, r = i >> 5, j = r & 1, o = r >> 1, o0 = o & 3, o1 = o >> 2;
+      const int st = a == 0 ? 1 : (a == 1 ? 4 : 16);
+      const int base = a == 0 ? 4 * o0 + 16 * o1 : (a == 1 ? o0 + 16 * o1 : o0 + 4 * o1);
+      double &x = Wd[e][base + j * st], &y = Wd[e][base + (3 - j) * st];
+      const double s = x + y, d = x - y;
+      x = s;
+      y = d;
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < AE * 64; i += PT) {
+    const int e = i & 31, b = i >> 5, s = b >> 3, j = b & 7;
+    int node = 0;
+    for (int a = 2; a >= 0; --a) {
+      const int ja = (j >> a) & 1;
+      node = node * 4 + ((s >> a) & 1 ? 3 - ja : ja);
+    }
+    Ws[b][e] = df_split(Wd[e][node]);
+  }
+  __syncthreads();
+  for (int i0 = 2 * warp; i0 < K; i0 += 2 * (PT / 32)) {
+    df v[2][8];
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      v[0][s] = v[1][s] = df{0.f, 0.f};
+      // (an odd K: the last pair's second offset repeats the first, unused)
+      const float4* h0 = reinterpret_cast<const float4*>(Hs + (s * K + i0) * 8);
+      const float4* h1 = i0 + 1 < K ? h0 + 4 : h0;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const df w0 = Ws[8 * s + 2 * j][lane], w1 = Ws[8 * s + 2 * j + 1][lane];
+        const float4 a = h0[j], b = h1[j];
+        df_fma(v[0][s], w0, df{a.x, a.y});
+        df_fma(v[0][s], w1, df{a.z, a.w});
+        df_fma(v[1][s], w0, df{b.x, b.y});
+        df_fma(v[1][s], w1, df{b.z, b.w});
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const int i = i0 + t;
+      if (i >= K) break;
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+          if ((s >> a) & 1) continue;
+          const df x = v[t][s], y = v[t][s | (1 << a)];
+          v[t][s] = df_add(x, y);
+          v[t][s | (1 << a)] = df_add(x, df{-y.h, -y.l});
+        }
+      const int ix = i % kh, iy = (i / kh) % kh, iz = i / (kh * kh);
+      if (e0 + lane >= ne) continue;
+#pragma unroll
+      for (int f = 0; f < 8; ++f) {
+        const int ox = f & 1 ? noff - 1 - ix : ix, oy = f & 2 ? noff - 1 - iy : iy, oz = f & 4 ? noff - 1 - iz : iz;
+        if (oz >= z0 && oz < z1) D[((int64_t)(oz - z0) * plane + oy * noff + ox) * ne + e0 + lane] = v[t][f];
+      }
+    }
+  }
+}
 
 // Screen adjoint, gathered by vertex:
 //   A[s][k] = sum over the offsets o with o + k inside the block of D(o, s + k + o).
@@ -1499,8 +1909,8 @@ __device__ __forceinline__ double acc_value(double a) { return a; }
 // combined in shared memory in warp order, one thread per (vertex, corner):
 // deterministic.  FP32 path (H0 set): D holds the contraction with the
 // node-0-relative table, and each term gains H(o, 0) Wsum(v + o)
-// (pair_adjoint_table); terms and sums in double-float arithmetic.  FP64
-// path: D is the whole contraction, summed in FP64.
+// (pair_adjoint_table).  FP64 path: D is the whole contraction, as pairs.  Terms
+// and sums in double-float arithmetic.
 constexpr int AV_WARPS = 8;
 template <class T, int NSR>
 __global__ void __launch_bounds__(32 * AV_WARPS) k_adj_vertex(int n, int z0, int z1, int first,
@@ -1508,8 +1918,8 @@ __global__ void __launch_bounds__(32 * AV_WARPS) k_adj_vertex(int n, int z0, int
                                                               const float2* __restrict__ H0,
                                                               const float2* __restrict__ wsum, double* __restrict__ A) {
   constexpr int KEEP = NSR + 1, NOFF = 2 * NSR + 2, PLANE = NOFF * NOFF;
-  constexpr bool DF = sizeof(T) == 4;
-  typedef typename std::conditional<DF, dfacc, double>::type Acc;
+  constexpr bool DF = sizeof(T) == 4;   // T: float, or df (FP64)
+  typedef dfacc Acc;
   extern __shared__ __align__(16) unsigned char av_smem[];
   Acc(*part)[27][32] = reinterpret_cast<Acc(*)[27][32]>(av_smem);   // [AV_WARPS][27][32]: each warp's classes
   __shared__ int live[32];
@@ -1557,7 +1967,7 @@ __global__ void __launch_bounds__(32 * AV_WARPS) k_adj_vertex(int n, int z0, int
           acc_add(P[cx], p);
           acc_add(P[cx], d + r);
         } else {
-          P[cx] += d;
+          acc_merge(P[cx], dfacc{d.h, d.l});
         }
       }
       Acc* row = &part[warp][cz * 9 + cy * 3][lane];
@@ -1591,16 +2001,18 @@ __global__ void __launch_bounds__(PT) k_pair_adj_warp(int64_t N, int n, int n_sr
                                                       const typename vec4<T>::type* __restrict__ part,
                                                       const int* __restrict__ ecoord, const double* __restrict__ w,
                                                       double* __restrict__ psi, double* __restrict__ gpsi) {
-  __shared__ int runs_all[PT / 32][MAXRUN];
-  __shared__ int pre_all[PT / 32][MAXRUN + 1];
+  __shared__ int4 rows_all[PT / 32][MAXROW];
+  __shared__ int pre_all[PT / 32][MAXROW + 1];
+  __shared__ char2 tab[MAXROW];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t t = blockIdx.x * (int64_t)(PT / 32) + warp;
+  row_table(n_sr, tab);
   if (t >= N) return;
   const typename vec4<T>::type pt = part[t];
   const int ec = ecoord[t];
   T sg[4];
-  warp_singular<T, GRAD>(n, n_sr, h, ec & 1023, (ec >> 10) & 1023, ec >> 20, (int)t, pt, start, part, ecoord,
-                         runs_all[warp], pre_all[warp], w, sg);
+  warp_singular<T, GRAD>(n, n_sr, tab, h, ec & 1023, (ec >> 10) & 1023, ec >> 20, (int)t, pt, start, part, ecoord,
+                         rows_all[warp], pre_all[warp], w, sg);
   if (lane == 0) {
     psi[t] = (double)sg[0];
     if (GRAD) {
@@ -1757,8 +2169,8 @@ static cudaError_t launch_pair_screen(fep3m_ctx* c, cudaStream_t s, bool half) {
   cudaError_t e = smem_limit((const void*)kern, smem);
   if (e != cudaSuccess) return e;
   FEP3M_CL kern<<<(unsigned)pair_bricks(c), TC ? PTC : PT, smem, s>>>(
-      c->n, c->n_sr, (T)c->h, c->start, c->count, (const typename vec4<T>::type*)c->part, (const T*)c->Cv,
-      (const T*)c->rv, (const uint4*)c->Hb, (const float2*)c->H0df, (const float2*)c->Hdf, (T*)c->Gscr, c->phi_s, c->E_s,
+      c->n, c->n_sr, (T)c->h, c->start, c->count, (const typename vec4<T>::type*)c->part, (const T*)c->Vc,
+      (const uint4*)c->Hb, (const float2*)c->H0df, (const float2*)c->Hdf, (T*)c->Gscr, c->phi_s, c->E_s,
       half ? c->psi_s : nullptr,
       half ? c->gpsi_s : nullptr, c->iflags + 2);
   return cudaGetLastError();
@@ -1775,13 +2187,21 @@ static const float2* mesh_potential_pairs(const fep3m_ctx* c) {
   return c->box ? (const float2*)c->phi_hl : (const float2*)c->phi64;
 }
 
-template <class T, bool GRAD>
+template <bool GRAD>
 static cudaError_t launch_pair_eval(fep3m_ctx* c, double* phi_out) {
-  FEP3M_CL k_pair_eval<T, GRAD><<<(unsigned)pair_bricks(c), PT, 0, c->stream>>>(
-      c->n, mesh_nodes_per_axis(c), (T)c->inv_h, c->start, c->count, (const typename vec4<T>::type*)c->part, c->phi64,
-      mesh_potential_pairs(c), (const T*)c->Gscr, c->perm, c->phi_s, c->E_s, phi_out);
+  const unsigned g = (unsigned)pair_bricks(c);
+  if (c->precision == FEP3M_MIXED)
+    FEP3M_CL k_pair_eval<GRAD><<<g, PT, 0, c->stream>>>(
+        c->n, mesh_nodes_per_axis(c), (float)c->inv_h, c->start, c->count, (const float4*)c->part,
+        mesh_potential_pairs(c), (const float*)c->Gscr, c->perm, c->phi_s, c->E_s, phi_out);
+  else
+    FEP3M_CL k_pair_eval64<GRAD><<<g, PT, 0, c->stream>>>(
+        c->n, mesh_nodes_per_axis(c), c->inv_h, c->start, c->count, (const vec4<double>::type*)c->part, c->phi64,
+        (const double*)c->Gscr, c->perm, c->phi_s, c->E_s, phi_out);
   return cudaGetLastError();
 }
+
+static cudaError_t singular64(fep3m_ctx* c, bool grad, bool half, cudaStream_t s);
 
 cudaError_t pair_screen(fep3m_ctx* c, int want_grad, cudaStream_t s, bool energy_adjoint) {
   const bool half = energy_adjoint && want_grad;
@@ -1792,8 +2212,13 @@ cudaError_t pair_screen(fep3m_ctx* c, int want_grad, cudaStream_t s, bool energy
     return want_grad ? launch_pair_screen<float, true, false>(c, s, half)
                      : launch_pair_screen<float, false, false>(c, s, half);
   }
-  return want_grad ? launch_pair_screen<double, true, false>(c, s, half)
-                   : launch_pair_screen<double, false, false>(c, s, half);
+  const size_t smem = screen64_smem(c->n_sr);
+  cudaError_t e = smem_limit((const void*)k_screen64, smem);
+  if (e != cudaSuccess) return e;
+  FEP3M_CL k_screen64<<<dim3((unsigned)pair_bricks(c), 4), PT, smem, s>>>(
+      c->n, c->n_sr, c->count, (const df*)c->Vc, (const df*)c->HP, 1.0 / c->q_scale,
+      (double*)c->Gscr);
+  return singular64(c, want_grad != 0, half, s);
 }
 
 // Corner structure of an element's 64 order-3 nodes (m = mx + 4 my + 16 mz):
@@ -1852,6 +2277,32 @@ void pair_adjoint_table(int n_sr, const double* Hw, double* Hd, float* H0) {
     H0[2 * o] = hi;
     H0[2 * o + 1] = (float)(h0 - (double)hi);
   }
+}
+
+// the FP64 path's table by parity: HP[s][k][j], s = sx + 2 sy + 4 sz, k the offsets
+// 0 .. n_sr and j the nodes 0, 1 per axis (x fastest): the mean over the mirror
+// images (which agree to rounding) with the parities' signs, as float pairs
+void pair_parity_table(int n_sr, const double* Hw, float* out) {
+  const int kh = n_sr + 1, noff = 2 * kh, K = kh * kh * kh;
+  for (int s = 0; s < 8; ++s)
+    for (int k = 0; k < K; ++k)
+      for (int j = 0; j < 8; ++j) {
+        const int kk[3] = {k % kh, (k / kh) % kh, k / (kh * kh)};
+        double v = 0.0;
+        for (int f = 0; f < 64; ++f) {   // bit a: mirror the offset along axis a; bit 3 + a: the node
+          int o = 0, m = 0, sign = 1;
+          for (int a = 2; a >= 0; --a) {
+            const int fo = (f >> a) & 1, fm = (f >> (3 + a)) & 1, ja = (j >> a) & 1;
+            o = o * noff + (fo ? noff - 1 - kk[a] : kk[a]);
+            m = m * 4 + (fm ? 3 - ja : ja);
+            if (((s >> a) & 1) && fo != fm) sign = -sign;
+          }
+          v += sign * Hw[(size_t)o * 64 + m];
+        }
+        const df d = df_split(v / 64.0);
+        out[2 * ((size_t)(s * K + k) * 8 + j)] = d.h;
+        out[2 * ((size_t)(s * K + k) * 8 + j) + 1] = d.l;
+      }
 }
 
 // the table's three bf16 pieces for the screen adjoint's contraction
@@ -1934,9 +2385,7 @@ cudaError_t pair_prepare(fep3m_ctx* c) {
 }
 
 cudaError_t pair_eval(fep3m_ctx* c, double* phi_out, int want_grad) {
-  if (c->precision == FEP3M_MIXED)
-    return want_grad ? launch_pair_eval<float, true>(c, phi_out) : launch_pair_eval<float, false>(c, phi_out);
-  return want_grad ? launch_pair_eval<double, true>(c, phi_out) : launch_pair_eval<double, false>(c, phi_out);
+  return want_grad ? launch_pair_eval<true>(c, phi_out) : launch_pair_eval<false>(c, phi_out);
 }
 
 cudaError_t energy(fep3m_ctx* c, double* U_dev, cudaStream_t s) {
@@ -1949,18 +2398,18 @@ cudaError_t energy(fep3m_ctx* c, double* U_dev, cudaStream_t s) {
 template <class T, int NSR>
 static void launch_adj_vertex(fep3m_ctx* c, int z0, int z1, const T* D, double* A, cudaStream_t s) {
   const int64_t ne = (int64_t)c->n * c->n * c->n;
-  const bool df = sizeof(T) == 4;
-  const size_t smem = (size_t)AV_WARPS * 27 * 32 * 8;   // dfacc and double: 8 bytes
+  const bool rel = sizeof(T) == 4;   // D relative to node 0 (FP32 path)
+  const size_t smem = (size_t)AV_WARPS * 27 * 32 * sizeof(dfacc);
   (void)smem_limit((const void*)k_adj_vertex<T, NSR>, smem);   // a failure shows as the launch's error
   FEP3M_CL k_adj_vertex<T, NSR><<<(unsigned)((ne + 31) / 32), 32 * AV_WARPS, smem, s>>>(
-      c->n, z0, z1, z0 == 0, c->count, D, df ? (const float2*)c->H0df : nullptr, df ? (const float2*)c->Wsum : nullptr,
-      A);
+      c->n, z0, z1, z0 == 0, c->count, D, rel ? (const float2*)c->H0df : nullptr,
+      rel ? (const float2*)c->Wsum : nullptr, A);
 }
 
 // D-GEMM + gather over chunks of whole offset planes (all offsets with one
 // oz), sized so D stays within a memory budget
 template <class T>
-static cudaError_t screen_adjoint(fep3m_ctx* c, const T* W, const double* Hw, double* A) {
+static cudaError_t screen_adjoint(fep3m_ctx* c, const T* W, double* A) {
   const int n = c->n;
   const int64_t ne = (int64_t)n * n * n;
   const int noff = c->noff, plane = noff * noff;
@@ -1993,16 +2442,22 @@ static cudaError_t screen_adjoint(fep3m_ctx* c, const T* W, const double* Hw, do
       cudaError_t e = tc_rows_gemm(ne, 64, o0, o0 + no, ADJ_NT, (const float*)W, c->HbA, (float*)c->D_adj,
                                    c->iflags + 2, s);
       if (e != cudaSuccess) return e;
+    } else if constexpr (sizeof(T) == 8) {
+      const size_t smem = adj64_smem(c->n_sr);
+      (void)smem_limit((const void*)k_adj64, smem);   // a failure shows as the launch's error
+      FEP3M_CL k_adj64<<<(unsigned)((ne + AE - 1) / AE), PT, smem, s>>>(ne, c->n_sr, z0, z1, (const double*)W,
+                                                                       (const df*)c->HP, (df*)c->D_adj);
     } else {
       dim3 grid((unsigned)((ne + GT - 1) / GT), (unsigned)((no + GT - 1) / GT));
-      FEP3M_CL k_adj_gemm<T><<<grid, PT, 0, s>>>(ne, o0, no, W, Hw, (T*)c->D_adj);
+      FEP3M_CL k_adj_gemm<<<grid, PT, 0, s>>>(ne, o0, no, W, c->Ha64, (float*)c->D_adj);
     }
-    const T* D = (const T*)c->D_adj;
+    typedef typename std::conditional<sizeof(T) == 4, float, df>::type DT;
+    const DT* D = (const DT*)c->D_adj;
     switch (c->n_sr) {
-      case 1: launch_adj_vertex<T, 1>(c, z0, z1, D, A, s); break;
-      case 2: launch_adj_vertex<T, 2>(c, z0, z1, D, A, s); break;
-      case 3: launch_adj_vertex<T, 3>(c, z0, z1, D, A, s); break;
-      default: launch_adj_vertex<T, 4>(c, z0, z1, D, A, s); break;
+      case 1: launch_adj_vertex<DT, 1>(c, z0, z1, D, A, s); break;
+      case 2: launch_adj_vertex<DT, 2>(c, z0, z1, D, A, s); break;
+      case 3: launch_adj_vertex<DT, 3>(c, z0, z1, D, A, s); break;
+      default: launch_adj_vertex<DT, 4>(c, z0, z1, D, A, s); break;
     }
   }
   return cudaGetLastError();
@@ -2013,7 +2468,7 @@ cudaError_t adjoint_pre(fep3m_ctx* c, double gU, const double* gphi, cudaStream_
   const int n = c->n;
   const int64_t ne = (int64_t)n * n * n, nodes = 27 * ne, N = c->N;
   FEP3M_CL k_weights<<<gsz(N), PT, 0, s>>>(N, gU, gphi, c->perm, c->Q_s, c->w_s, c->w_s32);
-  const int per = PT / 64;
+  const int per = PT;   // elements per CTA: 32 per warp
   if (c->precision == FEP3M_MIXED) {
     FEP3M_CL k_elem_deposit<float><<<gsz(ne, per), PT, 0, s>>>(ne, c->start, c->count, (const float4*)c->part, c->w_s,
                                                                c->w_s32, (float*)c->W_el, (float2*)c->Wsum);
@@ -2036,12 +2491,12 @@ cudaError_t adjoint_sweeps(fep3m_ctx* c, cudaStream_t s, bool singular) {
   c->stream = s;   // screen_adjoint issues on c->stream
   cudaError_t e;
   if (c->precision == FEP3M_MIXED) {
-    e = screen_adjoint<float>(c, (const float*)c->W_el, c->Ha64, (double*)c->A_el);
+    e = screen_adjoint<float>(c, (const float*)c->W_el, (double*)c->A_el);
     if (e == cudaSuccess && singular)
       FEP3M_CL k_pair_adj_warp<float, true><<<(unsigned)((N + 7) / 8), PT, 0, s>>>(N, n, c->n_sr, (float)c->h, c->start,
                                                          (const float4*)c->part, c->ecoord, c->w_s, c->psi_s, c->gpsi_s);
   } else {
-    e = screen_adjoint<double>(c, (const double*)c->W_el, c->Hw64, (double*)c->A_el);
+    e = screen_adjoint<double>(c, (const double*)c->W_el, (double*)c->A_el);
     if (e == cudaSuccess && singular)
       FEP3M_CL k_pair_adj_warp<double, true><<<(unsigned)((N + 7) / 8), PT, 0, s>>>(N, n, c->n_sr, c->h, c->start,
                                                           (const vec4<double>::type*)c->part, c->ecoord, c->w_s,
@@ -2063,10 +2518,11 @@ cudaError_t adjoint_vertex(fep3m_ctx* c, cudaStream_t s) {
 static cudaError_t singular64(fep3m_ctx* c, bool grad, bool half, cudaStream_t s) {
   const int64_t N = c->N;
   PairCharge* ch = (PairCharge*)c->part_pairs;
-  FEP3M_CL k_pair_charges<<<gsz(N), PT, 0, s>>>(N, (const vec4<double>::type*)c->part, c->q_scale, ch);
+  FEP3M_CL k_pair_charges<<<gsz(N), PT, 0, s>>>(N, (const vec4<double>::type*)c->part, c->ecoord, c->q_scale, ch);
   double *psi = half ? c->psi_s : nullptr, *gpsi = half ? c->gpsi_s : nullptr;
   auto k = grad ? k_singular64<true> : k_singular64<false>;
-  FEP3M_CL k<<<(unsigned)((N + 7) / 8), PT, 0, s>>>(N, c->n, c->n_sr, c->h, 1.0 / c->q_scale, c->start, ch, c->ecoord,
+  FEP3M_CL k<<<(unsigned)((N + 7) / 8), PT, 0, s>>>(N, c->n, c->n_sr, c->inv_h / c->q_scale,
+                                                    c->inv_h * c->inv_h / c->q_scale, c->start, ch, c->ecoord,
                                                     c->phi_s, c->E_s, psi, gpsi);
   return cudaGetLastError();
 }
