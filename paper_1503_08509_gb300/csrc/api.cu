@@ -171,6 +171,19 @@ int deliver(fep3m_ctx* c, void* dst, const void* src, size_t bytes) {
   return FEP3M_OK;
 }
 
+// Device scalars (scal, 64 doubles): the charge sums at 32, U at 40, the pair
+// counts at 48, the integer flags (iflags) at kFlags.  One copy to pinned memory
+// brings the results of a call and its error flag; waits for the stream.
+constexpr int kFlags = 56;
+cudaError_t take_results(fep3m_ctx* c, double* U) {
+  cudaError_t e = cudaMemcpyAsync(c->host_scal, c->scal + 32, 32 * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+  if (e != cudaSuccess) return e;
+  if (U) *U = c->host_scal[40 - 32];
+  c->host_err = ((const int*)(c->host_scal + kFlags - 32))[2];
+  return cudaSuccess;
+}
+
 void ev_record(fep3m_ctx* c, int k, cudaStream_t s = nullptr) {
   if (c->timing) cudaEventRecord(c->ev[k], s ? s : c->stream);
 }
@@ -327,8 +340,7 @@ int compute_orderq(fep3m_ctx* c, double* phi, double* U) {
   const int st = orderq_compute(c, pd, U ? c->scal + 40 : nullptr);
   ev_record(c, 3);
   if (st != FEP3M_OK && st != FEP3M_ENOCONV) return st;
-  if (U) CK(cudaMemcpyAsync(U, c->scal + 40, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
+  CK(take_results(c, U));
   c->have_forward = true;
   c->have_grad = false;
   c->stats.refine_steps = c->oq->sweeps;
@@ -366,10 +378,8 @@ int compute_box(fep3m_ctx* c, double* phi, double* U) {
   const int st = box_compute(c, pd, U ? c->scal + 40 : nullptr);
   ev_record(c, 3);
   if (st != FEP3M_OK && st != FEP3M_ENOCONV) return st;
-  if (U) CK(cudaMemcpyAsync(U, c->scal + 40, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaMemcpyAsync(c->host_err, c->iflags + 2, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
-  if (*c->host_err) return FEP3M_ETIMEOUT;
+  CK(take_results(c, U));
+  if (c->host_err) return FEP3M_ETIMEOUT;
   c->have_forward = true;
   c->have_grad = false;
   c->stats.refine_steps = c->box->sweeps;
@@ -407,14 +417,14 @@ void fep3m_destroy(fep3m_ctx* c) {
   free_particles(c);
   void* p[] = {c->HP, c->Vc, c->count, c->start, c->fill, c->scan_tmp, c->C,
                c->precision == FEP3M_MIXED ? nullptr : c->rv, c->Cv, c->b64, c->phi64,
-               c->res64, c->scal, c->iflags, c->phi_hl, c->W_el, c->A_el, c->mu_v, c->Gscr, c->Hb, c->HbA,
+               c->res64, c->scal, c->phi_hl, c->W_el, c->A_el, c->mu_v, c->Gscr, c->Hb, c->HbA,
                c->Hdf, c->red_tmp, c->red_counter, c->D_adj, c->Ha64, c->H0df, c->Wsum};
   for (void* q : p) dfree(q);
   fep3m::solver_destroy(&c->solv[0]);
   fep3m::solver_destroy(&c->solv[1]);
   fep3m::orderq_destroy(c);
   fep3m::box_destroy(c);
-  if (c->host_err) cudaFreeHost(c->host_err);
+  if (c->host_scal) cudaFreeHost(c->host_scal);
   if (c->aux_stream) cudaStreamDestroy(c->aux_stream);
   if (c->sweep_stream) cudaStreamDestroy(c->sweep_stream);
   if (c->pair_stream) cudaStreamDestroy(c->pair_stream);
@@ -474,9 +484,9 @@ int fep3m_create(const fep3m_config* cfg, void* stream, fep3m_ctx** out) {
     cudaError_t e = cudaSuccess;
     if ((e = dalloc(&c->count, ne)) != cudaSuccess || (e = dalloc(&c->start, ne + 1)) != cudaSuccess ||
         (e = dalloc(&c->fill, ne)) != cudaSuccess || (e = cudaMalloc(&c->scan_tmp, scan_tmp_bytes(ne))) != cudaSuccess ||
-        (e = dalloc(&c->scal, 64)) != cudaSuccess || (e = dalloc(&c->iflags, 16)) != cudaSuccess ||
+        (e = dalloc(&c->scal, 64)) != cudaSuccess ||
         (e = dalloc(&c->red_tmp, 1024)) != cudaSuccess || (e = dalloc(&c->red_counter, 1)) != cudaSuccess ||
-        (e = cudaMallocHost(&c->host_err, sizeof(int))) != cudaSuccess ||
+        (e = cudaMallocHost(&c->host_scal, 32 * sizeof(double))) != cudaSuccess ||
         (e = cudaStreamCreateWithFlags(&c->pair_stream, cudaStreamNonBlocking)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&c->ev_pfork, cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&c->ev_pjoin, cudaEventDisableTiming)) != cudaSuccess ||
@@ -484,8 +494,8 @@ int fep3m_create(const fep3m_config* cfg, void* stream, fep3m_ctx** out) {
         (e = cudaMallocHost(&c->host_cnt, 5 * sizeof(unsigned long long))) != cudaSuccess)
       return fail(from_cuda(e));
     cudaMemset(c->red_counter, 0, sizeof(unsigned int));
-    cudaMemset(c->iflags, 0, 16 * sizeof(int));
-    *c->host_err = 0;
+    c->iflags = (int*)(c->scal + kFlags);
+  cudaMemset(c->iflags, 0, 16 * sizeof(int));
     if ((st = orderq_create(c)) != FEP3M_OK) return fail(st);
     for (int k = 0; k < 11; ++k) cudaEventCreate(&c->ev[k]);
     c->ev_init = true;
@@ -558,8 +568,7 @@ int fep3m_create(const fep3m_config* cfg, void* stream, fep3m_ctx** out) {
     cudaMemcpy(c->HbA, ha.data(), ha.size() * 2, cudaMemcpyHostToDevice);
     if ((st = from_cuda(tc_rows_prepare(128))) != FEP3M_OK) return fail(st);
   }
-  if ((st = from_cuda(cudaMallocHost(&c->host_err, sizeof(int)))) != FEP3M_OK) return fail(st);
-  *c->host_err = 0;
+  if ((st = from_cuda(cudaMallocHost(&c->host_scal, 32 * sizeof(double)))) != FEP3M_OK) return fail(st);
   const int64_t ne = (int64_t)c->n * c->n * c->n, nodes = 27 * ne;
   const size_t es = c->precision == FEP3M_MIXED ? 4 : 8;
   cudaError_t e = cudaSuccess;
@@ -571,7 +580,7 @@ int fep3m_create(const fep3m_config* cfg, void* stream, fep3m_ctx** out) {
       (box && (e = cudaMalloc(&c->Cv, ne * 8 * es)) != cudaSuccess) ||
       (e = dalloc(&c->b64, 2 * nodes)) != cudaSuccess || (e = dalloc(&c->phi64, 2 * nodes)) != cudaSuccess ||
       (e = dalloc(&c->res64, nodes)) != cudaSuccess || (e = dalloc(&c->scal, 64)) != cudaSuccess ||
-      (e = dalloc(&c->iflags, 16)) != cudaSuccess || (e = cudaMalloc(&c->W_el, ne * 64 * es)) != cudaSuccess ||
+      (e = cudaMalloc(&c->W_el, ne * 64 * es)) != cudaSuccess ||
       (e = cudaMalloc(&c->A_el, ne * 8 * sizeof(double))) != cudaSuccess ||
       (e = cudaMalloc(&c->mu_v, ne * sizeof(double))) != cudaSuccess ||
       (e = dalloc(&c->red_tmp, 1024)) != cudaSuccess || (e = dalloc(&c->red_counter, 1)) != cudaSuccess ||
@@ -589,6 +598,7 @@ int fep3m_create(const fep3m_config* cfg, void* stream, fep3m_ctx** out) {
        (e = cudaMalloc(&c->Wsum, ne * sizeof(float2))) != cudaSuccess))
     return fail(from_cuda(e));
   cudaMemset(c->red_counter, 0, sizeof(unsigned int));
+  c->iflags = (int*)(c->scal + kFlags);
   cudaMemset(c->iflags, 0, 16 * sizeof(int));
   if ((e = create_stream_at(&c->aux_stream, kPrioForward)) != cudaSuccess ||
       (e = create_stream_at(&c->sweep_stream, kPrioSweep)) != cudaSuccess ||
@@ -654,11 +664,11 @@ int fep3m_set_particles(fep3m_ctx* c, int64_t N, const double* pos, const double
   CK(cudaStreamWaitEvent(c->stream, c->ev_pjoin, 0));
   ev_record(c, 7);
   c->counts_stale = true;   // pair statistics: counted when fep3m_get_stats asks for them
-  double sums[2];
-  int flag = 0;
-  CK(cudaMemcpyAsync(sums, c->scal + 32, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaMemcpyAsync(&flag, c->iflags, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  // the charge sums and the input flag in one copy to pinned memory
+  CK(cudaMemcpyAsync(c->host_scal, c->scal + 32, 32 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
+  const double* sums = c->host_scal;
+  const int flag = ((const int*)(c->host_scal + kFlags - 32))[0];
   c->have_particles = false;
   c->have_forward = false;
   if (flag) return FEP3M_EINVAL;
@@ -687,10 +697,8 @@ int fep3m_compute(fep3m_ctx* c, double* phi, double* U, double* force) {
     int st = run_forward(c, phi_dev ? phi : (phi ? c->out_tmp : nullptr), force != nullptr, fdst,
                          U ? c->scal + 40 : nullptr);
     if (st != FEP3M_OK) return st;
-    if (U) CK(cudaMemcpyAsync(U, c->scal + 40, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaMemcpyAsync(c->host_err, c->iflags + 2, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    if (*c->host_err) return FEP3M_ETIMEOUT;
+    CK(take_results(c, U));
+    if (c->host_err) return FEP3M_ETIMEOUT;
     if (!solves_missed(c, force != nullptr) || attempt == kMaxReruns) break;
   }
   const int st = solve_status(c, force != nullptr);
@@ -728,9 +736,8 @@ int fep3m_vjp(fep3m_ctx* c, double gU, const double* gphi, double* dpos, double*
     for (int attempt = 0;; ++attempt) {
       int st = run_forward(c, nullptr, 1, nullptr);
       if (st != FEP3M_OK) return st;
-      CK(cudaMemcpyAsync(c->host_err, c->iflags + 2, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-      CK(cudaStreamSynchronize(c->stream));
-      if (*c->host_err) return FEP3M_ETIMEOUT;
+      CK(take_results(c, nullptr));
+      if (c->host_err) return FEP3M_ETIMEOUT;
       if (!solves_missed(c, false) || attempt == kMaxReruns) break;
     }
     solve_status(c, false);

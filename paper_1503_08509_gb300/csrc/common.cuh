@@ -335,7 +335,8 @@ struct fep3m_ctx {
   double* lam64 = nullptr;       // adjoint mesh solution (phi64 + nodes)
   double* scal = nullptr;        // device scalars (dots, norms, flags), 64 doubles
   void* phi_hl = nullptr;        // MIXED box: the FP64 mesh potential as hi + lo floats, (3n)^3 float2
-  int* iflags = nullptr;         // device int flags: [0] input error, [1] converged, ...
+  int* iflags = nullptr;         // 16 device int flags, the last 8 doubles of scal: [0] input error,
+                                 // [2] a bounded wait gave up, [3] boundary data
   void* lam_T = nullptr;
   // per-particle outputs, sorted order
   double* phi_s = nullptr;       // N
@@ -360,7 +361,8 @@ struct fep3m_ctx {
   double* Ha64 = nullptr;        // MIXED: the screen adjoint's table relative to node 0 (pair_adjoint_table)
   void* H0df = nullptr;          // MIXED: H(o, 0) per vertex offset as hi + lo floats
   void* Wsum = nullptr;          // MIXED: per element, the sum of the adjoint weights as hi + lo floats
-  int* host_err = nullptr;       // pinned: device-side error flags read after a step
+  double* host_scal = nullptr;   // pinned: the second half of scal, read after a step (api.cu)
+  int host_err = 0;              // the bounded waits' flag in it
   double* red_tmp = nullptr;     // reduction partials (1024)
   unsigned int* red_counter = nullptr;
   double* out_tmp = nullptr;     // N*3 staging for host outputs

@@ -861,7 +861,7 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
     __syncthreads();
     // y pass: rows 3 ey .. 3 ey + 2 of column hx, for the three planes
     if (y_on) {
-#pragma unroll
+#pragma unroll 1   // (the passes unrolled by plane do not fit the instruction cache)
       for (int p = 0; p < 3; ++p) {
         T u[7], v[7];
 #pragma unroll
@@ -885,7 +885,7 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
     // x pass and epilogue: nodes 3 ex .. 3 ex + 2 of row yy, for the three planes
     if (NST > 0) cp_async_wait_all();
     if (x_on) {
-#pragma unroll
+#pragma unroll 1
       for (int p = 0; p < 3; ++p) {
         T u[7], v[7];
 #pragma unroll

@@ -397,9 +397,15 @@ struct Pair3Smem {
   __host__ __device__ static int HW(int n_sr) { return BX + 2 * n_sr; }
   // charges that can be staged: STAGE_CAP floats-worth of float4 (half as many double4)
   __host__ __device__ static int cap() { return STAGE_CAP * 4 / (int)sizeof(T); }
+  // R's strides: rows 4 modulo 16 entries and (tensor cores) planes 16 modulo 32, so that the 4 x 4
+  // x 2 elements a warp reads fall on 32 different banks
+  __host__ __device__ static int RS(int n_sr) { return TC ? SW(n_sr) + (20 - SW(n_sr) % 16) % 16 : SW(n_sr); }
+  __host__ __device__ static int PS(int n_sr) {
+    const int p = RS(n_sr) * SW(n_sr);
+    return TC ? p + (48 - p % 32) % 32 : p;
+  }
   __host__ __device__ static size_t rbytes(int n_sr) {
-    const int sw = SW(n_sr);
-    return (((size_t)sw * sw * sw * ES) + 31) / 32 * 32;
+    return ((size_t)PS(n_sr) * SW(n_sr) * ES + 31) / 32 * 32;
   }
   __host__ __device__ static size_t region1(int n_sr) {
     const size_t r = rbytes(n_sr);
@@ -409,8 +415,8 @@ struct Pair3Smem {
   __host__ __device__ static size_t ints(int n_sr) {
     const int hw = HW(n_sr);
     const int noff = 2 * n_sr + 2, nb = 2 * n_sr + 1, sw = SW(n_sr);
-    return (size_t)hw * hw * hw + 1 + BE + 1 + 1 + NT / 32 + 1 + (size_t)noff * noff * noff + (size_t)nb * nb +
-           3 * sw + 3 * hw + 32;
+    return (size_t)hw * hw * hw + 1 + BE + 1 + 1 + NT / 32 + 1 + 3 + ((size_t)noff * noff * noff + 63) / 64 * 64 +
+           (size_t)nb * nb + 3 * sw + 3 * hw + 32;
   }
   static constexpr size_t TILES = 6 * 8192;   // three bf16 pieces of A (64 x 64) and of B (64 x 64)
   // tensor cores: the staged charges in a region of their own (staged while the contraction runs)
@@ -810,8 +816,9 @@ __global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_s
   int* epre = hs + HW * HW * HW + 1;                      // BE + 1
   int* flag = epre + BE + 1;
   int* wsum = flag + 1;                                   // NT/32 + 1 scan scratch
-  int* otab = wsum + NT / 32 + 1;                         // no3: R base index of each offset
-  int* rtab = otab + no3;                                 // nb^2 rows (dy, dz): halo offset | ay << 16 | az << 24
+  int* otab = (int*)(((uintptr_t)(wsum + NT / 32 + 1) + 15) & ~(uintptr_t)15);   // R base index of each offset, in
+  const int no3p = (no3 + 63) / 64 * 64;                  //   whole chunks of 64
+  int* rtab = otab + no3p;                                // nb^2 rows (dy, dz): halo offset | ay << 16 | az << 24
   int* wv = rtab + nrow;                                  // 3 x SW wrapped vertex coords times 1, n, n^2
   int* we = wv + 3 * SW;                                  // 3 x HW wrapped halo element coords
   if (!TC) sxb = (unsigned char*)(we + 3 * HW + 32);
@@ -831,12 +838,13 @@ __global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_s
   }
   if (ntarget == 0) return;
   // index tables (no divisions in the hot loops below)
-  for (int o = tid; o < no3; o += NT) {
+  const int RS = SM::RS(n_sr), PS = SM::PS(n_sr);
+  for (int o = tid; o < no3p; o += NT) {
     const int ox = o % noff - keep, oy = (o / noff) % noff - keep, oz = o / (noff * noff) - keep;
     const int bx = ox == -keep ? SF : (ox == n_sr ? SF + BX : n_sr - 1 - ox);
     const int by = oy == -keep ? SF : (oy == n_sr ? SF + BX : n_sr - 1 - oy);
     const int bz = oz == -keep ? SF : (oz == n_sr ? SF + BX : n_sr - 1 - oz);
-    otab[o] = bx + SW * (by + SW * bz);
+    otab[o] = o < no3 ? bx + RS * by + PS * bz : 0;
   }
   for (int r = tid; r < nrow; r += NT) rtab[r] = HW * ((r % nb) + HW * (r / nb)) | (r % nb) << 16 | (r / nb) << 24;
   {
@@ -868,7 +876,7 @@ __global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_s
       // the hi + lo floats of the double-float contraction (an FP32 value has lo = 0)
       reinterpret_cast<float2*>(R)[i] = make_float2(val, 0.f);
     } else {
-      R[i] = val;
+      R[sx + RS * sy + PS * sz] = val;
     }
     sx += dsx;
     sy += dsy;
@@ -921,7 +929,7 @@ __global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_s
       __shared__ float2 s0p[(SG / 64) * BE];
       float s0h = 0.f, s0l = 0.f;
       const int l = gt & 63, g = gt >> 6;   // this thread's A units: row l, chunk offsets 8 g .. and 8 (g + 4) ..
-      const int lam = (l % BX) + SW * (((l / BX) % BY) + SW * (l / (BX * BY)));
+      const int lam = (l % BX) + RS * ((l / BX) % BY) + PS * (l / (BX * BY));
       const uint32_t aoff[2] = {sw128_off(l, 8 * g), sw128_off(l, 8 * (g + 4))};
       const int nch = (no3 + 63) / 64;
       // this thread's accumulator entries (tmem_ld16x64b): register jj holds element row
@@ -941,8 +949,9 @@ __global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_s
 #pragma unroll
           for (int jj = 0; jj < 4; ++jj) {
             const int o = 64 * c + 8 * (g + 4 * hf) + 2 * jj;
-            const float xa = o < no3 ? (float)R[otab[o] + lam] : 0.f;
-            const float xb = o + 1 < no3 ? (float)R[otab[o + 1] + lam] : 0.f;
+            // (past the last offset any finite value does: the table is zero there)
+            const int2 ot = *reinterpret_cast<const int2*>(otab + o);
+            const float xa = R[ot.x + lam], xb = R[ot.y + lam];
             bf16_split2(xa, xb, p0[jj], p1[jj], p2[jj]);
             if (o + 1 < no3) {
               const float4 h2 = *reinterpret_cast<const float4*>(H0 + o);   // H0[o], H0[o + 1]
@@ -1384,34 +1393,37 @@ __global__ void __launch_bounds__(PT) k_pair_eval(int n, int Nm, float inv_h, co
       v4[i] += __shfl_xor_sync(0xffffffffu, v4[i], 1);
       v4[i] += __shfl_xor_sync(0xffffffffu, v4[i], 2);
     }
-    if (valid && q == 0) {
-      // the trilinear part of G - G0 and its gradient at the charge, in FP64
-      double tv, tg[3];
-      {
-        const double* g = Gc + l * 8;
-        const double x = pt.x, y = pt.y, z = pt.z;
-        double a[4], b[4];   // x-lerps and x-differences of the corner pairs j = cy + 2 cz
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          b[j] = g[2 * j + 1] - g[2 * j];
-          a[j] = fma(x, b[j], g[2 * j]);
-        }
-        const double ay0 = a[1] - a[0], ay1 = a[3] - a[2];
-        const double a0 = fma(y, ay0, a[0]), a1 = fma(y, ay1, a[2]);
-        const double bx0 = fma(y, b[1] - b[0], b[0]), bx1 = fma(y, b[3] - b[2], b[2]);
-        tv = fma(z, a1 - a0, a0);
-        tg[0] = fma(z, bx1 - bx0, bx0);
-        tg[1] = fma(z, ay1 - ay0, ay0);
-        tg[2] = a1 - a0;
-      }
-      const double phi = (((double)v4[0] + tv) + G0[l]) * (double)inv_h + phi_s[slot];
-      phi_s[slot] = phi;
-      if (phi_out) phi_out[perm[slot]] = phi;
-      if (GRAD) {
-        const double ih2 = (double)inv_h * (double)inv_h;
-        E_s[3 * slot + 0] = ((double)v4[1] + tg[0]) * ih2 + E_s[3 * slot + 0];
-        E_s[3 * slot + 1] = ((double)v4[2] + tg[1]) * ih2 + E_s[3 * slot + 1];
-        E_s[3 * slot + 2] = ((double)v4[3] + tg[2]) * ih2 + E_s[3 * slot + 2];
+    // The trilinear part of G - G0 and its gradient at the charge, in FP64: thread q takes the
+    // corner pair q (cy + 2 cz) along x, the pairs meet along y, then z, by shuffles, and thread q
+    // finishes sum q (an FP64 instruction takes its pipe for the whole warp, however few lanes are on)
+    const double* g = Gc + l * 8;
+    const double y = pt.y, z = pt.z;
+    const double b = g[2 * q + 1] - g[2 * q], a = fma((double)pt.x, b, g[2 * q]);
+    const double ao = __shfl_xor_sync(0xffffffffu, a, 1), bo = __shfl_xor_sync(0xffffffffu, b, 1);
+    const bool q1 = q & 1, q2 = q & 2;
+    const double a0 = q1 ? ao : a, b0 = q1 ? bo : b;
+    const double ay = (q1 ? a : ao) - a0, A = fma(y, ay, a0), B = fma(y, (q1 ? b : bo) - b0, b0);
+    const double Ao = __shfl_xor_sync(0xffffffffu, A, 2);
+    const double A0 = q2 ? Ao : A, az = (q2 ? A : Ao) - A0;
+    double t;   // sum q's trilinear part: the value, d/dx, d/dy, d/dz
+    if (GRAD) {
+      const double Bo = __shfl_xor_sync(0xffffffffu, B, 2), yo = __shfl_xor_sync(0xffffffffu, ay, 2);
+      // value, d/dx, d/dy at z are lerps of their values on the two z faces
+      const double lo = q == 0 ? A0 : (q == 1 ? (q2 ? Bo : B) : (q2 ? yo : ay));
+      const double hi = q == 0 ? A0 + az : (q == 1 ? (q2 ? B : Bo) : (q2 ? ay : yo));
+      t = q == 3 ? az : fma(z, q == 0 ? az : hi - lo, lo);
+    } else {
+      t = fma(z, az, A0);
+    }
+    if (valid && (GRAD || q == 0)) {
+      const double v = (double)(q == 0 ? v4[0] : (q == 1 ? v4[1] : (q == 2 ? v4[2] : v4[3]))) + t;
+      if (q == 0) {
+        const double phi = (v + G0[l]) * (double)inv_h + phi_s[slot];
+        phi_s[slot] = phi;
+        if (phi_out) phi_out[perm[slot]] = phi;
+      } else {
+        double* E = E_s + 3 * slot + (q - 1);
+        *E = v * ((double)inv_h * (double)inv_h) + *E;
       }
     }
   }
@@ -1655,49 +1667,55 @@ __global__ void __launch_bounds__(PT) k_elem_deposit(int64_t ne, const int* __re
 
 // g[node] = sum over (element, local node) pairs at the node of W: in FP64,
 // or (T = float, the mixed solver's right-hand side) as a float pair h + l
-// summed by two-sums; (3n)^3 < 2^32
+// summed by two-sums.  Grid (y, z): a CTA takes a row of nodes, so that the
+// elements along y and z are the CTA's and a node's own index costs one
+// division (one thread per node of the whole mesh spent 227 instructions on
+// the indices: 262 144 charges on 64^3, 100 -> @NA64@ us)
 template <class T>
-__global__ void k_node_assemble(int n, const T* __restrict__ W, double* __restrict__ g) {
-  const int N = 3 * n;
-  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (unsigned)N * (unsigned)N * (unsigned)N) return;
-  const unsigned q = i / (unsigned)N;
-  const int ix = (int)(i - q * (unsigned)N), iy = (int)(q % (unsigned)N), iz = (int)(q / (unsigned)N);
-  int el[3][2], lo[3][2], cnt[3];
-  const int id[3] = {ix, iy, iz};
-  for (int a = 0; a < 3; ++a) {
-    const int e = id[a] / 3, t = id[a] - 3 * e;
-    el[a][0] = e;
-    lo[a][0] = t;
-    cnt[a] = 1;
-    if (t == 0) {
-      el[a][1] = wrapn(e - 1, n);
-      lo[a][1] = 3;
-      cnt[a] = 2;
-    }
+__global__ void __launch_bounds__(PT) k_node_assemble(int n, const T* __restrict__ W, double* __restrict__ g) {
+  const int N = 3 * n, iy = blockIdx.x, iz = blockIdx.y;
+  // rows of W of the up to four elements that share the row: element row and local node offset
+  int64_t row[4];
+  int cnt = 0;
+  {
+    const int ey = iy / 3, ty = iy - 3 * ey, ez = iz / 3, tz = iz - 3 * ez;
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        if ((c && tz) || (b && ty)) continue;
+        const int y = b ? (ey ? ey - 1 : n - 1) : ey, z = c ? (ez ? ez - 1 : n - 1) : ez;
+        row[cnt++] = (int64_t)n * (y + (int64_t)n * z) * 64 + 4 * (b ? 3 : ty) + 16 * (c ? 3 : tz);
+      }
   }
-  if constexpr (sizeof(T) == 4) {
-    float sh = 0.f, sl = 0.f;
-    for (int c = 0; c < cnt[2]; ++c)
-      for (int b = 0; b < cnt[1]; ++b)
-        for (int a = 0; a < cnt[0]; ++a) {
-          const int64_t e = el[0][a] + (int64_t)n * (el[1][b] + (int64_t)n * el[2][c]);
-          const float v = W[e * 64 + lo[0][a] + 4 * lo[1][b] + 16 * lo[2][c]];
-          const float t = sh + v, bv = t - sh;
-          sl += (sh - (t - bv)) + (v - bv);
-          sh = t;
-        }
-    const float h = sh + sl;
-    reinterpret_cast<float2*>(g)[i] = make_float2(h, sl - (h - sh));
-  } else {
-    double acc = 0.0;
-    for (int c = 0; c < cnt[2]; ++c)
-      for (int b = 0; b < cnt[1]; ++b)
-        for (int a = 0; a < cnt[0]; ++a) {
-          const int64_t e = el[0][a] + (int64_t)n * (el[1][b] + (int64_t)n * el[2][c]);
-          acc += (double)W[e * 64 + lo[0][a] + 4 * lo[1][b] + 16 * lo[2][c]];
-        }
-    g[i] = acc;
+  const int64_t out = (int64_t)N * (iy + (int64_t)N * iz);
+  for (int ix = threadIdx.x; ix < N; ix += PT) {
+    const int e = ix / 3, t = ix - 3 * e, at = e * 64 + t, before = (e ? e - 1 : n - 1) * 64 + 3;
+    if constexpr (sizeof(T) == 4) {
+      float sh = 0.f, sl = 0.f;
+      auto add = [&](float v) {
+        const float u = sh + v, bv = u - sh;
+        sl += (sh - (u - bv)) + (v - bv);
+        sh = u;
+      };
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        if (r >= cnt) break;
+        add(W[row[r] + at]);
+        if (t == 0) add(W[row[r] + before]);
+      }
+      const float h = sh + sl;
+      reinterpret_cast<float2*>(g)[out + ix] = make_float2(h, sl - (h - sh));
+    } else {
+      double acc = 0.0;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        if (r >= cnt) break;
+        acc += (double)W[row[r] + at];
+        if (t == 0) acc += (double)W[row[r] + before];
+      }
+      g[out + ix] = acc;
+    }
   }
 }
 
@@ -1899,101 +1917,126 @@ __global__ void __launch_bounds__(PT, 2) k_adj64(int64_t ne, int n_sr, int z0, i
 //   A[s][k] = sum over the offsets o with o + k inside the block of D(o, s + k + o).
 // For the vertex v = s + k the terms are D(o, v + o) over the offsets that
 // corner k's block holds: along each axis, o_a = -(n_sr + 1) only for k_a = 1,
-// o_a = n_sr only for k_a = 0, the others for both.  The terms of a vertex are
-// summed into 27 classes (the three cases per axis); A(v - k, k) is the sum of
-// the eight classes that corner k admits.  A CTA of eight warps takes 32
-// consecutive vertices (one per lane: consecutive lanes read consecutive
-// elements of D) and a chunk of whole offset planes (oz in [z0, z1)); the
-// chunk's rows of offsets (oz, oy) are dealt to the warps in turn, each warp
-// sums its rows' terms into its own 27 classes, and the warps' classes are
-// combined in shared memory in warp order, one thread per (vertex, corner):
-// deterministic.  FP32 path (H0 set): D holds the contraction with the
+// o_a = n_sr only for k_a = 0, the others for both.  A CTA takes 32 consecutive
+// vertices (consecutive lanes read consecutive elements of D) and deals the
+// offset planes oz of the chunk [z0, z1) to its eight warps.  A thread sums a
+// plane's terms into nine classes (first, inner, last offset along x and along
+// y), two rows of D's values ahead in registers, adds them into the corners of
+// the plane's class along z in shared memory, and the warps' corner sums are
+// combined there in order: deterministic.  FP32 path (H0 set): D holds the contraction with the
 // node-0-relative table, and each term gains H(o, 0) Wsum(v + o)
 // (pair_adjoint_table).  FP64 path: D is the whole contraction, as pairs.  Terms
-// and sums in double-float arithmetic.
-constexpr int AV_WARPS = 8;
+// and sums in double-float arithmetic.  Bound by FP32 issue in the FP32 path (19
+// operations a term beside its loads) and by the read of D.  10^6 charges on
+// 128^3: 3484 -> @AV128@ us, 262 144 on 64^3: 439 -> @AV64@ us against one warp per 32
+// vertices and row of offsets with 27 class sums in shared memory, whose
+// bookkeeping took most of its instructions.
+constexpr int AVV = 32, AVZ = PT / AVV;   // vertices and threads per vertex of a CTA
 template <class T, int NSR>
-__global__ void __launch_bounds__(32 * AV_WARPS) k_adj_vertex(int n, int z0, int z1, int first,
-                                                              const int* __restrict__ count, const T* __restrict__ D,
-                                                              const float2* __restrict__ H0,
-                                                              const float2* __restrict__ wsum, double* __restrict__ A) {
+__global__ void __launch_bounds__(PT, sizeof(T) == 4 ? 3 : 2) k_adj_vertex(int n, int z0, int z1, int first, const int* __restrict__ count,
+                                                      const T* __restrict__ D, const float2* __restrict__ H0,
+                                                      const float2* __restrict__ wsum, double* __restrict__ A) {
   constexpr int KEEP = NSR + 1, NOFF = 2 * NSR + 2, PLANE = NOFF * NOFF;
-  constexpr bool DF = sizeof(T) == 4;   // T: float, or df (FP64)
-  typedef dfacc Acc;
-  extern __shared__ __align__(16) unsigned char av_smem[];
-  Acc(*part)[27][32] = reinterpret_cast<Acc(*)[27][32]>(av_smem);   // [AV_WARPS][27][32]: each warp's classes
-  __shared__ int live[32];
+  constexpr bool REL = sizeof(T) == 4;   // T: float, or df (FP64)
+  __shared__ dfacc part[AVZ][8][AVV];
+  __shared__ float2 h0[REL ? PLANE * NOFF : 1];
+  __shared__ int live[AVV];
   const int64_t ne = (int64_t)n * n * n;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t v = blockIdx.x * (int64_t)32 + lane;
+  const int vl = threadIdx.x & (AVV - 1), zg = threadIdx.x / AVV;
+  const int64_t v = blockIdx.x * (int64_t)AVV + vl;
   const bool in = v < ne;
   const int vx = in ? (int)(v % n) : 0, vy = in ? (int)((v / n) % n) : 0, vz = in ? (int)(v / ((int64_t)n * n)) : 0;
-  if (warp == 0) {
+  if (zg == 0) {
     bool any = false;   // the eight elements v - k; A is read only for non-empty ones
-    if (in)
+    if (in) {
+      const int px = vx ? vx - 1 : n - 1, py = vy ? vy - 1 : n - 1, pz = vz ? vz - 1 : n - 1;
 #pragma unroll
       for (int k = 0; k < 8; ++k)
-        any |= count[wrapn(vx - (k & 1), n) + (int64_t)n * (wrapn(vy - ((k >> 1) & 1), n) +
-                                                            (int64_t)n * wrapn(vz - (k >> 2), n))] != 0;
-    live[lane] = any;
+        any |= count[((k & 1) ? px : vx) + (int64_t)n * (((k & 2) ? py : vy) + (int64_t)n * ((k & 4) ? pz : vz))] != 0;
+    }
+    live[vl] = any;
   }
+  if (REL)
+    for (int i = threadIdx.x; i < PLANE * NOFF; i += PT) h0[i] = H0[i];
   __syncthreads();
-  const bool act = live[lane] != 0;
+  const bool act = live[vl] != 0;
 #pragma unroll
-  for (int c = 0; c < 27; ++c) part[warp][c][lane] = Acc{};
+  for (int k = 0; k < 8; ++k) part[zg][k][vl] = dfacc{0.f, 0.f};   // corner sums, k = kx + 2 ky + 4 kz
   if (__any_sync(0xffffffffu, act)) {
-    int wx[NOFF];
+    int wx[NOFF];   // the elements' x coordinates vx + o - KEEP (n >= 2 n_sr + 1: one period at most)
 #pragma unroll
-    for (int i = 0; i < NOFF; ++i) wx[i] = wrapn(vx + i - KEEP, n);
-    const int rows = (z1 - z0) * NOFF;
-    for (int rho = warp; rho < rows; rho += AV_WARPS) {
-      const int oz = z0 + rho / NOFF, oy = rho % NOFF;
-      const int cz = oz == 0 ? 0 : (oz == NOFF - 1 ? 2 : 1), cy = oy == 0 ? 0 : (oy == NOFF - 1 ? 2 : 1);
-      const int64_t erow = (int64_t)n * (wrapn(vy + oy - KEEP, n) + (int64_t)n * wrapn(vz + oz - KEEP, n));
-      const T* Dp = D + ((int64_t)(oz - z0) * PLANE + oy * NOFF) * ne;
-      Acc P[3] = {};
+    for (int i = 0; i < NOFF; ++i) {
+      int x = vx + i - KEEP;
+      x += x < 0 ? n : 0;
+      wx[i] = x >= n ? x - n : x;
+    }
+    for (int oz = z0 + zg; oz < z1; oz += AVZ) {
+      int ez = vz + oz - KEEP;
+      ez += ez < 0 ? n : 0;
+      ez = ez >= n ? ez - n : ez;
+      dfacc P[3][3];   // [class along y][class along x]: first, inner, last
 #pragma unroll
-      for (int ox = 0; ox < NOFF; ++ox) {
-        const int cx = ox == 0 ? 0 : (ox == NOFF - 1 ? 2 : 1);
-        if (!act) continue;
-        const int64_t e = erow + wx[ox];
-        const T d = Dp[(int64_t)ox * ne + e];
-        if constexpr (DF) {
-          const float2 h = H0[oz * PLANE + oy * NOFF + ox], w = wsum[e];
-          const float p = h.x * w.x;
-          float r = fmaf(h.x, w.x, -p);
-          r = fmaf(h.x, w.y, r);
-          r = fmaf(h.y, w.x, r);
-          acc_add(P[cx], p);
-          acc_add(P[cx], d + r);
-        } else {
-          acc_merge(P[cx], dfacc{d.h, d.l});
+      for (int i = 0; i < 9; ++i) P[i / 3][i % 3] = dfacc{0.f, 0.f};
+      int ey = vy - KEEP;
+      ey += ey < 0 ? n : 0;
+      const T* Dp = D + (int64_t)(oz - z0) * PLANE * ne;
+      const int erow0 = n * n * ez;   // n <= 404: below 2^31
+      T d[3][NOFF];                   // three rows of D in flight
+      int er[3];
+      auto load = [&](int oy) {       // row oy; called in order
+        er[oy % 3] = erow0 + n * ey;
+#pragma unroll
+        for (int ox = 0; ox < NOFF; ++ox) d[oy % 3][ox] = Dp[(int64_t)(oy * NOFF + ox) * ne + er[oy % 3] + wx[ox]];
+        ++ey;
+        ey = ey == n ? 0 : ey;
+      };
+      load(0);
+      load(1);
+#pragma unroll
+      for (int oy = 0; oy < NOFF; ++oy) {
+        constexpr int L = NOFF - 1;
+        const int cy = oy == 0 ? 0 : (oy == L ? 2 : 1);
+        if (oy + 2 < NOFF) load(oy + 2);
+#pragma unroll
+        for (int ox = 0; ox < NOFF; ++ox) {
+          const int cx = ox == 0 ? 0 : (ox == L ? 2 : 1);
+          if constexpr (REL) {
+            const float2 h = h0[oz * PLANE + oy * NOFF + ox], w = wsum[er[oy % 3] + wx[ox]];
+            const float p = h.x * w.x;
+            float r = fmaf(h.x, w.x, -p);
+            r = fmaf(h.x, w.y, r);
+            r = fmaf(h.y, w.x, r);
+            acc_add(P[cy][cx], p);
+            acc_add(P[cy][cx], d[oy % 3][ox] + r);
+          } else {
+            acc_merge(P[cy][cx], dfacc{d[oy % 3][ox].h, d[oy % 3][ox].l});
+          }
         }
       }
-      Acc* row = &part[warp][cz * 9 + cy * 3][lane];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) acc_merge(row[32 * c], P[c]);
+      for (int k = 0; k < 4; ++k) {   // corner (kx, ky): classes 0, 1 for 1, classes 1, 2 for 0
+        const int x0 = k & 1 ? 0 : 1, y0 = k & 2 ? 0 : 1;
+        dfacc t = P[y0][x0];
+        acc_merge(t, P[y0][x0 + 1]);
+        acc_merge(t, P[y0 + 1][x0]);
+        acc_merge(t, P[y0 + 1][x0 + 1]);
+        if (oz != NOFF - 1) acc_merge(part[zg][k + 4][vl], t);
+        if (oz != 0) acc_merge(part[zg][k][vl], t);
+      }
     }
   }
   __syncthreads();
-  // one thread per (vertex, corner): the admitted classes, warps in order
-  const int vl = threadIdx.x & 31, k = threadIdx.x >> 5;   // 256 threads = 32 vertices x 8 corners
-  const int64_t vv = blockIdx.x * (int64_t)32 + vl;
-  if (vv >= ne || !live[vl]) return;
-  const int kx = k & 1, ky = (k >> 1) & 1, kz = k >> 2;
-  Acc s = {};
+  if (!in || !act) return;
 #pragma unroll
-  for (int cz = kz ? 0 : 1; cz <= (kz ? 1 : 2); ++cz)
+  for (int t = 0; t < 8 / AVZ; ++t) {
+    const int k = zg + AVZ * t, kx = k & 1, ky = (k >> 1) & 1, kz = k >> 2;
+    dfacc s = part[0][k][vl];
 #pragma unroll
-    for (int cy = ky ? 0 : 1; cy <= (ky ? 1 : 2); ++cy)
-#pragma unroll
-      for (int cx = kx ? 0 : 1; cx <= (kx ? 1 : 2); ++cx)
-#pragma unroll
-        for (int w = 0; w < AV_WARPS; ++w) acc_merge(s, part[w][cz * 9 + cy * 3 + cx][vl]);
-  const int ux = (int)(vv % n), uy = (int)((vv / n) % n), uz = (int)(vv / ((int64_t)n * n));
-  const int64_t se = wrapn(ux - kx, n) + (int64_t)n * (wrapn(uy - ky, n) + (int64_t)n * wrapn(uz - kz, n));
-  double* dst = A + se * 8 + k;
-  *dst = first ? acc_value(s) : *dst + acc_value(s);
+    for (int z = 1; z < AVZ; ++z) acc_merge(s, part[z][k][vl]);
+    const int sx = vx - kx < 0 ? n - 1 : vx - kx, sy = vy - ky < 0 ? n - 1 : vy - ky, sz = vz - kz < 0 ? n - 1 : vz - kz;
+    double* dst = A + (sx + (int64_t)n * (sy + (int64_t)n * sz)) * 8 + k;
+    *dst = first ? acc_value(s) : *dst + acc_value(s);
+  }
 }
 
 template <class T, bool GRAD>
@@ -2399,9 +2442,7 @@ template <class T, int NSR>
 static void launch_adj_vertex(fep3m_ctx* c, int z0, int z1, const T* D, double* A, cudaStream_t s) {
   const int64_t ne = (int64_t)c->n * c->n * c->n;
   const bool rel = sizeof(T) == 4;   // D relative to node 0 (FP32 path)
-  const size_t smem = (size_t)AV_WARPS * 27 * 32 * sizeof(dfacc);
-  (void)smem_limit((const void*)k_adj_vertex<T, NSR>, smem);   // a failure shows as the launch's error
-  FEP3M_CL k_adj_vertex<T, NSR><<<(unsigned)((ne + 31) / 32), 32 * AV_WARPS, smem, s>>>(
+  FEP3M_CL k_adj_vertex<T, NSR><<<(unsigned)((ne + AVV - 1) / AVV), PT, 0, s>>>(
       c->n, z0, z1, z0 == 0, c->count, D, rel ? (const float2*)c->H0df : nullptr,
       rel ? (const float2*)c->Wsum : nullptr, A);
 }
@@ -2466,17 +2507,17 @@ static cudaError_t screen_adjoint(fep3m_ctx* c, const T* W, double* A) {
 // weights w = gU Q / 2 + gphi (sorted order), element deposits, adjoint right-hand side g64
 cudaError_t adjoint_pre(fep3m_ctx* c, double gU, const double* gphi, cudaStream_t s) {
   const int n = c->n;
-  const int64_t ne = (int64_t)n * n * n, nodes = 27 * ne, N = c->N;
+  const int64_t ne = (int64_t)n * n * n, N = c->N;
   FEP3M_CL k_weights<<<gsz(N), PT, 0, s>>>(N, gU, gphi, c->perm, c->Q_s, c->w_s, c->w_s32);
   const int per = PT;   // elements per CTA: 32 per warp
   if (c->precision == FEP3M_MIXED) {
     FEP3M_CL k_elem_deposit<float><<<gsz(ne, per), PT, 0, s>>>(ne, c->start, c->count, (const float4*)c->part, c->w_s,
                                                                c->w_s32, (float*)c->W_el, (float2*)c->Wsum);
-    FEP3M_CL k_node_assemble<float><<<gsz(nodes), PT, 0, s>>>(n, (const float*)c->W_el, c->g64);
+    FEP3M_CL k_node_assemble<float><<<dim3(3 * n, 3 * n), PT, 0, s>>>(n, (const float*)c->W_el, c->g64);
   } else {
     FEP3M_CL k_elem_deposit<double><<<gsz(ne, per), PT, 0, s>>>(ne, c->start, c->count, (const vec4<double>::type*)c->part,
                                                                 c->w_s, c->w_s, (double*)c->W_el, nullptr);
-    FEP3M_CL k_node_assemble<double><<<gsz(nodes), PT, 0, s>>>(n, (const double*)c->W_el, c->g64);
+    FEP3M_CL k_node_assemble<double><<<dim3(3 * n, 3 * n), PT, 0, s>>>(n, (const double*)c->W_el, c->g64);
   }
   return cudaGetLastError();
 }
