@@ -1933,7 +1933,7 @@ __global__ void __launch_bounds__(PT, 2) k_adj64(int64_t ne, int n_sr, int z0, i
 // bookkeeping took most of its instructions.
 constexpr int AVV = 32, AVZ = PT / AVV;   // vertices and threads per vertex of a CTA
 template <class T, int NSR>
-__global__ void __launch_bounds__(PT, sizeof(T) == 4 ? 3 : 2) k_adj_vertex(int n, int z0, int z1, int first, const int* __restrict__ count,
+__global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int first, const int* __restrict__ count,
                                                       const T* __restrict__ D, const float2* __restrict__ H0,
                                                       const float2* __restrict__ wsum, double* __restrict__ A) {
   constexpr int KEEP = NSR + 1, NOFF = 2 * NSR + 2, PLANE = NOFF * NOFF;
@@ -1981,35 +1981,37 @@ __global__ void __launch_bounds__(PT, sizeof(T) == 4 ? 3 : 2) k_adj_vertex(int n
       ey += ey < 0 ? n : 0;
       const T* Dp = D + (int64_t)(oz - z0) * PLANE * ne;
       const int erow0 = n * n * ez;   // n <= 404: below 2^31
-      T d[3][NOFF];                   // three rows of D in flight
-      int er[3];
+      T d[2][NOFF];                   // the row of D being summed and the next (and its weight sums)
+      float2 w[REL ? 2 : 1][NOFF];
       auto load = [&](int oy) {       // row oy; called in order
-        er[oy % 3] = erow0 + n * ey;
+        const int er = erow0 + n * ey;
 #pragma unroll
-        for (int ox = 0; ox < NOFF; ++ox) d[oy % 3][ox] = Dp[(int64_t)(oy * NOFF + ox) * ne + er[oy % 3] + wx[ox]];
+        for (int ox = 0; ox < NOFF; ++ox) {
+          d[oy & 1][ox] = Dp[(int64_t)(oy * NOFF + ox) * ne + er + wx[ox]];
+          if constexpr (REL) w[oy & 1][ox] = wsum[er + wx[ox]];
+        }
         ++ey;
         ey = ey == n ? 0 : ey;
       };
       load(0);
-      load(1);
 #pragma unroll
       for (int oy = 0; oy < NOFF; ++oy) {
         constexpr int L = NOFF - 1;
         const int cy = oy == 0 ? 0 : (oy == L ? 2 : 1);
-        if (oy + 2 < NOFF) load(oy + 2);
+        if (oy + 1 < NOFF) load(oy + 1);
 #pragma unroll
         for (int ox = 0; ox < NOFF; ++ox) {
           const int cx = ox == 0 ? 0 : (ox == L ? 2 : 1);
           if constexpr (REL) {
-            const float2 h = h0[oz * PLANE + oy * NOFF + ox], w = wsum[er[oy % 3] + wx[ox]];
-            const float p = h.x * w.x;
-            float r = fmaf(h.x, w.x, -p);
-            r = fmaf(h.x, w.y, r);
-            r = fmaf(h.y, w.x, r);
+            const float2 h = h0[oz * PLANE + oy * NOFF + ox], u = w[oy & 1][ox];
+            const float p = h.x * u.x;
+            float r = fmaf(h.x, u.x, -p);
+            r = fmaf(h.x, u.y, r);
+            r = fmaf(h.y, u.x, r);
             acc_add(P[cy][cx], p);
-            acc_add(P[cy][cx], d[oy % 3][ox] + r);
+            acc_add(P[cy][cx], d[oy & 1][ox] + r);
           } else {
-            acc_merge(P[cy][cx], dfacc{d[oy % 3][ox].h, d[oy % 3][ox].l});
+            acc_merge(P[cy][cx], dfacc{d[oy & 1][ox].h, d[oy & 1][ox].l});
           }
         }
       }
