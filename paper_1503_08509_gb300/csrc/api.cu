@@ -263,14 +263,20 @@ int run_forward(fep3m_ctx* c, double* phi_dev, int want_grad, double* force_dev,
     CK(cudaEventRecord(c->ev_solved, c->stream));
   } else {
     CK(mesh_solve_begin(F, c->b64, c->phi64));
+    CK(cudaEventRecord(c->ev_solved, c->stream));
   }
-  CK(cudaStreamWaitEvent(c->pair_stream, c->ev_pfork, 0));
+  // A solve whose passes hold whole SMs (large meshes) is not run beside the other kernels,
+  // which fill the GPU on their own too: its CTAs would wait for SMs the short CTAs keep
+  // refilling (10^6 charges on 128^3: 23.5 ms a step beside each other, 21.7 ms one after the other)
+  const bool alone = fep3m::mesh_solve_alone(F);
+  CK(cudaStreamWaitEvent(c->pair_stream, alone ? c->ev_solved : c->ev_pfork, 0));
   ev_record(c, 8, c->pair_stream);
   CK(pair_screen(c, want_grad, c->pair_stream, force_dev != nullptr));
   ev_record(c, 9, c->pair_stream);
   CK(cudaEventRecord(c->ev_pjoin, c->pair_stream));
   if (force_dev) {
     CK(cudaStreamWaitEvent(c->sweep_stream, c->ev_fork2, 0));
+    if (alone) CK(cudaStreamWaitEvent(c->sweep_stream, c->ev_solved, 0));
     CK(adjoint_sweeps(c, c->sweep_stream, false));   // singular part: from the screen kernel
     CK(cudaEventRecord(c->ev_join2, c->sweep_stream));
     if (paired) CK(cudaStreamWaitEvent(c->aux_stream, c->ev_solved, 0));
@@ -755,9 +761,11 @@ int fep3m_vjp(fep3m_ctx* c, double gU, const double* gphi, double* dpos, double*
   CK(adjoint_pre(c, gU, g, c->aux_stream));
   CK(cudaEventRecord(c->ev_fork2, c->aux_stream));
   CK(cudaStreamWaitEvent(c->sweep_stream, c->ev_fork2, 0));
+  const bool alone = fep3m::mesh_solve_alone(&c->solv[1]);   // (run_forward)
+  if (alone) CK(mesh_solve(&c->solv[1], c->g64, c->lam64));   // has finished when it returns
   CK(adjoint_sweeps(c, c->sweep_stream, true));
   CK(cudaEventRecord(c->ev_join2, c->sweep_stream));
-  CK(mesh_solve(&c->solv[1], c->g64, c->lam64));
+  if (!alone) CK(mesh_solve(&c->solv[1], c->g64, c->lam64));
   c->stats.adj_iterations = c->solv[1].iters;
   c->stats.adj_rel_residual = c->solv[1].relres;
   CK(adjoint_vertex(c, c->aux_stream));

@@ -123,6 +123,12 @@ struct FineFDM {
   void* BpF = nullptr;
   void* BpI = nullptr;
   int nt = 0, ntile = 0;
+  // the passes by parity (k_tc_pass; set for large periodic order-3 meshes): the pieces of both
+  // tables, the eigenvalues with even modes first, the constant mode's place among them
+  void* PpF = nullptr;
+  void* PpI = nullptr;
+  float* plam = nullptr;
+  int pnt = 0, pntile = 0, pnull = -1, psms = 0;
   int* err = nullptr;         // device flag: a bounded wait gave up
 };
 
@@ -418,9 +424,10 @@ cudaError_t solver_init(Solver* s, const fep3m_ctx* c, cudaStream_t stream, int 
 // fast-diagonalisation solve of a periodic N^3 mesh from its 1-D eigenpairs
 // (mesh.cu): device data, x = K^+ b in FP32 (six transform passes; w1, w2 N^3
 // scratch), release
-// (rhs: right-hand sides per pass the solve will usually take, for the tile shape)
+// (rhs: right-hand sides per pass the solve will usually take, for the tile shape;
+// periodic3: the eigenbasis of a periodic order-3 mesh, which may be split by parity)
 cudaError_t fdm_setup(FineFDM& f, int N, const std::vector<double>& lam, const std::vector<double>& V, int rhs,
-                      bool tensor_cores, bool null_mode = true);
+                      bool tensor_cores, bool null_mode = true, bool periodic3 = false);
 // V vectors at a stride of vs values (V = 2 with the tensor-core passes only)
 cudaError_t fdm_apply(const FineFDM& f, const float* b, float* x, float* w1, float* w2, cudaStream_t s, int V = 1,
                       int64_t vs = 0);
@@ -449,6 +456,7 @@ cudaError_t mesh_solve_begin2(Solver* s, const double* b, double* phi);
 // as mesh_solve_check, for both right-hand sides of the paired solve
 bool mesh_solve_check2(Solver* s);
 bool mesh_solve_paired(const Solver* s);   // the solver can pair right-hand sides
+bool mesh_solve_alone(const Solver* s);    // its passes take whole SMs (k_tc_pass)
 cudaError_t pair_counts(fep3m_ctx* c, unsigned long long* dev5, cudaStream_t s);
 // short-range part in two launches: the screen contraction and the singular
 // sums need only the binned charges and the vertex density, so they run on

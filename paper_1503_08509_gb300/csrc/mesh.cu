@@ -1490,6 +1490,293 @@ __global__ void __launch_bounds__(FT_THREADS) k_tc_rows(int64_t R, int K, int cb
   if (warp == 0) tmem_dealloc(tmem, ncols);
 }
 
+// ---- the transform pass by parity (periodic order-3 meshes)
+//
+// The 1-D operators are symmetric under reflection about an element's centre,
+// node k <-> 3 - k (mod N), so the eigenbasis is chosen with every mode even or
+// odd (parity_basis).  With the node pairs i = 0 .. P - 1, P = ceil(N / 2), of
+// nodes 2 + i and 1 - i (for an odd N the last pair is one node), a pass is two
+// independent products of half the length:
+//   analysis   c_e[j] = sum_i V[2 + i][e_j] (x[2 + i] + x[1 - i]),
+//              c_o[j] = sum_i V[2 + i][o_j] (x[2 + i] - x[1 - i])
+//   synthesis  s = sum_j V[2 + i][e_j] c_e[j], a = sum_j V[2 + i][o_j] c_o[j],
+//              x[2 + i] = s + a, x[1 - i] = s - a
+// with the modes stored even ones first.  Half the multiply-adds and half the
+// table of k_tc_rows; the pieces, the accumulators and the output with the axes
+// rotated are as there.
+//
+// A persistent CTA per SM takes jobs of 128 rows and nt pair columns (even and
+// odd: four TMEM accumulators of nt columns).  A contraction chunk is 32 entries
+// of each parity side by side in one 64-wide operand tile, its first half for
+// the even product and its second for the odd one; within it entry 8 t + 2 q + b
+// sits at place 8 q + 2 t + b (operand and table alike), so that the four
+// threads of a row read 32 consecutive bytes per load.  Two stages, each with a
+// group of eight producer warps of its own, which load their rows two chunks
+// ahead in registers (across jobs), form and split the operands, and share the
+// epilogue; one warp issues the MMAs, one copies the table's chunks
+// (cp.async.bulk).  (With one group for both stages a chunk waited for its
+// loads: N = 384 480-690 us.)  Every wait is bounded: a role that gives up sets
+// `dead`, the others see it at their next wait, and the CTA waits (bounded) for
+// its copies and MMAs in flight, frees its TMEM and returns (err set).
+//
+// Chosen for N >= TP_MIN (solver_init); below, a pass is a few microseconds of
+// latency and the small CTAs of k_tc_rows leave room for the step's concurrent
+// kernels.  Paired passes, two right-hand sides: N = 192 50 -> 41 us, N = 243 152
+// -> 91 us, N = 384 588 -> 430 us (the scaling pass 53, 118 and 531 us).
+constexpr int TP_GROUP = 256, TP_PROD = 2 * TP_GROUP, TP_THREADS = TP_PROD + 64, TP_MIN = 160;
+static size_t tc_pass_smem(int nt) { return 1024 + 2 * (size_t)(3 * 16384 + 3 * nt * 128) + 128; }
+
+struct TcPass {
+  int64_t R;            // rows, N^2
+  int N, P, nt, ntile;  // nodes, pairs, pair columns per tile, tiles
+  int rtiles, jobs;     // row tiles; rtiles x ntile x vectors
+  const float* in;
+  const uint4* Bp;      // the table's pieces [tile][chunk][piece][nt][64]
+  const float* lam;     // SCALE: eigenvalues in the stored order
+  int null_mode;
+  float* out;
+  int* err;
+  int64_t vs;
+};
+
+template <bool SYNTH, bool SCALE>
+__global__ void __launch_bounds__(TP_THREADS, 1) k_tc_pass(TcPass a) {
+  PDL_PROLOGUE
+  using namespace tc;
+  extern __shared__ __align__(16) unsigned char fsm[];
+  __shared__ uint64_t bars[7];   // afull[2], bfull[2], empty[2], done
+  __shared__ uint64_t tfree_bar;
+  __shared__ uint32_t tslot;
+  __shared__ int dead;
+  unsigned char* tiles = fsm + ((1024u - (smem_u32(fsm) & 1023u)) & 1023u);
+  const uint32_t bpiece = (uint32_t)a.nt * 128, stage = 3 * 16384 + 3 * bpiece, tl = smem_u32(tiles);
+  const uint32_t afull = smem_u32(&bars[0]), bfull = smem_u32(&bars[2]), empty = smem_u32(&bars[4]),
+                 done = smem_u32(&bars[6]), tfree = smem_u32(&tfree_bar);
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int kc = (a.P + 31) / 32, N = a.N, P = a.P, No = N - P;
+  uint32_t ncols = 32;
+  while (ncols < 4u * (uint32_t)a.nt) ncols <<= 1;
+  if (warp == 0) tmem_alloc(smem_u32(&tslot), ncols);
+  if (tid == 0) {
+    for (int k = 0; k < 7; ++k) mbar_init_n(afull + 8 * k, 1);
+    mbar_init_n(tfree, 1);
+    dead = 0;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tslot;
+  const volatile int* vdead = &dead;
+  auto wait = [&](uint32_t bar, uint32_t phase) -> bool {
+    if (*vdead) return false;
+    if (mbar_wait(bar, phase)) return true;
+    atomicExch(&dead, 1);
+    return false;
+  };
+  int it = 0;   // chunks so far (MMA and table warps); chunk it is in stage it mod 2
+  if (warp < TP_PROD / 32) {
+    // -------- producers and epilogue
+    // group st forms the chunks of stage st; two units per thread: a row and eight pairs (or modes of
+    // each parity) 8 t + 2 q + b of the chunk, t = 0 .. 3, b = 0, 1
+    const uint32_t st = warp >= TP_GROUP / 32;
+    const int gt = tid & (TP_GROUP - 1);
+    const int align = (N & 1) == 0 && (!SYNTH || (P & 1) == 0) ? 2 : 1;
+    float x1[2][8], x2[2][8];
+    auto load = [&](int job, int c) {
+      const int rt = (job / a.ntile) % a.rtiles, v = job / (a.ntile * a.rtiles);
+      const float* in = a.in + v * a.vs;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int u = gt + TP_GROUP * j, i0 = 32 * c + 2 * (u & 3);
+        const int64_t r = (int64_t)rt * 128 + (u >> 2);
+        const bool on = r < a.R;
+        const float* row = in + r * N;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const int i = i0 + 8 * t;
+          float2 s = make_float2(0.f, 0.f), d = s;
+          if (on && align == 2 && i + 2 <= No && (SYNTH || i >= 2)) {
+            // the mirrored nodes 1 - i (mod N) are N + 1 - i, descending, for i >= 2
+            s = *reinterpret_cast<const float2*>(row + (SYNTH ? i : 2 + i));
+            d = *reinterpret_cast<const float2*>(row + (SYNTH ? P + i : N - i));
+            if (!SYNTH) d = make_float2(d.y, d.x);
+          } else if (on) {
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+              const int k = i + b;
+              float u1 = 0.f, u2 = 0.f;
+              if (k < P) {
+                // (the middle node of an odd N: the sum is the node, the difference zero)
+                u1 = row[SYNTH ? k : (2 + k < N ? 2 + k : 2 + k - N)];
+                if (k < No) u2 = row[SYNTH ? P + k : (k < 2 ? 1 - k : N + 1 - k)];
+              }
+              (b ? s.y : s.x) = u1;
+              (b ? d.y : d.x) = u2;
+            }
+          }
+          x1[j][2 * t] = s.x; x1[j][2 * t + 1] = s.y;
+          x2[j][2 * t] = d.x; x2[j][2 * t + 1] = d.y;
+        }
+      }
+    };
+    // barrier of n producers (id): true in all of them if v was true in all of them
+    auto all_ok = [](int id, int n, bool v) -> bool {
+      uint32_t r;
+      asm volatile(
+          "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbar.red.and.pred q, %2, %3, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+          : "=r"(r)
+          : "r"((uint32_t)v), "r"(id), "r"(n)
+          : "memory");
+      return r != 0;
+    };
+    bool ok = true;
+    const uint32_t base = tl + st * stage;
+    if ((int)blockIdx.x < a.jobs) load(blockIdx.x, st);   // chunk st of the first job (kc >= 3)
+    int njob = 0, uses = 0;                               // uses: chunks this group has formed
+    for (int job = blockIdx.x; job < a.jobs; job += gridDim.x, ++njob) {
+      for (int c = (st + njob * kc) & 1; c < kc; c += 2, ++uses) {
+        if (uses > 0) ok = wait(empty + 8 * st, (uses - 1) & 1);
+        if (ok) {
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const int u = gt + TP_GROUP * j, row = u >> 2, g = u & 3;
+            uint32_t p0[4], p1[4], p2[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+              const float sa = x1[j][2 * t], sb = x1[j][2 * t + 1], da = x2[j][2 * t], db = x2[j][2 * t + 1];
+              bf16_split2(SYNTH ? sa : sa + da, SYNTH ? sb : sb + db, p0[t], p1[t], p2[t]);
+            }
+            const uint32_t eo = base + sw128_off(row, 8 * g);
+            sts128(eo, p0);
+            sts128(eo + 16384, p1);
+            sts128(eo + 32768, p2);
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+              const float sa = x1[j][2 * t], sb = x1[j][2 * t + 1], da = x2[j][2 * t], db = x2[j][2 * t + 1];
+              bf16_split2(SYNTH ? da : sa - da, SYNTH ? db : sb - db, p0[t], p1[t], p2[t]);
+            }
+            const uint32_t oo = base + sw128_off(row, 32 + 8 * g);
+            sts128(oo, p0);
+            sts128(oo + 16384, p1);
+            sts128(oo + 32768, p2);
+          }
+          fence_async_smem();
+        }
+        ok = all_ok(1 + st, TP_GROUP, ok);   // (uniform: a producer that gave up takes its group along)
+        if (!ok) break;
+        if (gt == 0) mbar_arrive(afull + 8 * st);
+        // this group's next chunk, or its first of the next job
+        if (c + 2 < kc) load(job, c + 2);
+        else if (job + (int)gridDim.x < a.jobs) load(job + gridDim.x, (st + (njob + 1) * kc) & 1);
+      }
+      // both groups come here for every job, also when one has given up
+      ok = all_ok(3, TP_PROD, ok && wait(done, njob & 1));
+      if (!ok) break;
+      tc_fence_after();
+      const int tile = job % a.ntile, rt = (job / a.ntile) % a.rtiles, v = job / (a.ntile * a.rtiles);
+      const int q4 = warp & 3;
+      const int64_t r = (int64_t)rt * 128 + 32 * q4 + (tid & 31);
+      float* out = a.out + v * a.vs + r;
+      float djk = 0.f;
+      bool jk_null = false;
+      if (SCALE && r < a.R) {
+        const unsigned k = (unsigned)r / (unsigned)N, j = (unsigned)r - k * (unsigned)N;   // r < N^2 < 2^21
+        djk = a.lam[j] + a.lam[k];
+        jk_null = (int)j == a.null_mode && (int)k == a.null_mode;
+      }
+      for (int grp = warp >> 2; 8 * grp < a.nt; grp += TP_PROD / 128) {
+        uint32_t eh[8], el[8], oh[8], ol[8];
+        const uint32_t ta = tmem + ((uint32_t)(32 * q4) << 16) + 8 * grp;
+        tmem_ld8(ta, eh);
+        tmem_ld8(ta + a.nt, el);
+        tmem_ld8(ta + 2 * a.nt, oh);
+        tmem_ld8(ta + 3 * a.nt, ol);
+        tmem_wait_ld();
+        if (r >= a.R) continue;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          const int i = tile * a.nt + 8 * grp + t;
+          if (i >= P) continue;
+          float e = __uint_as_float(eh[t]) + __uint_as_float(el[t]), o = __uint_as_float(oh[t]) + __uint_as_float(ol[t]);
+          if (SYNTH) {
+            const int n1 = 2 + i < N ? 2 + i : 2 + i - N, n2 = i < 2 ? 1 - i : N + 1 - i;
+            out[n1 * a.R] = e + o;
+            if (i < No) out[n2 * a.R] = e - o;
+          } else {
+            if (SCALE) {
+              e = jk_null && i == a.null_mode ? 0.f : e * rcp_approx(a.lam[i] + djk);
+              if (i < No) o = jk_null && P + i == a.null_mode ? 0.f : o * rcp_approx(a.lam[P + i] + djk);
+            }
+            out[i * a.R] = e;
+            if (i < No) out[(P + i) * a.R] = o;
+          }
+        }
+      }
+      tc_fence_before();
+      asm volatile("bar.sync 3, %0;" ::"r"(TP_PROD) : "memory");
+      if (tid == 0) mbar_arrive(tfree);
+    }
+  } else if (warp == TP_PROD / 32) {
+    // -------- MMA issue
+    if ((tid & 31) == 0) {
+      const uint32_t idesc = umma_idesc((uint32_t)a.nt);
+      bool ok = true;
+      int njob = 0;
+      for (int job = blockIdx.x; ok && job < a.jobs; job += gridDim.x, ++njob) {
+        if (njob > 0) ok = wait(tfree, (njob - 1) & 1);   // the accumulators were read
+        for (int c = 0; ok && c < kc; ++c, ++it) {
+          const uint32_t st = it & 1, ph = (it >> 1) & 1, ta = tl + st * stage, tb = ta + 3 * 16384;
+          ok = wait(afull + 8 * st, ph) && wait(bfull + 8 * st, ph);
+          if (!ok) break;
+          tc_fence_after();
+          for (int kk = 0; kk < 4; ++kk) {   // 0, 1: even entries; 2, 3: odd
+            const uint32_t x = ta + 32 * kk, b = tb + 32 * kk, hi = tmem + (kk >> 1) * 2 * a.nt, lo = hi + a.nt;
+            const uint32_t acc = (c > 0 || (kk & 1)) ? 1u : 0u;
+            umma_bf16(hi, umma_desc(x), umma_desc(b), idesc, acc);                           // a0 b0
+            umma_bf16(lo, umma_desc(x), umma_desc(b + bpiece), idesc, acc);                  // a0 b1
+            umma_bf16(lo, umma_desc(x + 16384), umma_desc(b), idesc, 1u);                    // a1 b0
+            umma_bf16(lo, umma_desc(x), umma_desc(b + 2 * bpiece), idesc, 1u);               // a0 b2
+            umma_bf16(lo, umma_desc(x + 16384), umma_desc(b + bpiece), idesc, 1u);           // a1 b1
+            umma_bf16(lo, umma_desc(x + 32768), umma_desc(b), idesc, 1u);                    // a2 b0
+          }
+          umma_commit(empty + 8 * st);
+          if (c == kc - 1) umma_commit(done);
+        }
+      }
+      // MMAs in flight when a role gave up: their commits arrive on both stages
+      if (!ok) {
+        for (int k = 0; k < 2; ++k) {
+          (void)mbar_wait(empty + 8 * k, 0u);
+          (void)mbar_wait(empty + 8 * k, 1u);
+        }
+      }
+    }
+  } else {
+    // -------- the table's chunks
+    if ((tid & 31) == 0) {
+      bool ok = true;
+      for (int job = blockIdx.x; ok && job < a.jobs; job += gridDim.x) {
+        const uint4* src = a.Bp + (size_t)(job % a.ntile) * kc * 3 * (bpiece / 16);
+        for (int c = 0; c < kc; ++c, ++it) {
+          const uint32_t st = it & 1;
+          if (it >= 2) ok = wait(empty + 8 * st, ((it >> 1) - 1) & 1);
+          if (!ok) break;
+          mbar_expect(bfull + 8 * st, 3 * bpiece);
+          bulk_copy(tl + st * stage + 3 * 16384, src + (size_t)c * 3 * (bpiece / 16), 3 * bpiece, bfull + 8 * st);
+        }
+      }
+      // copies still in flight (they write this CTA's shared memory): the last one of each stage
+      for (int k = it - 2; k < it; ++k)
+        if (k >= 0) (void)mbar_wait(bfull + 8 * (k & 1), (k >> 1) & 1);
+    }
+  }
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  if (tid == 0 && dead) atomicExch(a.err, 1);
+  if (warp == 0) tmem_dealloc(tmem, ncols);
+}
+
 static size_t tc_rows_smem(int nt) { return 1024 + 3 * 16384 + (size_t)3 * nt * 128 + 16; }
 
 
@@ -2250,7 +2537,7 @@ static cudaError_t mg_setup(Solver* c) {
     const int Nf = 3 * c->n;
     std::vector<double> lamf, Vf;
     periodic_eigen(c->n, c->st, lamf, Vf);
-    if ((e = fdm_setup(H.fdm, Nf, lamf, Vf, c->nv, !(c->cfg.flags & FEP3M_CUDA_CORES))) != cudaSuccess) return e;
+    if ((e = fdm_setup(H.fdm, Nf, lamf, Vf, c->nv, !(c->cfg.flags & FEP3M_CUDA_CORES), true, true)) != cudaSuccess) return e;
   }
   return cudaGetLastError();
 }
@@ -2644,6 +2931,7 @@ cudaError_t mesh_solve(Solver* c, const double* b, double* phi) {
   return mesh_solve_end(c);
 }
 
+bool mesh_solve_alone(const Solver* c) { return c->mg.fdm.PpF != nullptr; }
 bool mesh_solve_paired(const Solver* c) { return c->nv == 2 && c->mg.fdm.BpF != nullptr; }
 
 cudaError_t mesh_solve_begin2(Solver* c, const double* b, double* phi) {
@@ -2714,9 +3002,124 @@ static void solver_plan_free(Solver* c) {
 // FP32 eigenbasis for the CUDA-core passes and, with tensor_cores, its bf16
 // pieces in the layout of the tensor-core row GEMM (column tiles of nt modes,
 // chunks of 64 nodes).  Used by the order-3 fine level and the order-p mesh.
+// The eigenbasis of a periodic order-3 mesh with every mode even or odd under
+// node k -> 3 - k (mod N): degenerate pairs (one cosine, one sine) are rotated;
+// modes of the others have a parity already.  order: the modes, even ones first.
+// False if the basis does not come out that way (the plain passes serve then).
+static bool parity_basis(int N, const std::vector<double>& lam, std::vector<double>& V, std::vector<int>& order) {
+  auto mirror = [&](int k) { return ((3 - k) % N + N) % N; };
+  std::vector<int> ord(N), even, odd;
+  for (int i = 0; i < N; ++i) ord[i] = i;
+  std::sort(ord.begin(), ord.end(), [&](int a, int b) { return lam[a] < lam[b]; });
+  const double top = lam[ord[N - 1]];
+  auto dot = [&](int a, int b, bool mir) {
+    double s = 0.0;
+    for (int k = 0; k < N; ++k) s += V[(size_t)k * N + a] * V[(size_t)(mir ? mirror(k) : k) * N + b];
+    return s;
+  };
+  auto put = [&](int m) -> bool {   // mode m: its parity, made exact
+    const double p = dot(m, m, true) / dot(m, m, false);
+    if (std::fabs(std::fabs(p) - 1.0) > 1e-6) return false;
+    const double s = p > 0 ? 1.0 : -1.0;
+    for (int k = 0; k < N; ++k) {
+      const int j = mirror(k);
+      if (j < k) continue;
+      const double v = 0.5 * (V[(size_t)k * N + m] + s * V[(size_t)j * N + m]);
+      V[(size_t)k * N + m] = v;
+      V[(size_t)j * N + m] = s * v;
+    }
+    (p > 0 ? even : odd).push_back(m);
+    return true;
+  };
+  for (int i = 0; i < N;) {
+    int c = 1;
+    while (i + c < N && lam[ord[i + c]] - lam[ord[i]] < 1e-9 * top) ++c;
+    if (c > 2) return false;
+    if (c == 2) {
+      // the reflection in the pair's span, (G^-1 A)_ij with A = V^T mirror V and G = V^T V: its
+      // eigenvectors for +1 and -1 are orthonormal combinations (the modes are M-orthonormal)
+      const int a = ord[i], b = ord[i + 1];
+      const double gaa = dot(a, a, false), gab = dot(a, b, false), gbb = dot(b, b, false);
+      const double aaa = dot(a, a, true), aab = dot(a, b, true), abb = dot(b, b, true), det = gaa * gbb - gab * gab;
+      const double q00 = (gbb * aaa - gab * aab) / det, q01 = (gbb * aab - gab * abb) / det;
+      if (std::fabs(q01) > 1e-12) {
+        // eigenvector for +1: (q01, 1 - q00), normalised; for -1: its perpendicular
+        const double n = std::hypot(q01, 1.0 - q00), cs = q01 / n, sn = (1.0 - q00) / n;
+        for (int k = 0; k < N; ++k) {
+          const double u = V[(size_t)k * N + a], w = V[(size_t)k * N + b];
+          V[(size_t)k * N + a] = cs * u + sn * w;
+          V[(size_t)k * N + b] = -sn * u + cs * w;
+        }
+      }
+    }
+    for (int t = 0; t < c; ++t)
+      if (!put(ord[i + t])) return false;
+    i += c;
+  }
+  if ((int)even.size() != (N + 1) / 2) return false;
+  order = even;
+  order.insert(order.end(), odd.begin(), odd.end());
+  return true;
+}
+
+// the parity passes' data: the eigenvalues in the stored order and the pieces of
+// both tables per tile of nt pair columns and chunk of 32 entries of each parity
+static cudaError_t fdm_setup_parity(FineFDM& f, int N, const std::vector<double>& lam, std::vector<double> V) {
+  std::vector<int> order;
+  if (!parity_basis(N, lam, V, order)) return cudaSuccess;
+  const int P = (N + 1) / 2, No = N - P;
+  // the fewest tiles of at most 128 columns (a row's operands are formed once per tile)
+  const int ntile = (P + 127) / 128, nt = ((P + ntile - 1) / ntile + 15) / 16 * 16, kc = (P + 31) / 32;
+  const size_t per = (size_t)3 * nt * 64;
+  std::vector<uint16_t> bf((size_t)ntile * kc * per, 0), bi((size_t)ntile * kc * per, 0);
+  for (int t = 0; t < ntile; ++t)
+    for (int ch = 0; ch < kc; ++ch)
+      for (int ii = 0; ii < nt; ++ii)
+        for (int k = 0; k < 64; ++k) {
+          const bool odd = k >= 32;
+          // column, and the contraction index at place k (k_tc_pass)
+          const int i = t * nt + ii, b = 32 * ch + 8 * ((k & 7) >> 1) + 2 * ((k & 31) >> 3) + (k & 1);
+          uint16_t pf[3] = {0, 0, 0}, pi[3] = {0, 0, 0};
+          auto val = [&](int pair, int j) { return V[(size_t)((2 + pair) % N) * N + order[odd ? P + j : j]]; };
+          const int lim = odd ? No : P;
+          if (i < lim && b < P && (!odd || b < No)) tc::bf16_pieces(val(b, i), pf);   // analysis: column = mode
+          if (i < P && b < lim && (!odd || i < No)) tc::bf16_pieces(val(i, b), pi);   // synthesis: column = pair
+          for (int p = 0; p < 3; ++p) {
+            const size_t o = ((size_t)(t * kc + ch) * 3 + p) * nt * 64 + tc::sw128_off(ii, k) / 2;
+            bf[o] = pf[p];
+            bi[o] = pi[p];
+          }
+        }
+  std::vector<float> l32(N);
+  f.pnull = -1;
+  for (int i = 0; i < N; ++i) {
+    l32[i] = (float)lam[order[i]];
+    if (order[i] == f.null_mode) f.pnull = i;
+  }
+  cudaError_t e;
+  if ((e = cudaMalloc(&f.PpF, bf.size() * 2)) != cudaSuccess || (e = cudaMalloc(&f.PpI, bi.size() * 2)) != cudaSuccess ||
+      (e = cudaMalloc(&f.plam, N * sizeof(float))) != cudaSuccess)
+    return e;
+  cudaMemcpy(f.PpF, bf.data(), bf.size() * 2, cudaMemcpyHostToDevice);
+  cudaMemcpy(f.PpI, bi.data(), bi.size() * 2, cudaMemcpyHostToDevice);
+  cudaMemcpy(f.plam, l32.data(), N * sizeof(float), cudaMemcpyHostToDevice);
+  f.pnt = nt;
+  f.pntile = ntile;
+  int dev = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+      (e = cudaDeviceGetAttribute(&f.psms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+    return e;
+  const size_t sm = tc_pass_smem(nt);
+  if ((e = smem_limit((const void*)k_tc_pass<false, false>, sm)) != cudaSuccess ||
+      (e = smem_limit((const void*)k_tc_pass<false, true>, sm)) != cudaSuccess ||
+      (e = smem_limit((const void*)k_tc_pass<true, false>, sm)) != cudaSuccess)
+    return e;
+  return cudaSuccess;
+}
+
 cudaError_t fdm_setup(FineFDM& f, int Nf, const std::vector<double>& lamf, const std::vector<double>& Vf,
                       int rhs,
-                      bool tensor_cores, bool null_mode) {
+                      bool tensor_cores, bool null_mode, bool periodic3) {
   cudaError_t e;
   {
     // the constant mode of a periodic (or fully Neumann) mesh: the eigenvalue
@@ -2775,13 +3178,14 @@ cudaError_t fdm_setup(FineFDM& f, int Nf, const std::vector<double>& lamf, const
       if ((e = tc_rows_prepare(nt)) != cudaSuccess) return e;
       if ((e = cudaMalloc(&f.err, sizeof(int))) != cudaSuccess) return e;
       cudaMemset(f.err, 0, sizeof(int));
+      if (periodic3 && Nf >= TP_MIN && (e = fdm_setup_parity(f, Nf, lamf, Vf)) != cudaSuccess) return e;
     }
   }
   return cudaGetLastError();
 }
 
 void fdm_free(FineFDM& f) {
-  void* p[] = {f.BpF, f.BpI, f.err, f.V32, f.VT32, f.lam32};
+  void* p[] = {f.BpF, f.BpI, f.err, f.V32, f.VT32, f.lam32, f.PpF, f.PpI, f.plam};
   for (void* q : p)
     if (q) cudaFree(q);
   f = FineFDM();
@@ -2792,6 +3196,35 @@ void fdm_free(FineFDM& f) {
 cudaError_t fdm_apply(const FineFDM& f, const float* b, float* x, float* w1, float* w2, cudaStream_t s, int V,
                       int64_t vs) {
   const int N = f.N;
+  if (f.PpF) {
+    TcPass a;
+    a.R = (int64_t)N * N;
+    a.N = N;
+    a.P = (N + 1) / 2;
+    a.nt = f.pnt;
+    a.ntile = f.pntile;
+    a.rtiles = (int)((a.R + 127) / 128);
+    a.jobs = a.rtiles * a.ntile * V;
+    a.lam = f.plam;
+    a.null_mode = f.pnull;
+    a.err = f.err;
+    a.vs = vs;
+    const dim3 g((unsigned)std::min(a.jobs, f.psms));
+    const size_t sm = tc_pass_smem(f.pnt);
+    auto pass = [&](void (*k)(TcPass), const float* in, float* out, const void* Bp) {
+      a.in = in;
+      a.out = out;
+      a.Bp = (const uint4*)Bp;
+      launch_pdl(k, g, TP_THREADS, sm, s, a);
+    };
+    pass(k_tc_pass<false, false>, b, w1, f.PpF);
+    pass(k_tc_pass<false, false>, w1, w2, f.PpF);
+    pass(k_tc_pass<false, true>, w2, w1, f.PpF);
+    pass(k_tc_pass<true, false>, w1, w2, f.PpI);
+    pass(k_tc_pass<true, false>, w2, w1, f.PpI);
+    pass(k_tc_pass<true, false>, w1, x, f.PpI);
+    return cudaGetLastError();
+  }
   if (f.BpF) {
     const dim3 g((unsigned)(((int64_t)N * N + 127) / 128 * f.ntile), (unsigned)V);
     const size_t sm = tc_rows_smem(f.nt);

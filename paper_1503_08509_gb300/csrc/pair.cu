@@ -1670,7 +1670,7 @@ __global__ void __launch_bounds__(PT) k_elem_deposit(int64_t ne, const int* __re
 // summed by two-sums.  Grid (y, z): a CTA takes a row of nodes, so that the
 // elements along y and z are the CTA's and a node's own index costs one
 // division (one thread per node of the whole mesh spent 227 instructions on
-// the indices: 262 144 charges on 64^3, 100 -> @NA64@ us)
+// the indices: 262 144 charges on 64^3, 100 -> 45 us)
 template <class T>
 __global__ void __launch_bounds__(PT) k_node_assemble(int n, const T* __restrict__ W, double* __restrict__ g) {
   const int N = 3 * n, iy = blockIdx.x, iz = blockIdx.y;
@@ -1921,14 +1921,14 @@ __global__ void __launch_bounds__(PT, 2) k_adj64(int64_t ne, int n_sr, int z0, i
 // vertices (consecutive lanes read consecutive elements of D) and deals the
 // offset planes oz of the chunk [z0, z1) to its eight warps.  A thread sums a
 // plane's terms into nine classes (first, inner, last offset along x and along
-// y), two rows of D's values ahead in registers, adds them into the corners of
+// y), a row of D's values and weight sums ahead in registers, adds them into the corners of
 // the plane's class along z in shared memory, and the warps' corner sums are
 // combined there in order: deterministic.  FP32 path (H0 set): D holds the contraction with the
 // node-0-relative table, and each term gains H(o, 0) Wsum(v + o)
 // (pair_adjoint_table).  FP64 path: D is the whole contraction, as pairs.  Terms
 // and sums in double-float arithmetic.  Bound by FP32 issue in the FP32 path (19
 // operations a term beside its loads) and by the read of D.  10^6 charges on
-// 128^3: 3484 -> @AV128@ us, 262 144 on 64^3: 439 -> @AV64@ us against one warp per 32
+// 128^3: 3484 -> 2301 us, 262 144 on 64^3: 439 -> 285 us against one warp per 32
 // vertices and row of offsets with 27 class sums in shared memory, whose
 // bookkeeping took most of its instructions.
 constexpr int AVV = 32, AVZ = PT / AVV;   // vertices and threads per vertex of a CTA
