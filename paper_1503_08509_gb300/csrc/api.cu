@@ -234,6 +234,7 @@ int run_forward(fep3m_ctx* c, double* phi_dev, int want_grad, double* force_dev,
     ~Restore() { c->stream = s; }
   } restore{c, c->stream};
   const cudaStream_t caller = c->stream;
+  c->have_mesh = false;
   CK(cudaEventRecord(c->ev_ffork, caller));
   CK(cudaStreamWaitEvent(c->fwd_stream, c->ev_ffork, 0));
   c->stream = c->fwd_stream;
@@ -676,7 +677,7 @@ int fep3m_set_particles(fep3m_ctx* c, int64_t N, const double* pos, const double
   const double* sums = c->host_scal;
   const int flag = ((const int*)(c->host_scal + kFlags - 32))[0];
   c->have_particles = false;
-  c->have_forward = false;
+  c->have_forward = c->have_mesh = false;
   if (flag) return FEP3M_EINVAL;
   if (!c->box && !(c->cfg.flags & FEP3M_NEUTRALIZE) && std::fabs(sums[0]) > 1e-12 * sums[1])
     return FEP3M_ENOTNEUTRAL;
@@ -708,6 +709,7 @@ int fep3m_compute(fep3m_ctx* c, double* phi, double* U, double* force) {
     if (!solves_missed(c, force != nullptr) || attempt == kMaxReruns) break;
   }
   const int st = solve_status(c, force != nullptr);
+  c->have_mesh = force || st == FEP3M_OK;
   if (phi && !phi_dev) {
     int s2 = deliver(c, phi, c->out_tmp, N * sizeof(double));
     if (s2 != FEP3M_OK) return s2;
@@ -734,11 +736,44 @@ int fep3m_compute(fep3m_ctx* c, double* phi, double* U, double* force) {
   return st;
 }
 
+// The adjoint's kernels: forked from c->stream and joined back to it.  The mesh
+// solution's replay is checked by the caller (mesh_solve_check), after the
+// stream has completed.  fields: the charges' gradients are missing (the
+// forward was without forces) and are evaluated beside the adjoint, from the
+// forward's mesh solution and class sums, which the context keeps until the
+// next set_particles.
+int run_adjoint(fep3m_ctx* c, double gU, const double* g, bool fields, double* dp, double* dq) {
+  fep3m::Solver* A = &c->solv[1];
+  CK(cudaMemsetAsync(c->iflags + 2, 0, sizeof(int), c->stream));
+  CK(cudaEventRecord(c->ev_fork, c->stream));
+  CK(cudaStreamWaitEvent(c->aux_stream, c->ev_fork, 0));
+  CK(adjoint_pre(c, gU, g, c->aux_stream));
+  CK(cudaEventRecord(c->ev_fork2, c->aux_stream));
+  CK(mesh_solve_begin(A, c->g64, c->lam64));
+  const bool alone = fep3m::mesh_solve_alone(A);   // as in run_forward
+  if (alone) CK(cudaEventRecord(c->ev_solved, c->aux_stream));
+  CK(cudaStreamWaitEvent(c->sweep_stream, alone ? c->ev_solved : c->ev_fork2, 0));
+  CK(adjoint_sweeps(c, c->sweep_stream, true));
+  CK(cudaEventRecord(c->ev_join2, c->sweep_stream));
+  if (fields) {
+    CK(cudaStreamWaitEvent(c->pair_stream, alone ? c->ev_solved : c->ev_fork, 0));
+    CK(pair_fields(c, c->pair_stream));
+    CK(cudaEventRecord(c->ev_pjoin, c->pair_stream));
+    CK(cudaStreamWaitEvent(c->stream, c->ev_pjoin, 0));
+  }
+  CK(adjoint_vertex(c, c->aux_stream));
+  CK(cudaEventRecord(c->ev_join, c->aux_stream));
+  CK(cudaStreamWaitEvent(c->stream, c->ev_join, 0));
+  CK(cudaStreamWaitEvent(c->stream, c->ev_join2, 0));
+  CK(adjoint_final(c, gU, dp, dq, 1.0, c->stream));
+  return FEP3M_OK;
+}
+
 int fep3m_vjp(fep3m_ctx* c, double gU, const double* gphi, double* dpos, double* dQ) {
   if (!c || !std::isfinite(gU) || c->oq || c->box) return FEP3M_EINVAL;
   if (!c->have_particles) return FEP3M_ESTATE;
   const int64_t N = c->N;
-  if (!c->have_forward || !c->have_grad) {
+  if (!c->have_mesh) {   // no forward for these charges, or one that did not succeed
     for (int attempt = 0;; ++attempt) {
       int st = run_forward(c, nullptr, 1, nullptr);
       if (st != FEP3M_OK) return st;
@@ -747,6 +782,7 @@ int fep3m_vjp(fep3m_ctx* c, double gU, const double* gphi, double* dpos, double*
       if (!solves_missed(c, false) || attempt == kMaxReruns) break;
     }
     solve_status(c, false);
+    c->have_mesh = true;
   }
   const double* g = gphi;
   if (gphi && !is_device_ptr(gphi)) {
@@ -756,23 +792,17 @@ int fep3m_vjp(fep3m_ctx* c, double gU, const double* gphi, double* dpos, double*
   const bool pdev = is_device_ptr(dpos), qdev = is_device_ptr(dQ);
   double* dp = dpos ? (pdev ? dpos : c->out_tmp + N) : nullptr;
   double* dq = dQ ? (qdev ? dQ : c->out_tmp + 4 * N) : nullptr;
-  CK(cudaEventRecord(c->ev_fork, c->stream));
-  CK(cudaStreamWaitEvent(c->aux_stream, c->ev_fork, 0));
-  CK(adjoint_pre(c, gU, g, c->aux_stream));
-  CK(cudaEventRecord(c->ev_fork2, c->aux_stream));
-  CK(cudaStreamWaitEvent(c->sweep_stream, c->ev_fork2, 0));
-  const bool alone = fep3m::mesh_solve_alone(&c->solv[1]);   // (run_forward)
-  if (alone) CK(mesh_solve(&c->solv[1], c->g64, c->lam64));   // has finished when it returns
-  CK(adjoint_sweeps(c, c->sweep_stream, true));
-  CK(cudaEventRecord(c->ev_join2, c->sweep_stream));
-  if (!alone) CK(mesh_solve(&c->solv[1], c->g64, c->lam64));
+  const bool fields = !c->have_grad;
+  for (int attempt = 0;; ++attempt) {   // again if the replayed solve missed its tolerance (it re-calibrates then)
+    const int st = run_adjoint(c, gU, g, fields, dp, dq);
+    if (st != FEP3M_OK) return st;
+    CK(take_results(c, nullptr));
+    if (c->host_err) return FEP3M_ETIMEOUT;
+    if (mesh_solve_check(&c->solv[1]) || attempt == kMaxReruns) break;
+  }
+  c->have_grad = true;
   c->stats.adj_iterations = c->solv[1].iters;
   c->stats.adj_rel_residual = c->solv[1].relres;
-  CK(adjoint_vertex(c, c->aux_stream));
-  CK(cudaEventRecord(c->ev_join, c->aux_stream));
-  CK(cudaStreamWaitEvent(c->stream, c->ev_join, 0));
-  CK(cudaStreamWaitEvent(c->stream, c->ev_join2, 0));
-  CK(adjoint_final(c, gU, dp, dq, 1.0, c->stream));
   if (dpos && !pdev) {
     int s = deliver(c, dpos, c->out_tmp + N, 3 * N * sizeof(double));
     if (s != FEP3M_OK) return s;
@@ -990,7 +1020,7 @@ int fep3m_set_boundary(fep3m_ctx* c, const double* g) {
   CK(cudaStreamSynchronize(c->stream));
   if (flag) return FEP3M_EINVAL;
   const int st = box_set_boundary(c, stage);
-  c->have_forward = false;
+  c->have_forward = c->have_mesh = false;
   return st;
 }
 

@@ -312,6 +312,7 @@ struct fep3m_ctx {
   int64_t N = 0, cap = 0;
   double q_scale = 1;            // power of two near the inverse mean |Q| of the charges last set
   bool have_particles = false, have_forward = false, have_grad = false;
+  bool have_mesh = false;   // phi64 solves the mesh problem of these charges (fep3m_vjp)
   double* pos_in = nullptr;      // N*3 (staging for host inputs)
   double* Q_in = nullptr;        // N
   int* cell = nullptr;           // N
@@ -487,6 +488,7 @@ cudaError_t tc_rows_prepare(int nt);
 cudaError_t tc_rows_gemm(int64_t R, int K, int cb, int ce, int nt, const float* in, const void* Bp, float* out,
                          int* err, cudaStream_t s);
 cudaError_t pair_eval(fep3m_ctx* c, double* phi_out, int want_grad);
+cudaError_t pair_fields(fep3m_ctx* c, cudaStream_t s);
 // adjoint in three parts: weights and deposit (-> g64), the parts that need
 // lam (vertex adjoint, screen sweep, singular adjoint), and the per-charge assembly
 cudaError_t adjoint_pre(fep3m_ctx* c, double gU, const double* gphi, cudaStream_t s);

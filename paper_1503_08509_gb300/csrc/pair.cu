@@ -2433,6 +2433,20 @@ cudaError_t pair_eval(fep3m_ctx* c, double* phi_out, int want_grad) {
   return want_grad ? launch_pair_eval<true>(c, phi_out) : launch_pair_eval<false>(c, phi_out);
 }
 
+// Potentials and their gradients at the charges, on stream s, after a forward
+// without gradients: the mesh potential and the screens' class sums are there.
+// FP64 keeps the screen field too; the FP32 screen kernel writes it again, as the
+// singular sums are made there.
+cudaError_t pair_fields(fep3m_ctx* c, cudaStream_t s) {
+  cudaError_t e = c->precision == FEP3M_MIXED ? pair_screen(c, 1, s, false) : singular64(c, true, false, s);
+  if (e != cudaSuccess) return e;
+  const cudaStream_t keep = c->stream;
+  c->stream = s;   // launch_pair_eval issues on c->stream
+  e = pair_eval(c, nullptr, 1);
+  c->stream = keep;
+  return e;
+}
+
 cudaError_t energy(fep3m_ctx* c, double* U_dev, cudaStream_t s) {
   const int64_t N = c->N;
   const int nb = (int)std::min<int64_t>(std::max<int64_t>(gsz(N), 1), 1024);
