@@ -47,7 +47,7 @@ __constant__ float cDinv32[27];
 // two-product) plus the cross terms; a sum keeps its exact rounding error
 // (two-sum, Knuth) in l.  Values stay unnormalised (|l| may exceed half an
 // ulp of h); the represented number is always h + l.
-struct dfv {
+struct alignas(8) dfv {   // (one 64-bit access)
   float h, l;
 };
 __device__ __forceinline__ dfv operator*(dfv c, dfv x) {
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(256) k_coarse_pencil(int N, const T* __restric
 }
 
 // ------------------------------------------------------------ operator apply
-enum { EPI_Y = 0, EPI_RESID = 1, EPI_CHEB = 2, EPI_CHEB0 = 3 };
+enum { EPI_Y = 0, EPI_RESID = 1, EPI_CHEB = 2, EPI_CHEB0 = 3, EPI_CHECK = 4 };
 
 // scalars derived on the device by the reductions: doubles at
 // scal[SC_DERIVED + k], floats at ((float*)(scal + SC_DERIVED_F))[k]
@@ -554,6 +554,8 @@ struct ApplyDot {
 //   EPI_CHEB0  the second Chebyshev step from a zero start, whose first step
 //              is d = x = c0 D^-1 b: the input is formed from b on the fly
 //              (x must point at b), then as EPI_CHEB with that d and x
+//   EPI_CHECK  no output: |b - y|^2, and the integral of the iterate xo + x / s
+//              (the last correction x of a refinement, k_ref_out)
 constexpr int AEX = 16, AEY = 4;                  // elements per tile in x, y
 constexpr int AFX = 3 * AEX, AFY = 3 * AEY;       // output nodes per tile
 constexpr int AHX = AFX + 6, AHY = AFY + 6;       // halo column extents
@@ -563,7 +565,7 @@ constexpr int APL = (ANC + AT - 1) / AT;          // halo columns per thread
 static_assert(AHX * AEY <= AT && AEX * AFY <= AT, "one y item and one x item per thread");
 
 template <class T>
-struct Pair2 {
+struct alignas(2 * sizeof(T)) Pair2 {   // one access in shared memory
   T a, b;
 };
 
@@ -573,13 +575,14 @@ struct Pair2 {
 // (with DOT, EPI_Y stages x for the dot x.Kx)
 template <class T, int EPI, bool DOT = false>
 __host__ __device__ constexpr int apply_nst() {
-  return EPI == EPI_CHEB ? (sizeof(T) == 4 ? 3 : 2) : (EPI == EPI_Y ? (DOT ? 1 : 0) : 1);
+  return EPI == EPI_CHEB ? (sizeof(T) == 4 ? 3 : 2) : EPI == EPI_CHECK ? 2 : (EPI == EPI_Y ? (DOT ? 1 : 0) : 1);
 }
 
 template <class T, int EPI, bool DOT = false>
 struct ApplySmem {
   Pair2<T> tz[3][AHY][AHX];        // z pass: (Mz x, Kz x)
   Pair2<T> ac[3][AFY][AHX];        // y pass: (a, c)
+  dfv it[EPI == EPI_CHECK ? 3 : 1][EPI == EPI_CHECK ? AFY : 1][EPI == EPI_CHECK ? AFX : 1];   // EPI_CHECK: the iterate
   T dinv[27];                      // D^-1 by node types: x + 3 y + 9 z
   T stg[apply_nst<T, EPI, DOT>() > 0 ? apply_nst<T, EPI, DOT>() : 1][3][AFY][AFX];
 };
@@ -644,6 +647,16 @@ __device__ __forceinline__ T st_KM(const T* u, const T* w) {
   return s;
 }
 
+// the iterate p plus a correction t, rounded to a pair (two-sum, then renormalised)
+__device__ __forceinline__ dfv df_iterate(dfv p, float t) {
+  const float sum = p.h + t;
+  const float bv = sum - p.h;
+  const float err = (p.h - (sum - bv)) + (t - bv);
+  const float lo = p.l + err;
+  const float h = sum + lo;
+  return {h, lo - (h - sum)};
+}
+
 // the epilogue at node g with y = (K x)_g and the staged b_g, d_g, x_g
 // returns y (EPI_Y) or the new iterate (EPI_CHEB), the factor of the fused dots
 template <class T, int EPI>
@@ -661,6 +674,9 @@ __device__ __forceinline__ T apply_epilogue(int64_t g, T y, T bg, T dg, T xg, T*
     return y;
   } else if constexpr (EPI == EPI_Y) {
     out[g] = y;
+    return y;
+  } else if constexpr (EPI == EPI_CHECK) {
+    rsd = bg - y;
     return y;
   } else if constexpr (EPI == EPI_RESID) {
     if constexpr (std::is_same<T, float>::value) out[g] = bg - y;
@@ -709,16 +725,19 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
                T* __restrict__ d, T* __restrict__ xo, T c0, T c1, T c2, double* __restrict__ scal, ApplyDot dt,
                int64_t vs) {
   PDL_PROLOGUE
-  static_assert(!DOT || EPI == EPI_Y || EPI == EPI_CHEB || (EPI == EPI_RESID && (BOX || std::is_same<T, dfv>::value)),
+  static_assert(EPI != EPI_CHECK || (DOT && sizeof(T) == 4 && !F32IN && !BOX), "the correction's check: FP32");
+  static_assert(!DOT || EPI == EPI_Y || EPI == EPI_CHEB || EPI == EPI_CHECK || (EPI == EPI_RESID && (BOX || std::is_same<T, dfv>::value)),
                 "fused dots: EPI_Y, EPI_CHEB, the double-float residual and a box's");
   static_assert(!BOX || (EPI == EPI_RESID && DOT && !F32IN && !std::is_same<T, float>::value), "box: residuals only");
   static_assert(!F32IN || (EPI == EPI_RESID && std::is_same<T, dfv>::value), "FP32 input: the double-float residual");
   extern __shared__ __align__(16) unsigned char apply_smem_raw[];
   ApplySmem<T, EPI, DOT>& S = *reinterpret_cast<ApplySmem<T, EPI, DOT>*>(apply_smem_raw);
   constexpr int NST = apply_nst<T, EPI, DOT>();
+  constexpr bool NORM = EPI == EPI_RESID || EPI == EPI_CHECK;   // with DOT: |r|^2, and the integral for dt.wout
   double dacc = 0.0;
-  float facc = 0.f;          // EPI_RESID dot: |r|^2 in FP32
-  dfv wacc = {0.f, 0.f};     // EPI_RESID dot with dt.wout: the iterate's integral
+  float facc = 0.f;          // NORM: |r|^2 in FP32
+  dfv wacc = {0.f, 0.f};     // NORM with dt.wout: the iterate's integral
+  const dfv* itx = reinterpret_cast<const dfv*>(xo);   // EPI_CHECK: the iterate
   const int n = BOX ? (N + 2) / 3 : N / 3;
   const int64_t NN = (int64_t)N * N;
   const int x0 = blockIdx.x * AFX, y0 = blockIdx.y * AFY;
@@ -731,19 +750,20 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
     else x += o;
     if constexpr (EPI == EPI_RESID && !std::is_same<T, float>::value)
       out = reinterpret_cast<T*>(reinterpret_cast<float*>(out) + o);   // the FP32 residual
-    else
+    else if constexpr (EPI != EPI_CHECK)
       out += o;
     if (b) b += o;
     if (d) d += o;
     if (xo) xo += o;
+    itx += o;
     scal += 64 * vi;
   }
   const int tid = threadIdx.x;
   float rs = 0.0f;   // power-of-two scale of the refinement residual (FP64, double-float)
   if constexpr (BOX) rs = dt.bscale ? *dt.bscale : 1.f;
   else if constexpr (!std::is_same<T, float>::value) rs = reinterpret_cast<const float*>(scal + SC_DERIVED_F)[SD_SCALE];
-  float ris = 0.0f;  // F32IN: 1 / s
-  if constexpr (F32IN) ris = reinterpret_cast<const float*>(scal + SC_DERIVED_F)[SD_INVSCALE];
+  float ris = 0.0f;  // F32IN, EPI_CHECK: 1 / s
+  if constexpr (F32IN || EPI == EPI_CHECK) ris = reinterpret_cast<const float*>(scal + SC_DERIVED_F)[SD_INVSCALE];
   const float* xf = reinterpret_cast<const float*>(x);   // F32IN: the correction e
   auto ldx = [&](int64_t off) -> T {
     if constexpr (F32IN) return T{xf[off] * ris, 0.f};
@@ -834,7 +854,9 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
         for (int r = 0; r < 3; ++r) {
           if (BOX && (gx0 + r >= N || 3 * e + p >= N)) continue;
           cp_async<sizeof(T)>(&S.stg[0][p][x_yy][3 * x_ex + r], (EPI == EPI_Y ? x : b) + g + r);
-          if constexpr (NST > 1) cp_async<sizeof(T)>(&S.stg[NST > 1 ? 1 : 0][p][x_yy][3 * x_ex + r], d + g + r);
+          if constexpr (NST > 1)
+            cp_async<sizeof(T)>(&S.stg[NST > 1 ? 1 : 0][p][x_yy][3 * x_ex + r], (EPI == EPI_CHECK ? x : d) + g + r);
+          if constexpr (EPI == EPI_CHECK) cp_async<sizeof(dfv)>(&S.it[p][x_yy][3 * x_ex + r], itx + g + r);
           if constexpr (NST > 2) cp_async<sizeof(T)>(&S.stg[NST > 2 ? 2 : 0][p][x_yy][3 * x_ex + r], x + g + r);
         }
       }
@@ -942,19 +964,21 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
           float rsd = 0.f;
           const T f = apply_epilogue<T, EPI>(g + r, y[r], bg, dg, xg, out, d, xo, c0, c1, c2, dv[r], rs, rsd);
           if constexpr (F32IN) xo[g + r] = T{xf[g + r] * ris, 0.f};   // the iterate after the first sweep
-          if constexpr (DOT && EPI == EPI_RESID && !BOX) {
+          if constexpr (DOT && NORM && !BOX) {
             if (dt.wout) {   // the node weight (1/4 or 3/8 per axis) times the iterate, as a two-product
               const float wn = (r ? 0.375f : 0.25f) * (ty3 ? 0.375f : 0.25f) * (p ? 0.375f : 0.25f);
-              const T xv = ldx(g + r);
+              dfv xv;
+              if constexpr (EPI == EPI_CHECK) xv = df_iterate(S.it[p][x_yy][3 * x_ex + r], dg * ris);
+              else xv = ldx(g + r);
               const float pr = wn * xv.h;
               wacc += dfv{pr, fmaf(wn, xv.l, fmaf(wn, xv.h, -pr))};
             }
           }
-          if constexpr (DOT && EPI == EPI_RESID) dres = fmaf(rsd, rsd, dres);
+          if constexpr (DOT && NORM) dres = fmaf(rsd, rsd, dres);
           else if constexpr (DOT) dsum = r == 0 ? bg * f : dsum + bg * f;   // EPI_Y stages x in the b slot
         }
-        if constexpr (DOT && EPI != EPI_RESID) dacc += (double)dsum;
-        if constexpr (DOT && EPI == EPI_RESID) facc += dres;
+        if constexpr (DOT && !NORM) dacc += (double)dsum;
+        if constexpr (DOT && NORM) facc += dres;
       }
     }
     // next element: slots 0..3 <- 3..6, slots 4..6 <- the prefetched planes
@@ -972,7 +996,7 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
   if constexpr (DOT) {
     const unsigned nbv = gridDim.x * gridDim.y * zsb;   // blocks per vector
     const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * (blockIdx.z - vi * zsb));
-    if constexpr (EPI == EPI_RESID) {
+    if constexpr (NORM) {
       if (dt.wout) {   // two totals: |r|^2 and the integral (partials two per block)
         double tr, tw;
         if (block_sum2_finish(dfv{facc, 0.f}, wacc, bid, nbv, dt.partials + (size_t)vi * 2 * nbv, dt.counter + vi,
@@ -1010,6 +1034,7 @@ static cudaError_t apply_set_smem() {
   if (e == cudaSuccess) e = apply_set_smem_one<float, EPI_CHEB0>();
   if (e == cudaSuccess) e = apply_set_smem_one<float, EPI_Y, true>();
   if (e == cudaSuccess) e = apply_set_smem_one<float, EPI_CHEB, true>();
+  if (e == cudaSuccess) e = apply_set_smem_one<float, EPI_CHECK, true>();
   if (e == cudaSuccess) e = apply_set_smem_one<double, EPI_RESID>();
   if (e == cudaSuccess) e = apply_set_smem_one<dfv, EPI_RESID>();
   if (e == cudaSuccess) e = apply_set_smem_one<dfv, EPI_RESID, true>();
@@ -1952,14 +1977,7 @@ __global__ void k_df_update(int64_t n, dfv* __restrict__ phi, const float* __res
   e += blockIdx.y * vs;
   scal += 64 * blockIdx.y;
   const float is = reinterpret_cast<const float*>(scal + SC_DERIVED_F)[SD_INVSCALE];
-  const float t = e[g] * is;
-  dfv p = phi[g];
-  const float sum = p.h + t;
-  const float bv = sum - p.h;
-  const float err = (p.h - (sum - bv)) + (t - bv);
-  const float lo = p.l + err;
-  const float h = sum + lo;
-  phi[g] = {h, lo - (h - sum)};
+  phi[g] = df_iterate(phi[g], e[g] * is);
 }
 
 // ---- double-float refinement bookkeeping (MIXED).  FP64 arithmetic runs at a
@@ -2090,21 +2108,38 @@ __global__ void k_ref_wsum(int N, const dfv* __restrict__ v, double* __restrict_
 }
 
 // finish, second pass: phi = v - m as normalised float pairs (m the mean just
-// derived)
-__global__ void k_ref_out(int64_t n, const dfv* __restrict__ v, dfv* __restrict__ phi, const double* __restrict__ scal,
-                          int64_t vs) {
+// derived); with e, v + e / s in place of v, where the last correction was
+// checked without adding it to the iterate (EPI_CHECK).  Bound by memory: four
+// nodes per thread, their loads first (two right-hand sides on 128^3, 16 bytes a
+// node: one node per thread 459 us; now with e, 20 bytes, 310 us, and the
+// update's own pass, 393 us, is gone)
+constexpr int RO_PER = 4;
+__global__ void __launch_bounds__(TPB) k_ref_out(int64_t n, const dfv* __restrict__ v, dfv* __restrict__ phi,
+                                                 const float* __restrict__ e, const double* __restrict__ scal,
+                                                 int64_t vs) {
   PDL_PROLOGUE
   const int vi = blockIdx.y;
   v += vi * vs;
   phi += vi * vs;
   scal += 64 * vi;
   const float* dfs = reinterpret_cast<const float*>(scal + SC_DERIVED_F);
-  const float mh = dfs[SD_MEAN], ml = dfs[SD_MEANLO];
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += stride) {
-    dfv y = v[g];
-    y += dfv{-mh, -ml};
-    phi[g] = df_norm(y);
+  const float mh = dfs[SD_MEAN], ml = dfs[SD_MEANLO], is = dfs[SD_INVSCALE];
+  const int64_t g0 = (int64_t)blockIdx.x * (TPB * RO_PER) + threadIdx.x;
+  dfv y[RO_PER];
+  float t[RO_PER];
+#pragma unroll
+  for (int k = 0; k < RO_PER; ++k) {
+    const int64_t g = g0 + k * TPB;
+    y[k] = g < n ? v[g] : dfv{0.f, 0.f};
+    t[k] = e && g < n ? e[vi * vs + g] : 0.f;
+  }
+#pragma unroll
+  for (int k = 0; k < RO_PER; ++k) {
+    const int64_t g = g0 + k * TPB;
+    if (g >= n) break;
+    if (e) y[k] = df_iterate(y[k], t[k] * is);
+    y[k] += dfv{-mh, -ml};
+    phi[g] = df_norm(y[k]);
   }
 }
 
@@ -2646,6 +2681,30 @@ static cudaError_t refine_resid(Solver* c, const double* phi64, float* r, double
   return cudaGetLastError();
 }
 
+// MIXED, the second and last sweep of a replayed solve: the norm of the residual
+// after the correction e, r - s K (e / s) = r - K e, in FP32, and the integral
+// of the iterate plus e / s (k_ref_out adds it).  r = s (Pi b - K phi) came from
+// the double-float apply, and the sum of the first sweep's FP32 iterate and an
+// FP32 correction is exact as a pair, so this is the residual of the returned
+// solution but for the FP32 rounding of K e, about 2^-24 |K| |e|, below what the
+// FP32 inner solve leaves of r (8^3 to 86^3 elements, random and smooth right-hand
+// sides: within 10% of the residual in FP64).  A later sweep rounds the iterate,
+// and a residual as small as that rounding has to be formed anew.  A double-float
+// apply to the new iterate takes some eight times the instructions (two
+// right-hand sides on 128^3: 2431 us, here 775; 64^3 322 us, here 119; 32^3
+// 54 us, here 28).
+static cudaError_t refine_check(Solver* c, const float* e, const float* r, double* norm_out, double* wsum_out) {
+  const int N = c->mg.lv[0].N;
+  const int steps = apply_steps(N);
+  dim3 grid = apply_grid(N, steps);
+  grid.z *= c->V;
+  const ApplyDot dt = {(double*)c->red_tmp, c->red_counter, norm_out, POST_NONE, wsum_out, apply_invW(c)};
+  launch_pdl(k_apply_el<float, EPI_CHECK, true>, grid, AT, sizeof(ApplySmem<float, EPI_CHECK, true>), c->stream, N,
+             steps, e, (float*)nullptr, r, (float*)nullptr, reinterpret_cast<float*>(c->phidf), 0.f, 0.f, 0.f, c->scal,
+             dt, c->vs);
+  return cudaGetLastError();
+}
+
 // start: Pi b, the scale s, phi = 0 (FP64; MIXED: the first update assigns),
 // r = s Pi b in FP32 and |r|^2 into scal[10]
 static void refine_setup(Solver* c, const double* b, double* phi64, float* r) {
@@ -2688,8 +2747,9 @@ static void refine_update(Solver* c, double* phi64, const float* e) {
 }
 
 // end: phi with mean zero (FP64; MIXED: float pairs); have_mean: the last
-// residual apply already summed the integral and derived the mean
-static void refine_finish(Solver* c, double* phi, bool have_mean = false) {
+// residual apply already summed the integral and derived the mean; e_last
+// (MIXED): the last correction, not yet in the iterate (refine_check)
+static void refine_finish(Solver* c, double* phi, bool have_mean = false, const float* e_last = nullptr) {
   const Level& L0 = c->mg.lv[0];
   const int N = L0.N;
   const size_t n = L0.size;
@@ -2699,8 +2759,9 @@ static void refine_finish(Solver* c, double* phi, bool have_mean = false) {
     if (!have_mean)
       launch_pdl(k_ref_wsum, dim3((unsigned)reduce_blocks(n), (unsigned)c->V), TPB, 0, c->stream, N, v,
                (double*)c->red_tmp, c->red_counter, c->scal, 1.0 / W, c->vs);
-    launch_pdl(k_ref_out, dim3((unsigned)grid_for(n), (unsigned)c->V), TPB, 0, c->stream, (int64_t)n, v,
-               reinterpret_cast<dfv*>(phi), (const double*)c->scal, c->vs);
+    const int per = TPB * RO_PER;
+    launch_pdl(k_ref_out, dim3((unsigned)((n + per - 1) / per), (unsigned)c->V), TPB, 0, c->stream, (int64_t)n, v,
+               reinterpret_cast<dfv*>(phi), e_last, (const double*)c->scal, c->vs);
     return;
   }
   reduce<double>(c, N, RD_WSUM, phi, nullptr, c->scal + 6, POST_MEAN, 1.0 / W);
@@ -2710,6 +2771,8 @@ static void refine_finish(Solver* c, double* phi, bool have_mean = false) {
 static double solver_rtol(const Solver* c) {
   return c->cfg.mg_rtol > 0 ? c->cfg.mg_rtol : (c->precision == FEP3M_FP64 ? 1e-13 : 1e-10);
 }
+
+constexpr double kCheckRtol = 1e-11;   // solve_fixed: the tightest tolerance checked by refine_check
 
 // host-checked solve (used once to calibrate the iteration counts, and as the
 // fallback when a replayed solve misses its tolerance)
@@ -2783,6 +2846,9 @@ static cudaError_t solve_fixed(Solver* c, const double* b, double* phi, int kout
   float* e32 = (float*)sb[4];
   refine_setup(c, b, phi, r32);   // |r|^2 into sc[10]
   const bool mixed = c->precision != FEP3M_FP64;
+  // MIXED, the exact inner solve in two sweeps: the last residual is formed from the correction
+  // (refine_check), unless the tolerance is near the double-float residual's own rounding
+  const bool check = mixed && kout == 2 && c->mg.fdm.N > 0 && solver_rtol(c) >= kCheckRtol;
   for (int step = 0; step < kout; ++step) {
     if (step == 0 && c->ev_in0) cudaEventRecordWithFlags(c->ev_in0, c->stream, cudaEventRecordExternal);
     if (c->mg.fdm.N > 0) mg.fdm_solve(r32, e32, (float*)sb[0], (float*)sb[1]);
@@ -2791,6 +2857,11 @@ static cudaError_t solve_fixed(Solver* c, const double* b, double* phi, int kout
     // MIXED: the first sweep's apply forms the iterate e / s itself, and the
     // last residual's |r|^2 is accumulated by its apply
     const bool first_df = mixed && step == 0;
+    if (check && step == kout - 1) {
+      const cudaError_t e = refine_check(c, e32, r32, sc + 11, sc + 6);
+      if (e != cudaSuccess) return e;
+      break;
+    }
     if (!first_df) refine_update(c, phi, e32);
     const bool last = mixed && step == kout - 1;   // also the iterate's integral, for the finish
     cudaError_t e = refine_resid(c, phi, r32, last ? sc + 11 : nullptr, first_df ? e32 : nullptr, last ? sc + 6 : nullptr);
@@ -2799,7 +2870,7 @@ static cudaError_t solve_fixed(Solver* c, const double* b, double* phi, int kout
   if (mixed && kout == 0)
     cudaMemsetAsync(c->phidf, 0, (c->V > 1 ? c->V * c->vs : (int64_t)L0.size) * sizeof(dfv), c->stream);
   if (!mixed || kout == 0) reduce<float>(c, N, RD_NORM2, r32, nullptr, sc + 11);
-  refine_finish(c, phi, mixed && kout > 0);
+  refine_finish(c, phi, mixed && kout > 0, check ? e32 : nullptr);
   return cudaGetLastError();
 }
 
