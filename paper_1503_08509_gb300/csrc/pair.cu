@@ -1917,32 +1917,54 @@ __global__ void __launch_bounds__(PT, 2) k_adj64(int64_t ne, int n_sr, int z0, i
 //   A[s][k] = sum over the offsets o with o + k inside the block of D(o, s + k + o).
 // For the vertex v = s + k the terms are D(o, v + o) over the offsets that
 // corner k's block holds: along each axis, o_a = -(n_sr + 1) only for k_a = 1,
-// o_a = n_sr only for k_a = 0, the others for both.  A CTA takes 32 consecutive
-// vertices (consecutive lanes read consecutive elements of D) and deals the
-// offset planes oz of the chunk [z0, z1) to its eight warps.  A thread sums a
-// plane's terms into nine classes (first, inner, last offset along x and along
-// y), a row of D's values and weight sums ahead in registers, adds them into the corners of
-// the plane's class along z in shared memory, and the warps' corner sums are
-// combined there in order: deterministic.  FP32 path (H0 set): D holds the contraction with the
+// o_a = n_sr only for k_a = 0, the others for both.  A CTA takes 256 / AVZ
+// consecutive vertices (consecutive lanes read consecutive elements of D) and
+// deals the offset planes oz of the chunk [z0, z1) to AVZ threads per vertex.  A
+// thread sums a plane's terms into nine classes (first, inner, last offset along
+// x and along y); planes of one class along z add up there (AVZ = 1), then go to
+// the corners' sums in shared memory, which are combined in order:
+// deterministic.  The rows of D come by cp.async into a ring of the thread's own
+// (av_ring rows of 2 n_sr + 2 values in flight), the weight sums a row ahead in
+// registers.  FP32 path (H0 set): D holds the contraction with the
 // node-0-relative table, and each term gains H(o, 0) Wsum(v + o)
 // (pair_adjoint_table).  FP64 path: D is the whole contraction, as pairs.  Terms
-// and sums in double-float arithmetic.  Bound by FP32 issue in the FP32 path (19
-// operations a term beside its loads) and by the read of D.  10^6 charges on
-// 128^3: 3484 -> 2301 us, 262 144 on 64^3: 439 -> 285 us against one warp per 32
-// vertices and row of offsets with 27 class sums in shared memory, whose
-// bookkeeping took most of its instructions.
-constexpr int AVV = 32, AVZ = PT / AVV;   // vertices and threads per vertex of a CTA
-template <class T, int NSR>
+// and sums in double-float arithmetic (19 operations a term in the FP32 path, of
+// 36 instructions).  Bound by instruction issue, at 2/3 of its rate.  10^6
+// charges on 128^3: 3484 us with one warp per 32 vertices and row of offsets and 27
+// class sums in shared memory, 2301 with a row ahead in registers and AVZ = 8, 1458
+// now; 262 144 on 64^3: 439, 285 and 195 us.
+//
+// One thread per vertex (AVZ = 1) from 40 elements per axis on, eight below,
+// where one leaves too few warps (8 / 1, us: 16^3 9.9 / 35, 32^3 37 / 39, 40^3
+// 68 / 61, 48^3 110 / 92, 64^3 249 / 195).
+// asynchronous copy of one value (4 or 8 bytes) to shared memory
+template <class T>
+__device__ __forceinline__ void cp_async_val(T* dst, const T* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "n"(sizeof(T))
+               : "memory");
+}
+// rows of D in flight per thread: a divisor of the rows of a plane (a row's place is the same in every plane)
+template <int NSR>
+constexpr int av_ring = NSR == 2 ? 3 : (NSR == 4 ? 5 : 4);
+template <class T, int NSR, int AVZ>
+struct AdjVertexSmem {
+  static constexpr int NOFF = 2 * NSR + 2;
+  T ring[av_ring<NSR>][NOFF][PT];
+  dfacc part[AVZ][8][PT / AVZ];
+  float2 h0[sizeof(T) == 4 ? NOFF * NOFF * NOFF : 1];
+  int live[PT / AVZ];
+};
+template <class T, int NSR, int AVZ>
 __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int first, const int* __restrict__ count,
                                                       const T* __restrict__ D, const float2* __restrict__ H0,
                                                       const float2* __restrict__ wsum, double* __restrict__ A) {
-  constexpr int KEEP = NSR + 1, NOFF = 2 * NSR + 2, PLANE = NOFF * NOFF;
+  constexpr int KEEP = NSR + 1, NOFF = 2 * NSR + 2, PLANE = NOFF * NOFF, AVV = PT / AVZ, AV_RING = av_ring<NSR>;
   constexpr bool REL = sizeof(T) == 4;   // T: float, or df (FP64)
-  __shared__ dfacc part[AVZ][8][AVV];
-  __shared__ float2 h0[REL ? PLANE * NOFF : 1];
-  __shared__ int live[AVV];
+  extern __shared__ __align__(16) unsigned char av_smem[];
+  AdjVertexSmem<T, NSR, AVZ>& S = *reinterpret_cast<AdjVertexSmem<T, NSR, AVZ>*>(av_smem);
   const int64_t ne = (int64_t)n * n * n;
-  const int vl = threadIdx.x & (AVV - 1), zg = threadIdx.x / AVV;
+  const int tid = threadIdx.x, vl = tid & (AVV - 1), zg = AVZ == 1 ? 0 : tid / AVV;
   const int64_t v = blockIdx.x * (int64_t)AVV + vl;
   const bool in = v < ne;
   const int vx = in ? (int)(v % n) : 0, vy = in ? (int)((v / n) % n) : 0, vz = in ? (int)(v / ((int64_t)n * n)) : 0;
@@ -1954,15 +1976,16 @@ __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int
       for (int k = 0; k < 8; ++k)
         any |= count[((k & 1) ? px : vx) + (int64_t)n * (((k & 2) ? py : vy) + (int64_t)n * ((k & 4) ? pz : vz))] != 0;
     }
-    live[vl] = any;
+    S.live[vl] = any;
   }
   if (REL)
-    for (int i = threadIdx.x; i < PLANE * NOFF; i += PT) h0[i] = H0[i];
+    for (int i = tid; i < PLANE * NOFF; i += PT) S.h0[i] = H0[i];
   __syncthreads();
-  const bool act = live[vl] != 0;
+  const bool act = S.live[vl] != 0;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) part[zg][k][vl] = dfacc{0.f, 0.f};   // corner sums, k = kx + 2 ky + 4 kz
-  if (__any_sync(0xffffffffu, act)) {
+  for (int k = 0; k < 8; ++k) S.part[zg][k][vl] = dfacc{0.f, 0.f};   // corner sums, k = kx + 2 ky + 4 kz
+  const int oz0 = z0 + zg;
+  if (oz0 < z1 && __any_sync(0xffffffffu, act)) {
     int wx[NOFF];   // the elements' x coordinates vx + o - KEEP (n >= 2 n_sr + 1: one period at most)
 #pragma unroll
     for (int i = 0; i < NOFF; ++i) {
@@ -1970,51 +1993,79 @@ __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int
       x += x < 0 ? n : 0;
       wx[i] = x >= n ? x - n : x;
     }
-    for (int oz = z0 + zg; oz < z1; oz += AVZ) {
+    int ey0 = vy - KEEP;
+    ey0 += ey0 < 0 ? n : 0;
+    auto plane_row = [&](int oz) {   // the first element of the plane's elements (n <= 404: below 2^31)
       int ez = vz + oz - KEEP;
       ez += ez < 0 ? n : 0;
       ez = ez >= n ? ez - n : ez;
-      dfacc P[3][3];   // [class along y][class along x]: first, inner, last
+      return n * n * ez;
+    };
+    dfacc P[3][3];   // [class along y][class along x]: first, inner, last
 #pragma unroll
-      for (int i = 0; i < 9; ++i) P[i / 3][i % 3] = dfacc{0.f, 0.f};
-      int ey = vy - KEEP;
-      ey += ey < 0 ? n : 0;
-      const T* Dp = D + (int64_t)(oz - z0) * PLANE * ne;
-      const int erow0 = n * n * ez;   // n <= 404: below 2^31
-      T d[2][NOFF];                   // the row of D being summed and the next (and its weight sums)
-      float2 w[REL ? 2 : 1][NOFF];
-      auto load = [&](int oy) {       // row oy; called in order
-        const int er = erow0 + n * ey;
+    for (int i = 0; i < 9; ++i) P[i / 3][i % 3] = dfacc{0.f, 0.f};
+    float2 w[REL ? 2 : 1][NOFF];   // the weight sums of the row being summed and of the next
+    int eyd = ey0, eyw = ey0;      // element rows of the next fetch and the next load
+    // row oy of plane oz of D into this thread's ring; called in order of the rows
+    auto fetch = [&](int oz, int oy, int prow) {
+      if (oz < z1) {
+        const T* Dr = D + ((int64_t)(oz - z0) * PLANE + oy * NOFF) * ne;
+        const int er = prow + n * eyd;
 #pragma unroll
-        for (int ox = 0; ox < NOFF; ++ox) {
-          d[oy & 1][ox] = Dp[(int64_t)(oy * NOFF + ox) * ne + er + wx[ox]];
-          if constexpr (REL) w[oy & 1][ox] = wsum[er + wx[ox]];
-        }
-        ++ey;
-        ey = ey == n ? 0 : ey;
-      };
-      load(0);
+        for (int ox = 0; ox < NOFF; ++ox)
+          cp_async_val(&S.ring[oy % AV_RING][ox][tid], Dr + ox * ne + (unsigned)(er + wx[ox]));
+        eyd = eyd + 1 == n ? 0 : eyd + 1;
+        if (oy == NOFF - 1) eyd = ey0;
+      }
+      tc::cp_async_commit();       // (past the last row an empty group, for the count below)
+    };
+    auto load = [&](int oy, int prow) {   // row oy's weight sums; called in order of the rows
+      if constexpr (REL) {
+        const int er = prow + n * eyw;
+#pragma unroll
+        for (int ox = 0; ox < NOFF; ++ox) w[oy & 1][ox] = wsum[(unsigned)(er + wx[ox])];
+        eyw = eyw + 1 == n ? 0 : eyw + 1;
+        if (oy == NOFF - 1) eyw = ey0;
+      }
+    };
+    int prow = plane_row(oz0);
+#pragma unroll
+    for (int oy = 0; oy < AV_RING; ++oy) fetch(oz0, oy, prow);
+    load(0, prow);
+#pragma unroll 1
+    for (int oz = oz0; oz < z1; oz += AVZ) {
+      const int pnext = plane_row(oz + AVZ);
 #pragma unroll
       for (int oy = 0; oy < NOFF; ++oy) {
         constexpr int L = NOFF - 1;
         const int cy = oy == 0 ? 0 : (oy == L ? 2 : 1);
-        if (oy + 1 < NOFF) load(oy + 1);
+        if (oy + 1 < NOFF) load(oy + 1, prow);
+        else if (oz + AVZ < z1) load(0, pnext);
+        asm volatile("cp.async.wait_group %0;" ::"n"(AV_RING - 1) : "memory");   // row oy (this thread's own copies)
+        T d[NOFF];
+#pragma unroll
+        for (int ox = 0; ox < NOFF; ++ox) d[ox] = S.ring[oy % AV_RING][ox][tid];
+        if (oy + AV_RING < NOFF) fetch(oz, oy + AV_RING, prow);   // into the row just read
+        else fetch(oz + AVZ, oy + AV_RING - NOFF, pnext);
 #pragma unroll
         for (int ox = 0; ox < NOFF; ++ox) {
           const int cx = ox == 0 ? 0 : (ox == L ? 2 : 1);
           if constexpr (REL) {
-            const float2 h = h0[oz * PLANE + oy * NOFF + ox], u = w[oy & 1][ox];
+            const float2 h = S.h0[oz * PLANE + oy * NOFF + ox], u = w[oy & 1][ox];
             const float p = h.x * u.x;
             float r = fmaf(h.x, u.x, -p);
             r = fmaf(h.x, u.y, r);
             r = fmaf(h.y, u.x, r);
             acc_add(P[cy][cx], p);
-            acc_add(P[cy][cx], d[oy & 1][ox] + r);
+            acc_add(P[cy][cx], d[ox] + r);
           } else {
-            acc_merge(P[cy][cx], dfacc{d[oy & 1][ox].h, d[oy & 1][ox].l});
+            acc_merge(P[cy][cx], dfacc{d[ox].h, d[ox].l});
           }
         }
       }
+      prow = pnext;
+      // the inner planes of a thread count alike for both corners: their sums stay in P
+      if (AVZ == 1 && oz > 0 && oz < NOFF - 2 && oz < z1 - 1) continue;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {   // corner (kx, ky): classes 0, 1 for 1, classes 1, 2 for 0
         const int x0 = k & 1 ? 0 : 1, y0 = k & 2 ? 0 : 1;
@@ -2022,9 +2073,11 @@ __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int
         acc_merge(t, P[y0][x0 + 1]);
         acc_merge(t, P[y0 + 1][x0]);
         acc_merge(t, P[y0 + 1][x0 + 1]);
-        if (oz != NOFF - 1) acc_merge(part[zg][k + 4][vl], t);
-        if (oz != 0) acc_merge(part[zg][k][vl], t);
+        if (oz != NOFF - 1) acc_merge(S.part[zg][k + 4][vl], t);
+        if (oz != 0) acc_merge(S.part[zg][k][vl], t);
       }
+#pragma unroll
+      for (int i = 0; i < 9; ++i) P[i / 3][i % 3] = dfacc{0.f, 0.f};
     }
   }
   __syncthreads();
@@ -2032,9 +2085,9 @@ __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int
 #pragma unroll
   for (int t = 0; t < 8 / AVZ; ++t) {
     const int k = zg + AVZ * t, kx = k & 1, ky = (k >> 1) & 1, kz = k >> 2;
-    dfacc s = part[0][k][vl];
+    dfacc s = S.part[0][k][vl];
 #pragma unroll
-    for (int z = 1; z < AVZ; ++z) acc_merge(s, part[z][k][vl]);
+    for (int z = 1; z < AVZ; ++z) acc_merge(s, S.part[z][k][vl]);
     const int sx = vx - kx < 0 ? n - 1 : vx - kx, sy = vy - ky < 0 ? n - 1 : vy - ky, sz = vz - kz < 0 ? n - 1 : vz - kz;
     double* dst = A + (sx + (int64_t)n * (sy + (int64_t)n * sz)) * 8 + k;
     *dst = first ? acc_value(s) : *dst + acc_value(s);
@@ -2454,13 +2507,22 @@ cudaError_t energy(fep3m_ctx* c, double* U_dev, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <class T, int NSR>
-static void launch_adj_vertex(fep3m_ctx* c, int z0, int z1, const T* D, double* A, cudaStream_t s) {
+constexpr int AV_LARGE = 40;   // k_adj_vertex
+template <class T, int NSR, int AVZ>
+static void launch_adj_vertex_z(fep3m_ctx* c, int z0, int z1, const T* D, double* A, cudaStream_t s) {
   const int64_t ne = (int64_t)c->n * c->n * c->n;
   const bool rel = sizeof(T) == 4;   // D relative to node 0 (FP32 path)
-  FEP3M_CL k_adj_vertex<T, NSR><<<(unsigned)((ne + AVV - 1) / AVV), PT, 0, s>>>(
+  const size_t smem = sizeof(AdjVertexSmem<T, NSR, AVZ>);
+  (void)smem_limit((const void*)k_adj_vertex<T, NSR, AVZ>, smem);   // a failure shows as the launch's error
+  constexpr int AVV = PT / AVZ;
+  FEP3M_CL k_adj_vertex<T, NSR, AVZ><<<(unsigned)((ne + AVV - 1) / AVV), PT, smem, s>>>(
       c->n, z0, z1, z0 == 0, c->count, D, rel ? (const float2*)c->H0df : nullptr,
       rel ? (const float2*)c->Wsum : nullptr, A);
+}
+template <class T, int NSR>
+static void launch_adj_vertex(fep3m_ctx* c, int z0, int z1, const T* D, double* A, cudaStream_t s) {
+  if (c->n >= AV_LARGE) launch_adj_vertex_z<T, NSR, 1>(c, z0, z1, D, A, s);
+  else launch_adj_vertex_z<T, NSR, 8>(c, z0, z1, D, A, s);
 }
 
 // D-GEMM + gather over chunks of whole offset planes (all offsets with one
