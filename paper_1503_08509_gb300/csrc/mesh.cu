@@ -1546,8 +1546,9 @@ __global__ void __launch_bounds__(FT_THREADS) k_tc_rows(int64_t R, int K, int cb
 //
 // Chosen for N >= TP_MIN (solver_init); below, a pass is a few microseconds of
 // latency and the small CTAs of k_tc_rows leave room for the step's concurrent
-// kernels.  Paired passes, two right-hand sides: N = 192 50 -> 41 us, N = 243 152
-// -> 91 us, N = 384 588 -> 430 us (the scaling pass 53, 118 and 531 us).
+// kernels.  Paired passes, two right-hand sides: N = 192 50 -> 40 us, N = 243 152
+// -> 86 us, N = 384 588 -> 405 us (the scaling pass 51, 108 and 488 us).  Three
+// operand stages leave the L1 too little room for the rows' lines (N = 384 +20%).
 constexpr int TP_GROUP = 256, TP_PROD = 2 * TP_GROUP, TP_THREADS = TP_PROD + 64, TP_MIN = 160;
 static size_t tc_pass_smem(int nt) { return 1024 + 2 * (size_t)(3 * 16384 + 3 * nt * 128) + 128; }
 
@@ -1607,13 +1608,15 @@ __global__ void __launch_bounds__(TP_THREADS, 1) k_tc_pass(TcPass a) {
     const int gt = tid & (TP_GROUP - 1);
     const int align = (N & 1) == 0 && (!SYNTH || (P & 1) == 0) ? 2 : 1;
     float x1[2][8], x2[2][8];
+    // a unit's row: eight lanes take rows 4 apart, whose places in the swizzled tile are in different banks
+    auto unit_row = [](int u) { return ((u >> 2) & ~7) | ((u & 4) ? 4 : 0) | ((u >> 3) & 3); };
     auto load = [&](int job, int c) {
       const int rt = (job / a.ntile) % a.rtiles, v = job / (a.ntile * a.rtiles);
       const float* in = a.in + v * a.vs;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         const int u = gt + TP_GROUP * j, i0 = 32 * c + 2 * (u & 3);
-        const int64_t r = (int64_t)rt * 128 + (u >> 2);
+        const int64_t r = (int64_t)rt * 128 + unit_row(u);
         const bool on = r < a.R;
         const float* row = in + r * N;
 #pragma unroll
@@ -1664,7 +1667,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1) k_tc_pass(TcPass a) {
         if (ok) {
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
-            const int u = gt + TP_GROUP * j, row = u >> 2, g = u & 3;
+            const int u = gt + TP_GROUP * j, row = unit_row(u), g = u & 3;
             uint32_t p0[4], p1[4], p2[4];
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
