@@ -1805,6 +1805,198 @@ __global__ void __launch_bounds__(TP_THREADS, 1) k_tc_pass(TcPass a) {
   if (warp == 0) tmem_dealloc(tmem, ncols);
 }
 
+// The same GEMM for many rows of 64 (the screen adjoint's contraction on large
+// meshes): out[(i - cb) R + r] = sum_a in[64 r + a] B[i][a], column tiles of 128.
+// k_tc_rows splits a row tile's operands once per column tile and its store, its
+// MMAs and its loads follow one another.  Here a persistent CTA per SM takes 128
+// rows through all column tiles: four warps load and split the next rows, one
+// copies the table's tiles (cp.async.bulk, two stages), one issues the MMAs, and
+// eight store a tile's results from one half of TMEM (128 columns for the leading
+// product, 128 for the other five) while the other half fills.  Bound by the write
+// of D (512 values an element at n_sr = 3): 64^3 elements 214 -> 106 us, 128^3 1675
+// -> 846 us (5.1 TB/s).  Every wait is bounded, as in k_tc_pass.
+constexpr int SW_NT = 128, SW_PROD = 128, SW_EPI = 256, SW_THREADS = SW_PROD + SW_EPI + 64;
+constexpr size_t SW_SMEM = 1024 + 2 * 3 * 16384 + 2 * (size_t)(3 * SW_NT * 128);
+__global__ void __launch_bounds__(SW_THREADS, 1) k_tc_sweep(int64_t R, int cb, int ce, const float* __restrict__ in,
+                                                            const uint4* __restrict__ Bp, float* __restrict__ out,
+                                                            int* __restrict__ err) {
+  using namespace tc;
+  extern __shared__ __align__(16) unsigned char fsm[];
+  __shared__ uint64_t bars[10];   // afull[2], aempty[2], bfull[2], mdone[2], tempty[2]
+  __shared__ uint32_t tslot;
+  __shared__ int dead;
+  unsigned char* tiles = fsm + ((1024u - (smem_u32(fsm) & 1023u)) & 1023u);
+  constexpr uint32_t BP = SW_NT * 128, ASTAGE = 3 * 16384, BSTAGE = 3 * BP;
+  const uint32_t tl = smem_u32(tiles), tbl = tl + 2 * ASTAGE;
+  const uint32_t afull = smem_u32(&bars[0]), aempty = smem_u32(&bars[2]), bfull = smem_u32(&bars[4]),
+                 mdone = smem_u32(&bars[6]), tempty = smem_u32(&bars[8]);
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int t0 = cb / SW_NT, t1 = (ce + SW_NT - 1) / SW_NT, rtiles = (int)((R + 127) / 128);
+  if (warp == 0) tmem_alloc(smem_u32(&tslot), 512);
+  if (tid == 0) {
+    for (int k = 0; k < 8; ++k) mbar_init_n(afull + 8 * k, 1);
+    for (int k = 0; k < 2; ++k) mbar_init_n(tempty + 8 * k, SW_EPI / 32);
+    dead = 0;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tslot;
+  const volatile int* vdead = &dead;
+  auto wait = [&](uint32_t bar, uint32_t phase) -> bool {
+    if (*vdead) return false;
+    if (mbar_wait(bar, phase)) return true;
+    atomicExch(&dead, 1);
+    return false;
+  };
+  int it = 0;   // tiles so far: table stage, TMEM half and their barriers it mod 2
+  if (warp < SW_PROD / 32) {
+    // -------- the rows' operands: eight units of eight values per thread, eight threads per row
+    float x[8][8];
+    auto load = [&](int rt) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int u = tid + SW_PROD * j;
+        const int64_t r = (int64_t)rt * 128 + (u >> 3);
+        float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0;
+        if (r < R) {
+          const float4* src = reinterpret_cast<const float4*>(in + r * 64 + 8 * (u & 7));
+          v0 = src[0];
+          v1 = src[1];
+        }
+        x[j][0] = v0.x; x[j][1] = v0.y; x[j][2] = v0.z; x[j][3] = v0.w;
+        x[j][4] = v1.x; x[j][5] = v1.y; x[j][6] = v1.z; x[j][7] = v1.w;
+      }
+    };
+    if ((int)blockIdx.x < rtiles) load(blockIdx.x);
+    int k = 0;
+    for (int rt = blockIdx.x; rt < rtiles; rt += gridDim.x, ++k) {
+      const uint32_t st = k & 1, base = tl + st * ASTAGE;
+      bool ok = k < 2 || wait(aempty + 8 * st, ((k >> 1) - 1) & 1);
+      if (ok) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int u = tid + SW_PROD * j;
+          uint32_t p0[4], p1[4], p2[4];
+#pragma unroll
+          for (int t = 0; t < 4; ++t) bf16_split2(x[j][2 * t], x[j][2 * t + 1], p0[t], p1[t], p2[t]);
+          const uint32_t o = base + sw128_off(u >> 3, 8 * (u & 7));
+          sts128(o, p0);
+          sts128(o + 16384, p1);
+          sts128(o + 32768, p2);
+        }
+        fence_async_smem();
+      }
+      uint32_t all;   // (uniform: a thread that gave up takes the four warps along)
+      asm volatile(
+          "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbar.red.and.pred q, 1, %2, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+          : "=r"(all)
+          : "r"((uint32_t)ok), "r"(SW_PROD)
+          : "memory");
+      if (!all) break;
+      if (tid == 0) mbar_arrive(afull + 8 * st);
+      if (rt + (int)gridDim.x < rtiles) load(rt + gridDim.x);
+    }
+  } else if (warp < (SW_PROD + SW_EPI) / 32) {
+    // -------- results: a warp reads 32 rows of half a tile's columns and stores them column by column
+    const int q4 = warp & 3, half = (warp - SW_PROD / 32) >> 2, lane = tid & 31;
+    bool ok = true;
+    for (int rt = blockIdx.x; ok && rt < rtiles; rt += gridDim.x) {
+      const int64_t r = (int64_t)rt * 128 + 32 * q4 + lane;
+      for (int ct = t0; ct < t1; ++ct, ++it) {
+        const uint32_t st = it & 1;
+        ok = __all_sync(0xffffffffu, wait(mdone + 8 * st, (it >> 1) & 1));
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t ta = tmem + ((uint32_t)(32 * q4) << 16) + 256 * st + 64 * half;
+        float v[64];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          uint32_t vh[16], vl[16];
+          tmem_ld16(ta + 16 * g, vh);
+          tmem_ld16(ta + SW_NT + 16 * g, vl);
+          tmem_wait_ld();
+#pragma unroll
+          for (int t = 0; t < 16; ++t) v[16 * g + t] = __uint_as_float(vh[t]) + __uint_as_float(vl[t]);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty + 8 * st);
+        const int i0 = ct * SW_NT + 64 * half;
+        float* dst = out + (int64_t)(i0 - cb) * R + r;
+        if (r < R) {
+          if (i0 >= cb && i0 + 64 <= ce) {
+#pragma unroll
+            for (int t = 0; t < 64; ++t) dst[t * R] = v[t];
+          } else {
+#pragma unroll
+            for (int t = 0; t < 64; ++t)
+              if (i0 + t >= cb && i0 + t < ce) dst[t * R] = v[t];
+          }
+        }
+      }
+    }
+  } else if (warp == (SW_PROD + SW_EPI) / 32) {
+    // -------- MMA issue
+    if ((tid & 31) == 0) {
+      const uint32_t idesc = umma_idesc(SW_NT);
+      bool ok = true;
+      int k = 0;
+      for (int rt = blockIdx.x; ok && rt < rtiles; rt += gridDim.x, ++k) {
+        const uint32_t as = k & 1, ta = tl + as * ASTAGE;
+        ok = wait(afull + 8 * as, (k >> 1) & 1);
+        for (int ct = t0; ok && ct < t1; ++ct, ++it) {
+          const uint32_t st = it & 1, tb = tbl + st * BSTAGE, hi = tmem + 256 * st, lo = hi + SW_NT;
+          ok = wait(bfull + 8 * st, (it >> 1) & 1) && (it < 2 || wait(tempty + 8 * st, ((it >> 1) - 1) & 1));
+          if (!ok) break;
+          tc_fence_after();
+          for (int kk = 0; kk < 4; ++kk) {
+            const uint32_t a = ta + 32 * kk, b = tb + 32 * kk;
+            const uint32_t acc = kk > 0 ? 1u : 0u;
+            umma_bf16(hi, umma_desc(a), umma_desc(b), idesc, acc);                  // a0 b0
+            umma_bf16(lo, umma_desc(a), umma_desc(b + BP), idesc, acc);             // a0 b1
+            umma_bf16(lo, umma_desc(a + 16384), umma_desc(b), idesc, 1u);           // a1 b0
+            umma_bf16(lo, umma_desc(a), umma_desc(b + 2 * BP), idesc, 1u);          // a0 b2
+            umma_bf16(lo, umma_desc(a + 16384), umma_desc(b + BP), idesc, 1u);      // a1 b1
+            umma_bf16(lo, umma_desc(a + 32768), umma_desc(b), idesc, 1u);           // a2 b0
+          }
+          umma_commit(mdone + 8 * st);
+          if (ct == t1 - 1) umma_commit(aempty + 8 * as);
+        }
+      }
+      if (ok && k > 0) (void)mbar_wait(aempty + 8 * ((k - 1) & 1), ((k - 1) >> 1) & 1);   // the last commit has arrived
+      if (!ok) {   // MMAs in flight when a role gave up
+        for (int q = 0; q < 2; ++q) {
+          (void)mbar_wait(mdone + 8 * q, 0u);
+          (void)mbar_wait(mdone + 8 * q, 1u);
+        }
+      }
+    }
+  } else {
+    // -------- the table's tiles
+    if ((tid & 31) == 0) {
+      bool ok = true;
+      for (int rt = blockIdx.x; ok && rt < rtiles; rt += gridDim.x) {
+        for (int ct = t0; ct < t1; ++ct, ++it) {
+          const uint32_t st = it & 1;
+          if (it >= 2) ok = wait(mdone + 8 * st, ((it >> 1) - 1) & 1);
+          if (!ok) break;
+          mbar_expect(bfull + 8 * st, BSTAGE);
+          bulk_copy(tbl + st * BSTAGE, Bp + (size_t)ct * (BSTAGE / 16), BSTAGE, bfull + 8 * st);
+        }
+      }
+      // copies still in flight: the last one of each stage
+      for (int q = it - 2; q < it; ++q)
+        if (q >= 0) (void)mbar_wait(bfull + 8 * (q & 1), (q >> 1) & 1);
+    }
+  }
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  if (tid == 0 && dead) atomicExch(err, 1);
+  if (warp == 0) tmem_dealloc(tmem, 512);
+}
+
 static size_t tc_rows_smem(int nt) { return 1024 + 3 * 16384 + (size_t)3 * nt * 128 + 16; }
 
 
@@ -2186,6 +2378,19 @@ cudaError_t tc_rows_prepare(int nt) {
 }
 
 // out[(i - cb) R + r] = sum_{a < K} in[r K + a] B[i][a] for the columns cb <= i < ce
+// R rows of 64 on a GPU the caller has to itself (k_tc_sweep)
+cudaError_t tc_sweep_gemm(int64_t R, int cb, int ce, const float* in, const void* Bp, float* out, int* err,
+                          cudaStream_t s) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = smem_limit((const void*)k_tc_sweep, SW_SMEM);
+  if (e != cudaSuccess) return e;
+  const int64_t rt = (R + 127) / 128;
+  FEP3M_CL k_tc_sweep<<<(unsigned)std::min<int64_t>(rt, sms), SW_THREADS, SW_SMEM, s>>>(R, cb, ce, in, (const uint4*)Bp,
+                                                                                       out, err);
+  return cudaGetLastError();
+}
 cudaError_t tc_rows_gemm(int64_t R, int K, int cb, int ce, int nt, const float* in, const void* Bp, float* out,
                          int* err, cudaStream_t s) {
   const dim3 g((unsigned)((R + 127) / 128 * ((ce + nt - 1) / nt - cb / nt)));

@@ -2558,8 +2558,12 @@ static cudaError_t screen_adjoint(fep3m_ctx* c, const T* W, double* A) {
   for (int z0 = 0; z0 < noff; z0 += planes) {
     const int z1 = std::min(noff, z0 + planes), o0 = z0 * plane, no = (z1 - z0) * plane;
     if (tcore) {
-      cudaError_t e = tc_rows_gemm(ne, 64, o0, o0 + no, ADJ_NT, (const float*)W, c->HbA, (float*)c->D_adj,
-                                   c->iflags + 2, s);
+      // one CTA per SM (k_tc_sweep) where the sweep is not beside the mesh solve, whose short kernels on the
+      // critical path would wait for it (run_forward)
+      cudaError_t e = mesh_solve_alone(&c->solv[0])
+                          ? tc_sweep_gemm(ne, o0, o0 + no, (const float*)W, c->HbA, (float*)c->D_adj, c->iflags + 2, s)
+                          : tc_rows_gemm(ne, 64, o0, o0 + no, ADJ_NT, (const float*)W, c->HbA, (float*)c->D_adj,
+                                         c->iflags + 2, s);
       if (e != cudaSuccess) return e;
     } else if constexpr (sizeof(T) == 8) {
       const size_t smem = adj64_smem(c->n_sr);
