@@ -485,7 +485,7 @@ cudaError_t split_pairs(int64_t n, const double* v, void* out, cudaStream_t s);
 // = sum_{a < K} in[r K + a] B[i][a] for the columns cb <= i < ce; B in split
 // bf16 pieces per column tile of nt
 cudaError_t tc_rows_prepare(int nt);
-cudaError_t tc_sweep_gemm(int64_t R, int cb, int ce, const float* in, const void* Bp, float* out, int* err,
+cudaError_t tc_sweep_gemm(int64_t R, int64_t ld, int cb, int ce, const float* in, const void* Bp, float* out, int* err,
                           cudaStream_t s);
 cudaError_t tc_rows_gemm(int64_t R, int K, int cb, int ce, int nt, const float* in, const void* Bp, float* out,
                          int* err, cudaStream_t s);

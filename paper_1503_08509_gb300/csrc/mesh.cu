@@ -1806,7 +1806,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1) k_tc_pass(TcPass a) {
 }
 
 // The same GEMM for many rows of 64 (the screen adjoint's contraction on large
-// meshes): out[(i - cb) R + r] = sum_a in[64 r + a] B[i][a], column tiles of 128.
+// meshes): out[(i - cb) ld + r] = sum_a in[64 r + a] B[i][a], column tiles of 128.
 // k_tc_rows splits a row tile's operands once per column tile and its store, its
 // MMAs and its loads follow one another.  Here a persistent CTA per SM takes 128
 // rows through all column tiles: four warps load and split the next rows, one
@@ -1817,7 +1817,8 @@ __global__ void __launch_bounds__(TP_THREADS, 1) k_tc_pass(TcPass a) {
 // -> 846 us (5.1 TB/s).  Every wait is bounded, as in k_tc_pass.
 constexpr int SW_NT = 128, SW_PROD = 128, SW_EPI = 256, SW_THREADS = SW_PROD + SW_EPI + 64;
 constexpr size_t SW_SMEM = 1024 + 2 * 3 * 16384 + 2 * (size_t)(3 * SW_NT * 128);
-__global__ void __launch_bounds__(SW_THREADS, 1) k_tc_sweep(int64_t R, int cb, int ce, const float* __restrict__ in,
+__global__ void __launch_bounds__(SW_THREADS, 1) k_tc_sweep(int64_t R, int64_t ld, int cb, int ce,
+                                                            const float* __restrict__ in,
                                                             const uint4* __restrict__ Bp, float* __restrict__ out,
                                                             int* __restrict__ err) {
   using namespace tc;
@@ -1923,15 +1924,15 @@ __global__ void __launch_bounds__(SW_THREADS, 1) k_tc_sweep(int64_t R, int cb, i
         __syncwarp();
         if (lane == 0) mbar_arrive(tempty + 8 * st);
         const int i0 = ct * SW_NT + 64 * half;
-        float* dst = out + (int64_t)(i0 - cb) * R + r;
+        float* dst = out + (int64_t)(i0 - cb) * ld + r;
         if (r < R) {
           if (i0 >= cb && i0 + 64 <= ce) {
 #pragma unroll
-            for (int t = 0; t < 64; ++t) dst[t * R] = v[t];
+            for (int t = 0; t < 64; ++t) dst[t * ld] = v[t];
           } else {
 #pragma unroll
             for (int t = 0; t < 64; ++t)
-              if (i0 + t >= cb && i0 + t < ce) dst[t * R] = v[t];
+              if (i0 + t >= cb && i0 + t < ce) dst[t * ld] = v[t];
           }
         }
       }
@@ -2379,7 +2380,7 @@ cudaError_t tc_rows_prepare(int nt) {
 
 // out[(i - cb) R + r] = sum_{a < K} in[r K + a] B[i][a] for the columns cb <= i < ce
 // R rows of 64 on a GPU the caller has to itself (k_tc_sweep)
-cudaError_t tc_sweep_gemm(int64_t R, int cb, int ce, const float* in, const void* Bp, float* out, int* err,
+cudaError_t tc_sweep_gemm(int64_t R, int64_t ld, int cb, int ce, const float* in, const void* Bp, float* out, int* err,
                           cudaStream_t s) {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -2387,7 +2388,7 @@ cudaError_t tc_sweep_gemm(int64_t R, int cb, int ce, const float* in, const void
   if (e == cudaSuccess) e = smem_limit((const void*)k_tc_sweep, SW_SMEM);
   if (e != cudaSuccess) return e;
   const int64_t rt = (R + 127) / 128;
-  FEP3M_CL k_tc_sweep<<<(unsigned)std::min<int64_t>(rt, sms), SW_THREADS, SW_SMEM, s>>>(R, cb, ce, in, (const uint4*)Bp,
+  FEP3M_CL k_tc_sweep<<<(unsigned)std::min<int64_t>(rt, sms), SW_THREADS, SW_SMEM, s>>>(R, ld, cb, ce, in, (const uint4*)Bp,
                                                                                        out, err);
   return cudaGetLastError();
 }

@@ -1957,7 +1957,7 @@ struct AdjVertexSmem {
 };
 template <class T, int NSR, int AVZ>
 __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int first, const int* __restrict__ count,
-                                                      const T* __restrict__ D, const float2* __restrict__ H0,
+                                                      const T* __restrict__ D, int64_t ld, const float2* __restrict__ H0,
                                                       const float2* __restrict__ wsum, double* __restrict__ A) {
   constexpr int KEEP = NSR + 1, NOFF = 2 * NSR + 2, PLANE = NOFF * NOFF, AVV = PT / AVZ, AV_RING = av_ring<NSR>;
   constexpr bool REL = sizeof(T) == 4;   // T: float, or df (FP64)
@@ -2009,11 +2009,11 @@ __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int
     // row oy of plane oz of D into this thread's ring; called in order of the rows
     auto fetch = [&](int oz, int oy, int prow) {
       if (oz < z1) {
-        const T* Dr = D + ((int64_t)(oz - z0) * PLANE + oy * NOFF) * ne;
+        const T* Dr = D + ((int64_t)(oz - z0) * PLANE + oy * NOFF) * ld;
         const int er = prow + n * eyd;
 #pragma unroll
         for (int ox = 0; ox < NOFF; ++ox)
-          cp_async_val(&S.ring[oy % AV_RING][ox][tid], Dr + ox * ne + (unsigned)(er + wx[ox]));
+          cp_async_val(&S.ring[oy % AV_RING][ox][tid], Dr + ox * ld + (unsigned)(er + wx[ox]));
         eyd = eyd + 1 == n ? 0 : eyd + 1;
         if (oy == NOFF - 1) eyd = ey0;
       }
@@ -2509,20 +2509,20 @@ cudaError_t energy(fep3m_ctx* c, double* U_dev, cudaStream_t s) {
 
 constexpr int AV_LARGE = 40;   // k_adj_vertex
 template <class T, int NSR, int AVZ>
-static void launch_adj_vertex_z(fep3m_ctx* c, int z0, int z1, const T* D, double* A, cudaStream_t s) {
+static void launch_adj_vertex_z(fep3m_ctx* c, int z0, int z1, const T* D, int64_t ld, double* A, cudaStream_t s) {
   const int64_t ne = (int64_t)c->n * c->n * c->n;
   const bool rel = sizeof(T) == 4;   // D relative to node 0 (FP32 path)
   const size_t smem = sizeof(AdjVertexSmem<T, NSR, AVZ>);
   (void)smem_limit((const void*)k_adj_vertex<T, NSR, AVZ>, smem);   // a failure shows as the launch's error
   constexpr int AVV = PT / AVZ;
   FEP3M_CL k_adj_vertex<T, NSR, AVZ><<<(unsigned)((ne + AVV - 1) / AVV), PT, smem, s>>>(
-      c->n, z0, z1, z0 == 0, c->count, D, rel ? (const float2*)c->H0df : nullptr,
+      c->n, z0, z1, z0 == 0, c->count, D, ld, rel ? (const float2*)c->H0df : nullptr,
       rel ? (const float2*)c->Wsum : nullptr, A);
 }
 template <class T, int NSR>
-static void launch_adj_vertex(fep3m_ctx* c, int z0, int z1, const T* D, double* A, cudaStream_t s) {
-  if (c->n >= AV_LARGE) launch_adj_vertex_z<T, NSR, 1>(c, z0, z1, D, A, s);
-  else launch_adj_vertex_z<T, NSR, 8>(c, z0, z1, D, A, s);
+static void launch_adj_vertex(fep3m_ctx* c, int z0, int z1, const T* D, int64_t ld, double* A, cudaStream_t s) {
+  if (c->n >= AV_LARGE) launch_adj_vertex_z<T, NSR, 1>(c, z0, z1, D, ld, A, s);
+  else launch_adj_vertex_z<T, NSR, 8>(c, z0, z1, D, ld, A, s);
 }
 
 // D-GEMM + gather over chunks of whole offset planes (all offsets with one
@@ -2544,8 +2544,13 @@ static cudaError_t screen_adjoint(fep3m_ctx* c, const T* W, double* A) {
   }
   // tensor cores (FP32 path, table pieces prepared): column tiles of ADJ_NT offsets
   const bool tcore = sizeof(T) == 4 && c->HbA != nullptr;
+  // one CTA per SM (k_tc_sweep) where the sweep is not beside the mesh solve, whose short kernels on the
+  // critical path would wait for it (run_forward); its stores take D's rows as whole 128-byte lines
+  // (81^3 elements, rows unpadded: 406 us, padded 221; the gather 387 and 375)
+  const bool sweep = tcore && mesh_solve_alone(&c->solv[0]);
+  const int64_t ld = sweep ? (ne + 31) / 32 * 32 : ne;
   const int planes = c->adj_planes;
-  const size_t need = (size_t)planes * plane * ne * sizeof(T);
+  const size_t need = (size_t)planes * plane * ld * sizeof(T);
   if (c->D_bytes < need) {
     if (c->D_adj) cudaFree(c->D_adj);
     c->D_adj = nullptr;
@@ -2558,10 +2563,8 @@ static cudaError_t screen_adjoint(fep3m_ctx* c, const T* W, double* A) {
   for (int z0 = 0; z0 < noff; z0 += planes) {
     const int z1 = std::min(noff, z0 + planes), o0 = z0 * plane, no = (z1 - z0) * plane;
     if (tcore) {
-      // one CTA per SM (k_tc_sweep) where the sweep is not beside the mesh solve, whose short kernels on the
-      // critical path would wait for it (run_forward)
-      cudaError_t e = mesh_solve_alone(&c->solv[0])
-                          ? tc_sweep_gemm(ne, o0, o0 + no, (const float*)W, c->HbA, (float*)c->D_adj, c->iflags + 2, s)
+      cudaError_t e = sweep
+                          ? tc_sweep_gemm(ne, ld, o0, o0 + no, (const float*)W, c->HbA, (float*)c->D_adj, c->iflags + 2, s)
                           : tc_rows_gemm(ne, 64, o0, o0 + no, ADJ_NT, (const float*)W, c->HbA, (float*)c->D_adj,
                                          c->iflags + 2, s);
       if (e != cudaSuccess) return e;
@@ -2577,10 +2580,10 @@ static cudaError_t screen_adjoint(fep3m_ctx* c, const T* W, double* A) {
     typedef typename std::conditional<sizeof(T) == 4, float, df>::type DT;
     const DT* D = (const DT*)c->D_adj;
     switch (c->n_sr) {
-      case 1: launch_adj_vertex<DT, 1>(c, z0, z1, D, A, s); break;
-      case 2: launch_adj_vertex<DT, 2>(c, z0, z1, D, A, s); break;
-      case 3: launch_adj_vertex<DT, 3>(c, z0, z1, D, A, s); break;
-      default: launch_adj_vertex<DT, 4>(c, z0, z1, D, A, s); break;
+      case 1: launch_adj_vertex<DT, 1>(c, z0, z1, D, ld, A, s); break;
+      case 2: launch_adj_vertex<DT, 2>(c, z0, z1, D, ld, A, s); break;
+      case 3: launch_adj_vertex<DT, 3>(c, z0, z1, D, ld, A, s); break;
+      default: launch_adj_vertex<DT, 4>(c, z0, z1, D, ld, A, s); break;
     }
   }
   return cudaGetLastError();
