@@ -166,62 +166,58 @@ __global__ void k_vertex_density(int n, const T* __restrict__ C, double* __restr
   }
 }
 
-// one axis of the order-3 x order-1 mixed mass: global order-3 node g -> up to
-// three vertices with weights.  FP32: the weights times 120, which are exact
-// integers (the element entries are 13/120, 1/60, 3/10 and 3/40), so that the
-// load vector carries no systematic rounding of the weights (it would scale
-// each charge's own smooth potential against its screen and bias U); the
-// last pass divides by 120^3 in FP64.
+// weights of one axis of the order-3 x order-1 mixed mass: element node t, vertex
+// j.  FP32: the weights times 120, which are exact integers (the element entries
+// are 13/120, 1/60, 3/10 and 3/40), so that the load vector carries no systematic
+// rounding of the weights (it would scale each charge's own smooth potential
+// against its screen and bias U); the last pass divides by 120^3 in FP64.
 template <class T>
 __device__ __forceinline__ T mpq_w(int t, int j) {
   if constexpr (sizeof(T) == 4) return cMpq120[t][j];
   else return cMpq64[t][j];
 }
-template <class T>
-__device__ __forceinline__ int mpq_row(int g, int n, int vtx[3], T wgt[3]) {
-  const int e = g / 3, t = g - 3 * e;
-  if (t == 0) {
-    vtx[0] = wrapi(e - 1, n); wgt[0] = mpq_w<T>(3, 0);
-    vtx[1] = e;               wgt[1] = mpq_w<T>(0, 0) + mpq_w<T>(3, 1);
-    vtx[2] = wrapi(e + 1, n); wgt[2] = mpq_w<T>(0, 1);
-    return 3;
-  }
-  vtx[0] = e;               wgt[0] = mpq_w<T>(t, 0);
-  vtx[1] = wrapi(e + 1, n); wgt[1] = mpq_w<T>(t, 1);
-  return 2;
-}
-
 // One axis of b = 4 pi (Mpq (x) Mpq (x) Mpq) r, three separable passes (x, y,
 // then z): out[.., g, ..] = scale sum_k w_k in[.., v_k, ..], vertices v_k of
-// order-3 node g along `axis` (mpq_row; FP32: integer weights, the caller's
-// scale divides by 120^3 at the last pass).  d[3]: the output's extents (3n
-// along the axes done, n along the others; their product < 2^32).  The scale:
-// s64 for an FP64 output, s32 for FP32, the pair s32 + s32lo for float pairs
-// (dfv: the FP32 sum times the scale as a two-product).
-template <class Tin, class Tout>
-__global__ void k_load_axis(int n, int axis, int d0, int d1, int d2, const Tin* __restrict__ in,
-                            Tout* __restrict__ out, double s64, float s32, float s32lo) {
+// order-3 node g along AXIS (FP32: integer weights, the caller's scale divides by
+// 120^3 at the last pass).  inner: the values per vertex (AXIS 0: rows of n; 1 and
+// 2: consecutive values, gridDim.y times).  A thread takes a vertex e and forms the
+// nodes 3 e, 3 e + 1 and 3 e + 2 of its element.  The scale: s64 for an FP64 output, s32 for FP32,
+// the pair s32 + s32lo for float pairs (dfv: the FP32 sum times the scale as a
+// two-product).  Bound by memory.  One thread per node took 52 us for the last axis
+// of 64^3 elements and 394 us of 128^3, its indices most of it; now 12 and 88 us.
+template <int AXIS, class Tin, class Tout>
+__global__ void __launch_bounds__(TPB) k_load_axis(int n, unsigned inner, const Tin* __restrict__ in,
+                                                   Tout* __restrict__ out, double s64, float s32, float s32lo) {
+  // AXIS 0: g = vertex + n row; else g = inner index + inner * vertex, outer index blockIdx.y
   const unsigned g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= (unsigned)d0 * (unsigned)d1 * (unsigned)d2) return;
-  const unsigned q = g / (unsigned)d0;
-  int idx[3] = {(int)(g - q * (unsigned)d0), (int)(q % (unsigned)d1), (int)(q / (unsigned)d1)};
-  int din[3] = {d0, d1, d2};
-  din[axis] = n;
-  const int64_t st[3] = {1, din[0], (int64_t)din[0] * din[1]};
-  int vtx[3];
-  Tin w[3];
-  const int k = mpq_row<Tin>(idx[axis], n, vtx, w);
-  idx[axis] = 0;
-  const int64_t base = idx[0] * st[0] + idx[1] * st[1] + idx[2] * st[2];
-  Tin acc = Tin(0);
-  for (int j = 0; j < k; ++j) acc += w[j] * in[base + vtx[j] * st[axis]];
-  if constexpr (std::is_same<Tout, dfv>::value) {
-    const float p = acc * s32;
-    out[g] = {p, fmaf(acc, s32lo, fmaf(acc, s32, -p))};
-  } else if constexpr (std::is_same<Tout, float>::value) {
-    out[g] = acc * s32;
-  } else {
-    out[g] = (Tout)(s64 * (double)acc);
+  const unsigned span = inner * (unsigned)n;
+  if (g >= span) return;
+  const unsigned e = AXIS == 0 ? g % (unsigned)n : g / inner, i = g - (AXIS == 0 ? e : e * inner);
+  const int64_t st = AXIS == 0 ? 1 : inner;
+  const Tin* src = in + (AXIS == 0 ? (int64_t)i : (int64_t)blockIdx.y * span + i);
+  Tout* dst = out + (AXIS == 0 ? 3 * (int64_t)g : 3 * ((int64_t)blockIdx.y * span) + i + 3 * (int64_t)e * inner);
+  const Tin v0 = src[(e == 0 ? n - 1 : (int)e - 1) * st], v1 = src[e * st],
+            v2 = src[((int)e + 1 == n ? 0 : (int)e + 1) * st];
+  // node 3 e: the vertex itself, shared with the element before; then the element's two inner nodes
+  Tin acc[3];
+  acc[0] = mpq_w<Tin>(3, 0) * v0;
+  acc[0] = fma(mpq_w<Tin>(0, 0) + mpq_w<Tin>(3, 1), v1, acc[0]);
+  acc[0] = fma(mpq_w<Tin>(0, 1), v2, acc[0]);
+#pragma unroll
+  for (int t = 1; t < 3; ++t) {
+    acc[t] = mpq_w<Tin>(t, 0) * v1;
+    acc[t] = fma(mpq_w<Tin>(t, 1), v2, acc[t]);
+  }
+#pragma unroll
+  for (int t = 0; t < 3; ++t) {
+    if constexpr (std::is_same<Tout, dfv>::value) {
+      const float p = acc[t] * s32;
+      dst[t * st] = {p, fmaf(acc[t], s32lo, fmaf(acc[t], s32, -p))};
+    } else if constexpr (std::is_same<Tout, float>::value) {
+      dst[t * st] = acc[t] * s32;
+    } else {
+      dst[t * st] = (Tout)(s64 * (double)acc[t]);
+    }
   }
 }
 
@@ -3642,28 +3638,28 @@ cudaError_t assemble_forward(fep3m_ctx* c) {
   // fine-level scratch (free until its solve, which follows on this stream)
   const Level& L0 = c->solv[0].mg.lv[0];
   const int N3 = 3 * n;
+  // n <= 404: every pass's spans are below 2^32
+  const unsigned gx = (unsigned)grid_for((int64_t)n * n * n);
+  const dim3 gy((unsigned)grid_for((int64_t)N3 * n), (unsigned)n);
+  const unsigned gz = (unsigned)grid_for((int64_t)N3 * N3 * n);
   if (c->precision == FEP3M_MIXED) {
     // b as float pairs (the mixed solver's right-hand side): the FP32 sums of the
     // integer-weighted passes times 4 pi / 120^3 as a two-product
     const double sc = 4.0 * M_PI / (120.0 * 120.0 * 120.0);
     const float sh = (float)sc, sl = (float)(sc - (double)sh);
     float *t1 = (float*)L0.t1, *t2 = (float*)L0.t2;
-    FEP3M_CL k_load_axis<float, float><<<grid_for((int64_t)N3 * n * n), TPB, 0, s>>>(n, 0, N3, n, n, (const float*)c->rv,
-                                                                                    t1, 1.0, 1.0f, 0.0f);
-    FEP3M_CL k_load_axis<float, float><<<grid_for((int64_t)N3 * N3 * n), TPB, 0, s>>>(n, 1, N3, N3, n, t1, t2, 1.0,
-                                                                                     1.0f, 0.0f);
-    FEP3M_CL k_load_axis<float, dfv><<<grid_for((int64_t)N3 * N3 * N3), TPB, 0, s>>>(n, 2, N3, N3, N3, t2,
-                                                                                    reinterpret_cast<dfv*>(c->b64), sc,
-                                                                                    sh, sl);
+    FEP3M_CL k_load_axis<0, float, float><<<gx, TPB, 0, s>>>(n, (unsigned)(n * n), (const float*)c->rv, t1, 1.0, 1.0f,
+                                                             0.0f);
+    FEP3M_CL k_load_axis<1, float, float><<<gy, TPB, 0, s>>>(n, (unsigned)N3, t1, t2, 1.0, 1.0f, 0.0f);
+    FEP3M_CL k_load_axis<2, float, dfv><<<gz, TPB, 0, s>>>(n, (unsigned)(N3 * N3), t2, reinterpret_cast<dfv*>(c->b64),
+                                                           sc, sh, sl);
   } else {
     double *t1 = (double*)L0.t1, *t2 = (double*)L0.t2;
-    FEP3M_CL k_load_axis<double, double><<<grid_for((int64_t)N3 * n * n), TPB, 0, s>>>(n, 0, N3, n, n,
-                                                                                      (const double*)c->rv, t1, 1.0,
-                                                                                      1.0f, 0.0f);
-    FEP3M_CL k_load_axis<double, double><<<grid_for((int64_t)N3 * N3 * n), TPB, 0, s>>>(n, 1, N3, N3, n, t1, t2, 1.0,
-                                                                                       1.0f, 0.0f);
-    FEP3M_CL k_load_axis<double, double><<<grid_for((int64_t)N3 * N3 * N3), TPB, 0, s>>>(n, 2, N3, N3, N3, t2, c->b64,
-                                                                                        4.0 * M_PI, 1.0f, 0.0f);
+    FEP3M_CL k_load_axis<0, double, double><<<gx, TPB, 0, s>>>(n, (unsigned)(n * n), (const double*)c->rv, t1, 1.0, 1.0f,
+                                                               0.0f);
+    FEP3M_CL k_load_axis<1, double, double><<<gy, TPB, 0, s>>>(n, (unsigned)N3, t1, t2, 1.0, 1.0f, 0.0f);
+    FEP3M_CL k_load_axis<2, double, double><<<gz, TPB, 0, s>>>(n, (unsigned)(N3 * N3), t2, c->b64, 4.0 * M_PI, 1.0f,
+                                                               0.0f);
   }
   return cudaGetLastError();
 }
