@@ -116,8 +116,8 @@ typedef struct {
                           screen basis on Gauss-Lobatto nodes, potentials and
                           energy only (fep3m_compute with force = NULL;
                           fep3m_vjp returns FEP3M_EINVAL), the screen
-                          contraction in FP64 in both precisions; p n_el <=
-                          1024                                                  */
+                          contraction in double-float in both precisions;
+                          p n_el <= 1024                                         */
   int n_sr;            /* short-range block half-width in elements, 1..4 (3 in
                           the paper's tests, Sec. 4: a 7 x 7 x 7 block)         */
   int precision;       /* FEP3M_FP64 or FEP3M_MIXED.  Both solve the mesh
@@ -129,8 +129,9 @@ typedef struct {
                           refinement residual, for speed -- FP64 issues at
                           1/64 of the FP32 rate on this GPU -- accurate to
                           about 2e-14 relative, far inside the 1e-10 the
-                          refinement reaches).  Pair sums run in FP64
-                          (FP64) or FP32 (MIXED); the screen contractions in
+                          refinement reaches).  Pair sums run in
+                          double-float with FP64 for close pairs (FP64) or
+                          FP32 (MIXED); the screen contractions in
                           double-float arithmetic on the FP32 pipes (FP64, and
                           MIXED with FEP3M_CUDA_CORES) or as split-precision
                           bf16 tensor-core MMAs against tables relative to
@@ -156,7 +157,9 @@ typedef struct {
   int mg_levels;
   int mg_iterations;        /* last forward solve: total inner CG iterations     */
   int refine_steps;         /* last forward solve: refinement sweeps              */
-  double mg_rel_residual;   /* last forward solve, FP64 residual / |b|            */
+  double mg_rel_residual;   /* last forward solve, residual / |b| (FP64; MIXED:
+                               double-float, or from the last correction alone
+                               after two sweeps at a tolerance >= 1e-11)         */
   int adj_iterations;       /* last adjoint solve                                 */
   double adj_rel_residual;
   int64_t singular_pairs;   /* ordered (target, source) pairs in the blocks       */
@@ -222,7 +225,9 @@ int fep3m_compute(fep3m_ctx* ctx, double* phi, double* U, double* force);
  * writes dLf/dx (N x 3) into dpos and dLf/dQ (N) into dQ (host or device;
  * either may be NULL).  gphi may be NULL (zero).  The derivative is that of
  * the discrete method (element and block membership held fixed); the mesh
- * part uses the same mesh solver on the adjoint right-hand side.           */
+ * part uses the same mesh solver on the adjoint right-hand side.  After a
+ * fep3m_compute without forces the charges' fields are evaluated here, from
+ * that call's mesh solution.                                                */
 int fep3m_vjp(fep3m_ctx* ctx, double gU, const double* gphi, double* dpos, double* dQ);
 
 /* Counters of the last calls (see fep3m_stats).  The pair statistics
