@@ -1745,7 +1745,7 @@ __global__ void __launch_bounds__(TP_THREADS, 1) k_tc_pass(TcPass a) {
     if ((tid & 31) == 0) {
       const uint32_t idesc = umma_idesc((uint32_t)a.nt);
       bool ok = true;
-      int njob = 0;
+      int njob = 0, ndone = 0;
       for (int job = blockIdx.x; ok && job < a.jobs; job += gridDim.x, ++njob) {
         if (njob > 0) ok = wait(tfree, (njob - 1) & 1);   // the accumulators were read
         for (int c = 0; ok && c < kc; ++c, ++it) {
@@ -1764,16 +1764,17 @@ __global__ void __launch_bounds__(TP_THREADS, 1) k_tc_pass(TcPass a) {
             umma_bf16(lo, umma_desc(x + 32768), umma_desc(b), idesc, 1u);                    // a2 b0
           }
           umma_commit(empty + 8 * st);
-          if (c == kc - 1) umma_commit(done);
+          if (c == kc - 1) {
+            umma_commit(done);
+            ++ndone;
+          }
         }
       }
-      // MMAs in flight when a role gave up: their commits arrive on both stages
-      if (!ok) {
-        for (int k = 0; k < 2; ++k) {
-          (void)mbar_wait(empty + 8 * k, 0u);
-          (void)mbar_wait(empty + 8 * k, 1u);
-        }
-      }
+      // The commits arrive on their own, on barriers in this CTA's shared memory: the last one of each
+      // barrier has arrived before the CTA returns (also the MMAs in flight when a role gave up)
+      for (int k = it - 2; k < it; ++k)
+        if (k >= 0) (void)mbar_wait(empty + 8 * (k & 1), (k >> 1) & 1);
+      if (ndone > 0) (void)mbar_wait(done, (ndone - 1) & 1);
     }
   } else {
     // -------- the table's chunks
@@ -1938,7 +1939,7 @@ __global__ void __launch_bounds__(SW_THREADS, 1) k_tc_sweep(int64_t R, int64_t l
     if ((tid & 31) == 0) {
       const uint32_t idesc = umma_idesc(SW_NT);
       bool ok = true;
-      int k = 0;
+      int k = 0, nempty = 0;
       for (int rt = blockIdx.x; ok && rt < rtiles; rt += gridDim.x, ++k) {
         const uint32_t as = k & 1, ta = tl + as * ASTAGE;
         ok = wait(afull + 8 * as, (k >> 1) & 1);
@@ -1958,16 +1959,17 @@ __global__ void __launch_bounds__(SW_THREADS, 1) k_tc_sweep(int64_t R, int64_t l
             umma_bf16(lo, umma_desc(a + 32768), umma_desc(b), idesc, 1u);           // a2 b0
           }
           umma_commit(mdone + 8 * st);
-          if (ct == t1 - 1) umma_commit(aempty + 8 * as);
+          if (ct == t1 - 1) {
+            umma_commit(aempty + 8 * as);
+            ++nempty;
+          }
         }
       }
-      if (ok && k > 0) (void)mbar_wait(aempty + 8 * ((k - 1) & 1), ((k - 1) >> 1) & 1);   // the last commit has arrived
-      if (!ok) {   // MMAs in flight when a role gave up
-        for (int q = 0; q < 2; ++q) {
-          (void)mbar_wait(mdone + 8 * q, 0u);
-          (void)mbar_wait(mdone + 8 * q, 1u);
-        }
-      }
+      // the last commit of each barrier has arrived (k_tc_pass)
+      for (int q = it - 2; q < it; ++q)
+        if (q >= 0) (void)mbar_wait(mdone + 8 * (q & 1), (q >> 1) & 1);
+      for (int q = nempty - 2; q < nempty; ++q)
+        if (q >= 0) (void)mbar_wait(aempty + 8 * (q & 1), (q >> 1) & 1);
     }
   } else {
     // -------- the table's tiles
