@@ -646,7 +646,7 @@ double box_rtol(const fep3m_ctx* c) {
 // B->red: partials of the sums (1024) or of the fused applies from PART on
 // (box_apply_blocks), and before them the sums' results and the scale
 constexpr int RED_SUM = 1024, RED_SCALE = 1027, RED_NORM = 1028, PART = 1060;   // norms: the start's, one per sweep
-constexpr int MAX_SWEEPS = PART - RED_NORM - 1;
+constexpr int NORMS = PART - RED_NORM - 1;   // (the sweeps past them share the last)
 
 void box_sum(Box* B, int mode, const double* v, double* dst, cudaStream_t s) {
   const int64_t len = (int64_t)B->Nn * B->Nn * B->Nn;
@@ -669,7 +669,7 @@ cudaError_t box_refine(fep3m_ctx* c, Box* B, const double* rhs, double* phi) {
   const int64_t len = (int64_t)Ns * Ns * Ns, nn3 = (int64_t)Nn * Nn * Nn;
   cudaStream_t s = c->stream;
   const double rtol = box_rtol(c);
-  const int max_sweeps = std::min(c->cfg.mg_max_cycles > 0 ? c->cfg.mg_max_cycles : 10, MAX_SWEEPS);
+  const int max_sweeps = c->cfg.mg_max_cycles > 0 ? c->cfg.mg_max_cycles : 10;
   const bool mixed = c->precision == FEP3M_MIXED;
   df* pairs = mixed ? (df*)c->phi_hl : nullptr;
   float* scale = (float*)(B->red + RED_SCALE);
@@ -699,15 +699,16 @@ cudaError_t box_refine(fep3m_ctx* c, Box* B, const double* rhs, double* phi) {
   ap.r = B->r32;
   B->sweeps = 0;
   B->relres = 0.0;
-  int read = std::max(1, std::min(B->plan, max_sweeps));   // sweeps before the norms are looked at
+  const int read = std::max(1, std::min(B->plan, std::min(max_sweeps, NORMS)));   // sweeps before the norms are looked at
   for (int k = 0; k < max_sweeps; ++k) {
     if ((e = fdm_apply(B->fdm, B->r32, B->x32, B->w1, B->w2, s)) != cudaSuccess) return e;
     FEP3M_CL k_box_add<<<gsz(len), BT, 0, s>>>(Ns, Nn, B->off, B->x32, scale, phi, pairs);
-    ap.norm = norm + 1 + k;
+    const int at = std::min(k, NORMS - 1);
+    ap.norm = norm + 1 + at;
     if ((e = box_apply(ap, s)) != cudaSuccess) return e;
     if (k + 1 < read) continue;
     // host_red: the scale (two floats), then the norms
-    cudaMemcpyAsync(B->host_red, B->red + RED_SCALE, (k + 3) * sizeof(double), cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(B->host_red, B->red + RED_SCALE, (at + 3) * sizeof(double), cudaMemcpyDeviceToHost, s);
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
     const double n0 = std::sqrt(B->host_red[1]), sc = *(const float*)B->host_red;
     if (!(n0 > 0.0)) {
@@ -718,13 +719,13 @@ cudaError_t box_refine(fep3m_ctx* c, Box* B, const double* rhs, double* phi) {
       return cudaGetLastError();
     }
     bool done = false;
-    for (int j = 0; j <= k && !done; ++j) {   // the sweeps that were needed: the next solve's plan
+    for (int j = 0; j <= at && !done; ++j) {   // the sweeps that were needed: the next solve's plan
       const double rel = std::sqrt(B->host_red[2 + j]) / (sc * n0);
       done = !(rel > rtol);
       B->plan = j + 1;
     }
     B->sweeps = k + 1;
-    B->relres = std::sqrt(B->host_red[2 + k]) / (sc * n0);
+    B->relres = std::sqrt(B->host_red[2 + at]) / (sc * n0);
     if (done || !(B->relres > rtol)) break;
   }
   return cudaGetLastError();
@@ -819,7 +820,7 @@ int box_create(fep3m_ctx* c, int nb, bool neumann, const double* Hw) {
   al((void**)&B->tab, tab.size() * sizeof(df));
   if (neumann) al((void**)&B->sface, (size_t)6 * nb * nb * 16 * sizeof(double));
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? FEP3M_ENOMEM : FEP3M_ECUDA;
-  if (cudaMallocHost(&B->host_red, (MAX_SWEEPS + 2) * sizeof(double)) != cudaSuccess) return FEP3M_ENOMEM;
+  if (cudaMallocHost(&B->host_red, (NORMS + 2) * sizeof(double)) != cudaSuccess) return FEP3M_ENOMEM;
   cudaMemset(B->counter, 0, sizeof(unsigned int));
   if ((e = box_apply_setup(c->st)) != cudaSuccess) return FEP3M_ECUDA;
   cudaMemset(B->g, 0, box_data_size(c) * sizeof(double));

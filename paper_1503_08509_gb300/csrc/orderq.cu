@@ -558,7 +558,8 @@ __global__ void __launch_bounds__(OT) k_oq_eval(int64_t N, int n, OQParams prm, 
 // ---------------------------------------------------------------- host side
 // o->red: partials of the sums from OQ_PART on (one per block), before them the
 // sums' results: the scale, then the norms of the right-hand side and of each sweep's residual
-constexpr int OQ_SUM = 0, OQ_SCALE = 1, OQ_NORM = 2, OQ_PART = 34, OQ_MAX_SWEEPS = OQ_PART - OQ_NORM - 1;
+// (the sweeps past OQ_NORMS share the last)
+constexpr int OQ_SUM = 0, OQ_SCALE = 1, OQ_NORM = 2, OQ_PART = 34, OQ_NORMS = OQ_PART - OQ_NORM - 1;
 inline int sum_blocks(int64_t len) { return (int)std::min<int64_t>(1024, std::max<int64_t>(1, len / (OT * 4))); }
 
 void oq_sum(OrderQ* o, int64_t len, int weighted, const double* v, cudaStream_t s) {
@@ -576,12 +577,12 @@ cudaError_t oq_solve(fep3m_ctx* ctx, OrderQ* o, double rtol, int max_sweeps) {
   cudaStream_t s = ctx->stream;
   const float* scale = (const float*)(o->red + OQ_SCALE);
   double *part = o->red + OQ_PART, *norm = o->red + OQ_NORM;
-  max_sweeps = std::min(max_sweeps, OQ_MAX_SWEEPS);
   o->sweeps = 0;
   o->relres = 0.0;
   FEP3M_CL k_oq_round<<<gsz(len), OT, 0, s>>>(len, o->pb, scale, o->r32);
-  const int read = std::max(1, std::min(o->plan, max_sweeps));
+  const int read = std::max(1, std::min(o->plan, std::min(max_sweeps, OQ_NORMS)));
   for (int k = 0; k < max_sweeps; ++k) {
+    const int at = std::min(k, OQ_NORMS - 1);
     cudaError_t e = fdm_apply(o->fdm, o->r32, o->x32, o->w1, o->w2, s);
     if (e != cudaSuccess) return e;
     FEP3M_CL k_oq_add<<<gsz(len), OT, 0, s>>>(len, o->x32, scale, o->phi, k == 0);
@@ -591,9 +592,9 @@ cudaError_t oq_solve(fep3m_ctx* ctx, OrderQ* o, double rtol, int max_sweeps) {
     FEP3M_CL k_oq_band<1><<<gsz(len), OT, 0, s>>>(Np, o->prm, a, b, c, f, nullptr, nullptr, nullptr, nullptr, nullptr,
                                                   nullptr);
     FEP3M_CL k_oq_band<0><<<gsz(len), OT, 0, s>>>(Np, o->prm, c, f, nullptr, nullptr, o->pb, scale, o->r32, part,
-                                                  o->counter, norm + 1 + k);
+                                                  o->counter, norm + 1 + at);
     if (k + 1 < read) continue;
-    cudaMemcpyAsync(o->host_red, o->red + OQ_SCALE, (k + 3) * sizeof(double), cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(o->host_red, o->red + OQ_SCALE, (at + 3) * sizeof(double), cudaMemcpyDeviceToHost, s);
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
     const double nb = std::sqrt(o->host_red[1]), sc = *(const float*)o->host_red;
     if (!(nb > 0.0)) {
@@ -601,12 +602,12 @@ cudaError_t oq_solve(fep3m_ctx* ctx, OrderQ* o, double rtol, int max_sweeps) {
       return cudaGetLastError();
     }
     bool done = false;
-    for (int j = 0; j <= k && !done; ++j) {   // the sweeps that were needed: the next solve's plan
+    for (int j = 0; j <= at && !done; ++j) {   // the sweeps that were needed: the next solve's plan
       done = std::sqrt(o->host_red[2 + j]) / (sc * nb) <= rtol;
       o->plan = j + 1;
     }
     o->sweeps = k + 1;
-    o->relres = std::sqrt(o->host_red[2 + k]) / (sc * nb);
+    o->relres = std::sqrt(o->host_red[2 + at]) / (sc * nb);
     if (done || o->relres <= rtol) break;
   }
   // int phi = 0: remove the node-integral weighted mean the FP32 corrections leave
@@ -730,7 +731,7 @@ int orderq_create(fep3m_ctx* c) {
   al((void**)&o->red, (OQ_PART + std::max<int64_t>(1024, gsz(np3))) * sizeof(double));
   al((void**)&o->counter, sizeof(unsigned int));
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? FEP3M_ENOMEM : FEP3M_ECUDA;
-  if (cudaMallocHost(&o->host_red, (OQ_MAX_SWEEPS + 2) * sizeof(double)) != cudaSuccess) return FEP3M_ENOMEM;
+  if (cudaMallocHost(&o->host_red, (OQ_NORMS + 2) * sizeof(double)) != cudaSuccess) return FEP3M_ENOMEM;
   cudaMemcpy(o->H, tab.data(), tab.size() * sizeof(df), cudaMemcpyHostToDevice);
   cudaMemset(o->counter, 0, sizeof(unsigned int));
   e = fdm_setup(o->fdm, o->Np, h.lam, h.V, 1, !(c->cfg.flags & FEP3M_CUDA_CORES));
