@@ -555,13 +555,12 @@ __device__ __forceinline__ double box_w1(int g, int Nn, const BoxBand& bd) {
 }
 
 // deterministic FP64 sums: mode 0, sum of squares of v at the solved nodes
-// into *out, with the power of two near the inverse RMS and its inverse into
-// scale[0], scale[1]; mode 1, sum of v over all nodes; mode 2, sum of w3 v
-// over all nodes (w3 the 3-D node integrals)
+// into *out, with the refinement's state for it; mode 1, sum of v over all
+// nodes; mode 2, sum of w3 v over all nodes (w3 the 3-D node integrals)
 __global__ void __launch_bounds__(BT) k_box_sum(int mode, int Ns, int Nn, int off, BoxBand bd,
                                                 const double* __restrict__ v, double* __restrict__ partial,
                                                 unsigned int* __restrict__ counter, double* __restrict__ out,
-                                                float* __restrict__ scale) {
+                                                double rtol, RefineState* __restrict__ st) {
   static_assert(BT == 256, "grid_sum256");
   const int64_t len = mode == 0 ? (int64_t)Ns * Ns * Ns : (int64_t)Nn * Nn * Nn;
   double acc = 0.0;
@@ -579,23 +578,24 @@ __global__ void __launch_bounds__(BT) k_box_sum(int mode, int Ns, int Nn, int of
   double s;
   if (grid_sum256(acc, gridDim.x, blockIdx.x, partial, counter, s)) {
     *out = s;
-    if (mode == 0) rms_scale(s, (double)len, scale);
+    if (mode == 0) refine_begin(s, (double)len, rtol, st);
   }
 }
 
 // the first residual at the solved nodes, scaled into FP32; the FP32
 // correction added back (pairs: the new iterate as float pairs too)
-__global__ void k_box_round(int Ns, int Nn, int off, const double* __restrict__ res, const float* __restrict__ scale,
-                            float* __restrict__ out) {
+__global__ void k_box_round(int Ns, int Nn, int off, const double* __restrict__ res,
+                            const RefineState* __restrict__ st, float* __restrict__ out) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < (int64_t)Ns * Ns * Ns) out[i] = (float)(res[solved_node(i, Ns, Nn, off)] * (double)scale[0]);
+  if (i < (int64_t)Ns * Ns * Ns) out[i] = (float)(res[solved_node(i, Ns, Nn, off)] * (double)st->scale);
 }
-__global__ void k_box_add(int Ns, int Nn, int off, const float* __restrict__ x, const float* __restrict__ scale,
+__global__ void k_box_add(int Ns, int Nn, int off, const float* __restrict__ x, const RefineState* __restrict__ st,
                           double* __restrict__ phi, df* __restrict__ pairs) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < (int64_t)Ns * Ns * Ns) {
+  const float inv = st->inv;   // a power of two, or zero: an earlier sweep reached the tolerance
+  if (inv != 0.f && i < (int64_t)Ns * Ns * Ns) {
     const int64_t j = solved_node(i, Ns, Nn, off);
-    const double v = phi[j] + (double)(x[i] * scale[1]);   // the scale is a power of two
+    const double v = phi[j] + (double)(x[i] * inv);
     phi[j] = v;
     if (pairs) pairs[j] = df_split(v);
   }
@@ -644,15 +644,16 @@ double box_rtol(const fep3m_ctx* c) {
 }
 
 // B->red: partials of the sums (1024) or of the fused applies from PART on
-// (box_apply_blocks), and before them the sums' results and the scale
-constexpr int RED_SUM = 1024, RED_SCALE = 1027, RED_NORM = 1028, PART = 1060;   // norms: the start's, one per sweep
+// (box_apply_blocks), and before them the sums' results and the refinement's state
+constexpr int RED_SUM = 1024, RED_STATE = 1026, RED_NORM = 1028, PART = 1060;   // norms: the start's, one per sweep
 constexpr int NORMS = PART - RED_NORM - 1;   // (the sweeps past them share the last)
+static_assert(sizeof(RefineState) == 2 * sizeof(double), "RED_STATE");
 
-void box_sum(Box* B, int mode, const double* v, double* dst, cudaStream_t s) {
+void box_sum(Box* B, int mode, const double* v, double* dst, cudaStream_t s, double rtol = 0.0) {
   const int64_t len = (int64_t)B->Nn * B->Nn * B->Nn;
   const int nblk = (int)std::min<int64_t>(1024, std::max<int64_t>(1, len / (BT * 8)));
   FEP3M_CL k_box_sum<<<nblk, BT, 0, s>>>(mode, B->Ns, B->Nn, B->off, B->band, v, B->red, B->counter, dst,
-                                         (float*)(B->red + RED_SCALE));
+                                         rtol, (RefineState*)(B->red + RED_STATE));
 }
 
 // K phi = rhs at the solved nodes (Dirichlet: the interior, phi's boundary
@@ -662,7 +663,8 @@ void box_sum(Box* B, int mode, const double* v, double* dst, cudaStream_t s) {
 // MIXED the residual is formed in double-float arithmetic (as the periodic
 // solver's; about 2e-14 relative) from a copy of the iterate as float pairs.
 // The norms stay on the device: they are read once after as many sweeps as
-// the last solve took (and after each further one).  Sets B->sweeps and
+// the last solve took (and after each further one); sweeps past the first that
+// reached the tolerance change nothing (RefineState).  Sets B->sweeps and
 // B->relres (the residual relative to that of phi's starting values)
 cudaError_t box_refine(fep3m_ctx* c, Box* B, const double* rhs, double* phi) {
   const int Ns = B->Ns, Nn = B->Nn;
@@ -672,7 +674,7 @@ cudaError_t box_refine(fep3m_ctx* c, Box* B, const double* rhs, double* phi) {
   const int max_sweeps = c->cfg.mg_max_cycles > 0 ? c->cfg.mg_max_cycles : 10;
   const bool mixed = c->precision == FEP3M_MIXED;
   df* pairs = mixed ? (df*)c->phi_hl : nullptr;
-  float* scale = (float*)(B->red + RED_SCALE);
+  RefineState* st = (RefineState*)(B->red + RED_STATE);
   double* norm = B->red + RED_NORM;
   cudaError_t e;
   if (mixed && (e = split_pairs(nn3, rhs, B->t[0], s)) != cudaSuccess) return e;
@@ -693,24 +695,25 @@ cudaError_t box_refine(fep3m_ctx* c, Box* B, const double* rhs, double* phi) {
     ap.r64 = nullptr;
     r0 = B->res;
   }
-  box_sum(B, 0, r0, norm, s);
-  FEP3M_CL k_box_round<<<gsz(len), BT, 0, s>>>(Ns, Nn, B->off, r0, scale, B->r32);
-  ap.scale = scale;
+  box_sum(B, 0, r0, norm, s, rtol);
+  FEP3M_CL k_box_round<<<gsz(len), BT, 0, s>>>(Ns, Nn, B->off, r0, st, B->r32);
+  ap.state = st;
   ap.r = B->r32;
   B->sweeps = 0;
   B->relres = 0.0;
   const int read = std::max(1, std::min(B->plan, std::min(max_sweeps, NORMS)));   // sweeps before the norms are looked at
   for (int k = 0; k < max_sweeps; ++k) {
     if ((e = fdm_apply(B->fdm, B->r32, B->x32, B->w1, B->w2, s)) != cudaSuccess) return e;
-    FEP3M_CL k_box_add<<<gsz(len), BT, 0, s>>>(Ns, Nn, B->off, B->x32, scale, phi, pairs);
+    FEP3M_CL k_box_add<<<gsz(len), BT, 0, s>>>(Ns, Nn, B->off, B->x32, st, phi, pairs);
     const int at = std::min(k, NORMS - 1);
     ap.norm = norm + 1 + at;
     if ((e = box_apply(ap, s)) != cudaSuccess) return e;
     if (k + 1 < read) continue;
-    // host_red: the scale (two floats), then the norms
-    cudaMemcpyAsync(B->host_red, B->red + RED_SCALE, (at + 3) * sizeof(double), cudaMemcpyDeviceToHost, s);
+    // host_red: the state, then the norms
+    cudaMemcpyAsync(B->host_red, B->red + RED_STATE, (at + 4) * sizeof(double), cudaMemcpyDeviceToHost, s);
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-    const double n0 = std::sqrt(B->host_red[1]), sc = *(const float*)B->host_red;
+    const RefineState& hs = *(const RefineState*)B->host_red;
+    const double n0 = std::sqrt(B->host_red[2]), *nr = B->host_red + 3;
     if (!(n0 > 0.0)) {
       // a zero (or, for non-finite data, NaN) residual: nothing to solve.  MIXED: an infinite
       // boundary value is NaN in the float pairs, reported as not converged, as in FP64
@@ -718,15 +721,12 @@ cudaError_t box_refine(fep3m_ctx* c, Box* B, const double* rhs, double* phi) {
       FEP3M_CL k_box_clear<<<gsz(len), BT, 0, s>>>(Ns, Nn, B->off, phi);
       return cudaGetLastError();
     }
-    bool done = false;
-    for (int j = 0; j <= at && !done; ++j) {   // the sweeps that were needed: the next solve's plan
-      const double rel = std::sqrt(B->host_red[2 + j]) / (sc * n0);
-      done = !(rel > rtol);
-      B->plan = j + 1;
-    }
-    B->sweeps = k + 1;
-    B->relres = std::sqrt(B->host_red[2 + at]) / (sc * n0);
-    if (done || !(B->relres > rtol)) break;
+    int j = 0;   // the first sweep that reached the tolerance (as the device decided), or the last one
+    while (j < at && nr[j] > hs.limit) ++j;
+    B->plan = j + 1;
+    B->sweeps = j == at ? k + 1 : j + 1;
+    B->relres = std::sqrt(nr[j]) / (hs.scale * n0);
+    if (!(nr[j] > hs.limit)) break;
   }
   return cudaGetLastError();
 }
@@ -820,7 +820,7 @@ int box_create(fep3m_ctx* c, int nb, bool neumann, const double* Hw) {
   al((void**)&B->tab, tab.size() * sizeof(df));
   if (neumann) al((void**)&B->sface, (size_t)6 * nb * nb * 16 * sizeof(double));
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? FEP3M_ENOMEM : FEP3M_ECUDA;
-  if (cudaMallocHost(&B->host_red, (NORMS + 2) * sizeof(double)) != cudaSuccess) return FEP3M_ENOMEM;
+  if (cudaMallocHost(&B->host_red, (NORMS + 3) * sizeof(double)) != cudaSuccess) return FEP3M_ENOMEM;
   cudaMemset(B->counter, 0, sizeof(unsigned int));
   if ((e = box_apply_setup(c->st)) != cudaSuccess) return FEP3M_ECUDA;
   cudaMemset(B->g, 0, box_data_size(c) * sizeof(double));

@@ -241,10 +241,19 @@ struct BoxBand {
   double wn[3];         // node integrals by node type t (t = 0: a vertex shared by two elements)
   double wend;          // the node integral of the first and last node
 };
+// A box's or order-q refinement's state on the device: the residuals' power-of-two
+// scale into FP32 and its inverse, and the sum of squares of a scaled residual that
+// reaches the tolerance.  A sweep that reaches it sets inv to zero: the corrections
+// of sweeps already queued behind it then leave the iterate as it is, so that the
+// solution does not depend on how many sweeps were queued before the norms were read
+struct RefineState {
+  float scale, inv;
+  double limit;
+};
 // one residual r = b - K x on the open mesh (box_apply, mesh.cu): x and b in
 // FP64 or float pairs; r64: the FP64 residual of every node; else r receives
-// scale times it at the solved nodes (Ns per axis from index off), packed, in
-// FP32, and norm the sum of its squares
+// the state's scale times it at the solved nodes (Ns per axis from index off),
+// packed, in FP32, and norm the sum of its squares (checked against the limit)
 struct BoxApply {
   int N = 0, Ns = 0, off = 0;
   bool pairs = false;
@@ -252,7 +261,7 @@ struct BoxApply {
   const void* b = nullptr;
   float* r = nullptr;
   double* r64 = nullptr;
-  const float* scale = nullptr;   // device
+  RefineState* state = nullptr;   // device
   double* partials = nullptr;     // box_apply_blocks(N)
   unsigned int* counter = nullptr;
   double* norm = nullptr;

@@ -2,6 +2,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "common.cuh"
+
 namespace fep3m {
 
 __device__ __forceinline__ double block_sum256(double a, double* sh /* 8 */) {   // in thread 0
@@ -40,13 +42,16 @@ __device__ __forceinline__ bool grid_sum256(double acc, unsigned nblocks, unsign
 }
 
 // The power of two 2^-k with 2^k near the RMS sqrt(sum / n), and its inverse,
-// into scale[0], scale[1]: what a residual is scaled by into FP32
-__device__ __forceinline__ void rms_scale(double sum, double n, float* scale) {
+// into the state: what a residual is scaled by into FP32, and the sum of
+// squares of a scaled residual of rtol times the first one's norm
+__device__ __forceinline__ void refine_begin(double sum, double n, double rtol, RefineState* st) {
   const double rms = sqrt(sum / n);
   int k = rms > 0.0 && isfinite(rms) ? ilogb(rms) : 0;
   k = max(-100, min(100, k));
-  scale[0] = (float)ldexp(1.0, -k);
-  scale[1] = (float)ldexp(1.0, k);
+  st->scale = (float)ldexp(1.0, -k);
+  st->inv = (float)ldexp(1.0, k);
+  const double f = rtol * ldexp(1.0, -k);
+  st->limit = f * f * sum;
 }
 
 }  // namespace fep3m

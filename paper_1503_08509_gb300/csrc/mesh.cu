@@ -365,7 +365,7 @@ constexpr int SC_DERIVED = 16, SC_DERIVED_F = 32;
 enum { SD_ALPHA = 0, SD_BETA = 1, SD_MEAN = 2, SD_SCALE = 3, SD_INVSCALE = 4, SD_MEANLO = 5 };
 // what the last block derives from the total t (written next to it, so that
 // the consumers read one ready scalar instead of recomputing it per node)
-enum { POST_NONE = 0, POST_ALPHA = 1, POST_BETA = 2, POST_MEAN = 3, POST_SCALE = 4 };
+enum { POST_NONE = 0, POST_ALPHA = 1, POST_BETA = 2, POST_MEAN = 3, POST_SCALE = 4, POST_STOP = 5 };
 
 // Deterministic block-then-grid sum (blockDim.x == 256): the block's total
 // (in thread 0) goes to partials[bid]; the last block to finish adds the
@@ -395,6 +395,11 @@ __device__ void block_total_finish(double total, unsigned bid, unsigned nblocks,
   for (int k = 0; k < 8; ++k) t += sh[k];
   *out = t;
   *counter = 0u;
+  if (post == POST_STOP) {   // scal: a box's RefineState (NaN ends too)
+    RefineState* st = reinterpret_cast<RefineState*>(scal);
+    if (!(t > st->limit)) st->inv = 0.f;
+    return;
+  }
   double* dd = scal + SC_DERIVED;
   float* df = (float*)(scal + SC_DERIVED_F);
   if (post == POST_ALPHA) {          // alpha = (r.z) / (p.q), t = p.q
@@ -523,10 +528,10 @@ struct ApplyDot {
   double* wout = nullptr;
   double invW = 0.0;
   // box: the solved nodes (Ns per axis from index off) that the packed FP32
-  // residual and its sum take, their scale, or (out64) the FP64 residual of
-  // every node instead
+  // residual and its sum take, the refinement's state (scale; POST_STOP), or
+  // (out64) the FP64 residual of every node instead
   int Ns = 0, off = 0;
-  const float* bscale = nullptr;
+  RefineState* state = nullptr;
   double* out64 = nullptr;
 };
 
@@ -756,7 +761,7 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
   }
   const int tid = threadIdx.x;
   float rs = 0.0f;   // power-of-two scale of the refinement residual (FP64, double-float)
-  if constexpr (BOX) rs = dt.bscale ? *dt.bscale : 1.f;
+  if constexpr (BOX) rs = dt.state ? dt.state->scale : 1.f;
   else if constexpr (!std::is_same<T, float>::value) rs = reinterpret_cast<const float*>(scal + SC_DERIVED_F)[SD_SCALE];
   float ris = 0.0f;  // F32IN, EPI_CHECK: 1 / s
   if constexpr (F32IN || EPI == EPI_CHECK) ris = reinterpret_cast<const float*>(scal + SC_DERIVED_F)[SD_INVSCALE];
@@ -1008,7 +1013,7 @@ __global__ void __launch_bounds__(AT, sizeof(T) == 4 ? 3 : 2)
         }
       } else {
         block_sum_finish_df(dfv{facc, 0.f}, bid, nbv, dt.partials + (size_t)vi * nbv, dt.counter + vi,
-                            dt.out + 64 * vi, dt.post, 0.0, scal);
+                            dt.out + 64 * vi, dt.post, 0.0, BOX ? reinterpret_cast<double*>(dt.state) : scal);
       }
     } else
       block_sum_finish(dacc, bid, nbv, dt.partials + (size_t)vi * nbv, dt.counter + vi, dt.out + 64 * vi, dt.post,
@@ -3594,10 +3599,10 @@ cudaError_t box_apply_setup(const Stencils& st) {
   return apply_set_smem();
 }
 cudaError_t box_apply(const BoxApply& a, cudaStream_t s) {
-  ApplyDot dt = {a.partials, a.counter, a.norm, POST_NONE};
+  ApplyDot dt = {a.partials, a.counter, a.norm, POST_STOP};
   dt.Ns = a.Ns;
   dt.off = a.off;
-  dt.bscale = a.scale;
+  dt.state = a.state;
   dt.out64 = a.r64;
   const dim3 g = box_apply_grid(a.N);
   const int steps = box_apply_steps(a.N);

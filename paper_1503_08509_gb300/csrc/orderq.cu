@@ -165,11 +165,12 @@ __global__ void __launch_bounds__(OT) k_oq_sum(int64_t len, int Np, OQParams prm
 }
 
 // out = in - s w3 (the load less its uniform background), s = *sum / n^3, with
-// sum out^2 into *norm and the residuals' power-of-two scale
+// sum out^2 into *norm and the refinement's state
 __global__ void __launch_bounds__(OT) k_oq_project(int Np, OQParams prm, const double* __restrict__ sum, double inv,
                                                    const double* __restrict__ in, double* __restrict__ out,
                                                    double* __restrict__ partial, unsigned int* __restrict__ counter,
-                                                   double* __restrict__ norm, float* __restrict__ scale) {
+                                                   double* __restrict__ norm, double rtol,
+                                                   RefineState* __restrict__ st) {
   const int64_t len = (int64_t)Np * Np * Np;
   const double m = *sum * inv;
   double acc = 0.0;
@@ -181,7 +182,7 @@ __global__ void __launch_bounds__(OT) k_oq_project(int Np, OQParams prm, const d
   double t;
   if (grid_sum256(acc, gridDim.x, blockIdx.x, partial, counter, t)) {
     *norm = t;
-    rms_scale(t, (double)len, scale);
+    refine_begin(t, (double)len, rtol, st);
   }
 }
 // v -= *sum / n^3 (the mean)
@@ -202,7 +203,7 @@ template <int AXIS>
 __global__ void __launch_bounds__(OT) k_oq_band(int Np, OQParams prm, const double* __restrict__ in,
                                                 const double* __restrict__ in2, double* __restrict__ o1,
                                                 double* __restrict__ o2, const double* __restrict__ pb,
-                                                const float* __restrict__ scale, float* __restrict__ r32,
+                                                RefineState* state, float* __restrict__ r32,
                                                 double* __restrict__ partial, unsigned int* __restrict__ counter,
                                                 double* __restrict__ norm) {
   const int64_t g = blockIdx.x * (int64_t)OT + threadIdx.x, len = (int64_t)Np * Np * Np;
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(OT) k_oq_band(int Np, OQParams prm, const doub
       }
     }
     if (AXIS == 0) {
-      const float r = (float)((pb[g] - s1) * (double)scale[0]);
+      const float r = (float)((pb[g] - s1) * (double)state->scale);
       r32[g] = r;
       sq = (double)r * (double)r;
     } else {
@@ -241,19 +242,23 @@ __global__ void __launch_bounds__(OT) k_oq_band(int Np, OQParams prm, const doub
   }
   if (AXIS == 0) {
     double total;
-    if (grid_sum256(sq, gridDim.x, blockIdx.x, partial, counter, total)) *norm = total;
+    if (grid_sum256(sq, gridDim.x, blockIdx.x, partial, counter, total)) {
+      *norm = total;
+      if (total <= state->limit) state->inv = 0.f;
+    }
   }
 }
 
-__global__ void k_oq_round(int64_t n, const double* __restrict__ in, const float* __restrict__ scale,
+__global__ void k_oq_round(int64_t n, const double* __restrict__ in, const RefineState* __restrict__ st,
                            float* __restrict__ out) {
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (g < n) out[g] = (float)(in[g] * (double)scale[0]);
+  if (g < n) out[g] = (float)(in[g] * (double)st->scale);
 }
-__global__ void k_oq_add(int64_t n, const float* __restrict__ x, const float* __restrict__ scale,
+__global__ void k_oq_add(int64_t n, const float* __restrict__ x, const RefineState* __restrict__ st,
                          double* __restrict__ phi, int first) {
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (g < n) phi[g] = (first ? 0.0 : phi[g]) + (double)(x[g] * scale[1]);   // the scale is a power of two
+  const float inv = st->inv;   // a power of two, or zero: an earlier sweep reached the tolerance
+  if (inv != 0.f && g < n) phi[g] = (first ? 0.0 : phi[g]) + (double)(x[g] * inv);
 }
 
 // ------------------------------------------------------------ screen field
@@ -557,9 +562,9 @@ __global__ void __launch_bounds__(OT) k_oq_eval(int64_t N, int n, OQParams prm, 
 
 // ---------------------------------------------------------------- host side
 // o->red: partials of the sums from OQ_PART on (one per block), before them the
-// sums' results: the scale, then the norms of the right-hand side and of each sweep's residual
+// sums' results: the refinement's state, then the norms of the right-hand side and of each sweep's residual
 // (the sweeps past OQ_NORMS share the last)
-constexpr int OQ_SUM = 0, OQ_SCALE = 1, OQ_NORM = 2, OQ_PART = 34, OQ_NORMS = OQ_PART - OQ_NORM - 1;
+constexpr int OQ_SUM = 0, OQ_STATE = 2, OQ_NORM = 4, OQ_PART = 36, OQ_NORMS = OQ_PART - OQ_NORM - 1;
 inline int sum_blocks(int64_t len) { return (int)std::min<int64_t>(1024, std::max<int64_t>(1, len / (OT * 4))); }
 
 void oq_sum(OrderQ* o, int64_t len, int weighted, const double* v, cudaStream_t s) {
@@ -570,45 +575,45 @@ void oq_sum(OrderQ* o, int64_t len, int weighted, const double* v, cudaStream_t 
 // K phi = pb (pb neutral, with its norm and scale: oq_project), int phi = 0:
 // iterative refinement around the FP32 fast-diagonalisation solve.  The norms
 // stay on the device and are read once after as many sweeps as the last solve
-// took (and after each further one)
-cudaError_t oq_solve(fep3m_ctx* ctx, OrderQ* o, double rtol, int max_sweeps) {
+// took (and after each further one); sweeps past the first that reached the
+// tolerance change nothing (RefineState)
+cudaError_t oq_solve(fep3m_ctx* ctx, OrderQ* o, int max_sweeps) {
   const int n = ctx->n, Np = o->Np;
   const int64_t len = (int64_t)Np * Np * Np;
   cudaStream_t s = ctx->stream;
-  const float* scale = (const float*)(o->red + OQ_SCALE);
+  RefineState* st = (RefineState*)(o->red + OQ_STATE);
   double *part = o->red + OQ_PART, *norm = o->red + OQ_NORM;
   o->sweeps = 0;
   o->relres = 0.0;
-  FEP3M_CL k_oq_round<<<gsz(len), OT, 0, s>>>(len, o->pb, scale, o->r32);
+  FEP3M_CL k_oq_round<<<gsz(len), OT, 0, s>>>(len, o->pb, st, o->r32);
   const int read = std::max(1, std::min(o->plan, std::min(max_sweeps, OQ_NORMS)));
   for (int k = 0; k < max_sweeps; ++k) {
     const int at = std::min(k, OQ_NORMS - 1);
     cudaError_t e = fdm_apply(o->fdm, o->r32, o->x32, o->w1, o->w2, s);
     if (e != cudaSuccess) return e;
-    FEP3M_CL k_oq_add<<<gsz(len), OT, 0, s>>>(len, o->x32, scale, o->phi, k == 0);
+    FEP3M_CL k_oq_add<<<gsz(len), OT, 0, s>>>(len, o->x32, st, o->phi, k == 0);
     double *a = o->t[0], *b = o->t[1], *c = o->t[2], *f = o->t[3];
     FEP3M_CL k_oq_band<2><<<gsz(len), OT, 0, s>>>(Np, o->prm, o->phi, nullptr, a, b, nullptr, nullptr, nullptr,
                                                   nullptr, nullptr, nullptr);
     FEP3M_CL k_oq_band<1><<<gsz(len), OT, 0, s>>>(Np, o->prm, a, b, c, f, nullptr, nullptr, nullptr, nullptr, nullptr,
                                                   nullptr);
-    FEP3M_CL k_oq_band<0><<<gsz(len), OT, 0, s>>>(Np, o->prm, c, f, nullptr, nullptr, o->pb, scale, o->r32, part,
+    FEP3M_CL k_oq_band<0><<<gsz(len), OT, 0, s>>>(Np, o->prm, c, f, nullptr, nullptr, o->pb, st, o->r32, part,
                                                   o->counter, norm + 1 + at);
     if (k + 1 < read) continue;
-    cudaMemcpyAsync(o->host_red, o->red + OQ_SCALE, (at + 3) * sizeof(double), cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(o->host_red, o->red + OQ_STATE, (at + 4) * sizeof(double), cudaMemcpyDeviceToHost, s);
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-    const double nb = std::sqrt(o->host_red[1]), sc = *(const float*)o->host_red;
+    const RefineState& hs = *(const RefineState*)o->host_red;
+    const double nb = std::sqrt(o->host_red[2]), *nr = o->host_red + 3;
     if (!(nb > 0.0)) {
       cudaMemsetAsync(o->phi, 0, len * sizeof(double), s);
       return cudaGetLastError();
     }
-    bool done = false;
-    for (int j = 0; j <= at && !done; ++j) {   // the sweeps that were needed: the next solve's plan
-      done = std::sqrt(o->host_red[2 + j]) / (sc * nb) <= rtol;
-      o->plan = j + 1;
-    }
-    o->sweeps = k + 1;
-    o->relres = std::sqrt(o->host_red[2 + at]) / (sc * nb);
-    if (done || o->relres <= rtol) break;
+    int j = 0;   // the first sweep that reached the tolerance (as the device decided), or the last one
+    while (j < at && !(nr[j] <= hs.limit)) ++j;
+    o->plan = j + 1;
+    o->sweeps = j == at ? k + 1 : j + 1;
+    o->relres = std::sqrt(nr[j]) / (hs.scale * nb);
+    if (nr[j] <= hs.limit) break;
   }
   // int phi = 0: remove the node-integral weighted mean the FP32 corrections leave
   oq_sum(o, len, 1, o->phi, s);
@@ -731,7 +736,7 @@ int orderq_create(fep3m_ctx* c) {
   al((void**)&o->red, (OQ_PART + std::max<int64_t>(1024, gsz(np3))) * sizeof(double));
   al((void**)&o->counter, sizeof(unsigned int));
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? FEP3M_ENOMEM : FEP3M_ECUDA;
-  if (cudaMallocHost(&o->host_red, (OQ_NORMS + 2) * sizeof(double)) != cudaSuccess) return FEP3M_ENOMEM;
+  if (cudaMallocHost(&o->host_red, (OQ_NORMS + 3) * sizeof(double)) != cudaSuccess) return FEP3M_ENOMEM;
   cudaMemcpy(o->H, tab.data(), tab.size() * sizeof(df), cudaMemcpyHostToDevice);
   cudaMemset(o->counter, 0, sizeof(unsigned int));
   e = fdm_setup(o->fdm, o->Np, h.lam, h.V, 1, !(c->cfg.flags & FEP3M_CUDA_CORES));
@@ -755,6 +760,10 @@ void orderq_destroy(fep3m_ctx* c) {
   c->oq = nullptr;
 }
 
+static double oq_rtol(const fep3m_ctx* c) {
+  return c->cfg.mg_rtol > 0 ? c->cfg.mg_rtol : (c->precision == FEP3M_FP64 ? 1e-13 : 1e-10);
+}
+
 // the load vector less its background, from b (device), with its norm and scale
 static void oq_project(fep3m_ctx* c, OrderQ* o, cudaStream_t s) {
   const int n = c->n, Np = o->Np;
@@ -762,11 +771,7 @@ static void oq_project(fep3m_ctx* c, OrderQ* o, cudaStream_t s) {
   oq_sum(o, len, 0, o->b, s);
   FEP3M_CL k_oq_project<<<sum_blocks(len), OT, 0, s>>>(Np, o->prm, o->red + OQ_SUM, 1.0 / ((double)n * n * n), o->b,
                                                        o->pb, o->red + OQ_PART, o->counter, o->red + OQ_NORM,
-                                                       (float*)(o->red + OQ_SCALE));
-}
-
-static double oq_rtol(const fep3m_ctx* c) {
-  return c->cfg.mg_rtol > 0 ? c->cfg.mg_rtol : (c->precision == FEP3M_FP64 ? 1e-13 : 1e-10);
+                                                       oq_rtol(c), (RefineState*)(o->red + OQ_STATE));
 }
 
 int orderq_compute(fep3m_ctx* c, double* phi_dev, double* U_dev) {
@@ -792,7 +797,7 @@ int orderq_compute(fep3m_ctx* c, double* phi_dev, double* U_dev) {
     FEP3M_CL k_oq_load<<<gsz(np3), OT, 0, s>>>(n, 2, Np, Np, Np, o->prm, o->t[1], o->b, 4.0 * M_PI);
   }
   oq_project(c, o, s);
-  cudaError_t e = oq_solve(c, o, oq_rtol(c), c->cfg.mg_max_cycles > 0 ? c->cfg.mg_max_cycles : 10);
+  cudaError_t e = oq_solve(c, o, c->cfg.mg_max_cycles > 0 ? c->cfg.mg_max_cycles : 10);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? FEP3M_ENOMEM : FEP3M_ECUDA;
   const ParityBlocks pb = parity_blocks(o->U, P1);
   for (int64_t e0 = 0; e0 < ne; e0 += o->piece) {
@@ -828,7 +833,7 @@ int orderq_solve(fep3m_ctx* c, const double* b_dev, double* phi_dev) {
   cudaStream_t s = c->stream;
   cudaMemcpyAsync(o->b, b_dev, np3 * sizeof(double), cudaMemcpyDeviceToDevice, s);
   oq_project(c, o, s);
-  cudaError_t e = oq_solve(c, o, oq_rtol(c), c->cfg.mg_max_cycles > 0 ? c->cfg.mg_max_cycles : 10);
+  cudaError_t e = oq_solve(c, o, c->cfg.mg_max_cycles > 0 ? c->cfg.mg_max_cycles : 10);
   if (e != cudaSuccess) return FEP3M_ECUDA;
   cudaMemcpyAsync(phi_dev, o->phi, np3 * sizeof(double), cudaMemcpyDeviceToDevice, s);
   return o->relres <= 10 * oq_rtol(c) ? FEP3M_OK : FEP3M_ENOCONV;

@@ -1,6 +1,9 @@
 """The refinement of the boxes and of the order-q mesh: its cap on the sweeps is the
-caller's (also past the residual norms kept on the device).
+caller's (also past the residual norms kept on the device), and a solution does not depend
+on what the engine solved before (the sweeps queued before the norms are read follow the
+last solve).
 """
+import numpy as np
 import pytest
 
 from paper_1503_08509_gb300 import workloads
@@ -40,3 +43,34 @@ def test_cap_on_the_sweeps(api, precision, kind, cap):
         assert out["status"] != 0 and st["refine_steps"] == cap
         assert 0.0 < st["mg_rel_residual"] < (1e-3 if cap == 1 else 1e-11)
     eng.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("kind", KINDS)
+def test_no_memory_of_earlier_solves(api, precision, kind):
+    """An easy right-hand side (alternating: the largest eigenvalues, no level to remove) after a
+    harder one and on a fresh engine, and the harder one after the easy one: the same bits."""
+    import torch
+
+    def easy(eng):
+        m = round(eng.nodes ** (1 / 3))
+        s = (-1.0) ** np.arange(m)
+        b = torch.tensor((s[:, None, None] * s[:, None] * s).ravel(), device="cuda")
+        b += 0.1 * torch.randn(eng.nodes, dtype=torch.float64, device="cuda",
+                               generator=torch.Generator("cuda").manual_seed(2))
+        phi, st = eng.solve_mesh(b), eng.stats()
+        return phi, st["refine_steps"], st["mg_rel_residual"]
+
+    def hard(eng):
+        phi, st = eng.compute(forces=False)["phi"].clone(), eng.stats()
+        return phi, st["refine_steps"], st["mg_rel_residual"]
+
+    for first, second in ((easy, hard), (hard, easy)):
+        eng = engine(api, precision, kind)
+        want = second(eng)
+        eng.close()
+        eng = engine(api, precision, kind)
+        first(eng)
+        got = second(eng)
+        eng.close()
+        assert torch.equal(got[0], want[0]) and got[1:] == want[1:], (got[1:], want[1:])
