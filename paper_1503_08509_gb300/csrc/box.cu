@@ -661,18 +661,22 @@ void box_sum(Box* B, int mode, const double* v, double* dst, cudaStream_t s, dou
 // iterative refinement around the FP32 fast-diagonalisation solve, the
 // residuals scaled by one power of two near the first one's inverse RMS.  In
 // MIXED the residual is formed in double-float arithmetic (as the periodic
-// solver's; about 2e-14 relative) from a copy of the iterate as float pairs.
+// solver's) from a copy of the iterate as float pairs, down to tolerances of
+// BOX_PAIR_RTOL: the pairs' rounding leaves 1e-13 (8^3 elements) to 7e-13 (48^3)
+// of the Dirichlet residual and 6e-13 to 3e-12 of the Neumann one, FP64 2e-15 and
+// 2e-14 (8^3), so a tighter tolerance takes the FP64 residual.
 // The norms stay on the device: they are read once after as many sweeps as
 // the last solve took (and after each further one); sweeps past the first that
 // reached the tolerance change nothing (RefineState).  Sets B->sweeps and
 // B->relres (the residual relative to that of phi's starting values)
+constexpr double BOX_PAIR_RTOL = 1e-11;
 cudaError_t box_refine(fep3m_ctx* c, Box* B, const double* rhs, double* phi) {
   const int Ns = B->Ns, Nn = B->Nn;
   const int64_t len = (int64_t)Ns * Ns * Ns, nn3 = (int64_t)Nn * Nn * Nn;
   cudaStream_t s = c->stream;
   const double rtol = box_rtol(c);
   const int max_sweeps = c->cfg.mg_max_cycles > 0 ? c->cfg.mg_max_cycles : 10;
-  const bool mixed = c->precision == FEP3M_MIXED;
+  const bool mixed = c->precision == FEP3M_MIXED && rtol >= BOX_PAIR_RTOL;
   df* pairs = mixed ? (df*)c->phi_hl : nullptr;
   RefineState* st = (RefineState*)(B->red + RED_STATE);
   double* norm = B->red + RED_NORM;

@@ -1,5 +1,5 @@
 """The refinement of the boxes and of the order-q mesh: its cap on the sweeps is the
-caller's (also past the residual norms kept on the device), and a solution does not depend
+caller's (also past the residual norms kept on the device), a tight tolerance is met, and a solution does not depend
 on what the engine solved before (the sweeps queued before the norms are read follow the
 last solve).
 """
@@ -42,6 +42,17 @@ def test_cap_on_the_sweeps(api, precision, kind, cap):
         st = eng.stats()
         assert out["status"] != 0 and st["refine_steps"] == cap
         assert 0.0 < st["mg_rel_residual"] < (1e-3 if cap == 1 else 1e-11)
+    eng.close()
+
+
+@pytest.mark.parametrize("n_el", [8, 20])
+@pytest.mark.parametrize("kind", KINDS)
+def test_tight_tolerance(api, kind, n_el):
+    """Mixed contexts: residuals that FP64 arithmetic reaches (2e-15 to 2e-14 at 8^3, growing with
+    the mesh) and float pairs do not (1e-13 and more)."""
+    eng = engine(api, "mixed", kind, n_el, mg_rtol=5e-15 * (n_el / 8))
+    out = eng.compute(forces=False)
+    assert out["status"] == 0 and eng.stats()["mg_rel_residual"] <= 5e-14 * (n_el / 8)
     eng.close()
 
 
