@@ -664,19 +664,21 @@ void box_sum(Box* B, int mode, const double* v, double* dst, cudaStream_t s, dou
 // solver's) from a copy of the iterate as float pairs, down to tolerances of
 // BOX_PAIR_RTOL: the pairs' rounding leaves 1e-13 (8^3 elements) to 7e-13 (48^3)
 // of the Dirichlet residual and 6e-13 to 3e-12 of the Neumann one, FP64 2e-15 and
-// 2e-14 (8^3), so a tighter tolerance takes the FP64 residual.
+// 2e-14 (8^3), so a tighter tolerance takes the FP64 residual.  So do values a
+// pair cannot hold (an infinite boundary value, beside a charge on its node, is
+// NaN as a pair): a NaN norm is looked at again in FP64, which tells an infinite
+// residual from none.
 // The norms stay on the device: they are read once after as many sweeps as
 // the last solve took (and after each further one); sweeps past the first that
 // reached the tolerance change nothing (RefineState).  Sets B->sweeps and
 // B->relres (the residual relative to that of phi's starting values)
 constexpr double BOX_PAIR_RTOL = 1e-11;
-cudaError_t box_refine(fep3m_ctx* c, Box* B, const double* rhs, double* phi) {
+cudaError_t box_refine(fep3m_ctx* c, Box* B, const double* rhs, double* phi, bool mixed) {
   const int Ns = B->Ns, Nn = B->Nn;
   const int64_t len = (int64_t)Ns * Ns * Ns, nn3 = (int64_t)Nn * Nn * Nn;
   cudaStream_t s = c->stream;
   const double rtol = box_rtol(c);
   const int max_sweeps = c->cfg.mg_max_cycles > 0 ? c->cfg.mg_max_cycles : 10;
-  const bool mixed = c->precision == FEP3M_MIXED && rtol >= BOX_PAIR_RTOL;
   df* pairs = mixed ? (df*)c->phi_hl : nullptr;
   RefineState* st = (RefineState*)(B->red + RED_STATE);
   double* norm = B->red + RED_NORM;
@@ -719,10 +721,9 @@ cudaError_t box_refine(fep3m_ctx* c, Box* B, const double* rhs, double* phi) {
     const RefineState& hs = *(const RefineState*)B->host_red;
     const double n0 = std::sqrt(B->host_red[2]), *nr = B->host_red + 3;
     if (!(n0 > 0.0)) {
-      // a zero (or, for non-finite data, NaN) residual: nothing to solve.  MIXED: an infinite
-      // boundary value is NaN in the float pairs, reported as not converged, as in FP64
-      if (mixed && !(n0 == 0.0)) B->relres = n0;
+      // a zero (or, for non-finite data, NaN) residual: nothing to solve
       FEP3M_CL k_box_clear<<<gsz(len), BT, 0, s>>>(Ns, Nn, B->off, phi);
+      if (mixed && n0 != 0.0) return box_refine(c, B, rhs, phi, false);
       return cudaGetLastError();
     }
     int j = 0;   // the first sweep that reached the tolerance (as the device decided), or the last one
@@ -733,6 +734,9 @@ cudaError_t box_refine(fep3m_ctx* c, Box* B, const double* rhs, double* phi) {
     if (!(nr[j] > hs.limit)) break;
   }
   return cudaGetLastError();
+}
+cudaError_t box_refine(fep3m_ctx* c, Box* B, const double* rhs, double* phi) {
+  return box_refine(c, B, rhs, phi, c->precision == FEP3M_MIXED && box_rtol(c) >= BOX_PAIR_RTOL);
 }
 
 }  // namespace
