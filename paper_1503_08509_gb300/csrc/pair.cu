@@ -1817,6 +1817,9 @@ __device__ __forceinline__ void acc_merge(dfacc& a, const dfacc& b) {
   a.h = s;
 }
 __device__ __forceinline__ double acc_value(const dfacc& a) { return (double)a.h + (double)a.l; }
+// the FP64 path's: three floats
+__device__ __forceinline__ void acc_merge(tf& a, tf b) { tf_add(a, b); }
+__device__ __forceinline__ double acc_value(tf a) { return df_value(a); }
 
 // The FP64 path's D by parity (see k_screen64): with W+-(j) = W(j) +- W(3 - j)
 // along each axis, D+-(i) = sum_j E+-(i, j) W+-(j) and D(i) = D+(i) + D-(i),
@@ -1927,9 +1930,11 @@ __global__ void __launch_bounds__(PT, 2) k_adj64(int64_t ne, int n_sr, int z0, i
 // (av_ring rows of 2 n_sr + 2 values in flight), the weight sums a row ahead in
 // registers.  FP32 path (H0 set): D holds the contraction with the
 // node-0-relative table, and each term gains H(o, 0) Wsum(v + o)
-// (pair_adjoint_table).  FP64 path: D is the whole contraction, as pairs.  Terms
-// and sums in double-float arithmetic (19 operations a term in the FP32 path, of
-// 36 instructions).  Bound by instruction issue, at 2/3 of its rate.  10^6
+// (pair_adjoint_table); terms and sums in double-float arithmetic (19 operations
+// a term, of 36 instructions).  FP64 path: D is the whole contraction, as pairs,
+// summed in three floats: the up to (2 n_sr)^3 terms of a class are of one sign
+// where the weights are, and the low word of a pair's sum would round each of
+// them at 2^-48 of the running sum.  Bound by instruction issue, at 2/3 of its rate.  10^6
 // charges on 128^3: 3484 us with one warp per 32 vertices and row of offsets and 27
 // class sums in shared memory, 2301 with a row ahead in registers and AVZ = 8, 1458
 // now; 262 144 on 64^3: 439, 285 and 195 us.
@@ -1951,7 +1956,8 @@ template <class T, int NSR, int AVZ>
 struct AdjVertexSmem {
   static constexpr int NOFF = 2 * NSR + 2;
   T ring[av_ring<NSR>][NOFF][PT];
-  dfacc part[AVZ][8][PT / AVZ];
+  typedef typename std::conditional<sizeof(T) == 4, dfacc, tf>::type Acc;   // (tf: three floats)
+  Acc part[AVZ][8][PT / AVZ];
   float2 h0[sizeof(T) == 4 ? NOFF * NOFF * NOFF : 1];
   int live[PT / AVZ];
 };
@@ -1961,6 +1967,7 @@ __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int
                                                       const float2* __restrict__ wsum, double* __restrict__ A) {
   constexpr int KEEP = NSR + 1, NOFF = 2 * NSR + 2, PLANE = NOFF * NOFF, AVV = PT / AVZ, AV_RING = av_ring<NSR>;
   constexpr bool REL = sizeof(T) == 4;   // T: float, or df (FP64)
+  typedef typename AdjVertexSmem<T, NSR, AVZ>::Acc Acc;
   extern __shared__ __align__(16) unsigned char av_smem[];
   AdjVertexSmem<T, NSR, AVZ>& S = *reinterpret_cast<AdjVertexSmem<T, NSR, AVZ>*>(av_smem);
   const int64_t ne = (int64_t)n * n * n;
@@ -1983,7 +1990,7 @@ __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int
   __syncthreads();
   const bool act = S.live[vl] != 0;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) S.part[zg][k][vl] = dfacc{0.f, 0.f};   // corner sums, k = kx + 2 ky + 4 kz
+  for (int k = 0; k < 8; ++k) S.part[zg][k][vl] = Acc{};   // corner sums, k = kx + 2 ky + 4 kz
   const int oz0 = z0 + zg;
   if (oz0 < z1 && __any_sync(0xffffffffu, act)) {
     int wx[NOFF];   // the elements' x coordinates vx + o - KEEP (n >= 2 n_sr + 1: one period at most)
@@ -2001,9 +2008,9 @@ __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int
       ez = ez >= n ? ez - n : ez;
       return n * n * ez;
     };
-    dfacc P[3][3];   // [class along y][class along x]: first, inner, last
+    Acc P[3][3];   // [class along y][class along x]: first, inner, last
 #pragma unroll
-    for (int i = 0; i < 9; ++i) P[i / 3][i % 3] = dfacc{0.f, 0.f};
+    for (int i = 0; i < 9; ++i) P[i / 3][i % 3] = Acc{};
     float2 w[REL ? 2 : 1][NOFF];   // the weight sums of the row being summed and of the next
     int eyd = ey0, eyw = ey0;      // element rows of the next fetch and the next load
     // row oy of plane oz of D into this thread's ring; called in order of the rows
@@ -2059,7 +2066,7 @@ __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int
             acc_add(P[cy][cx], p);
             acc_add(P[cy][cx], d[ox] + r);
           } else {
-            acc_merge(P[cy][cx], dfacc{d[ox].h, d[ox].l});
+            tf_add(P[cy][cx], d[ox]);
           }
         }
       }
@@ -2069,7 +2076,7 @@ __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int
 #pragma unroll
       for (int k = 0; k < 4; ++k) {   // corner (kx, ky): classes 0, 1 for 1, classes 1, 2 for 0
         const int x0 = k & 1 ? 0 : 1, y0 = k & 2 ? 0 : 1;
-        dfacc t = P[y0][x0];
+        Acc t = P[y0][x0];
         acc_merge(t, P[y0][x0 + 1]);
         acc_merge(t, P[y0 + 1][x0]);
         acc_merge(t, P[y0 + 1][x0 + 1]);
@@ -2077,7 +2084,7 @@ __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int
         if (oz != 0) acc_merge(S.part[zg][k][vl], t);
       }
 #pragma unroll
-      for (int i = 0; i < 9; ++i) P[i / 3][i % 3] = dfacc{0.f, 0.f};
+      for (int i = 0; i < 9; ++i) P[i / 3][i % 3] = Acc{};
     }
   }
   __syncthreads();
@@ -2085,7 +2092,7 @@ __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int
 #pragma unroll
   for (int t = 0; t < 8 / AVZ; ++t) {
     const int k = zg + AVZ * t, kx = k & 1, ky = (k >> 1) & 1, kz = k >> 2;
-    dfacc s = S.part[0][k][vl];
+    Acc s = S.part[0][k][vl];
 #pragma unroll
     for (int z = 1; z < AVZ; ++z) acc_merge(s, S.part[z][k][vl]);
     const int sx = vx - kx < 0 ? n - 1 : vx - kx, sy = vy - ky < 0 ? n - 1 : vy - ky, sz = vz - kz < 0 ? n - 1 : vz - kz;
