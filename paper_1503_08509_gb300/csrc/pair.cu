@@ -1431,7 +1431,10 @@ __global__ void __launch_bounds__(PT) k_pair_eval(int n, int Nm, float inv_h, co
 
 // The same in an FP64 context.  The screen field comes in its even and odd
 // parts (k_screen64); its nodal values are formed in shared memory, three
-// sums and differences each, and subtracted from the mesh potential.  Four
+// sums and differences each, and subtracted from the mesh potential.  They are held
+// relative to node 0's (G0): the shape functions sum to one and their gradients to
+// zero, so an element's level enters the potential alone and the rounding acts on
+// the variation only (charges of one sign give a level of hundreds).  Four
 // threads per target take the four z layers of nodes: each evaluates one shape
 // function and derivative per axis (shared by shuffles) and contracts its
 // layer along x, then y: about 400 FP64 operations per target where the terms
@@ -1453,6 +1456,7 @@ __global__ void __launch_bounds__(PT) k_pair_eval64(int n, int Nm, double inv_h,
                                                     double* __restrict__ E_s, double* __restrict__ phi_out) {
   typedef vec4<double>::type V4;
   __shared__ __align__(32) double G[BE * 64];
+  __shared__ double G0[BE];
   __shared__ int epre[BE + 1];
   __shared__ int wsum[PT / 32 + 1];
   const int nbx = (n + BX - 1) / BX, nby = (n + BY - 1) / BY;
@@ -1512,10 +1516,11 @@ __global__ void __launch_bounds__(PT) k_pair_eval64(int n, int Nm, double inv_h,
     const int gx = 3 * (E0x + l % BX) + m[0], gy = 3 * (E0y + (l / BX) % BY) + m[1], gz = 3 * (E0z + l / (BX * BY)) + m[2];
     val[k] = phi64[(gx >= Nm ? gx - Nm : gx) +
                    (int64_t)Nm * ((gy >= Nm ? gy - Nm : gy) + (int64_t)Nm * (gz >= Nm ? gz - Nm : gz))] - G[i];
+    if ((at[k] & 63) == 0) G0[l] = val[k];
   }
   __syncthreads();
 #pragma unroll
-  for (int k = 0; k < PER; ++k) G[at[k]] = val[k];
+  for (int k = 0; k < PER; ++k) G[at[k]] = val[k] - G0[at[k] >> 6];
   __syncthreads();
   const int q = tid & 3, lane0 = (tid & 31) & ~3;
   for (int tb = 0; tb < ntarget; tb += PT / 4) {
@@ -1568,7 +1573,7 @@ __global__ void __launch_bounds__(PT) k_pair_eval64(int n, int Nm, double inv_h,
     if (!valid) continue;
     // thread q writes sum q
     if (q == 0) {
-      const double phi = v4[0] * inv_h + phi_s[slot];
+      const double phi = (v4[0] + G0[l]) * inv_h + phi_s[slot];
       phi_s[slot] = phi;
       if (phi_out) phi_out[perm[slot]] = phi;
     } else if (GRAD) {
