@@ -540,6 +540,7 @@ int fep3m_create(const fep3m_config* cfg, void* stream, fep3m_ctx** out) {
     pair_adjoint_table(c->n_sr, Hw.data(), Hd.data(), H0.data());
   }
   if (c->precision == FEP3M_FP64) {
+    pair_mirror_table(c->n_sr, Hw.data());
     const int kh = c->n_sr + 1;
     std::vector<float> hp((size_t)2 * 64 * kh * kh * kh);
     pair_parity_table(c->n_sr, Hw.data(), hp.data());

@@ -482,7 +482,9 @@ void pair_adj_table(int n_sr, const double* Hw, uint16_t* out);
 // floats, 2 per offset)
 void pair_relative_table(int n_sr, const double* Hw, double* Hrel);
 void pair_adjoint_table(int n_sr, const double* Hw, double* Hd, float* H0);
-// the FP64 path's table by parity, as hi + lo floats (2 x 64 (n_sr + 1)^3)
+// the FP64 path's table, symmetric under reflection of each axis
+void pair_mirror_table(int n_sr, double* Hw);
+// the same by parity, as hi + lo floats (2 x 64 (n_sr + 1)^3)
 void pair_parity_table(int n_sr, const double* Hw, float* out);
 // energy_adjoint: also leave half the singular sums in psi_s / gpsi_s (the
 // singular adjoint of the energy's weights Q / 2)

@@ -2389,6 +2389,27 @@ void pair_adjoint_table(int n_sr, const double* Hw, double* Hd, float* H0) {
   }
 }
 
+// The table as the mean over its mirror images along each axis, H(noff - 1 - o, 3 - m) =
+// H(o, m), which agree to the rounding of the solve that made them.  The FP64 path's
+// contractions by parity are of this table, so whatever else the path forms from it (a
+// box's boundary values and fluxes) takes it too: what a screen adds at the boundary and
+// what it subtracts at a charge is then the same field.
+void pair_mirror_table(int n_sr, double* Hw) {
+  const int noff = 2 * n_sr + 2, no3 = noff * noff * noff;
+  for (int a = 0; a < 3; ++a) {
+    const int so = a == 0 ? 1 : (a == 1 ? noff : noff * noff), sm = a == 0 ? 1 : (a == 1 ? 4 : 16);
+    for (int o = 0; o < no3; ++o) {
+      const int oa = (o / so) % noff;
+      if (2 * oa >= noff) continue;   // with its image (noff is even)
+      for (int m = 0; m < 64; ++m) {
+        double &x = Hw[(size_t)o * 64 + m];
+        double &y = Hw[(size_t)(o + (noff - 1 - 2 * oa) * so) * 64 + m + (3 - 2 * ((m / sm) & 3)) * sm];
+        x = y = 0.5 * (x + y);
+      }
+    }
+  }
+}
+
 // the FP64 path's table by parity: HP[s][k][j], s = sx + 2 sy + 4 sz, k the offsets
 // 0 .. n_sr and j the nodes 0, 1 per axis (x fastest): the mean over the mirror
 // images (which agree to rounding) with the parities' signs, as float pairs
