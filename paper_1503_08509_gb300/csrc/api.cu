@@ -171,7 +171,7 @@ int deliver(fep3m_ctx* c, void* dst, const void* src, size_t bytes) {
   return FEP3M_OK;
 }
 
-// Device scalars (scal, 64 doubles): the charge sums at 32, U at 40, the pair
+// Device scalars (scal, 64 doubles): the adjoint weights' scale at kWeightScale, the charge sums at 32, U at 40, the pair
 // counts at 48, the integer flags (iflags) at kFlags.  One copy to pinned memory
 // brings the results of a call and its error flag; waits for the stream.
 constexpr int kFlags = 56;

@@ -320,6 +320,7 @@ struct fep3m_ctx {
   // particles
   int64_t N = 0, cap = 0;
   double q_scale = 1;            // power of two near the inverse mean |Q| of the charges last set
+  bool weights_given = false;    // the adjoint's weights have a part from the caller (k_weight_scale)
   bool have_particles = false, have_forward = false, have_grad = false;
   bool have_mesh = false;   // phi64 solves the mesh problem of these charges (fep3m_vjp)
   double* pos_in = nullptr;      // N*3 (staging for host inputs)
@@ -409,6 +410,7 @@ struct fep3m_ctx {
 #define FEP3M_PAIR_CHARGE_BYTES 48   // sizeof a charge of part_pairs
 
 namespace fep3m {
+constexpr int kWeightScale = 24;   // in fep3m_ctx::scal: the adjoint weights' scale and its inverse (FP64)
 // host setup (setup.cpp)
 // Raises a kernel's dynamic shared-memory limit to at least `bytes` on the
 // current device, calling the runtime only when the limit has to grow (the

@@ -1585,14 +1585,38 @@ __global__ void __launch_bounds__(PT) k_pair_eval64(int n, int Nm, double inv_h,
 
 // ----------------------------------------------------------------- adjoint
 __global__ void k_weights(int64_t N, double gU, const double* __restrict__ gphi, const int* __restrict__ perm,
-                          const double* __restrict__ Qs, double* __restrict__ w, float* __restrict__ w32) {
+                          const double* __restrict__ Qs, double* __restrict__ w, float* __restrict__ w32,
+                          double scale, double* __restrict__ ws) {
   int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (k >= N) return;
   const double v = 0.5 * gU * Qs[k] + (gphi ? gphi[perm[k]] : 0.0);
   w[k] = v;
   if (w32) w32[k] = (float)v;
+  if (k == 0 && scale > 0.0) {
+    ws[0] = scale;
+    ws[1] = 1.0 / scale;
+  }
 }
 
+// FP64: the power of two that takes the largest weight near 2^100, and its inverse, for
+// weights that only the device knows (fep3m_vjp's gphi).  The screen adjoint's float pairs
+// are of the scaled weights (the field they give is within 2^12 of them, n_sr <= 4), so that
+// their low words stay normal FP32 numbers whatever the weights' unit; non-finite weights
+// stay as they are.  One CTA: the weights are read once more, beside the mesh solve.
+__global__ void __launch_bounds__(1024) k_weight_scale(int64_t N, const double* __restrict__ w,
+                                                       double* __restrict__ ws) {
+  __shared__ int top[32];
+  int hi = 0;   // the largest exponent, by the high words
+  for (int64_t k = threadIdx.x; k < N; k += 1024) hi = max(hi, __double2hiint(w[k]) & 0x7fffffff);
+  for (int o = 16; o > 0; o >>= 1) hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = hi;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int i = 1; i < 32; ++i) hi = max(hi, top[i]);
+  const int e = (hi >> 20) - 1023, k = e == 1024 ? 0 : max(-900, min(900, 100 - e));
+  ws[0] = ldexp(1.0, k);
+  ws[1] = ldexp(1.0, -k);
+}
 
 // W[e][m] = sum_{t in e} w_t u_m(tau_t): the adjoint's point deposit, per
 // element.  wsum (FP32 path): sum_{t in e} w_t in FP64 as hi + lo floats, the
@@ -1832,8 +1856,8 @@ __device__ __forceinline__ double acc_value(tf a) { return df_value(a); }
 // 768 (n_sr = 3), in float pairs, and three sums and differences per value.  A
 // CTA takes 32 consecutive elements, one per lane; a warp forms the eight
 // parities of two offsets i at a time for them and writes their sixteen
-// mirrored values of D as pairs (rows of 32 consecutive elements).  HP: the
-// table by parity, [s][i][j].  Bound by FP32 issue; rock salt 32^3: 778 ->
+// mirrored values of D as pairs (rows of 32 consecutive elements), times the
+// weights' scale ws[0] (k_weight_scale).  HP: the table by parity, [s][i][j].  Bound by FP32 issue; rock salt 32^3: 778 ->
 // 143 us against the full product in pairs with D rounded to FP64.
 constexpr int AE = 32;
 static size_t adj64_smem(int n_sr) {
@@ -1841,7 +1865,8 @@ static size_t adj64_smem(int n_sr) {
   return (size_t)AE * 65 * sizeof(double) + (size_t)64 * AE * sizeof(df) + (size_t)kh * kh * kh * 64 * sizeof(df);
 }
 __global__ void __launch_bounds__(PT, 2) k_adj64(int64_t ne, int n_sr, int z0, int z1, const double* __restrict__ W,
-                                                 const df* __restrict__ HP, df* __restrict__ D) {
+                                                 const double* __restrict__ ws, const df* __restrict__ HP,
+                                                 df* __restrict__ D) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int kh = n_sr + 1, noff = 2 * kh, K = kh * kh * kh, plane = noff * noff;
   double(*Wd)[65] = reinterpret_cast<double(*)[65]>(smem_raw);                                      // [AE]
@@ -1869,6 +1894,7 @@ __global__ void __launch_bounds__(PT, 2) k_adj64(int64_t ne, int n_sr, int z0, i
     }
   }
   __syncthreads();
+  const double scale = ws[0];
   for (int i = tid; i < AE * 64; i += PT) {
     const int e = i & 31, b = i >> 5, s = b >> 3, j = b & 7;
     int node = 0;
@@ -1876,7 +1902,7 @@ __global__ void __launch_bounds__(PT, 2) k_adj64(int64_t ne, int n_sr, int z0, i
       const int ja = (j >> a) & 1;
       node = node * 4 + ((s >> a) & 1 ? 3 - ja : ja);
     }
-    Ws[b][e] = df_split(Wd[e][node]);
+    Ws[b][e] = df_split(Wd[e][node] * scale);
   }
   __syncthreads();
   for (int i0 = 2 * warp; i0 < K; i0 += 2 * (PT / 32)) {
@@ -1969,7 +1995,8 @@ struct AdjVertexSmem {
 template <class T, int NSR, int AVZ>
 __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int first, const int* __restrict__ count,
                                                       const T* __restrict__ D, int64_t ld, const float2* __restrict__ H0,
-                                                      const float2* __restrict__ wsum, double* __restrict__ A) {
+                                                      const float2* __restrict__ wsum, const double* __restrict__ ws,
+                                                      double* __restrict__ A) {
   constexpr int KEEP = NSR + 1, NOFF = 2 * NSR + 2, PLANE = NOFF * NOFF, AVV = PT / AVZ, AV_RING = av_ring<NSR>;
   constexpr bool REL = sizeof(T) == 4;   // T: float, or df (FP64)
   typedef typename AdjVertexSmem<T, NSR, AVZ>::Acc Acc;
@@ -2102,7 +2129,8 @@ __global__ void __launch_bounds__(PT, 2) k_adj_vertex(int n, int z0, int z1, int
     for (int z = 1; z < AVZ; ++z) acc_merge(s, S.part[z][k][vl]);
     const int sx = vx - kx < 0 ? n - 1 : vx - kx, sy = vy - ky < 0 ? n - 1 : vy - ky, sz = vz - kz < 0 ? n - 1 : vz - kz;
     double* dst = A + (sx + (int64_t)n * (sy + (int64_t)n * sz)) * 8 + k;
-    *dst = first ? acc_value(s) : *dst + acc_value(s);
+    const double a = REL ? acc_value(s) : acc_value(s) * ws[1];
+    *dst = first ? a : *dst + a;
   }
 }
 
@@ -2550,7 +2578,7 @@ static void launch_adj_vertex_z(fep3m_ctx* c, int z0, int z1, const T* D, int64_
   constexpr int AVV = PT / AVZ;
   FEP3M_CL k_adj_vertex<T, NSR, AVZ><<<(unsigned)((ne + AVV - 1) / AVV), PT, smem, s>>>(
       c->n, z0, z1, z0 == 0, c->count, D, ld, rel ? (const float2*)c->H0df : nullptr,
-      rel ? (const float2*)c->Wsum : nullptr, A);
+      rel ? (const float2*)c->Wsum : nullptr, c->scal + kWeightScale, A);
 }
 template <class T, int NSR>
 static void launch_adj_vertex(fep3m_ctx* c, int z0, int z1, const T* D, int64_t ld, double* A, cudaStream_t s) {
@@ -2605,7 +2633,8 @@ static cudaError_t screen_adjoint(fep3m_ctx* c, const T* W, double* A) {
       const size_t smem = adj64_smem(c->n_sr);
       (void)smem_limit((const void*)k_adj64, smem);   // a failure shows as the launch's error
       FEP3M_CL k_adj64<<<(unsigned)((ne + AE - 1) / AE), PT, smem, s>>>(ne, c->n_sr, z0, z1, (const double*)W,
-                                                                       (const df*)c->HP, (df*)c->D_adj);
+                                                                       c->scal + kWeightScale, (const df*)c->HP,
+                                                                       (df*)c->D_adj);
     } else {
       dim3 grid((unsigned)((ne + GT - 1) / GT), (unsigned)((no + GT - 1) / GT));
       FEP3M_CL k_adj_gemm<<<grid, PT, 0, s>>>(ne, o0, no, W, c->Ha64, (float*)c->D_adj);
@@ -2626,7 +2655,12 @@ static cudaError_t screen_adjoint(fep3m_ctx* c, const T* W, double* A) {
 cudaError_t adjoint_pre(fep3m_ctx* c, double gU, const double* gphi, cudaStream_t s) {
   const int n = c->n;
   const int64_t ne = (int64_t)n * n * n, N = c->N;
-  FEP3M_CL k_weights<<<gsz(N), PT, 0, s>>>(N, gU, gphi, c->perm, c->Q_s, c->w_s, c->w_s32);
+  // FP64: the scale of the screen adjoint's pairs, for weights gU Q / 2 from the charges' (their
+  // largest is below 2^31 times their mean), else from the weights (adjoint_sweeps)
+  c->weights_given = gphi != nullptr;
+  const double scale = c->weights_given || gU == 0.0 ? 0.0 : std::ldexp(c->q_scale, 64 - std::ilogb(gU));
+  FEP3M_CL k_weights<<<gsz(N), PT, 0, s>>>(N, gU, gphi, c->perm, c->Q_s, c->w_s, c->w_s32, scale,
+                                           c->scal + kWeightScale);
   const int per = PT;   // elements per CTA: 32 per warp
   if (c->precision == FEP3M_MIXED) {
     FEP3M_CL k_elem_deposit<float><<<gsz(ne, per), PT, 0, s>>>(ne, c->start, c->count, (const float4*)c->part, c->w_s,
@@ -2655,6 +2689,7 @@ cudaError_t adjoint_sweeps(fep3m_ctx* c, cudaStream_t s, bool singular) {
       FEP3M_CL k_pair_adj_warp<float, true><<<(unsigned)((N + 7) / 8), PT, 0, s>>>(N, n, c->n_sr, (float)c->h, c->start,
                                                          (const float4*)c->part, c->ecoord, c->w_s, c->psi_s, c->gpsi_s);
   } else {
+    if (c->weights_given) FEP3M_CL k_weight_scale<<<1, 1024, 0, s>>>(N, c->w_s, c->scal + kWeightScale);
     e = screen_adjoint<double>(c, (const double*)c->W_el, (double*)c->A_el);
     if (e == cudaSuccess && singular)
       FEP3M_CL k_pair_adj_warp<double, true><<<(unsigned)((N + 7) / 8), PT, 0, s>>>(N, n, c->n_sr, c->h, c->start,
