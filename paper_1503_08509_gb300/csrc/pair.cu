@@ -1627,70 +1627,136 @@ __global__ void __launch_bounds__(1024) k_weight_scale(int64_t N, const double* 
 // shuffles, two nodes per lane (with one thread per element and node each
 // element waited for three dependent loads: 262 144 charges on 64^3, 146 ->
 // 41 us, 10^6 on 128^3, 845 -> 145 us; FP64 rock salt 32^3, where every thread also evaluated twelve
-// shape functions, 208 -> 34 us).
+// shape functions, 208 -> 34 us).  That takes some 290 cycles a charge in series,
+// so rows of 32 elements with more than `run` charges are dealt by elements to the
+// CTA's warps, which put the shape functions of 32 charges, one per lane, into shared
+// memory and sum over them there (4096 charges in one row of 32^3 elements: 617 us in
+// one warp, now 29; 20 000 in a blob of 16^3: 1165 -> 90).  A CTA takes eight rows.
+//
+// Dealing costs a row two dependent loads per element, but on a small mesh the rows in
+// series leave the GPU idle: there (deposit_dealt) a CTA takes one row and deals it
+// whatever it holds.  FP32, 0.2 / 1 / 3 charges per element, in series and dealt (us):
+// 12^3 8.7 / 17 / 34 and 6.4 / 7.6 / 8.5; 28^3 9.3 / 18 / 37 and 17 / 18 / 19; 32^3 9.9 /
+// 20 / 35 and 25 / 26 / 28; 48^3 12 / 24 / 48 and 65 / 69 / 72: about 8 + 0.31 run against
+// 4 + 0.021 rows.  FP64: 12^3 11 / 32 / 82 and 12 / 19 / 22; 28^3 14 / 36 / 88 and 24 / 64 /
+// 92; 48^3 23 / 85 / 233 and 77 / 255 / 397.
+constexpr int DEP_RUN = 160;   // (64^3, FP32: 4 charges per element 119 us in series, 165 dealt)
+static bool deposit_dealt(int64_t ne, int64_t N, bool f32) {
+  const int64_t rows = (ne + 31) / 32, run = N * 32 / ne;
+  return rows < 200 + (f32 ? 15 : 5) * run || run > DEP_RUN;
+}
+// order-3 shape function i at t as q3_values forms it: k (t - r0) (t - r1) (t - r2)
 template <class T>
-__global__ void __launch_bounds__(PT) k_elem_deposit(int64_t ne, const int* __restrict__ start,
+__device__ __forceinline__ T q3_value(T t, int i) {
+  const T k = i == 0 ? T(-4.5) : (i == 1 ? T(13.5) : (i == 2 ? T(-13.5) : T(4.5)));
+  const T r0 = i == 0 ? T(1) / T(3) : T(0), r1 = i < 2 ? T(2) / T(3) : T(1) / T(3), r2 = i == 3 ? T(2) / T(3) : T(1);
+  return k * (t - r0) * (t - r1) * (t - r2);
+}
+template <class T>
+__global__ void __launch_bounds__(PT) k_elem_deposit(int64_t ne, int nrows, int run, const int* __restrict__ start,
                                                      const int* __restrict__ count,
                                                      const typename vec4<T>::type* __restrict__ part,
                                                      const double* __restrict__ w, const T* __restrict__ wT,
                                                      T* __restrict__ W, float2* __restrict__ wsum) {
-  const int lane = threadIdx.x & 31;
-  const int64_t e0 = (blockIdx.x * (int64_t)(PT / 32) + (threadIdx.x >> 5)) * 32;
-  if (e0 >= ne) return;
-  const int nel = (int)min((int64_t)32, ne - e0);
-  const int s0 = lane < nel ? start[e0 + lane] : 0, cnt = lane < nel ? count[e0 + lane] : 0;
-  if (wsum && lane < nel) {
-    double ws = 0.0;
-    for (int j = s0; j < s0 + cnt; ++j) ws += w[j];
-    const float hi = (float)ws;
-    wsum[e0 + lane] = make_float2(hi, (float)(ws - (double)hi));
-  }
+  __shared__ int crowded[PT / 32];
+  __shared__ T shape[PT / 32][12][33];   // of a warp's 32 charges: x (times the weight), y, z
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t cta0 = blockIdx.x * (int64_t)nrows * 32, e0 = cta0 + 32 * warp;
   // this lane's nodes: m = lane and lane + 32 (the same x and y index, z index 2 on)
   const int mx = lane & 3, my = (lane >> 2) & 3, mz = lane >> 4;
-  // order-3 shape function i at t as q3_values forms it: k (t - r0) (t - r1) (t - r2)
-  auto one = [](T t, int i) -> T {
-    const T k = i == 0 ? T(-4.5) : (i == 1 ? T(13.5) : (i == 2 ? T(-13.5) : T(4.5)));
-    const T r0 = i == 0 ? T(1) / T(3) : T(0), r1 = i < 2 ? T(2) / T(3) : T(1) / T(3), r2 = i == 3 ? T(2) / T(3) : T(1);
-    return k * (t - r0) * (t - r1) * (t - r2);
-  };
-  const int first = __shfl_sync(0xffffffffu, s0, 0), end = __shfl_sync(0xffffffffu, s0 + cnt, nel - 1);
-  int base = first;                 // the charges base .. base + 31 are held, one per lane
-  typename vec4<T>::type pc;
+  typename vec4<T>::type pc;   // charges held, one per lane
   T wc = T(0);
   pc.x = pc.y = pc.z = pc.w = T(0);
-  auto hold = [&]() {
-    if (base + lane < end) {
-      pc = part[base + lane];
-      wc = wT[base + lane];
-    }
-  };
-  hold();
-  for (int i = 0; i < nel; ++i) {
-    const int s = __shfl_sync(0xffffffffu, s0, i), c = __shfl_sync(0xffffffffu, cnt, i);
-    T a0 = T(0), a1 = T(0);
-    for (int j = s; j < s + c; ++j) {
-      if (j >= base + 32) {
-        base = j;
-        hold();
+  bool crowd = false;
+  if (warp < nrows && e0 < ne) {
+    const int nel = (int)min((int64_t)32, ne - e0);
+    const int s0 = lane < nel ? start[e0 + lane] : 0, cnt = lane < nel ? count[e0 + lane] : 0;
+    const int first = __shfl_sync(0xffffffffu, s0, 0), end = __shfl_sync(0xffffffffu, s0 + cnt, nel - 1);
+    crowd = end - first > run;
+    if (!crowd) {
+      if (wsum && lane < nel) {
+        double ws = 0.0;
+        for (int j = s0; j < s0 + cnt; ++j) ws += w[j];
+        const float hi = (float)ws;
+        wsum[e0 + lane] = make_float2(hi, (float)(ws - (double)hi));
       }
-      const int src = j - base;
-      const T x = __shfl_sync(0xffffffffu, pc.x, src), y = __shfl_sync(0xffffffffu, pc.y, src),
-              z = __shfl_sync(0xffffffffu, pc.z, src), wj = __shfl_sync(0xffffffffu, wc, src);
-      if constexpr (sizeof(T) == 4) {
-        const T xy = wj * one(x, mx) * one(y, my);
-        a0 += xy * one(z, mz);
-        a1 += xy * one(z, mz + 2);
-      } else {
-        // one shape function per lane (12 of them), then shuffles
-        const T u = one(lane < 4 ? x : (lane < 8 ? y : z), lane & 3);
-        const T xy = wj * __shfl_sync(0xffffffffu, u, mx) * __shfl_sync(0xffffffffu, u, 4 + my);
-        const T z0 = __shfl_sync(0xffffffffu, u, 8 + mz), z1 = __shfl_sync(0xffffffffu, u, 10 + mz);
-        a0 = fma(xy, z0, a0);
-        a1 = fma(xy, z1, a1);
+      int base = first;                 // the charges base .. base + 31 are held
+      auto hold = [&]() {
+        if (base + lane < end) {
+          pc = part[base + lane];
+          wc = wT[base + lane];
+        }
+      };
+      hold();
+      for (int i = 0; i < nel; ++i) {
+        const int s = __shfl_sync(0xffffffffu, s0, i), c = __shfl_sync(0xffffffffu, cnt, i);
+        T a0 = T(0), a1 = T(0);
+        for (int j = s; j < s + c; ++j) {
+          if (j >= base + 32) {
+            base = j;
+            hold();
+          }
+          const int src = j - base;
+          const T x = __shfl_sync(0xffffffffu, pc.x, src), y = __shfl_sync(0xffffffffu, pc.y, src),
+                  z = __shfl_sync(0xffffffffu, pc.z, src), wj = __shfl_sync(0xffffffffu, wc, src);
+          if constexpr (sizeof(T) == 4) {
+            const T xy = wj * q3_value(x, mx) * q3_value(y, my);
+            a0 += xy * q3_value(z, mz);
+            a1 += xy * q3_value(z, mz + 2);
+          } else {
+            // one shape function per lane (12 of them), then shuffles
+            const T u = q3_value(lane < 4 ? x : (lane < 8 ? y : z), lane & 3);
+            const T xy = wj * __shfl_sync(0xffffffffu, u, mx) * __shfl_sync(0xffffffffu, u, 4 + my);
+            const T z0 = __shfl_sync(0xffffffffu, u, 8 + mz), z1 = __shfl_sync(0xffffffffu, u, 10 + mz);
+            a0 = fma(xy, z0, a0);
+            a1 = fma(xy, z1, a1);
+          }
+        }
+        W[(e0 + i) * 64 + lane] = a0;
+        W[(e0 + i) * 64 + lane + 32] = a1;
       }
     }
-    W[(e0 + i) * 64 + lane] = a0;
-    W[(e0 + i) * 64 + lane + 32] = a1;
+  }
+  if (lane == 0) crowded[warp] = crowd;
+  if (!__syncthreads_or(crowd)) return;
+  T(*u)[33] = shape[warp];
+  for (int r = 0; r < nrows; ++r) {
+    if (!crowded[r]) continue;
+    const int64_t e1 = min(cta0 + 32 * r + 32, ne);
+    for (int64_t e = cta0 + 32 * r + warp; e < e1; e += PT / 32) {
+      const int s = start[e], c = count[e];
+      T a0 = T(0), a1 = T(0);
+      double ws = 0.0;
+      for (int base = 0; base < c; base += 32) {
+        const int m = min(32, c - base);
+        if (lane < m) {
+          pc = part[s + base + lane];
+          wc = wT[s + base + lane];
+          if (wsum) ws += w[s + base + lane];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            u[i][lane] = wc * q3_value(pc.x, i);
+            u[4 + i][lane] = q3_value(pc.y, i);
+            u[8 + i][lane] = q3_value(pc.z, i);
+          }
+        }
+        __syncwarp();
+#pragma unroll 4
+        for (int k = 0; k < m; ++k) {
+          const T xy = u[mx][k] * u[4 + my][k];
+          a0 = fma(xy, u[8 + mz][k], a0);
+          a1 = fma(xy, u[10 + mz][k], a1);
+        }
+        __syncwarp();
+      }
+      W[e * 64 + lane] = a0;
+      W[e * 64 + lane + 32] = a1;
+      if (wsum) {
+        warp_sum(ws);
+        const float hi = (float)ws;
+        if (lane == 0) wsum[e] = make_float2(hi, (float)(ws - (double)hi));
+      }
+    }
   }
 }
 
@@ -2661,13 +2727,14 @@ cudaError_t adjoint_pre(fep3m_ctx* c, double gU, const double* gphi, cudaStream_
   const double scale = c->weights_given || gU == 0.0 ? 0.0 : std::ldexp(c->q_scale, 64 - std::ilogb(gU));
   FEP3M_CL k_weights<<<gsz(N), PT, 0, s>>>(N, gU, gphi, c->perm, c->Q_s, c->w_s, c->w_s32, scale,
                                            c->scal + kWeightScale);
-  const int per = PT;   // elements per CTA: 32 per warp
+  const bool dealt = deposit_dealt(ne, N, c->precision == FEP3M_MIXED);
+  const int nrows = dealt ? 1 : PT / 32, run = dealt ? 0 : DEP_RUN, per = 32 * nrows;   // rows of 32 elements per CTA
   if (c->precision == FEP3M_MIXED) {
-    FEP3M_CL k_elem_deposit<float><<<gsz(ne, per), PT, 0, s>>>(ne, c->start, c->count, (const float4*)c->part, c->w_s,
+    FEP3M_CL k_elem_deposit<float><<<gsz(ne, per), PT, 0, s>>>(ne, nrows, run, c->start, c->count, (const float4*)c->part, c->w_s,
                                                                c->w_s32, (float*)c->W_el, (float2*)c->Wsum);
     FEP3M_CL k_node_assemble<float><<<dim3(3 * n, 3 * n), PT, 0, s>>>(n, (const float*)c->W_el, c->g64);
   } else {
-    FEP3M_CL k_elem_deposit<double><<<gsz(ne, per), PT, 0, s>>>(ne, c->start, c->count, (const vec4<double>::type*)c->part,
+    FEP3M_CL k_elem_deposit<double><<<gsz(ne, per), PT, 0, s>>>(ne, nrows, run, c->start, c->count, (const vec4<double>::type*)c->part,
                                                                 c->w_s, c->w_s, (double*)c->W_el, nullptr);
     FEP3M_CL k_node_assemble<double><<<dim3(3 * n, 3 * n), PT, 0, s>>>(n, (const double*)c->W_el, c->g64);
   }
