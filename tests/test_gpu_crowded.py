@@ -61,3 +61,40 @@ def test_deposit_on_a_small_mesh(api, groups):
     [(250, 12, 300)]])
 def test_deposit_of_crowded_rows(api, groups):
     check(api, 22, *charges(22, groups, len(groups) + groups[0][2]))
+
+
+@pytest.mark.parametrize("forces", [False, True])
+@pytest.mark.parametrize("counts", [(1600,), (1537, 1545), (1700, 5, 11, 12, 13)])
+def test_singular_sums_from_global_memory(api, counts, forces):
+    """An element over the staging area: its bricks' blocks are read from global memory, element
+    by element, eight (potentials: twelve) charges at a time.  Against the FP64 path, whose
+    singular sums have a kernel of their own.
+
+    Tolerance, per charge: the FP32 coordinates' rounding, 2^-24 of an element along each axis of
+    a difference, through 1 / r (and 1 / r^2); 64 roundings of the sum of the terms' sizes, for
+    their arithmetic and the sums; and the mixed path's 1e-6 (forces 1e-5) of the RMS.  A charge
+    left out or taken twice is a hundred times that."""
+    import torch
+    elements, n = [73, 74, 0, 511, 200], 8   # neighbours, the corners (rows that wrap)
+    groups = [(elements[i], 1, c) for i, c in enumerate(counts)] + [(0, 512, 60)]
+    pos, Q = charges(n, groups, len(counts))
+    p, q = torch.tensor(pos, device="cuda"), torch.tensor(Q, device="cuda")
+    out = {}
+    for precision in ("fp64", "mixed"):
+        eng = api.FEP3M(1.0, n, precision=precision)
+        eng.set_particles(p, q)
+        assert eng.stats()["max_per_element"] > 1536
+        out[precision] = eng.compute(forces=forces)
+        eng.close()
+    r = p[:, None] - p
+    r = (r - r.round()).norm(dim=2)
+    r.fill_diagonal_(float("inf"))
+    eps, shift = 2.0 ** -24, 3 ** 0.5 * 2.0 ** -24 / n
+    terms = [(q.abs() / r ** k).sum(1) for k in (1, 2, 3)]
+    ref = out["fp64"]["phi"]
+    tol = shift * terms[1] + 64 * eps * terms[0] + 1e-6 * ref.square().mean().sqrt()
+    assert bool(((out["mixed"]["phi"] - ref).abs() < tol).all())
+    if forces:
+        ref = out["fp64"]["forces"]
+        tol = q.abs() * (2 * shift * terms[2] + 64 * eps * terms[1]) + 1e-5 * ref.square().mean().sqrt()
+        assert bool(((out["mixed"]["forces"] - ref).abs() < tol[:, None]).all())
