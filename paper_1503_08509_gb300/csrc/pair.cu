@@ -2756,7 +2756,9 @@ cudaError_t adjoint_pre(fep3m_ctx* c, double gU, const double* gphi, cudaStream_
   // FP64: the scale of the screen adjoint's pairs, for weights gU Q / 2 from the charges' (their
   // largest is below 2^31 times their mean), else from the weights (adjoint_sweeps)
   c->weights_given = gphi != nullptr;
-  const double scale = c->weights_given || gU == 0.0 ? 0.0 : std::ldexp(c->q_scale, 64 - std::ilogb(gU));
+  double scale = 0.0;   // (none given)
+  if (!c->weights_given)
+    scale = gU == 0.0 ? 1.0 : std::ldexp(1.0, std::max(-900, std::min(900, 64 - std::ilogb(gU) + std::ilogb(c->q_scale))));
   FEP3M_CL k_weights<<<gsz(N), PT, 0, s>>>(N, gU, gphi, c->perm, c->Q_s, c->w_s, c->w_s32, scale,
                                            c->scal + kWeightScale);
   const bool dealt = deposit_dealt(ne, N, c->precision == FEP3M_MIXED);

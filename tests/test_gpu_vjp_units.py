@@ -56,6 +56,17 @@ def test_vjp_is_linear(api, n_el, n_sr, N, gU, gphi):
     eng.close()
 
 
+@pytest.mark.parametrize("gU", [0.0, 1e-300, 5e-324])
+def test_vanishing_weights_on_a_fresh_engine(api, gU):
+    """Weights of zero, and ones that the scale's exponent cannot take to its target: finite."""
+    import torch
+    eng, p, q = setup(api, 9, 2, 400)
+    eng.set_particles(p, q)
+    for t in eng.vjp(gU, None):
+        assert bool(torch.isfinite(t).all()) and (gU > 0.0 or float(t.abs().max()) == 0.0)
+    eng.close()
+
+
 @pytest.mark.parametrize("n_el,n_sr,N", [(9, 2, 400), (10, 4, 300)])
 def test_forces_scale_with_the_charges(api, n_el, n_sr, N):
     eng, p, q = setup(api, n_el, n_sr, N)
