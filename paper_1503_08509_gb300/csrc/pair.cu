@@ -381,22 +381,20 @@ __global__ void __launch_bounds__(PT) k_singular64(int64_t N, int n, int n_sr, d
 // offsets reach, then BX slots of corner-1-only sums (offset -(n_sr+1),
 // vertex e + n_sr + 1) and BX of corner-0-only sums (offset n_sr, vertex
 // e - n_sr).  A(e, o) is then the single value R[beta(o) + lambda(e)].
-constexpr int STAGE_CAP = 1536;   // halo charges staged in shared memory (T = float)
+constexpr int STAGE_CAP = 1536;   // halo charges staged in shared memory
 
 // CUDA-core layout (TC = false): region 1 holds R first, then the staged
 // charges; A and H chunks follow.  Tensor-core layout (TC = true): 48 KB of
-// operand tiles (1 KB aligned; the staged charges reuse them after the
-// contraction), then R.  Both end with the index tables.
-template <class T, bool TC = false>
+// operand tiles (1 KB aligned), then R, then the staged charges.  Both end with
+// the index tables.
+template <bool TC>
 struct Pair3Smem {
   static constexpr int NT = TC ? PTC : PT;
   // bytes per R and chunk-operand entry: one float (tensor cores) or a hi + lo
-  // float pair (the double-float CUDA-core contraction, both precisions)
+  // float pair (the double-float CUDA-core contraction)
   static constexpr int ES = TC ? 4 : 8;
   __host__ __device__ static int SW(int n_sr) { return 3 * BX + 2 * n_sr - 1; }
   __host__ __device__ static int HW(int n_sr) { return BX + 2 * n_sr; }
-  // charges that can be staged: STAGE_CAP floats-worth of float4 (half as many double4)
-  __host__ __device__ static int cap() { return STAGE_CAP * 4 / (int)sizeof(T); }
   // R's strides: rows 4 modulo 16 entries and (tensor cores) planes 16 modulo 32, so that the 4 x 4
   // x 2 elements a warp reads fall on 32 different banks
   __host__ __device__ static int RS(int n_sr) { return TC ? SW(n_sr) + (20 - SW(n_sr) % 16) % 16 : SW(n_sr); }
@@ -409,7 +407,7 @@ struct Pair3Smem {
   }
   __host__ __device__ static size_t region1(int n_sr) {
     const size_t r = rbytes(n_sr);
-    const size_t stg = (size_t)cap() * sizeof(typename vec4<T>::type);
+    const size_t stg = (size_t)STAGE_CAP * sizeof(float4);
     return r > stg ? r : stg;
   }
   __host__ __device__ static size_t ints(int n_sr) {
@@ -421,11 +419,11 @@ struct Pair3Smem {
   static constexpr size_t TILES = 6 * 8192;   // three bf16 pieces of A (64 x 64) and of B (64 x 64)
   // tensor cores: the staged charges in a region of their own (staged while the contraction runs)
   __host__ __device__ static size_t stgbytes() {
-    return (size_t)cap() * sizeof(typename vec4<T>::type) + ((size_t)cap() + 15) / 16 * 16;
+    return (size_t)STAGE_CAP * sizeof(float4) + ((size_t)STAGE_CAP + 15) / 16 * 16;
   }
   static size_t bytes(int n_sr) {
     if (TC) return 1024 + TILES + rbytes(n_sr) + stgbytes() + ints(n_sr) * sizeof(int) + 16;
-    return region1(n_sr) + 2 * (size_t)OCH * 64 * ES + ints(n_sr) * sizeof(int) + (size_t)cap();
+    return region1(n_sr) + 2 * (size_t)OCH * 64 * ES + ints(n_sr) * sizeof(int) + (size_t)STAGE_CAP;
   }
 };
 
@@ -520,10 +518,9 @@ __device__ __forceinline__ int halo_gid(int i, int n, int HW, const int* __restr
 // the charges are staged in shared memory in that order (with each charge's
 // halo x index) when they all fit (cap).  By SG threads (gt, barrier id).
 // Returns the HaloMode.
-template <class T>
 __device__ int stage_halo(int gt, int id, int n, int HW, const int* __restrict__ we, const int* __restrict__ start,
-                          const int* __restrict__ count, const typename vec4<T>::type* __restrict__ part, int cap,
-                          typename vec4<T>::type* stg, unsigned char* sxb, int* hs, int* flag, int* wsum) {
+                          const int* __restrict__ count, const float4* __restrict__ part, int cap, float4* stg,
+                          unsigned char* sxb, int* hs, int* flag, int* wsum) {
   const int nh = HW * HW * HW;
   const int per = (nh + SG - 1) / SG, i0 = gt * per;
   int cnt[8], gid[8];   // per <= 7 for n_sr <= 4 (nh <= 1728)
@@ -637,15 +634,14 @@ __device__ __noinline__ float4 global_target(int q, int tpt, int n, int n_sr, co
 // phi_s / E_s, element units, scaled at the last tile).  Global (an element
 // over the staging area): the same rows read from global memory, element by
 // element.  Writes phi_s and E_s (and half of them to psi, gpsi).
-template <class T, bool GRAD>
-__device__ void singular_targets(int gt, int id, int mode, int n, int n_sr, T h, int E0x, int E0y, int E0z, int HW,
+template <bool GRAD>
+__device__ void singular_targets(int gt, int id, int mode, int n, int n_sr, float h, int E0x, int E0y, int E0z, int HW,
                                  int ntarget, const int* __restrict__ epre, const int* __restrict__ hs,
                                  const int* __restrict__ rtab, const int* __restrict__ we,
-                                 typename vec4<T>::type* stg, unsigned char* sxb, int cap,
-                                 const int* __restrict__ start, const int* __restrict__ count,
-                                 const typename vec4<T>::type* __restrict__ part, double* __restrict__ phi_s,
-                                 double* __restrict__ E_s, double* __restrict__ psi, double* __restrict__ gpsi) {
-  typedef typename vec4<T>::type V4;
+                                 float4* stg, unsigned char* sxb, int cap, const int* __restrict__ start,
+                                 const int* __restrict__ count, const float4* __restrict__ part,
+                                 double* __restrict__ phi_s, double* __restrict__ E_s, double* __restrict__ psi,
+                                 double* __restrict__ gpsi) {
   constexpr int TPT = 4;
   const int nb = 2 * n_sr + 1, nrow = nb * nb, nh = HW * HW * HW;
   const int q = gt & (TPT - 1);
@@ -677,7 +673,7 @@ __device__ void singular_targets(int gt, int id, int mode, int n, int n_sr, T h,
     for (int tb = 0; tb < ntarget; tb += SG / TPT) {
       const int k = tb + gt / TPT;
       const bool valid = k < ntarget;
-      T v4[4] = {T(0), T(0), T(0), T(0)};
+      float v4[4] = {0.f, 0.f, 0.f, 0.f};
       int slot = 0;
       if (valid) {
         int lo = 0, hi2 = BE;                 // element of target k: epre[l] <= k < epre[l + 1]
@@ -693,13 +689,13 @@ __device__ void singular_targets(int gt, int id, int mode, int n, int n_sr, T h,
         slot = start[ex + (int64_t)n * (ey + (int64_t)n * ez)] + kk;
         const int base = lx + HW * (ly + HW * lz);          // halo index of block offset (-n_sr, -n_sr, -n_sr)
         const int cx = lx + n_sr;                           // the target's halo x index
-        Acc<T> ps, fx, fy, fz;
+        Acc<float> ps, fx, fy, fz;
         if (mode != HALO_GLOBAL) {
           const int selfh = base + n_sr * (1 + HW + HW * HW);   // the target's own halo element
           const int self = hs[selfh] + kk - c0;
-          const V4 pt = mode == HALO_STAGED ? stg[self] : part[slot];
-          const T cxf = T(cx);
-          T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0), ddy = T(0), ddz = T(0);
+          const float4 pt = mode == HALO_STAGED ? stg[self] : part[slot];
+          const float cxf = (float)cx;
+          float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f, ddy = 0.f, ddz = 0.f;
           int r = q, j = 0, je = 0;
           for (;;) {
             if (j >= je) {
@@ -709,31 +705,31 @@ __device__ void singular_targets(int gt, int id, int mode, int n, int n_sr, T h,
                 fy.add(s2);
                 fz.add(s3);
               }
-              s0 = s1 = s2 = s3 = T(0);
+              s0 = s1 = s2 = s3 = 0.f;
               if (r >= nrow) break;
               const int rt = rtab[r];
               const int h0 = base + (rt & 0xFFFF);
               const int ha = h0 > ta ? h0 : ta, hb = h0 + nb < tz ? h0 + nb : tz;   // the row's part in the tile
               j = ha < hb ? hs[ha] - c0 : 0;
               je = ha < hb ? hs[hb] - c0 : 0;
-              ddy = T(((rt >> 16) & 0xFF) - n_sr);
-              ddz = T((rt >> 24) - n_sr);
+              ddy = (float)(((rt >> 16) & 0xFF) - n_sr);
+              ddz = (float)((rt >> 24) - n_sr);
               r += TPT;
               continue;
             }
             const bool two = j + 1 < je;
             const int jb = two ? j + 1 : j;
-            const V4 pa = stg[j], pb = stg[jb];
+            const float4 pa = stg[j], pb = stg[jb];
             // element units (1/h applied once per target, in FP64), fused r^2 and sums
-            const T rxa = (T(sxb[j]) - cxf) + (pa.x - pt.x), rya = ddy + (pa.y - pt.y), rza = ddz + (pa.z - pt.z);
-            const T rxb = (T(sxb[jb]) - cxf) + (pb.x - pt.x), ryb = ddy + (pb.y - pt.y), rzb = ddz + (pb.z - pt.z);
-            const T ira = j == self ? T(0) : rsq<T>(fmaw(rxa, rxa, fmaw(rya, rya, rza * rza)));
-            const T irb = (!two || jb == self) ? T(0) : rsq<T>(fmaw(rxb, rxb, fmaw(ryb, ryb, rzb * rzb)));
-            const T qa = pa.w * ira, qb = pb.w * irb;
+            const float rxa = ((float)sxb[j] - cxf) + (pa.x - pt.x), rya = ddy + (pa.y - pt.y), rza = ddz + (pa.z - pt.z);
+            const float rxb = ((float)sxb[jb] - cxf) + (pb.x - pt.x), ryb = ddy + (pb.y - pt.y), rzb = ddz + (pb.z - pt.z);
+            const float ira = j == self ? 0.f : rsq<float>(fmaw(rxa, rxa, fmaw(rya, rya, rza * rza)));
+            const float irb = (!two || jb == self) ? 0.f : rsq<float>(fmaw(rxb, rxb, fmaw(ryb, ryb, rzb * rzb)));
+            const float qa = pa.w * ira, qb = pb.w * irb;
             s0 += qa;
             s0 += qb;
             if (GRAD) {
-              const T f3a = qa * (ira * ira), f3b = qb * (irb * irb);
+              const float f3a = qa * (ira * ira), f3b = qb * (irb * irb);
               s1 = fmaw(f3a, rxa, s1);
               s2 = fmaw(f3a, rya, s2);
               s3 = fmaw(f3a, rza, s3);
@@ -802,47 +798,46 @@ __device__ void singular_targets(int gt, int id, int mode, int n, int n_sr, T h,
 // of every target charge in the brick (written to phi_s and E_s; with psi,
 // half of them to psi and gpsi as well: the singular adjoint for the weights
 // Q / 2 of the energy, whose kernel 1/r is symmetric).  TC: the
-// contraction on the tensor cores (FP32 only; Hb holds the table's bf16
+// contraction on the tensor cores (Hb holds the table's bf16
 // pieces in the tiles' layout, err receives a bounded wait that gave up),
 // 512 threads and eight per target; otherwise CUDA cores, 256 threads and
 // four per target.
-template <class T, bool GRAD, bool TC>
-__global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_sr, T h, const int* __restrict__ start,
+template <bool GRAD, bool TC>
+__global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_sr, float h, const int* __restrict__ start,
                                                              const int* __restrict__ count,
-                                                             const typename vec4<T>::type* __restrict__ part,
-                                                             const T* __restrict__ Vc,
+                                                             const float4* __restrict__ part,
+                                                             const float* __restrict__ Vc,
                                                              const uint4* __restrict__ Hb, const float2* __restrict__ H0,
-                                                             const float2* __restrict__ Hdf, T* __restrict__ Gscr, double* __restrict__ phi_s,
-                                                             double* __restrict__ E_s, double* __restrict__ psi,
-                                                             double* __restrict__ gpsi, int* __restrict__ err) {
-  static_assert(!TC || sizeof(T) == 4, "the tensor-core contraction is the FP32 path's");
+                                                             const float2* __restrict__ Hdf, float* __restrict__ Gscr,
+                                                             double* __restrict__ phi_s, double* __restrict__ E_s,
+                                                             double* __restrict__ psi, double* __restrict__ gpsi,
+                                                             int* __restrict__ err) {
   static_assert(PT == SG && PTC == 2 * SG, "the short-range sums take the whole CUDA-core CTA, half the tensor-core one");
   constexpr int NT = TC ? PTC : PT;
-  typedef typename vec4<T>::type V4;
-  typedef Pair3Smem<T, TC> SM;
+  typedef Pair3Smem<TC> SM;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nbx = (n + BX - 1) / BX, nby = (n + BY - 1) / BY;
   const int E0x = (blockIdx.x % nbx) * BX, E0y = ((blockIdx.x / nbx) % nby) * BY, E0z = (blockIdx.x / (nbx * nby)) * BZ;
   const int keep = n_sr + 1, noff = 2 * n_sr + 2, no3 = noff * noff * noff;
   const int SW = 3 * BX + 2 * n_sr - 1, SF = BX + 2 * n_sr - 1, HW = BX + 2 * n_sr;
   const int nb = 2 * n_sr + 1, nrow = nb * nb;
-  T *R, *A_c = nullptr, *H_c = nullptr;
-  V4* stg;
+  float *R, *A_c = nullptr, *H_c = nullptr;
+  float4* stg;
   unsigned char* tiles = nullptr;
   int* hs;                                                // halo element prefix, HW^3 + 1
-  unsigned char* sxb;                                     // cap(): halo x index of each staged charge
+  unsigned char* sxb;                                     // STAGE_CAP: halo x index of each staged charge
   if (TC) {
     tiles = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // swizzle atoms on 1 KB
-    R = (T*)(tiles + SM::TILES);
-    stg = (V4*)((unsigned char*)R + SM::rbytes(n_sr));
-    sxb = (unsigned char*)(stg + SM::cap());
+    R = (float*)(tiles + SM::TILES);
+    stg = (float4*)((unsigned char*)R + SM::rbytes(n_sr));
+    sxb = (unsigned char*)(stg + STAGE_CAP);
     hs = (int*)((unsigned char*)stg + SM::stgbytes());
   } else {
     const size_t r1 = SM::region1(n_sr);
-    R = (T*)smem_raw;                                     // region 1: R, later the staged charges
-    stg = (V4*)smem_raw;
-    A_c = (T*)(smem_raw + r1);                            // [OCH][64] chunks of A and H (float pairs)
-    H_c = (T*)((unsigned char*)A_c + OCH * 64 * SM::ES);
+    R = (float*)smem_raw;                                     // region 1: R, later the staged charges
+    stg = (float4*)smem_raw;
+    A_c = (float*)(smem_raw + r1);                            // [OCH][64] chunks of A and H (float pairs)
+    H_c = (float*)((unsigned char*)A_c + OCH * 64 * SM::ES);
     hs = (int*)((unsigned char*)H_c + OCH * 64 * SM::ES);
   }
   int* epre = hs + HW * HW * HW + 1;                      // BE + 1
@@ -903,7 +898,7 @@ __global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_s
   int sx = tid % SW, sy = (tid / SW) % SW, sz = tid / (SW * SW);
 #pragma unroll 4
   for (int i = tid; i < SW * SW * SW; i += NT) {
-    const T val = Vc[wv[sx] + wv[SW + sy] + wv[2 * SW + sz]];   // class and vertex: < 27 n^3 < 2^31
+    const float val = Vc[wv[sx] + wv[SW + sy] + wv[2 * SW + sz]];   // class and vertex: < 27 n^3 < 2^31
     if constexpr (!TC) {
       // the hi + lo floats of the double-float contraction (an FP32 value has lo = 0)
       reinterpret_cast<float2*>(R)[i] = make_float2(val, 0.f);
@@ -1061,17 +1056,16 @@ __global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_s
       tc_fence_before();
     } else {
       const int gt = tid - SG;
-      const int mode = stage_halo<T>(gt, 2, n, HW, we, start, count, part, SM::cap(), stg, sxb, hs, flag, wsum);
-      singular_targets<T, GRAD>(gt, 2, mode, n, n_sr, h, E0x, E0y, E0z, HW, ntarget, epre, hs, rtab, we, stg, sxb,
-                                SM::cap(), start, count, part, phi_s, E_s, psi, gpsi);
+      const int mode = stage_halo(gt, 2, n, HW, we, start, count, part, STAGE_CAP, stg, sxb, hs, flag, wsum);
+      singular_targets<GRAD>(gt, 2, mode, n, n_sr, h, E0x, E0y, E0z, HW, ntarget, epre, hs, rtab, we, stg, sxb,
+                                STAGE_CAP, start, count, part, phi_s, E_s, psi, gpsi);
     }
     __syncthreads();   // every TMEM read done
     if (tid < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem));
   } else {
     // CUDA cores: 4 x 4 register tile, per-chunk partial sums added into a
-    // total, in double-float arithmetic on the FP32 pipes in both precisions
-    // (FP64 issues at a small fraction of the FP32 rate here): A and H are
-    // staged as hi + lo float pairs (the table's from FP64; an FP32 A has lo =
+    // total, in double-float arithmetic on the FP32 pipes (FP64 issues at a
+    // small fraction of the FP32 rate here): A and H are staged as hi + lo float pairs (the table's from FP64; an FP32 A has lo =
     // 0), each product keeps its exact leading part (fused two-product) and the
     // two cross terms, and the products are summed by two-sum into a hi + lo
     // accumulator; each chunk's sum goes into an FP64 total, which keeps the
@@ -1082,7 +1076,7 @@ __global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_s
     const int lst = tid & 63;
     const int lam = (lst % BX) + SW * (((lst / BX) % BY) + SW * (lst / (BX * BY)));
     constexpr int SPT = OCH * 64 / PT;   // staged entries per thread per chunk
-    T* gb = Gscr + (int64_t)blockIdx.x * (BE * 64);
+    float* gb = Gscr + (int64_t)blockIdx.x * (BE * 64);
     {
       // the table's hi + lo floats come precomputed (Hdf); R was split in (1)
       float2 hpf[SPT];                   // next chunk's table values, fetched during this chunk
@@ -1148,19 +1142,19 @@ __global__ void __launch_bounds__(TC ? PTC : PT, 2) k_pair_screen(int n, int n_s
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        V4 v;
-        v.x = (T)tot[i][0];
-        v.y = (T)tot[i][1];
-        v.z = (T)tot[i][2];
-        v.w = (T)tot[i][3];
-        *reinterpret_cast<V4*>(gb + (4 * eb + i) * 64 + 4 * mb) = v;
+        float4 v;
+        v.x = (float)tot[i][0];
+        v.y = (float)tot[i][1];
+        v.z = (float)tot[i][2];
+        v.w = (float)tot[i][3];
+        *reinterpret_cast<float4*>(gb + (4 * eb + i) * 64 + 4 * mb) = v;
       }
     }
     // Region 1 (R) was last read before the chunk loop's final barrier, so the
     // staging may overwrite it without another one.
-    const int mode = stage_halo<T>(tid, 0, n, HW, we, start, count, part, SM::cap(), stg, sxb, hs, flag, wsum);
-    singular_targets<T, GRAD>(tid, 0, mode, n, n_sr, h, E0x, E0y, E0z, HW, ntarget, epre, hs, rtab, we, stg, sxb,
-                              SM::cap(), start, count, part, phi_s, E_s, psi, gpsi);
+    const int mode = stage_halo(tid, 0, n, HW, we, start, count, part, STAGE_CAP, stg, sxb, hs, flag, wsum);
+    singular_targets<GRAD>(tid, 0, mode, n, n_sr, h, E0x, E0y, E0z, HW, ntarget, epre, hs, rtab, we, stg, sxb,
+                              STAGE_CAP, start, count, part, phi_s, E_s, psi, gpsi);
   }
 }
 
@@ -2323,13 +2317,6 @@ __global__ void k_energy(int64_t N, const double* __restrict__ Qs, const double*
   }
 }
 
-template <class A, class B>
-__global__ void k_cast(int64_t n, const A* __restrict__ in, B* __restrict__ out, double scale) {
-  int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (g >= n) return;
-  out[g] = (B)((double)in[g] * scale);
-}
-
 inline int gsz(int64_t n, int t = PT) { return (int)((n + t - 1) / t); }
 
 }  // namespace
@@ -2398,15 +2385,15 @@ size_t pair_screen_bytes(const fep3m_ctx* c) {
   return (size_t)pair_bricks(c) * BE * 64 * (c->precision == FEP3M_MIXED ? sizeof(float) : sizeof(double));
 }
 
-template <class T, bool GRAD, bool TC>
+template <bool GRAD, bool TC>
 static cudaError_t launch_pair_screen(fep3m_ctx* c, cudaStream_t s, bool half) {
-  const size_t smem = Pair3Smem<T, TC>::bytes(c->n_sr);
-  auto kern = k_pair_screen<T, GRAD, TC>;
+  const size_t smem = Pair3Smem<TC>::bytes(c->n_sr);
+  auto kern = k_pair_screen<GRAD, TC>;
   cudaError_t e = smem_limit((const void*)kern, smem);
   if (e != cudaSuccess) return e;
   FEP3M_CL kern<<<(unsigned)pair_bricks(c), TC ? PTC : PT, smem, s>>>(
-      c->n, c->n_sr, (T)c->h, c->start, c->count, (const typename vec4<T>::type*)c->part, (const T*)c->Vc,
-      (const uint4*)c->Hb, (const float2*)c->H0df, (const float2*)c->Hdf, (T*)c->Gscr, c->phi_s, c->E_s,
+      c->n, c->n_sr, (float)c->h, c->start, c->count, (const float4*)c->part, (const float*)c->Vc,
+      (const uint4*)c->Hb, (const float2*)c->H0df, (const float2*)c->Hdf, (float*)c->Gscr, c->phi_s, c->E_s,
       half ? c->psi_s : nullptr,
       half ? c->gpsi_s : nullptr, c->iflags + 2);
   return cudaGetLastError();
@@ -2443,10 +2430,10 @@ cudaError_t pair_screen(fep3m_ctx* c, int want_grad, cudaStream_t s, bool energy
   const bool half = energy_adjoint && want_grad;
   if (c->precision == FEP3M_MIXED) {
     if (c->Hb)
-      return want_grad ? launch_pair_screen<float, true, true>(c, s, half)
-                       : launch_pair_screen<float, false, true>(c, s, half);
-    return want_grad ? launch_pair_screen<float, true, false>(c, s, half)
-                     : launch_pair_screen<float, false, false>(c, s, half);
+      return want_grad ? launch_pair_screen<true, true>(c, s, half)
+                       : launch_pair_screen<false, true>(c, s, half);
+    return want_grad ? launch_pair_screen<true, false>(c, s, half)
+                     : launch_pair_screen<false, false>(c, s, half);
   }
   const size_t smem = screen64_smem(c->n_sr);
   cudaError_t e = smem_limit((const void*)k_screen64, smem);
