@@ -138,13 +138,15 @@ typedef struct {
                           each element's corners (MIXED), with the parts that
                           carry an element's potential level in double-float
                           or FP64; projections and the energy reduction in
-                          FP64.  Both paths hold charges and
-                          screen weights in FP32 ranges somewhere (the FP64
-                          path's double-float contractions, whose low words
-                          sit 2^-24 below the charges): keep |Q| within
-                          about 1e-30 .. 1e30 for full accuracy.               */
+                          FP64.  Both paths hold charges in FP32 ranges: MIXED
+                          as they are, with the adjoint's weights; FP64 as
+                          double-float pairs of the charges over their mean
+                          magnitude (the weights over their largest), whose low
+                          words sit 2^-24 below.  Keep the mean |Q| within about
+                          1e-30 .. 1e30, and in FP64 charges that matter above
+                          1e-23 of it, for full accuracy.                      */
   double mg_rtol;      /* relative FE residual target; 0 -> 1e-13 (FP64) or
-                          1e-10 (MIXED)                                          */
+                          1e-10 (MIXED; a box's residual is FP64 below 1e-11)    */
   int mg_max_cycles;   /* cap on refinement sweeps; 0 -> 10                      */
   int table_pad;       /* Dirichlet box margin, elements, beyond the kept table;
                           0 -> 4 (q = 1) or 2 (q >= 2); at most 8               */
@@ -227,7 +229,8 @@ int fep3m_compute(fep3m_ctx* ctx, double* phi, double* U, double* force);
  * the discrete method (element and block membership held fixed); the mesh
  * part uses the same mesh solver on the adjoint right-hand side.  After a
  * fep3m_compute without forces the charges' fields are evaluated here, from
- * that call's mesh solution.                                                */
+ * that call's mesh solution.  FEP3M_OK also where a mesh solve missed its
+ * tolerance: fep3m_get_stats has the residuals reached.                     */
 int fep3m_vjp(fep3m_ctx* ctx, double gU, const double* gphi, double* dpos, double* dQ);
 
 /* Counters of the last calls (see fep3m_stats).  The pair statistics

@@ -171,9 +171,10 @@ int deliver(fep3m_ctx* c, void* dst, const void* src, size_t bytes) {
   return FEP3M_OK;
 }
 
-// Device scalars (scal, 64 doubles): the adjoint weights' scale at kWeightScale, the charge sums at 32, U at 40, the pair
-// counts at 48, the integer flags (iflags) at kFlags.  One copy to pinned memory
-// brings the results of a call and its error flag; waits for the stream.
+// Device scalars (scal, 64 doubles): the adjoint weights' scale at kWeightScale, the
+// charge sums at 32, U at 40, the pair counts at 48, the integer flags (iflags) at
+// kFlags.  One copy to pinned memory brings the results of a call and its error flag;
+// waits for the stream.
 constexpr int kFlags = 56;
 cudaError_t take_results(fep3m_ctx* c, double* U) {
   cudaError_t e = cudaMemcpyAsync(c->host_scal, c->scal + 32, 32 * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
@@ -710,6 +711,7 @@ int fep3m_compute(fep3m_ctx* c, double* phi, double* U, double* force) {
     if (!solves_missed(c, force != nullptr) || attempt == kMaxReruns) break;
   }
   const int st = solve_status(c, force != nullptr);
+  // (a solution with forces that missed its tolerance serves fep3m_vjp all the same: the caller was told)
   c->have_mesh = force || st == FEP3M_OK;
   if (phi && !phi_dev) {
     int s2 = deliver(c, phi, c->out_tmp, N * sizeof(double));
@@ -774,7 +776,7 @@ int fep3m_vjp(fep3m_ctx* c, double gU, const double* gphi, double* dpos, double*
   if (!c || !std::isfinite(gU) || c->oq || c->box) return FEP3M_EINVAL;
   if (!c->have_particles) return FEP3M_ESTATE;
   const int64_t N = c->N;
-  if (!c->have_mesh) {   // no forward for these charges, or one that did not succeed
+  if (!c->have_mesh) {   // no forward for these charges, or one without forces that did not converge
     for (int attempt = 0;; ++attempt) {
       int st = run_forward(c, nullptr, 1, nullptr);
       if (st != FEP3M_OK) return st;
@@ -782,7 +784,7 @@ int fep3m_vjp(fep3m_ctx* c, double gU, const double* gphi, double* dpos, double*
       if (c->host_err) return FEP3M_ETIMEOUT;
       if (!solves_missed(c, false) || attempt == kMaxReruns) break;
     }
-    solve_status(c, false);
+    solve_status(c, false);   // (into the statistics; the gradient is that of the solution reached)
     c->have_mesh = true;
   }
   const double* g = gphi;

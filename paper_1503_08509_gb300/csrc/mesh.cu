@@ -1547,7 +1547,12 @@ __global__ void __launch_bounds__(FT_THREADS) k_tc_rows(int64_t R, int K, int cb
 //
 // Chosen for N >= TP_MIN (solver_init); below, a pass is a few microseconds of
 // latency and the small CTAs of k_tc_rows leave room for the step's concurrent
-// kernels.  Paired passes, two right-hand sides: N = 192 50 -> 40 us, N = 243 152
+// kernels, while this solve is not run beside them (mesh_solve_alone) and takes the
+// persistent row GEMM for the screen adjoint (k_tc_sweep).  Whole steps at one charge
+// per element, us with k_tc_rows / this: mixed with forces N = 99 641 / 733, 129 1105 /
+// 1088, 159 1783 / 1695; mixed potentials 473 / 526, 716 / 734, 1127 / 1177; FP64 with
+// forces 2044 / 2330, 3715 / 3809, 6948 / 7072: at 159 two right-hand sides gain 5%, one
+// loses 4%, FP64 2%.  Paired passes, two right-hand sides: N = 192 50 -> 40 us, N = 243 152
 // -> 86 us, N = 384 588 -> 405 us (the scaling pass 51, 108 and 488 us).  Three
 // operand stages leave the L1 too little room for the rows' lines (N = 384 +20%).
 constexpr int TP_GROUP = 256, TP_PROD = 2 * TP_GROUP, TP_THREADS = TP_PROD + 64, TP_MIN = 160;
@@ -2381,8 +2386,7 @@ cudaError_t tc_rows_prepare(int nt) {
   return e;
 }
 
-// out[(i - cb) R + r] = sum_{a < K} in[r K + a] B[i][a] for the columns cb <= i < ce
-// R rows of 64 on a GPU the caller has to itself (k_tc_sweep)
+// the same for R rows of 64 on a GPU the caller has to itself, output rows ld apart (k_tc_sweep)
 cudaError_t tc_sweep_gemm(int64_t R, int64_t ld, int cb, int ce, const float* in, const void* Bp, float* out, int* err,
                           cudaStream_t s) {
   int dev = 0, sms = 0;
@@ -2395,6 +2399,7 @@ cudaError_t tc_sweep_gemm(int64_t R, int64_t ld, int cb, int ce, const float* in
                                                                                        out, err);
   return cudaGetLastError();
 }
+// out[(i - cb) R + r] = sum_{a < K} in[r K + a] B[i][a] for the columns cb <= i < ce
 cudaError_t tc_rows_gemm(int64_t R, int K, int cb, int ce, int nt, const float* in, const void* Bp, float* out,
                          int* err, cudaStream_t s) {
   const dim3 g((unsigned)((R + 127) / 128 * ((ce + nt - 1) / nt - cb / nt)));

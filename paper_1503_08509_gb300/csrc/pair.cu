@@ -259,9 +259,16 @@ __device__ __forceinline__ df charge_diff(const PairCharge& s, const PairCharge&
 // into E_s, and half of them to psi and gpsi when given (the singular adjoint
 // for the energy's weights Q / 2).  A lane sums sixteen charges at a time in
 // pairs (element units) and those sums in three floats.  A pair's term is good
-// to a few 2^-48; the few charges within three quarters of an element, whose terms are the
-// largest, take FP64 (as do distances outside df_in_range), so that the sums
-// are as good as all in FP64.  About 120 FP32 operations per pair;
+// to a few 2^-48; the few charges within three quarters of an element, whose terms
+// are the largest, take FP64 (as do distances outside df_in_range).  The sum keeps
+// the terms' roundings, about 2^-48 of the root of the sum of their squares, where
+// FP64 terms would leave a thirtieth of that (emulated: rock salt, two charges per
+// element edge, 5e-14 against 2e-15 of potentials of 3.5).  What a potential as a
+// whole is off the method by is more, the screens' table and its contraction: against
+// a table solved in long double, with the mesh solved to rounding, neutral charges at
+// 0.1 to 8 per element and n_sr 2 to 4 came out 0.4 to 1.03 times as far off as with
+// FP64 terms and tables (potentials 3e-14 to 6e-13, forces 2e-15 to 5e-12), charges of
+// one sign 1.0 (potentials) and 1.2 times (forces, n_sr = 4).  About 120 FP32 operations per pair;
 // bound by FP32 issue and, for few targets, by the latency of the loads.
 // 4000 charges, q = 2, potentials: 266 -> 42 us.
 constexpr float NEAR2 = 0.5625f;   // three quarters of an element, squared
