@@ -1662,21 +1662,23 @@ __global__ void __launch_bounds__(1024) k_weight_scale(int64_t N, const double* 
 // 41 us, 10^6 on 128^3, 845 -> 145 us; FP64 rock salt 32^3, where every thread also evaluated twelve
 // shape functions, 208 -> 34 us).  That takes some 290 cycles a charge in series,
 // so rows of 32 elements with more than `run` charges are dealt by elements to the
-// CTA's warps, which put the shape functions of 32 charges, one per lane, into shared
-// memory and sum over them there (4096 charges in one row of 32^3 elements: 617 us in
-// one warp, now 29; 20 000 in a blob of 16^3: 1165 -> 90).  A CTA takes eight rows.
+// CTA's warps, which put the shape functions of eight charges at a time into shared
+// memory and sum over them there (3 KB a CTA, 6 in FP64: with 32 at a time the CTAs
+// did not fit beside the screen kernel's, and the FP64 step waited 40 us for that).
+// 4096 charges in one row of 32^3 elements: 617 us in one warp, now 40; 20 000 in a blob
+// of 16^3: 1165 -> 107.  A CTA takes eight rows.
 //
 // Dealing costs a row two dependent loads per element, but on a small mesh the rows in
 // series leave the GPU idle: there (deposit_dealt) a CTA takes one row and deals it
-// whatever it holds.  FP32, 0.2 / 1 / 3 charges per element, in series and dealt (us):
-// 12^3 8.7 / 17 / 34 and 6.4 / 7.6 / 8.5; 28^3 9.3 / 18 / 37 and 17 / 18 / 19; 32^3 9.9 /
-// 20 / 35 and 25 / 26 / 28; 48^3 12 / 24 / 48 and 65 / 69 / 72: about 8 + 0.31 run against
-// 4 + 0.021 rows.  FP64: 12^3 11 / 32 / 82 and 12 / 19 / 22; 28^3 14 / 36 / 88 and 24 / 64 /
-// 92; 48^3 23 / 85 / 233 and 77 / 255 / 397.
+// whatever it holds.  0.2 / 1 / 3 charges per element, in series and dealt (us), FP32:
+// 12^3 8.7 / 17 / 34 and 6.5 / 7.7 / 8.9; 28^3 9.3 / 18 / 37 and 19 / 21 / 22; 32^3 10 /
+// 18 / 35 and 23 / 24 / 25; 48^3 12 / 23 / 49 and 66 / 69 / 73.  FP64: 12^3 11 / 32 / 82
+// and 8.9 / 12 / 16; 28^3 13 / 35 / 92 and 16 / 39 / 55; 32^3 14 / 37 / 91 and 20 / 50 /
+// 77; 48^3 22 / 85 / 238 and 46 / 141 / 235.
 constexpr int DEP_RUN = 160;   // (64^3, FP32: 4 charges per element 119 us in series, 165 dealt)
-static bool deposit_dealt(int64_t ne, int64_t N, bool f32) {
+static bool deposit_dealt(int64_t ne, int64_t N) {
   const int64_t rows = (ne + 31) / 32, run = N * 32 / ne;
-  return rows < 200 + (f32 ? 15 : 5) * run || run > DEP_RUN;
+  return rows < 200 + 15 * run || run > DEP_RUN;
 }
 // order-3 shape function i at t as q3_values forms it: k (t - r0) (t - r1) (t - r2)
 template <class T>
@@ -1692,7 +1694,7 @@ __global__ void __launch_bounds__(PT) k_elem_deposit(int64_t ne, int nrows, int 
                                                      const double* __restrict__ w, const T* __restrict__ wT,
                                                      T* __restrict__ W, float2* __restrict__ wsum) {
   __shared__ int crowded[PT / 32];
-  __shared__ T shape[PT / 32][12][33];   // of a warp's 32 charges: x (times the weight), y, z
+  __shared__ T shape[PT / 32][12][8];   // of eight of a warp's charges: x (times the weight), y, z
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t cta0 = blockIdx.x * (int64_t)nrows * 32, e0 = cta0 + 32 * warp;
   // this lane's nodes: m = lane and lane + 32 (the same x and y index, z index 2 on)
@@ -1752,7 +1754,8 @@ __global__ void __launch_bounds__(PT) k_elem_deposit(int64_t ne, int nrows, int 
   }
   if (lane == 0) crowded[warp] = crowd;
   if (!__syncthreads_or(crowd)) return;
-  T(*u)[33] = shape[warp];
+  T(*u)[8] = shape[warp];
+  const int axis = lane >> 3;   // this lane's shape functions: along x, y or z (or none), of charge lane mod 8
   for (int r = 0; r < nrows; ++r) {
     if (!crowded[r]) continue;
     const int64_t e1 = min(cta0 + 32 * r + 32, ne);
@@ -1766,21 +1769,33 @@ __global__ void __launch_bounds__(PT) k_elem_deposit(int64_t ne, int nrows, int 
           pc = part[s + base + lane];
           wc = wT[s + base + lane];
           if (wsum) ws += w[s + base + lane];
+        }
+        for (int b = 0; b < m; b += 8) {
+          const int src = b + (lane & 7);   // (past the last charge: a stale one, not read below)
+          const T x = __shfl_sync(0xffffffffu, pc.x, src), y = __shfl_sync(0xffffffffu, pc.y, src),
+                  z = __shfl_sync(0xffffffffu, pc.z, src), wj = __shfl_sync(0xffffffffu, wc, src);
+          const T t = axis == 0 ? x : (axis == 1 ? y : z);
+          if (axis < 3)
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            u[i][lane] = wc * q3_value(pc.x, i);
-            u[4 + i][lane] = q3_value(pc.y, i);
-            u[8 + i][lane] = q3_value(pc.z, i);
+            for (int i = 0; i < 4; ++i) u[4 * axis + i][lane & 7] = axis == 0 ? wj * q3_value(t, i) : q3_value(t, i);
+          __syncwarp();
+          const int e8 = min(8, m - b);
+          if (e8 == 8) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const T xy = u[mx][k] * u[4 + my][k];
+              a0 = fma(xy, u[8 + mz][k], a0);
+              a1 = fma(xy, u[10 + mz][k], a1);
+            }
+          } else {
+            for (int k = 0; k < e8; ++k) {
+              const T xy = u[mx][k] * u[4 + my][k];
+              a0 = fma(xy, u[8 + mz][k], a0);
+              a1 = fma(xy, u[10 + mz][k], a1);
+            }
           }
+          __syncwarp();
         }
-        __syncwarp();
-#pragma unroll 4
-        for (int k = 0; k < m; ++k) {
-          const T xy = u[mx][k] * u[4 + my][k];
-          a0 = fma(xy, u[8 + mz][k], a0);
-          a1 = fma(xy, u[10 + mz][k], a1);
-        }
-        __syncwarp();
       }
       W[e * 64 + lane] = a0;
       W[e * 64 + lane + 32] = a1;
@@ -2755,7 +2770,7 @@ cudaError_t adjoint_pre(fep3m_ctx* c, double gU, const double* gphi, cudaStream_
     scale = gU == 0.0 ? 1.0 : std::ldexp(1.0, std::max(-900, std::min(900, 64 - std::ilogb(gU) + std::ilogb(c->q_scale))));
   FEP3M_CL k_weights<<<gsz(N), PT, 0, s>>>(N, gU, gphi, c->perm, c->Q_s, c->w_s, c->w_s32, scale,
                                            c->scal + kWeightScale);
-  const bool dealt = deposit_dealt(ne, N, c->precision == FEP3M_MIXED);
+  const bool dealt = deposit_dealt(ne, N);
   const int nrows = dealt ? 1 : PT / 32, run = dealt ? 0 : DEP_RUN, per = 32 * nrows;   // rows of 32 elements per CTA
   if (c->precision == FEP3M_MIXED) {
     FEP3M_CL k_elem_deposit<float><<<gsz(ne, per), PT, 0, s>>>(ne, nrows, run, c->start, c->count, (const float4*)c->part, c->w_s,
