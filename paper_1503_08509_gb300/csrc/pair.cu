@@ -1471,7 +1471,7 @@ __global__ void __launch_bounds__(PT) k_pair_eval(int n, int Nm, float inv_h, co
 // threads per target take the four z layers of nodes: each evaluates one shape
 // function and derivative per axis (shared by shuffles) and contracts its
 // layer along x, then y: about 400 FP64 operations per target where the terms
-// one by one took 3000 (rock salt 32^3 with forces: 98 -> 74 us; an FP64
+// one by one took 3000 (rock salt 32^3 with forces: 98 -> 79 us; an FP64
 // operation costs as much as 64 FP32 ones here).
 __device__ __forceinline__ void q3_one(double t, int i, double& v, double& d) {
   const double k = i == 0 ? -4.5 : (i == 1 ? 13.5 : (i == 2 ? -13.5 : 4.5));
@@ -1971,8 +1971,8 @@ __device__ __forceinline__ double acc_value(tf a) { return df_value(a); }
 // CTA takes 32 consecutive elements, one per lane; a warp forms the eight
 // parities of two offsets i at a time for them and writes their sixteen
 // mirrored values of D as pairs (rows of 32 consecutive elements), times the
-// weights' scale ws[0] (k_weight_scale).  HP: the table by parity, [s][i][j].  Bound by FP32 issue; rock salt 32^3: 778 ->
-// 143 us against the full product in pairs with D rounded to FP64.
+// weights' scale ws[0] (k_weight_scale).  HP: the table by parity, [s][i][j].
+// Bound by FP32 issue; rock salt 32^3: 778 -> 146 us against the full product in pairs with D rounded to FP64.
 constexpr int AE = 32;
 static size_t adj64_smem(int n_sr) {
   const int kh = n_sr + 1;
@@ -2079,7 +2079,8 @@ __global__ void __launch_bounds__(PT, 2) k_adj64(int64_t ne, int n_sr, int z0, i
 // a term, of 36 instructions).  FP64 path: D is the whole contraction, as pairs,
 // summed in three floats: the up to (2 n_sr)^3 terms of a class are of one sign
 // where the weights are, and the low word of a pair's sum would round each of
-// them at 2^-48 of the running sum.  Bound by instruction issue, at 2/3 of its rate.  10^6
+// them at 2^-48 of the running sum (rock salt 32^3, 28 us with two floats, 35 with
+// three).  Bound by instruction issue, at 2/3 of its rate.  10^6
 // charges on 128^3: 3484 us with one warp per 32 vertices and row of offsets and 27
 // class sums in shared memory, 2301 with a row ahead in registers and AVZ = 8, 1458
 // now; 262 144 on 64^3: 439, 285 and 195 us.
