@@ -1635,7 +1635,8 @@ __global__ void k_weights(int64_t N, double gU, const double* __restrict__ gphi,
 // weights that only the device knows (fep3m_vjp's gphi).  The screen adjoint's float pairs
 // are of the scaled weights (the field they give is within 2^12 of them, n_sr <= 4), so that
 // their low words stay normal FP32 numbers whatever the weights' unit; non-finite weights
-// stay as they are.  One CTA: the weights are read once more, beside the mesh solve.
+// stay as they are.  One CTA: the weights are read once more, beside the mesh solve (76 800
+// charges 8 us, 10^6 49 us).
 __global__ void __launch_bounds__(1024) k_weight_scale(int64_t N, const double* __restrict__ w,
                                                        double* __restrict__ ws) {
   __shared__ int top[32];
